@@ -108,9 +108,7 @@ int build_tiles(ising_batch* b)
         b->lane_tile0[k] = (int)tiles.size();
         for (int r : order) {
             if (k >= b->lanes || lane_of[r] != k) continue;
-            const Geom& g = b->geom[r];
-            const uint32_t items = (uint32_t)((g.L + 3) / 4) * (uint32_t)g.W;
-            for (uint32_t f = 0; f < items; f += (uint32_t)b->threads) tiles.push_back({r, (int)f});
+            add_tiles(tiles, r, b->geom[r], b->threads);
         }
         b->lane_ntiles[k] = (int)tiles.size() - b->lane_tile0[k];
     }
@@ -143,9 +141,9 @@ template <int ROUNDS>
 void launch_batch_pair_r(bool every1, dim3 grid, dim3 block, cudaStream_t st, const BatchReplica* reps,
                          const BatchTile* tiles, const uint32_t* chunk_base, uint32_t s)
 {
-    launch_pdl(batch_half_sweep_kernel<0, ROUNDS, 1>, grid, block, st, reps, tiles, chunk_base, s, 1u);
-    if (every1) launch_pdl(batch_half_sweep_kernel<1, ROUNDS, 2>, grid, block, st, reps, tiles, chunk_base, s, 1u);
-    else launch_pdl(batch_half_sweep_kernel<1, ROUNDS, 0>, grid, block, st, reps, tiles, chunk_base, s, 1u);
+    launch_pdl(batch_half_sweep_kernel<0, ROUNDS, 1>, grid, block, st, reps, tiles, chunk_base, s);
+    if (every1) launch_pdl(batch_half_sweep_kernel<1, ROUNDS, 2>, grid, block, st, reps, tiles, chunk_base, s);
+    else launch_pdl(batch_half_sweep_kernel<1, ROUNDS, 0>, grid, block, st, reps, tiles, chunk_base, s);
 }
 
 void launch_batch_pair(int rounds, bool every1, dim3 grid, dim3 block, cudaStream_t st, const BatchReplica* reps,
@@ -257,7 +255,6 @@ extern "C" int ising_batch_create(int32_t n, const int32_t* L, const double* bet
         R.thr0 = a.thr0; R.thr1 = a.thr1; R.all0 = a.all0; R.all1 = a.all1;
         R.every = 1;
         R.rounds = 10;
-        R.items = (uint32_t)((g.L + 3) / 4) * (uint32_t)g.W;
         b->h_reps.push_back(R);
     }
     if (e != cudaSuccess) { free_batch(b); return cuda_fail(e, "batch init"); }

@@ -397,7 +397,7 @@ cl_mask_draw_kernel(Geom g, SweepArgs a, const uint64_t* t_base, uint64_t t0, in
     const int w = item - grp * g.W;
     const uint64_t t = (t_base ? *t_base : 0) + t0 + (uint64_t)(jc >> 1) + 1;
     uint64_t p[4];
-    item_masks_thread<ROUNDS>(g, item, t, jc & 1, a.rk, a.thr0, a.thr1, a.one, p);
+    item_masks_thread<ROUNDS>(g, item, t, jc & 1, a, p);
     // a threshold of 2^32 accepts always: its bits set here, not in the update
     const uint64_t always = (((uint64_t)a.all1 << 32 | a.all1) & kSpinBits) |
                             ((((uint64_t)a.all0 << 32 | a.all0) & kSpinBits) << 1);

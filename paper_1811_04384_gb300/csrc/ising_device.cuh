@@ -17,10 +17,6 @@
 #include <cstdint>
 #include "philox.cuh"
 
-#ifndef ISING_INSERTS_ON_ALU
-#define ISING_INSERTS_ON_ALU 0
-#endif
-
 namespace ising {
 
 constexpr int kFields = 21;
@@ -36,11 +32,11 @@ struct Geom {
 
 // Per-launch constants of one half-sweep.
 struct SweepArgs {
-    const uint64_t* t_base;    // device: sweep counter before this chunk
-    uint32_t t_off;            // this half-sweep belongs to sweep *t_base + t_off
+    const uint64_t* t_base;    // device: sweep counter before this chunk, or null ...
+    uint64_t t0;               // ... and then the same on the host
+    uint32_t t_off;            // this half-sweep belongs to sweep (t_base ? *t_base : t0) + t_off
     uint32_t thr0, thr1;       // integer thresholds clamped to 2^32 - 1 ...
     uint32_t all0, all1;       // ... and ~0u where the threshold is 2^32
-    uint32_t one;              // the value 1, as a launch operand (see accept_insert)
     uint32_t rounds;           // Philox rounds of the sweep draws: 10 (default) or 7 (opt-in)
     PhiloxKeys rk;             // round keys of the key (lo32(seed), hi32(seed))
     unsigned long long* counts;  // E/M count slots of this record (RECORD only)
@@ -57,12 +53,27 @@ __device__ __forceinline__ unsigned long long* record_counts(const SweepArgs& a)
 // Programmatic dependent launch: a half-sweep launched with programmatic
 // stream serialization lets the next half-sweep be launched and its blocks be
 // placed as soon as every block of this one has started (launch_dependents),
-// and waits, before its first read, until the previous grid has completed
-// and its writes are visible (wait).  Both are no-ops in a plain launch.
+// and waits, before its first read of device memory, until the previous grid
+// has completed and its writes are visible (wait).  Both are no-ops in a
+// plain launch.  What a block does before the wait (its draws, which need
+// launch operands only) overlaps the end of the previous grid.
+__device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_enter()
 {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    pdl_launch();
+    pdl_wait();
+}
+
+// The sweep number of a half-sweep; where the counter is on the device, after
+// the grids that advance it.
+__device__ __forceinline__ uint64_t sweep_number(const SweepArgs& a)
+{
+    if (a.t_base) {
+        pdl_wait();
+        return *a.t_base + a.t_off;
+    }
+    return a.t0 + a.t_off;
 }
 
 // ---- Checked build (compiled with -DISING_CHECKED) -------------------------
@@ -132,6 +143,31 @@ __device__ __forceinline__ void half_st(uint32_t* p, uint64_t idx, uint32_t v, u
     p[idx] = v;
 }
 
+// The word, or the 32-bit half of one, at byte offset `o` of an array of n words.
+__device__ __forceinline__ uint64_t byte_ld64(const uint64_t* p, uint32_t o, uint64_t n, uint32_t line)
+{
+#ifdef ISING_CHECKED
+    if (!check_index(o / 8u, n, line)) return 0;
+#endif
+    return *reinterpret_cast<const uint64_t*>(reinterpret_cast<const char*>(p) + o);
+}
+
+__device__ __forceinline__ uint32_t byte_ld32(const uint64_t* p, uint32_t o, uint64_t n, uint32_t line)
+{
+#ifdef ISING_CHECKED
+    if (!check_index(o / 4u, 2 * n, line)) return 0;
+#endif
+    return *reinterpret_cast<const uint32_t*>(reinterpret_cast<const char*>(p) + o);
+}
+
+__device__ __forceinline__ void byte_st64(uint64_t* p, uint32_t o, uint64_t v, uint64_t n, uint32_t line)
+{
+#ifdef ISING_CHECKED
+    if (!check_index(o / 8u, n, line)) return;
+#endif
+    *reinterpret_cast<uint64_t*>(reinterpret_cast<char*>(p) + o) = v;
+}
+
 __device__ __forceinline__ uint64_t lattice_words(const Geom& g) { return (uint64_t)g.L * (uint64_t)g.P; }
 
 __device__ __forceinline__ int wrap_row(int i, int L)
@@ -169,161 +205,265 @@ __device__ __forceinline__ void block_add_counts(unsigned long long* target, uin
     }
 }
 
-// Accept bits of one field for one row.  A1 collects r < thr1 at bit K2 (the
-// spin bit of the field within its 32-bit half), A0 collects r < thr0 at bit
-// K2 + 1.  The inserts are predicated PTX, so a compare result never becomes
-// a 0/1 value and the bit is an immediate: the r < thr1 insert is an OR on the
-// ALU, the r < thr0 insert a multiply-add (K * one + A0) on the FMA pipe, which
-// balances the two pipes against the Philox XORs (ALU) and multiplies (FMA).
-template <int K2>
-__device__ __forceinline__ void accept_insert(uint32_t& A1, uint32_t& A0, uint32_t r, uint32_t thr0,
-                                              uint32_t thr1, uint32_t one)
+// d = LUT(a, b, c) bit by bit, LUT over kLutA, kLutB, kLutC: one instruction.
+constexpr int kLutA = 0xF0, kLutB = 0xCC, kLutC = 0xAA;
+template <int LUT>
+__device__ __forceinline__ uint32_t lop3(uint32_t a, uint32_t b, uint32_t c)
 {
-    asm("{\n\t.reg .pred p;\n\tsetp.lt.u32 p, %1, %2;\n\t@p or.b32 %0, %0, %3;\n\t}"
-        : "+r"(A1) : "r"(r), "r"(thr1), "n"(1u << K2));
-#if ISING_INSERTS_ON_ALU
-    asm("{\n\t.reg .pred p;\n\tsetp.lt.u32 p, %1, %2;\n\t@p or.b32 %0, %0, %3;\n\t}"
-        : "+r"(A0) : "r"(r), "r"(thr0), "n"(2u << K2));
-#else
-    asm("{\n\t.reg .pred p;\n\tsetp.lt.u32 p, %1, %2;\n\t@p mad.lo.u32 %0, %4, %3, %0;\n\t}"
-        : "+r"(A0) : "r"(r), "r"(thr0), "n"(2u << K2), "r"(one));
-#endif
+    uint32_t d;
+    asm("lop3.b32 %0, %1, %2, %3, %4;" : "=r"(d) : "r"(a), "r"(b), "r"(c), "n"(LUT & 0xFF));
+    return d;
 }
 
-// Accumulators of one row: [0] r < thr1 bits of fields 0..10, [1] r < thr0
-// (shifted up one bit) of fields 0..10, [2], [3] the same for fields 11..20.
-struct AcceptBits {
-    uint32_t a[4][4];   // [row][word]
+// The Metropolis step of Sec. 2 on one 32-bit half of a word: s the own
+// spins, u, d, h0, h1 the four neighbours', p the sites with r < thr1, q
+// those with r < thr0, live the spin bits.  With x_n = s ^ n (anti-aligned),
+// A = x_u | x_d, B = x_u & x_d, C = x_h0 | x_h1, D = x_h0 & x_h1 (Eq. 3
+// summed bitwise), two or more anti-aligned neighbours (dE <= 0, Table 1) are
+// B | D | A & C and one or more A | C.  thr0 <= thr1, so q implies p, and
+//   accept = B | D | A & C | (A | C) & p | q = (B | D | q) | majority(A, C, p):
+// eight three-input operations.
+__device__ __forceinline__ uint32_t flip_half(uint32_t s, uint32_t u, uint32_t d, uint32_t h0, uint32_t h1,
+                                              uint32_t p, uint32_t q, uint32_t live)
+{
+    constexpr int kOr = (kLutA ^ kLutB) | (kLutA ^ kLutC), kAnd = (kLutA ^ kLutB) & (kLutA ^ kLutC);
+    const uint32_t A = lop3<kOr>(s, u, d), B = lop3<kAnd>(s, u, d);
+    const uint32_t C = lop3<kOr>(s, h0, h1), D = lop3<kAnd>(s, h0, h1);
+    const uint32_t e = lop3<(kLutA | kLutB | kLutC)>(B, D, q);
+    const uint32_t m = lop3<(kLutA & kLutB) | (kLutA & kLutC) | (kLutB & kLutC)>(A, C, p);
+    return s ^ lop3<(kLutA | kLutB) & kLutC>(e, m, live);
+}
+
+// Anti-aligned bonds of the updated half word s with its four neighbours, and
+// its up spins plus those of h0, added to anti / up.  Two spin-bit words share
+// one population count (x + 2 y: the fields are three bits wide).
+__device__ __forceinline__ void count_half(uint32_t s, uint32_t u, uint32_t d, uint32_t h0, uint32_t h1,
+                                           uint32_t live, uint32_t& anti, uint32_t& up)
+{
+    const uint32_t xh1 = lop3<(kLutA ^ kLutB) & kLutC>(s, h1, live);
+    anti += __popc((s ^ u) + 2u * (s ^ d)) + __popc((s ^ h0) + 2u * xh1);
+    up += __popc(s + 2u * h0);
+}
+
+// Accept masks of an item (4 rows x 1 word of one colour): per row and 32-bit
+// half, r < thr1 of field k at bit 3k of the word and r < thr0 at bit 3k + 1.
+// One accumulator holds both (their other bits fall on no spin bit), so a row
+// needs two registers.
+struct ItemMasks {
+    uint32_t m[4][2];   // [row][half]
+};
+
+// The inserts are predicated PTX, so a compare result never becomes a 0/1
+// value and the bit is an immediate.  On GB300 the Philox products and the
+// ALU share issue: a product takes four cycles of the multiply pipe and two
+// of the ALU's, any ALU operation two.  The products, XORs and compares
+// already fill those, so the inserts have to go to the multiply pipe: as an
+// OR into bits that are known to be zero they do (the compiler turns it into
+// an add there; as an XOR they stayed on the ALU, 1,243 against 1,394
+// spin-updates/ns at L = 16384).
+template <int B>
+__device__ __forceinline__ void accept_insert(uint32_t& acc, uint32_t r, uint32_t thr0, uint32_t thr1)
+{
+    asm("{\n\t.reg .pred p;\n\tsetp.lt.u32 p, %1, %2;\n\t@p or.b32 %0, %0, %3;\n\t}"
+        : "+r"(acc) : "r"(r), "r"(thr1), "n"(1u << B));
+    asm("{\n\t.reg .pred p;\n\tsetp.lt.u32 p, %1, %2;\n\t@p or.b32 %0, %0, %3;\n\t}"
+        : "+r"(acc) : "r"(r), "r"(thr0), "n"(2u << B));
+}
+
+// The first Philox products of an item's fields: computed (m = m0 + k), or
+// read from a block's shared table (first_products).
+struct FirstDirect {
+    uint32_t key, m0;
+    __device__ __forceinline__ void get(int k, uint32_t& hi, uint32_t& lo) const
+    {
+        mul_hilo(kPhiloxM0, key ^ (m0 + (uint32_t)k), hi, lo);
+    }
+};
+constexpr int kStripWords = 32;   // most words of a strip
+struct FirstTable {
+    const uint2* col;             // the item's word in the table
+    __device__ __forceinline__ void get(int k, uint32_t& hi, uint32_t& lo) const
+    {
+        const uint2 e = col[k * kStripWords];
+        hi = e.x;
+        lo = e.y;
+    }
 };
 
 // Fields k .. 20 of one Philox row group (compile-time k: immediate bit masks).
-template <int k, int ROUNDS>
+template <int k, int ROUNDS, typename First>
 struct FieldLoop {
-    __device__ __forceinline__ static void run(const PhiloxRowKey& pk, const PhiloxKeys& rk, uint32_t m0,
-                                               AcceptBits& acc, uint32_t thr0, uint32_t thr1, uint32_t one)
+    __device__ __forceinline__ static void run(const First& first, const PhiloxRowKey& pk, const PhiloxKeys& rk,
+                                               ItemMasks& acc, uint32_t thr0, uint32_t thr1)
     {
-        uint32_t rnd[4];
-        philox_row<ROUNDS>(pk, rk, m0 + (uint32_t)k, rnd);
-        constexpr int half = k <= 10 ? 0 : 2;
-        constexpr int K2 = k <= 10 ? 3 * k : 3 * k - 32;
+        uint32_t hi, lo, rnd[4];
+        first.get(k, hi, lo);
+        philox_row_tail<ROUNDS>(pk, rk, hi, lo, rnd);
+        constexpr int half = k <= 10 ? 0 : 1;
+        constexpr int B = k <= 10 ? 3 * k : 3 * k - 32;
 #pragma unroll
-        for (int e = 0; e < 4; ++e)
-            accept_insert<K2>(acc.a[e][half], acc.a[e][half + 1], rnd[e], thr0, thr1, one);
-        FieldLoop<k + 1, ROUNDS>::run(pk, rk, m0, acc, thr0, thr1, one);
+        for (int e = 0; e < 4; ++e) accept_insert<B>(acc.m[e][half], rnd[e], thr0, thr1);
+        FieldLoop<k + 1, ROUNDS, First>::run(first, pk, rk, acc, thr0, thr1);
     }
 };
-template <int ROUNDS>
-struct FieldLoop<kFields, ROUNDS> {
-    __device__ __forceinline__ static void run(const PhiloxRowKey&, const PhiloxKeys&, uint32_t, AcceptBits&,
-                                               uint32_t, uint32_t, uint32_t)
+template <int ROUNDS, typename First>
+struct FieldLoop<kFields, ROUNDS, First> {
+    __device__ __forceinline__ static void run(const First&, const PhiloxRowKey&, const PhiloxKeys&, ItemMasks&,
+                                               uint32_t, uint32_t)
     {
     }
 };
 
-// The work of one thread: rows row0 .. row0+3 (those below L) of word column
-// w of colour C, at sweep t (Sec. 2 steps 1-3 for every site of the colour at
-// once; same-colour sites are never neighbours).  One Philox call covers the
-// four rows of one field.
-//
-// Per row, with s the own word and u, d, h0, h1 the four aligned neighbour
-// words, x_n = s ^ n has the spin bit of field k set iff neighbour n is
-// anti-aligned (Eq. 3 summed bitwise instead of with carries):
-//   any = x1|x2|x3|x4                     (a >= 1)
-//   ge2 = x1&x2 | x3&x4 | (x1^x2)&(x3^x4) (a >= 2: dE <= 0, Table 1)
-//   accept = ge2 | any & (r < thr1) | ~any & (r < thr0)
-// GLOBAL selects read-only-cache loads (lattice in global memory) or plain
-// loads (lattice in shared memory).  Offsets are 32-bit (L * pitch < 2^32).
-// UPDATE = false skips the flip (measurement only).  RECORD adds the
-// anti-aligned bond count of the (updated) colour-1 words and the up-spin
-// count of both colours to anti / up: E = 2 anti - 2 L^2, M = 2 up - L^2.
-template <int C, bool UPDATE, bool RECORD, bool GLOBAL = true, int ROUNDS = 10>
-__device__ __forceinline__ void sweep_rows(uint64_t* __restrict__ own, const uint64_t* __restrict__ other,
-                                           const Geom& g, int row0, int w, uint64_t t, const PhiloxKeys& rk,
-                                           uint32_t thr0, uint32_t thr1, uint32_t all0w, uint32_t all1w,
-                                           uint32_t one, uint32_t& anti, uint32_t& up)
+// The masks of row group grp at sweep t, colour `colour` (Sec. 2 steps 2-3;
+// one Philox call covers the four rows of one field).
+template <int ROUNDS, typename First>
+__device__ __forceinline__ void draw_item(const First& first, uint32_t grp, uint64_t t, int colour,
+                                          const PhiloxKeys& rk, uint32_t thr0, uint32_t thr1, uint32_t all0w,
+                                          uint32_t all1w, ItemMasks& acc)
 {
-    constexpr int ROWS = 4;
-    const int nrows = min(ROWS, g.L - row0);
-    const uint64_t live = live_mask(g, w);
-    const uint32_t P = (uint32_t)g.P;
-    const uint32_t base = (uint32_t)row0 * P + (uint32_t)w;
-    const uint32_t up_off = row0 == 0 ? (uint32_t)(g.L - 1) * P + (uint32_t)w : base - P;
-    const uint32_t dn_off = row0 + nrows >= g.L ? (uint32_t)w : base + (uint32_t)nrows * P;
-    const uint32_t wl = (uint32_t)((w > 0) ? w - 1 : g.W - 1);
-    const uint32_t wr = (uint32_t)((w < g.W - 1) ? w + 1 : 0);
-
-    const uint64_t n = lattice_words(g);
-    // All loads first: their latency overlaps the Philox work below.
-    // oc[r] = other-colour row row0 - 1 + r (periodic), column w.
-    uint64_t oc[ROWS + 2], sw[ROWS], side[ROWS];
-    oc[0] = word_ld<GLOBAL>(other, up_off, n, __LINE__);
 #pragma unroll
-    for (int r = 0; r < ROWS; ++r) {
-        if (r < nrows) {
-            const uint32_t o = base + (uint32_t)r * P;
-            oc[r + 1] = word_ld<GLOBAL>(other, o, n, __LINE__);
-            sw[r] = word_ld<false>(own, o, n, __LINE__);
-            const uint32_t os = o - (uint32_t)w + ((((r + C) & 1) == 0) ? wl : wr);   // row0 is a multiple of 4
-            side[r] = word_ld<GLOBAL>(other, os, n, __LINE__);
-        } else {
-            oc[r + 1] = 0;
-            sw[r] = 0;
-            side[r] = 0;
+    for (int e = 0; e < 4; ++e) acc.m[e][0] = acc.m[e][1] = 0;
+    const uint32_t tl = (uint32_t)t;
+    const uint32_t th = ((uint32_t)(t >> 32) << 1) | (uint32_t)colour;
+    const PhiloxRowKey pk = philox_row_key(grp, tl, th, rk);
+    FieldLoop<0, ROUNDS, First>::run(first, pk, rk, acc, thr0, thr1);
+    if (all1w | all0w) {     // a threshold of 2^32 accepts always
+        const uint64_t a = ((((uint64_t)all1w << 32 | all1w) & kSpinBits)) |
+                           ((((uint64_t)all0w << 32 | all0w) & kSpinBits) << 1);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            acc.m[e][0] |= (uint32_t)a;
+            acc.m[e][1] |= (uint32_t)(a >> 32);
         }
     }
-    {
-        const uint64_t dn = word_ld<GLOBAL>(other, dn_off, n, __LINE__);   // row below the last present row
-#pragma unroll
-        for (int r = 0; r < ROWS; ++r)
-            if (r + 1 == nrows) oc[r + 2] = dn;
-        if (nrows == ROWS) oc[ROWS + 1] = dn;
-    }
+}
 
-    AcceptBits acc;
+// Update (and/or record) rows 4 grp .. 4 grp + 3 (those below L) of word
+// column w of colour C with the masks `acc` (same-colour sites are never
+// neighbours).  Byte offsets are 32-bit (a colour array has less than 2^28
+// bytes).  Only rows 0 and 1 of a group can exist alone (L even): the
+// missing rows then read rows 0 and 1 of the lattice and are not stored.
+// The side word gives one field only, so only its half is read: field 20
+// (or the row's last field across the wrap) of the word to the left, shifted
+// down to field 0, or field 0 of the word to the right, moved up by a
+// multiply.  UPDATE = false skips the flip (measurement only).  RECORD adds
+// the anti-aligned bond count of the (updated) colour-1 words and the up-spin
+// count of both colours to anti / up: E = 2 anti - 2 L^2, M = 2 up - L^2.
+template <int C, bool UPDATE, bool RECORD>
+__device__ __forceinline__ void apply_item(uint64_t* own, const uint64_t* other, const Geom& g, uint32_t grp,
+                                           uint32_t w, const ItemMasks& acc, uint32_t& anti, uint32_t& up)
+{
+    const uint32_t P8 = (uint32_t)g.P * 8u, LP8 = (uint32_t)g.L * P8, row0 = grp * 4u, w8 = w * 8u;
+    const bool two = row0 + 2u >= (uint32_t)g.L;                       // rows 0 and 1 only
+    // byte offsets of rows row0 - 1 .. row0 + 4 (periodic), word w
+    const uint32_t o1 = row0 * P8 + w8, o2 = o1 + P8, o3 = o2 + P8 - (two ? LP8 : 0u), o4 = o3 + P8;
+    const uint32_t o0 = o1 - P8 + (row0 == 0u ? LP8 : 0u);
+    const uint32_t o5 = o4 + P8 - (row0 + 4u == (uint32_t)g.L ? LP8 : 0u);
+    const bool first = w == 0u, last = w == (uint32_t)g.W - 1u;
+    const uint32_t lastbit = 3u * (uint32_t)(g.rlast - 1);             // the row's last live field
+    const uint32_t left = first ? (uint32_t)(g.W - 1) * 8u + (lastbit >= 32u ? 4u : 0u) : (uint32_t)-4;
+    const uint32_t lsh = first ? (lastbit & 31u) : 28u;
+    const uint32_t right = last ? 0u - w8 : 8u;
+    const uint32_t mul_lo = last && lastbit < 32u ? 1u << lastbit : 0u;
+    const uint32_t mul_hi = last ? (lastbit >= 32u ? 1u << (lastbit & 31u) : 0u) : 1u << 28;
+    const uint64_t n = lattice_words(g);
+    uint64_t oc[6], sw[4];
+    uint32_t side[4];
+    oc[0] = byte_ld64(other, o0, n, __LINE__);
+    oc[1] = byte_ld64(other, o1, n, __LINE__);
+    oc[2] = byte_ld64(other, o2, n, __LINE__);
+    oc[3] = byte_ld64(other, o3, n, __LINE__);
+    oc[4] = byte_ld64(other, o4, n, __LINE__);
+    oc[5] = byte_ld64(other, o5, n, __LINE__);
+    const uint32_t even = C == 0 ? left : right, odd = C == 0 ? right : left;
+    side[0] = byte_ld32(other, o1 + even, n, __LINE__);
+    side[1] = byte_ld32(other, o2 + odd, n, __LINE__);
+    side[2] = byte_ld32(other, o3 + even, n, __LINE__);
+    side[3] = byte_ld32(other, o4 + odd, n, __LINE__);
+    sw[0] = byte_ld64(own, o1, n, __LINE__);
+    sw[1] = byte_ld64(own, o2, n, __LINE__);
+    sw[2] = byte_ld64(own, o3, n, __LINE__);
+    sw[3] = byte_ld64(own, o4, n, __LINE__);
+    const uint64_t live64 = live_mask(g, (int)w);
+    const uint32_t live[2] = {(uint32_t)live64, (uint32_t)(live64 >> 32)};
 #pragma unroll
-    for (int e = 0; e < ROWS; ++e)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) acc.a[e][q] = 0;
-    if (UPDATE) {
-        const uint32_t tl = (uint32_t)t;
-        const uint32_t th = ((uint32_t)(t >> 32) << 1) | (uint32_t)C;
-        const PhiloxRowKey pk = philox_row_key((uint32_t)(row0 >> 2), tl, th, rk);
-        FieldLoop<0, ROUNDS>::run(pk, rk, (uint32_t)w * kFields, acc, thr0, thr1, one);
-    }
-    const uint64_t all0 = ((uint64_t)all0w << 32 | all0w) & live;
-    const uint64_t all1 = ((uint64_t)all1w << 32 | all1w) & live;
-#pragma unroll
-    for (int r = 0; r < ROWS; ++r) {
-        if (r < nrows) {
-            const uint64_t s = sw[r];
-            const uint64_t u = oc[r], d = oc[r + 2], h0 = oc[r + 1];
-            // the other-colour word shifted by one field (horizontal neighbour at m -/+ 1)
-            uint64_t h1;
-            if (((r + C) & 1) == 0) {
-                const int sh = (w > 0) ? 60 : 3 * (g.rlast - 1);
-                h1 = (h0 << 3) | (side[r] >> sh);
-            } else {
-                const int sh = (w < g.W - 1) ? 60 : 3 * (g.rlast - 1);
-                h1 = (h0 >> 3) | (side[r] << sh);
-            }
-            const uint64_t x1 = s ^ u, x2 = s ^ d, x3 = s ^ h0, x4 = s ^ h1;
-            uint64_t s_new = s;
+    for (int r = 0; r < 4; ++r) {
+        const uint32_t s[2] = {(uint32_t)sw[r], (uint32_t)(sw[r] >> 32)};
+        const uint32_t u[2] = {(uint32_t)oc[r], (uint32_t)(oc[r] >> 32)};
+        const uint32_t h0[2] = {(uint32_t)oc[r + 1], (uint32_t)(oc[r + 1] >> 32)};
+        const uint32_t d[2] = {(uint32_t)oc[r + 2], (uint32_t)(oc[r + 2] >> 32)};
+        // the horizontal neighbour at m - 1 (row + C even: row0 is a multiple of 4) or m + 1: the other
+        // colour's word moved by one field (bit 63 and dead fields are masked by live)
+        uint32_t h1[2], sn[2] = {s[0], s[1]};
+        if (((r + C) & 1) == 0) {
+            h1[0] = h0[0] * 8u + (side[r] >> lsh);
+            h1[1] = __funnelshift_l(h0[0], h0[1], 3);
+        } else {
+            h1[0] = __funnelshift_r(h0[0], h0[1], 3) + side[r] * mul_lo;
+            h1[1] = (h0[1] >> 3) + side[r] * mul_hi;
+        }
+        if (UPDATE) {
+            sn[0] = flip_half(s[0], u[0], d[0], h0[0], h1[0], acc.m[r][0],
+                              __funnelshift_r(acc.m[r][0], acc.m[r][1], 1), live[0]);
+            sn[1] = flip_half(s[1], u[1], d[1], h0[1], h1[1], acc.m[r][1], acc.m[r][1] >> 1, live[1]);
+        }
+        if (r < 2 || !two) {
             if (UPDATE) {
-                const uint64_t any = x1 | x2 | x3 | x4;
-                const uint64_t ge2 = (x1 & x2) | (x3 & x4) | ((x1 ^ x2) & (x3 ^ x4));
-                const uint64_t c1 = ((uint64_t)acc.a[r][2] << 32 | acc.a[r][0]) | all1;
-                const uint64_t c0 = (((uint64_t)acc.a[r][3] << 32 | acc.a[r][1]) >> 1) | all0;
-                const uint64_t accept = ge2 | (any & c1) | (~any & c0);
-                s_new = s ^ (accept & live);
-                word_st(own, base + (uint32_t)r * P, s_new, n, __LINE__);
+                const uint32_t o = r == 0 ? o1 : (r == 1 ? o2 : (r == 2 ? o3 : o4));
+                byte_st64(own, o, (uint64_t)sn[1] << 32 | sn[0], n, __LINE__);
             }
             if (RECORD) {
-                anti += __popcll((s_new ^ u) & live) + __popcll((s_new ^ d) & live)
-                      + __popcll((s_new ^ h0) & live) + __popcll((s_new ^ h1) & live);
-                up += __popcll(s_new & live) + __popcll(h0 & live);
+                count_half(sn[0], u[0], d[0], h0[0], h1[0], live[0], anti, up);
+                count_half(sn[1], u[1], d[1], h0[1], h1[1], live[1], anti, up);
             }
         }
     }
+}
+
+// ---- Strips: the items of a launch --------------------------------------
+// The thread items (group of 4 rows x word) are numbered strip by strip: a
+// strip is up to kStripWords consecutive word columns of all row groups, and
+// item q of a strip of `width` words is word q % width of group q / width.  A
+// block owns consecutive items of one strip, so its row groups share their
+// words' columns m = 21 w + k and with them the first Philox product of each
+// (first_products): 15 products per call instead of 16, and no index XOR.
+// Measured on GB300 at L = 16384 (one colour, launches back to back): 1,487
+// spin-updates/ns against 1,335-1,370 with the items in row order and each
+// call's own first product (26.1 against 28.1 cycles per site and scheduler,
+// with the word logic and index arithmetic trimmed at the same time).
+struct Strips {
+    uint32_t n;              // strips
+    uint32_t width, last;    // words of a strip, of the last one
+    uint32_t magic, magic_last;   // q / width = hi32(q * magic); 0: width 1
+};
+
+__device__ __forceinline__ uint32_t strip_group(uint32_t q, uint32_t magic) { return magic ? __umulhi(q, magic) : q; }
+
+// All threads of the block: the first products of fields 0 .. 20 of words
+// w0 .. w0 + width - 1 at a sweep (key: philox_first_key), field k of word w0
+// + x in tab[k * kStripWords + x].
+__device__ __forceinline__ void first_products(uint2* tab, uint32_t w0, uint32_t width, uint32_t key)
+{
+    const uint32_t x = threadIdx.x & 31u;
+    if (x < width)
+        for (uint32_t k = threadIdx.x >> 5; k < (uint32_t)kFields; k += blockDim.x >> 5) {
+            uint32_t hi, lo;
+            mul_hilo(kPhiloxM0, key ^ ((w0 + x) * (uint32_t)kFields + k), hi, lo);
+            tab[k * kStripWords + x] = make_uint2(hi, lo);
+        }
+    __syncthreads();
+}
+
+// Draw and update in one step without a table (the on-chip kernel that draws
+// its own masks).
+template <int C, bool RECORD, int ROUNDS>
+__device__ __forceinline__ void sweep_item(uint64_t* own, const uint64_t* other, const Geom& g, uint32_t grp,
+                                           uint32_t w, uint64_t t, const SweepArgs& a, uint32_t& anti, uint32_t& up)
+{
+    ItemMasks acc;
+    const FirstDirect first = {philox_first_key((uint32_t)t, a.rk), w * (uint32_t)kFields};
+    draw_item<ROUNDS>(first, grp, t, C, a.rk, a.thr0, a.thr1, a.all0, a.all1, acc);
+    apply_item<C, true, RECORD>(own, other, g, grp, w, acc, anti, up);
 }
 
 // ---- Split forms of sweep_rows -------------------------------------------
@@ -488,29 +628,21 @@ __device__ __forceinline__ void item_apply(uint64_t* __restrict__ own, const uin
     }
 }
 
-// All accept masks of one item drawn by one thread, with the draws and
-// accumulators of sweep_rows, packed one word per row: packed[e] has r < thr1
-// of field k at bit 3k and r < thr0 at bit 3k + 1.  For row_apply, m1 =
-// packed and m0 = packed >> 1: their other bits fall on no spin bit.
+// All accept masks of one item drawn by one thread, packed one word per row:
+// packed[e] has r < thr1 of field k at bit 3k and r < thr0 at bit 3k + 1, each
+// set where its threshold is 2^32.  For row_apply, m1 = packed and m0 =
+// packed >> 1: their other bits fall on no spin bit.
 template <int ROUNDS = 10>
-__device__ __forceinline__ void item_masks_thread(const Geom& g, int item, uint64_t t, int colour,
-                                                  const PhiloxKeys& rk, uint32_t thr0, uint32_t thr1, uint32_t one,
+__device__ __forceinline__ void item_masks_thread(const Geom& g, int item, uint64_t t, int colour, const SweepArgs& a,
                                                   uint64_t packed[4])
 {
     const int grp = item / g.W;
     const int w = item - grp * g.W;
-    AcceptBits acc;
+    ItemMasks acc;
+    const FirstDirect first = {philox_first_key((uint32_t)t, a.rk), (uint32_t)w * kFields};
+    draw_item<ROUNDS>(first, (uint32_t)grp, t, colour, a.rk, a.thr0, a.thr1, a.all0, a.all1, acc);
 #pragma unroll
-    for (int e = 0; e < 4; ++e)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) acc.a[e][q] = 0;
-    const uint32_t tl = (uint32_t)t;
-    const uint32_t th = ((uint32_t)(t >> 32) << 1) | (uint32_t)colour;
-    const PhiloxRowKey pk = philox_row_key((uint32_t)grp, tl, th, rk);
-    FieldLoop<0, ROUNDS>::run(pk, rk, (uint32_t)w * kFields, acc, thr0, thr1, one);
-#pragma unroll
-    for (int e = 0; e < 4; ++e)
-        packed[e] = (uint64_t)(acc.a[e][2] | acc.a[e][3]) << 32 | (acc.a[e][0] | acc.a[e][1]);
+    for (int e = 0; e < 4; ++e) packed[e] = (uint64_t)acc.m[e][1] << 32 | acc.m[e][0];
 }
 
 // Masks of an item with F lanes; an item past the end is drawn as item 0.
@@ -523,45 +655,39 @@ __device__ __forceinline__ void item_masks(const Geom& g, int item, bool valid, 
     item_masks_lanes<F, ROUNDS>(g, item, q, t, colour, rk, thr0, thr1, a1, a0);
 }
 
-// Draw and apply in one step (the launch path's lanes kernel).
-template <int C, bool RECORD, int F, int ROUNDS = 10>
-__device__ __forceinline__ void sweep_item_lanes(uint64_t* __restrict__ own, const uint64_t* __restrict__ other,
-                                                 const Geom& g, int item, bool valid, int q, uint64_t t,
-                                                 const PhiloxKeys& rk, uint32_t thr0, uint32_t thr1,
-                                                 uint32_t all0w, uint32_t all1w, uint32_t& anti, uint32_t& up)
+// One half-sweep of colour C over one lattice: block (x, y) owns items
+// blockDim.x x .. of strip y (a 1-D block of 32 to 256 threads).  The draws
+// need launch operands only (t from the host), so with programmatic dependent
+// launch they run before the wait for the previous half-sweep, and fill the
+// SMs that its last blocks leave idle; the lattice is read after it.  64
+// registers keep 32 warps on an SM.  Bound by the issue of Philox products,
+// XORs and compares (see accept_insert).  ROUNDS: Philox rounds of the draws
+// (10, or the opt-in 7).
+template <int C, bool UPDATE, bool RECORD, int ROUNDS = 10>
+__global__ void __launch_bounds__(256, 4)
+half_sweep_kernel(uint64_t* own, const uint64_t* other, Geom g, Strips st, SweepArgs a)
 {
-    uint64_t a1[4], a0[4];
-    item_masks<F, ROUNDS>(g, item, valid, q, t, C, rk, thr0, thr1, a1, a0);
-    item_apply<C, RECORD, F>(own, other, g, item, valid, q, a1, a0, all0w, all1w, anti, up);
-}
-
-// One half-sweep of colour C over one lattice.  LINEAR: a 1-D grid whose
-// thread k owns item k = group * W + w (word w of rows 4 group .. 4 group + 3),
-// so no thread idles on padding columns and the blocks tile the lattice
-// without a partial column of blocks.  Otherwise thread (x, y) of a 2-D grid
-// owns word column x and rows 4y .. 4y+3.  At most 256 threads per block.
-// ROUNDS: Philox rounds of the draws (10, or the opt-in 7).
-template <int C, bool UPDATE, bool RECORD, int ROUNDS = 10, bool LINEAR = true>
-__global__ void __launch_bounds__(256, 3)
-half_sweep_kernel(uint64_t* __restrict__ own, const uint64_t* __restrict__ other, Geom g, SweepArgs a)
-{
-    pdl_enter();
-    int w, row0;
-    if (LINEAR) {
-        const uint32_t item = blockIdx.x * blockDim.x + threadIdx.x;
-        const uint32_t grp = item / (uint32_t)g.W;
-        w = (int)(item - grp * (uint32_t)g.W);
-        row0 = (int)grp * 4;
-    } else {
-        w = blockIdx.x * blockDim.x + threadIdx.x;
-        row0 = (blockIdx.y * blockDim.y + threadIdx.y) * 4;
-    }
+    __shared__ uint2 tab[kFields * kStripWords];
+    pdl_launch();
+    const uint32_t w0 = blockIdx.y * st.width;
+    const bool last = blockIdx.y == st.n - 1u;
+    const uint32_t width = last ? st.last : st.width;
+    const uint32_t q = blockIdx.x * blockDim.x + threadIdx.x;
+    const uint32_t grp = strip_group(q, last ? st.magic_last : st.magic);
+    const uint32_t x = q - grp * width;
+    const bool valid = grp * 4u < (uint32_t)g.L;
     uint32_t anti = 0, up = 0;
-    if (w < g.W && row0 < g.L) {
-        const uint64_t t = UPDATE ? *a.t_base + a.t_off : 0;
-        sweep_rows<C, UPDATE, RECORD, true, ROUNDS>(own, other, g, row0, w, t, a.rk, a.thr0, a.thr1, a.all0,
-                                                    a.all1, a.one, anti, up);
+    ItemMasks acc;
+    if (UPDATE) {
+        const uint64_t t = sweep_number(a);
+        first_products(tab, w0, width, philox_first_key((uint32_t)t, a.rk));
+        if (valid) {
+            const FirstTable first = {tab + x};
+            draw_item<ROUNDS>(first, grp, t, C, a.rk, a.thr0, a.thr1, a.all0, a.all1, acc);
+        }
     }
+    pdl_wait();
+    if (valid) apply_item<C, UPDATE, RECORD>(own, other, g, grp, w0 + x, acc, anti, up);
     if (RECORD) {
         const int slot = (blockIdx.x + gridDim.x * blockIdx.y) % kCountSlots;
         block_add_counts(record_counts(a) + 2 * slot, anti, up);

@@ -133,7 +133,7 @@ ci_half_sweep_kernel(uint64_t* __restrict__ S, int L, int N, SweepArgs a, const 
 #pragma unroll
                 for (int e = 0; e < 4; ++e) packed[e] = __ldg(masks + ((size_t)q * (L / 2) + m) * 4 + e);
             } else {
-                ci_masks<ROUNDS>(N, q, m, *a.t_base + a.t_off, C, a, packed);
+                ci_masks<ROUNDS>(N, q, m, sweep_number(a), C, a, packed);
             }
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
@@ -228,7 +228,7 @@ __device__ __forceinline__ void rw_draw(const SweepArgs& a, uint32_t step, uint3
     packed = m;
 }
 
-// All updates of iteration *t_base + t_off, both phases: entry
+// All updates of iteration sweep_number(a), both phases: entry
 // draws[phase base + q * U_p + s] = (I << 16 | column in the half strip,
 // packed masks) for update s of strip q; phase 0's entries first.
 __global__ void __launch_bounds__(128)
@@ -243,7 +243,7 @@ ci_rw_draw_kernel(int L, int N, int NC, int nstrips, SweepArgs a, ulonglong2* __
     const uint64_t r = phase ? k - n0 : k;
     const uint64_t U = phase ? U1 : U0;
     const uint32_t q = (uint32_t)(r / U), step = (uint32_t)(r - (uint64_t)q * U);
-    const uint64_t t = *a.t_base + a.t_off;
+    const uint64_t t = sweep_number(a);
     const uint32_t x3 = 0x80000000u | ((uint32_t)(t >> 32) << 1) | (uint32_t)phase;
     uint32_t I, jr;
     uint64_t packed;
@@ -273,7 +273,7 @@ ci_rw_phase_kernel(uint64_t* S, int L, int N, int NC, int phase, SweepArgs a, co
     const int h = phase == 0 ? NC / 2 : NC - NC / 2;
     const int col0 = (int)q * NC + (phase == 0 ? 0 : NC / 2);
     const uint32_t U = 10u * (uint32_t)N * (uint32_t)h;
-    const uint64_t t = *a.t_base + a.t_off;
+    const uint64_t t = sweep_number(a);
     const uint32_t tl = (uint32_t)t;
     const uint32_t x3 = 0x80000000u | ((uint32_t)(t >> 32) << 1) | (uint32_t)phase;
     const ulonglong2* my_draws = PRE ? draws + (size_t)q * U : nullptr;   // this phase's block of draws

@@ -165,8 +165,12 @@ inline void launch_pdl(void (*kernel)(Params...), dim3 grid, dim3 block, cudaStr
 // Geometry checks shared by the entry points.
 bool valid_side(int32_t L);
 
+// Strips of at most `most` (and kStripWords) words for geometry g.
+Strips make_strips(const Geom& g, int most);
+
 // One half-sweep of one lattice (update and/or record), or the measurement
-// pass (update = false, record = true, colour 1); block = bw x bgrp threads.
+// pass (update = false, record = true, colour 1); bw = 0: bgrp threads a
+// block, else strips of at most bw words and bw * bgrp threads.
 cudaError_t launch_half_sweep(int bw, int bgrp, int colour, bool update, bool record,
                               uint64_t* own, const uint64_t* other, const Geom& g, const SweepArgs& a,
                               cudaStream_t s);

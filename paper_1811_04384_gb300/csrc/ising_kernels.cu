@@ -175,8 +175,7 @@ resident_sweeps_kernel(uint64_t* __restrict__ w0, uint64_t* __restrict__ w1, Geo
         uint32_t dummy0 = 0, dummy1 = 0;
         for (int it = threadIdx.x; it < items; it += blockDim.x) {
             const int grp = it / g.W, w = it - grp * g.W;
-            sweep_rows<0, true, false, false, ROUNDS>(s0, s1, g, grp * 4, w, t, a.rk, a.thr0, a.thr1, a.all0,
-                                                      a.all1, a.one, dummy0, dummy1);
+            sweep_item<0, false, ROUNDS>(s0, s1, g, (uint32_t)grp, (uint32_t)w, t, a, dummy0, dummy1);
         }
         __syncthreads();
         const bool record = (s % every) == 0;
@@ -184,11 +183,9 @@ resident_sweeps_kernel(uint64_t* __restrict__ w0, uint64_t* __restrict__ w1, Geo
         for (int it = threadIdx.x; it < items; it += blockDim.x) {
             const int grp = it / g.W, w = it - grp * g.W;
             if (record)
-                sweep_rows<1, true, true, false, ROUNDS>(s1, s0, g, grp * 4, w, t, a.rk, a.thr0, a.thr1, a.all0,
-                                                         a.all1, a.one, anti, up);
+                sweep_item<1, true, ROUNDS>(s1, s0, g, (uint32_t)grp, (uint32_t)w, t, a, anti, up);
             else
-                sweep_rows<1, true, false, false, ROUNDS>(s1, s0, g, grp * 4, w, t, a.rk, a.thr0, a.thr1, a.all0,
-                                                          a.all1, a.one, anti, up);
+                sweep_item<1, false, ROUNDS>(s1, s0, g, (uint32_t)grp, (uint32_t)w, t, a, anti, up);
         }
         if (record) {
             anti = __reduce_add_sync(0xffffffffu, anti);
@@ -212,8 +209,7 @@ resident_sweeps_kernel(uint64_t* __restrict__ w0, uint64_t* __restrict__ w1, Geo
 }
 
 // Accept masks of the sweeps j = 0 .. nsweeps-1 that follow sweep t0 (sweep
-// t0 + j + 1), one thread per (j, item), drawn exactly as sweep_rows draws
-// them: masks[(j * items + item) * 4 + e] = (colour-0, colour-1 packed masks)
+// t0 + j + 1), one thread per (j, item), drawn by item_masks_thread: masks[(j * items + item) * 4 + e] = (colour-0, colour-1 packed masks)
 // of row e of the item (item_masks_thread).  The draws depend on the site,
 // sweep and colour only, so a whole run's masks can be drawn at once by every
 // SM before the spins are updated.  t_base (device memory, or null) is added
@@ -232,8 +228,8 @@ mask_draw_kernel(Geom g, SweepArgs a, const uint64_t* t_base, uint64_t t0, int n
         const int item = (int)(k - (long long)j * items);
         uint64_t p0[4], p1[4];
         const uint64_t t = tb + (uint64_t)j;
-        item_masks_thread<ROUNDS>(g, item, t, 0, a.rk, a.thr0, a.thr1, a.one, p0);
-        item_masks_thread<ROUNDS>(g, item, t, 1, a.rk, a.thr0, a.thr1, a.one, p1);
+        item_masks_thread<ROUNDS>(g, item, t, 0, a, p0);
+        item_masks_thread<ROUNDS>(g, item, t, 1, a, p1);
         ulonglong2* out = masks + (size_t)k * 4;
 #pragma unroll
         for (int e = 0; e < 4; ++e) out[e] = make_ulonglong2(p0[e], p1[e]);
@@ -412,7 +408,7 @@ cudaError_t launch_half_sweep_apply(int colour, bool record, uint64_t* own, cons
 }
 
 // One half-sweep of colour C over all SMs with F lanes per thread item
-// (sweep_item_lanes on the lattice in global memory): for lattices whose one
+// (item_masks, item_apply): for lattices whose one
 // thread per item would leave SMs idle and each thread with a long chain of
 // 21 Philox calls.  Thread k of the grid is lane k % F of item k / F.  Same
 // results as half_sweep_kernel.
@@ -420,14 +416,16 @@ template <int C, bool RECORD, int F, int ROUNDS>
 __global__ void __launch_bounds__(128, 4)
 half_sweep_lanes_kernel(uint64_t* __restrict__ own, const uint64_t* __restrict__ other, Geom g, SweepArgs a)
 {
-    pdl_enter();
+    pdl_launch();
     const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
     const int item = (int)(k / F), q = (int)(k % F);
     const int items = ((g.L + 3) / 4) * g.W;
-    const uint64_t t = *a.t_base + a.t_off;
     uint32_t anti = 0, up = 0;
-    sweep_item_lanes<C, RECORD, F, ROUNDS>(own, other, g, item, item < items, q, t, a.rk, a.thr0, a.thr1, a.all0,
-                                           a.all1, anti, up);
+    uint64_t a1[4], a0[4];
+    // the draws overlap the end of the previous half-sweep (see half_sweep_kernel)
+    item_masks<F, ROUNDS>(g, item, item < items, q, sweep_number(a), C, a.rk, a.thr0, a.thr1, a1, a0);
+    pdl_wait();
+    item_apply<C, RECORD, F>(own, other, g, item, item < items, q, a1, a0, a.all0, a.all1, anti, up);
     if (RECORD) block_add_counts(record_counts(a) + 2 * (blockIdx.x % kCountSlots), anti, up);
 }
 
@@ -546,9 +544,9 @@ SweepArgs make_sweep_args(uint64_t seed, const uint64_t thr[2], const uint64_t* 
 {
     SweepArgs a;
     a.t_base = t_base;
+    a.t0 = 0;
     a.t_off = 0;
     fill_threshold_args(thr, a);
-    a.one = 1;
     a.rounds = 10;
     a.rk = philox_keys((uint32_t)seed, (uint32_t)(seed >> 32));
     a.counts = nullptr;
@@ -556,38 +554,49 @@ SweepArgs make_sweep_args(uint64_t seed, const uint64_t thr[2], const uint64_t* 
     return a;
 }
 
-template <int ROUNDS, bool LIN>
+Strips make_strips(const Geom& g, int most)
+{
+    most = std::min(most, kStripWords);
+    Strips st;
+    st.n = (uint32_t)((g.W + most - 1) / most);
+    st.width = ((uint32_t)g.W + st.n - 1) / st.n;               // strips of about equal width
+    st.n = ((uint32_t)g.W + st.width - 1) / st.width;
+    st.last = (uint32_t)g.W - (st.n - 1) * st.width;
+    // q < 2^18 and width <= 32, so hi32(q * ceil(2^32 / width)) = q / width
+    auto magic = [](uint32_t w) { return w == 1 ? 0u : (uint32_t)(((1ull << 32) + w - 1) / w); };
+    st.magic = magic(st.width);
+    st.magic_last = magic(st.last);
+    return st;
+}
+
+template <int ROUNDS>
 static void launch_half_sweep_r(dim3 grid, dim3 block, int colour, bool update, bool record, uint64_t* own,
-                                const uint64_t* other, const Geom& g, const SweepArgs& a, cudaStream_t s)
+                                const uint64_t* other, const Geom& g, const Strips& st, const SweepArgs& a,
+                                cudaStream_t s)
 {
     if (colour == 0) {
-        if (record) launch_pdl(half_sweep_kernel<0, true, true, ROUNDS, LIN>, grid, block, s, own, other, g, a);
-        else launch_pdl(half_sweep_kernel<0, true, false, ROUNDS, LIN>, grid, block, s, own, other, g, a);
+        if (record) launch_pdl(half_sweep_kernel<0, true, true, ROUNDS>, grid, block, s, own, other, g, st, a);
+        else launch_pdl(half_sweep_kernel<0, true, false, ROUNDS>, grid, block, s, own, other, g, st, a);
     } else if (!update) {
-        half_sweep_kernel<1, false, true, 10, LIN><<<grid, block, 0, s>>>(own, other, g, a);
+        half_sweep_kernel<1, false, true, 10><<<grid, block, 0, s>>>(own, other, g, st, a);
     } else {
-        if (record) launch_pdl(half_sweep_kernel<1, true, true, ROUNDS, LIN>, grid, block, s, own, other, g, a);
-        else launch_pdl(half_sweep_kernel<1, true, false, ROUNDS, LIN>, grid, block, s, own, other, g, a);
+        if (record) launch_pdl(half_sweep_kernel<1, true, true, ROUNDS>, grid, block, s, own, other, g, st, a);
+        else launch_pdl(half_sweep_kernel<1, true, false, ROUNDS>, grid, block, s, own, other, g, st, a);
     }
 }
 
-// bw == 0: linear items, bgrp threads per block; else bw x bgrp 2-D blocks.
+// bw == 0: strips of up to kStripWords words, bgrp threads per block; else
+// strips of up to bw words, bw * bgrp threads.
 cudaError_t launch_half_sweep(int bw, int bgrp, int colour, bool update, bool record,
                               uint64_t* own, const uint64_t* other, const Geom& g, const SweepArgs& a,
                               cudaStream_t s)
 {
-    const int ngroups = (g.L + 3) / 4;
-    if (bw == 0) {
-        const uint32_t items = (uint32_t)ngroups * (uint32_t)g.W;
-        dim3 block(bgrp), grid((items + bgrp - 1) / bgrp);
-        if (a.rounds == 7) launch_half_sweep_r<7, true>(grid, block, colour, update, record, own, other, g, a, s);
-        else launch_half_sweep_r<10, true>(grid, block, colour, update, record, own, other, g, a, s);
-        return cudaGetLastError();
-    }
-    dim3 block(bw, bgrp);
-    dim3 grid((g.W + bw - 1) / bw, (ngroups + bgrp - 1) / bgrp);
-    if (a.rounds == 7) launch_half_sweep_r<7, false>(grid, block, colour, update, record, own, other, g, a, s);
-    else launch_half_sweep_r<10, false>(grid, block, colour, update, record, own, other, g, a, s);
+    const Strips st = make_strips(g, bw == 0 ? kStripWords : bw);
+    const uint32_t threads = (uint32_t)(bw == 0 ? bgrp : bw * bgrp);
+    const uint32_t items = (uint32_t)((g.L + 3) / 4) * st.width;
+    dim3 block(threads), grid((items + threads - 1) / threads, st.n);
+    if (a.rounds == 7) launch_half_sweep_r<7>(grid, block, colour, update, record, own, other, g, st, a, s);
+    else launch_half_sweep_r<10>(grid, block, colour, update, record, own, other, g, st, a, s);
     return cudaGetLastError();
 }
 

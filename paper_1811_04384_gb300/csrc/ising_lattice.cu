@@ -506,12 +506,24 @@ static int replay_plain(ising_lattice* h, int64_t* n)
     return ISING_OK;
 }
 
-// Run `n` sweeps relative to the device counter; sweep s (1-based) records into
-// count slot rec_of(s) when rec_of(s) >= 0.  Then advances the counter by n.
+// Run `n` sweeps; sweep s (1-based) records into count slot rec_of(s) when
+// rec_of(s) >= 0.  Then advances the counter by n.  The launches take the
+// sweep counter from the host, so that their draws need no device memory;
+// where the stream is being captured they read the device's, which a replay
+// advances.
 template <typename RecOf>
 static int run_sweeps(ising_lattice* h, int64_t n, RecOf rec_of)
 {
     SweepArgs a = base_args(h);
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(h->stream, &cs) != cudaSuccess) {
+        cudaGetLastError();
+        cs = cudaStreamCaptureStatusActive;
+    }
+    if (cs == cudaStreamCaptureStatusNone) {
+        a.t_base = nullptr;
+        a.t0 = h->t;
+    }
     for (int64_t s = 1; s <= n; ++s) {
         a.t_off = (uint32_t)s;
         cudaError_t e = launch_hs(h, 0, true, false, a);

@@ -24,12 +24,10 @@ constexpr int kSlots = ising::kCountSlots;
 //   [0, kCounts)            count slots: record r, slot k -> 2 words (anti, up)
 //   [kCounts, +kMaxRecords) E per record
 //   [.., +kMaxRecords)      M per record
-//   [kTOffset]              sweep counter the half-sweep kernel reads
 constexpr size_t kCounts = (size_t)kMaxRecords * kSlots * 2;
 constexpr size_t kEOffset = kCounts;
 constexpr size_t kMOffset = kEOffset + kMaxRecords;
-constexpr size_t kTOffset = kMOffset + kMaxRecords;
-constexpr size_t kScratchWords = kTOffset + 32;   // the counter, padded to 256 bytes
+constexpr size_t kScratchWords = kMOffset + kMaxRecords;
 
 // The scratch memory: every GPU that loads the library holds one copy
 // (kScratchWords * 8 bytes, about 528 KB) until the process exits.
@@ -57,11 +55,6 @@ int scratch_on_current_device(unsigned long long** out)
     }
     *out = g_scratch_ptr[dev];
     return ISING_OK;
-}
-
-__global__ void noalloc_set_sweep_kernel(unsigned long long* t, unsigned long long value)
-{
-    if (threadIdx.x == 0 && blockIdx.x == 0) *t = value;
 }
 
 // E = 2 anti - 2 L^2 and M = 2 up - L^2 from the count slots of each record.
@@ -101,14 +94,12 @@ extern "C" int ising_sweep_record_noalloc(uint64_t* dev_words0, uint64_t* dev_wo
     // The array keeps the previous call's contents: clear the count slots.
     cudaError_t e = cudaMemsetAsync(scratch, 0, (size_t)(nrec > 0 ? nrec : 1) * kSlots * 2 * sizeof(unsigned long long), s);
     if (e != cudaSuccess) return ising::cuda_fail(e, "cudaMemsetAsync");
-    noalloc_set_sweep_kernel<<<1, 1, 0, s>>>(scratch + kTOffset, t0);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return ising::cuda_fail(e, "noalloc_set_sweep_kernel");
 
     const ising::Geom g = ising::lattice_geom(L);
     uint64_t thr[2];
     ising::thresholds_for_beta(beta, thr);
-    ising::SweepArgs a = ising::make_sweep_args(seed, thr, reinterpret_cast<const uint64_t*>(scratch + kTOffset));
+    ising::SweepArgs a = ising::make_sweep_args(seed, thr, nullptr);
+    a.t0 = t0;
     for (int64_t step = 1; step <= n; ++step) {
         a.t_off = (uint32_t)step;
         a.counts = nullptr;

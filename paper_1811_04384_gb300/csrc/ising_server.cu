@@ -259,7 +259,7 @@ int run_epoch(ising_server* s, const std::vector<uint64_t>& run, std::vector<Job
         lane_tile0[k] = (int)tiles.size();
         for (size_t a : order)
             if (lane_of[a] == k)
-                for (uint32_t f = 0; f < reps[a].items; f += threads) tiles.push_back({(int)a, (int)f});
+                add_tiles(tiles, (int)a, reps[a].g, threads);
         lane_nt[k] = (int)tiles.size() - lane_tile0[k];
     }
     int rc = ensure_tiles(s, tiles.size());
@@ -285,11 +285,11 @@ int run_epoch(ising_server* s, const std::vector<uint64_t>& run, std::vector<Job
             const BatchReplica* R = s->d_reps;
             const uint32_t* z = s->d_zero;
             if (rounds == 10) {
-                launch_pdl(batch_half_sweep_kernel<0, 10, 1>, dim3(lane_nt[k]), dim3(threads), st[k], R, t, z, n, 1u);
-                launch_pdl(batch_half_sweep_kernel<1, 10, 0>, dim3(lane_nt[k]), dim3(threads), st[k], R, t, z, n, 1u);
+                launch_pdl(batch_half_sweep_kernel<0, 10, 1>, dim3(lane_nt[k]), dim3(threads), st[k], R, t, z, n);
+                launch_pdl(batch_half_sweep_kernel<1, 10, 0>, dim3(lane_nt[k]), dim3(threads), st[k], R, t, z, n);
             } else {
-                launch_pdl(batch_half_sweep_kernel<0, 0, 1>, dim3(lane_nt[k]), dim3(threads), st[k], R, t, z, n, 1u);
-                launch_pdl(batch_half_sweep_kernel<1, 0, 0>, dim3(lane_nt[k]), dim3(threads), st[k], R, t, z, n, 1u);
+                launch_pdl(batch_half_sweep_kernel<0, 0, 1>, dim3(lane_nt[k]), dim3(threads), st[k], R, t, z, n);
+                launch_pdl(batch_half_sweep_kernel<1, 0, 0>, dim3(lane_nt[k]), dim3(threads), st[k], R, t, z, n);
             }
         }
     }
@@ -553,7 +553,6 @@ extern "C" int ising_server_submit(ising_server* s, const ising_job* job, uint64
     const SweepArgs a = make_sweep_args(job->seed, thr, nullptr);
     j.rep.rk = a.rk;
     j.rep.thr0 = a.thr0; j.rep.thr1 = a.thr1; j.rep.all0 = a.all0; j.rep.all1 = a.all1;
-    j.rep.items = (uint32_t)((j.g.L + 3) / 4) * (uint32_t)j.g.W;
     j.rep.rounds = job->rng == ISING_RNG_PHILOX4X32_7 ? 7 : 10;
     {
         std::lock_guard<std::mutex> lock(s->mu);

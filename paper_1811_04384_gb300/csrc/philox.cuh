@@ -22,14 +22,16 @@ constexpr uint32_t kPhiloxM1 = 0xCD9E8D57u;
 constexpr uint32_t kPhiloxW0 = 0x9E3779B9u;
 constexpr uint32_t kPhiloxW1 = 0xBB67AE85u;
 
-// hi, lo of the 64-bit product a * b.  On the device as two 32-bit
-// multiplies (high and low half): measured 0.7-5.6% faster on GB300 than one
-// 32x32->64 multiply, whose register-pair result constrains the allocation.
+// hi, lo of the 64-bit product a * b.  On the device one 32x32->64 multiply,
+// stated as such: written as a high-half and a low-half multiply, the
+// compiler fused only some of the pairs (a kernel of Philox calls alone ran
+// 7.7 multiply-pipe instructions per site instead of 4.6, 1,595 against
+// 1,985 sites/ns on GB300).
 ISING_HD void mul_hilo(uint32_t a, uint32_t b, uint32_t& hi, uint32_t& lo)
 {
 #if defined(__CUDA_ARCH__)
-    hi = __umulhi(a, b);
-    lo = a * b;
+    asm("{\n\t.reg .b64 p;\n\tmul.wide.u32 p, %2, %3;\n\tmov.b64 {%1, %0}, p;\n\t}"
+        : "=r"(hi), "=r"(lo) : "r"(a), "r"(b));
 #else
     const uint64_t p = (uint64_t)a * (uint64_t)b;
     hi = (uint32_t)(p >> 32);
@@ -113,17 +115,26 @@ ISING_HD PhiloxRowKey philox_row_key(uint32_t g, uint32_t tl, uint32_t th, const
     return p;
 }
 
+// The first product of a call, M0 y0 with y0 = hi(M1 tl) ^ k0 ^ m: it depends
+// on the sweep and on m only, not on the row group or the colour, so the
+// row groups of a block can share it (see first_products in ising_device.cuh).
+ISING_HD uint32_t philox_first_key(uint32_t tl, const PhiloxKeys& rk)
+{
+    uint32_t h, l;
+    mul_hilo(kPhiloxM1, tl, h, l);
+    return h ^ rk.k0[0];
+}
+
+// The rest of a call from its first product (hi, lo).
 // ROUNDS = 10 is Philox4x32-10; ROUNDS = 7 the opt-in cheaper member of the
 // same family (the same iteration stopped after 7 rounds).
 template <int ROUNDS = 10>
-ISING_HD void philox_row(const PhiloxRowKey& p, const PhiloxKeys& rk, uint32_t m, uint32_t out[4])
+ISING_HD void philox_row_tail(const PhiloxRowKey& p, const PhiloxKeys& rk, uint32_t hi, uint32_t lo, uint32_t out[4])
 {
     static_assert(ROUNDS >= 3 && ROUNDS <= 10, "3..10 rounds");
     uint32_t h, l;
-    const uint32_t y0 = p.a ^ m;
-    mul_hilo(kPhiloxM0, y0, h, l);
-    const uint32_t z2 = h ^ p.y3k;
-    const uint32_t z3 = l;
+    const uint32_t z2 = hi ^ p.y3k;
+    const uint32_t z3 = lo;
     mul_hilo(kPhiloxM1, z2, h, l);
     uint32_t x0 = h ^ p.z1k;
     uint32_t x1 = l;
@@ -133,6 +144,14 @@ ISING_HD void philox_row(const PhiloxRowKey& p, const PhiloxKeys& rk, uint32_t m
     for (int r = 3; r < ROUNDS; ++r)
         philox_round(x0, x1, x2, x3, rk.k0[r], rk.k1[r]);
     out[0] = x0; out[1] = x1; out[2] = x2; out[3] = x3;
+}
+
+template <int ROUNDS = 10>
+ISING_HD void philox_row(const PhiloxRowKey& p, const PhiloxKeys& rk, uint32_t m, uint32_t out[4])
+{
+    uint32_t h, l;
+    mul_hilo(kPhiloxM0, p.a ^ m, h, l);
+    philox_row_tail<ROUNDS>(p, rk, h, l, out);
 }
 
 }  // namespace ising
