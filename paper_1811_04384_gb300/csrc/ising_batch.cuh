@@ -76,7 +76,7 @@ batch_half_sweep_kernel(const BatchReplica* __restrict__ reps, const BatchTile* 
     const PhiloxKeys rk = R->rk;
     uint32_t anti = 0, up = 0;
     ItemMasks acc;
-    first_products(tab, w0, width, philox_first_key((uint32_t)t, rk));
+    first_products(tab, w0, width, tile.magic, philox_first_key((uint32_t)t, rk));
     if (valid) {
         const FirstTable first = {tab + x};
         if (ROUNDS == 7 || (ROUNDS == 0 && R->rounds == 7))

@@ -279,7 +279,7 @@ struct FirstDirect {
         mul_hilo(kPhiloxM0, key ^ (m0 + (uint32_t)k), hi, lo);
     }
 };
-constexpr int kStripWords = 32;   // most words of a strip
+constexpr int kStripWords = 16;   // most words of a strip
 struct FirstTable {
     const uint2* col;             // the item's word in the table
     __device__ __forceinline__ void get(int k, uint32_t& hi, uint32_t& lo) const
@@ -430,7 +430,10 @@ __device__ __forceinline__ void apply_item(uint64_t* own, const uint64_t* other,
 // Measured on GB300 at L = 16384 (one colour, launches back to back): 1,487
 // spin-updates/ns against 1,335-1,370 with the items in row order and each
 // call's own first product (26.1 against 28.1 cycles per site and scheduler,
-// with the word logic and index arithmetic trimmed at the same time).
+// with the word logic and index arithmetic trimmed at the same time).  Strips
+// of at most 32 / 24 / 20 / 16 / 12 words (blocks of 128, sweeps without
+// records): 1,537 / 1,551 / 1,558 / 1,567 / 1,574, but L = 2016: 1,136 /
+// 1,144 / 1,153 / 1,159 / 1,124; a 16-word strip reads whole 128-byte lines.
 struct Strips {
     uint32_t n;              // strips
     uint32_t width, last;    // words of a strip, of the last one
@@ -441,14 +444,17 @@ __device__ __forceinline__ uint32_t strip_group(uint32_t q, uint32_t magic) { re
 
 // All threads of the block: the first products of fields 0 .. 20 of words
 // w0 .. w0 + width - 1 at a sweep (key: philox_first_key), field k of word w0
-// + x in tab[k * kStripWords + x].
-__device__ __forceinline__ void first_products(uint2* tab, uint32_t w0, uint32_t width, uint32_t key)
+// + x in tab[k * kStripWords + x].  The threads fill whole columns of a field
+// at a time (blockDim / width fields per pass).
+__device__ __forceinline__ void first_products(uint2* tab, uint32_t w0, uint32_t width, uint32_t magic, uint32_t key)
 {
-    const uint32_t x = threadIdx.x & 31u;
-    if (x < width)
-        for (uint32_t k = threadIdx.x >> 5; k < (uint32_t)kFields; k += blockDim.x >> 5) {
+    const uint32_t k0 = strip_group(threadIdx.x, magic), x = threadIdx.x - k0 * width;
+    const uint32_t step = strip_group(blockDim.x, magic);      // >= 2: blocks have at least 32 threads
+    uint32_t m = (w0 + x) * (uint32_t)kFields + k0;
+    if (k0 < step)
+        for (uint32_t k = k0; k < (uint32_t)kFields; k += step, m += step) {
             uint32_t hi, lo;
-            mul_hilo(kPhiloxM0, key ^ ((w0 + x) * (uint32_t)kFields + k), hi, lo);
+            mul_hilo(kPhiloxM0, key ^ m, hi, lo);
             tab[k * kStripWords + x] = make_uint2(hi, lo);
         }
     __syncthreads();
@@ -672,15 +678,16 @@ half_sweep_kernel(uint64_t* own, const uint64_t* other, Geom g, Strips st, Sweep
     const uint32_t w0 = blockIdx.y * st.width;
     const bool last = blockIdx.y == st.n - 1u;
     const uint32_t width = last ? st.last : st.width;
+    const uint32_t magic = last ? st.magic_last : st.magic;
     const uint32_t q = blockIdx.x * blockDim.x + threadIdx.x;
-    const uint32_t grp = strip_group(q, last ? st.magic_last : st.magic);
+    const uint32_t grp = strip_group(q, magic);
     const uint32_t x = q - grp * width;
     const bool valid = grp * 4u < (uint32_t)g.L;
     uint32_t anti = 0, up = 0;
     ItemMasks acc;
     if (UPDATE) {
         const uint64_t t = sweep_number(a);
-        first_products(tab, w0, width, philox_first_key((uint32_t)t, a.rk));
+        first_products(tab, w0, width, magic, philox_first_key((uint32_t)t, a.rk));
         if (valid) {
             const FirstTable first = {tab + x};
             draw_item<ROUNDS>(first, grp, t, C, a.rk, a.thr0, a.thr1, a.all0, a.all1, acc);

@@ -562,7 +562,7 @@ Strips make_strips(const Geom& g, int most)
     st.width = ((uint32_t)g.W + st.n - 1) / st.n;               // strips of about equal width
     st.n = ((uint32_t)g.W + st.width - 1) / st.width;
     st.last = (uint32_t)g.W - (st.n - 1) * st.width;
-    // q < 2^18 and width <= 32, so hi32(q * ceil(2^32 / width)) = q / width
+    // q < 2^18 and width <= 16, so hi32(q * ceil(2^32 / width)) = q / width
     auto magic = [](uint32_t w) { return w == 1 ? 0u : (uint32_t)(((1ull << 32) + w - 1) / w); };
     st.magic = magic(st.width);
     st.magic_last = magic(st.last);
