@@ -65,7 +65,10 @@ batch_half_sweep_kernel(const BatchReplica* __restrict__ reps, const BatchTile* 
     const BatchTile tile = tiles[blockIdx.x];
     const BatchReplica* R = reps + tile.rep;
     const uint32_t s = *chunk_base + s_local;      // sweep of this run, 1-based
-    if (s > R->nsweeps) return;                    // uniform over the block
+    if (s > R->nsweeps) {                          // uniform over the block
+        pdl_wait();    // every block waits, so a grid that has completed implies all those before it
+        return;
+    }
     const Geom g = R->g;
     const uint32_t w0 = tile.strip & 0xffffu, width = tile.strip >> 16;
     const uint32_t q = tile.first + threadIdx.x;
