@@ -433,7 +433,7 @@ __device__ __forceinline__ void apply_item(uint64_t* own, const uint64_t* other,
 // with the word logic and index arithmetic trimmed at the same time).  Strips
 // of at most 32 / 24 / 20 / 16 / 12 words (blocks of 128, sweeps without
 // records): 1,537 / 1,551 / 1,558 / 1,567 / 1,574, but L = 2016: 1,136 /
-// 1,144 / 1,153 / 1,159 / 1,124; a 16-word strip reads whole 128-byte lines.
+// 1,144 / 1,153 / 1,159 / 1,124; 16 words are 128 bytes of a row.
 struct Strips {
     uint32_t n;              // strips
     uint32_t width, last;    // words of a strip, of the last one
