@@ -129,8 +129,7 @@ int ising_get_thresholds(ising_lattice *h, uint64_t host_thr[2]);
 /* Run n >= 0 full sweeps t+1 .. t+n (t += n).  A sweep is the paper's Monte
  * Carlo iteration (Sec. 2: every spin proposed once), in checkerboard order:
  * all colour-0 sites, then all colour-1 sites.  Asynchronous on the stream
- * (the first call on the on-chip path or with graph replays allocates its
- * mask buffer), except on the cluster path with several clusters, where the
+ * (the first call on the on-chip path allocates its mask buffer), except on the cluster path with several clusters, where the
  * call synchronises the stream to read the status of the waits between
  * clusters.  Errors: EINVAL (NULL, n < 0), ENOMEM (that buffer), ETIMEOUT
  * (a wait between clusters gave up; see ising_set_clusters), ECUDA. */
@@ -141,7 +140,7 @@ int ising_sweep(ising_lattice *h, int64_t n);
  * each; either may be NULL.  n >= 0, 1 <= every <= 2^22.  Synchronises the stream.
  * The counts come from the reduction fused into the colour-1 half-sweep.
  * Errors: EINVAL (NULL, n < 0, every out of range), ENOMEM (the mask
- * buffer of the on-chip path or of the graph replays), ETIMEOUT (as for
+ * buffer of the on-chip path), ETIMEOUT (as for
  * ising_sweep), ECUDA. */
 int ising_sweep_record(ising_lattice *h, int64_t n, int64_t every,
                        int64_t *host_E, int64_t *host_M);
@@ -214,41 +213,36 @@ int ising_set_sweep(ising_lattice *h, uint64_t t);
 int ising_set_stream(ising_lattice *h, void *stream);
 
 /* Launch shape of the half-sweep kernels: rows_per_thread must be 4 (one
- * Philox call serves four rows).  block_words == 0 selects a 1-D grid over
- * the thread items (item = row group * W + word, no padding columns) with
- * block_groups threads per block, in {64, 128, 192, 256}.  Otherwise a 2-D
- * grid: block_words (threads along a row) in {16, 32, 64}; block_groups
- * (threads down the columns) in {1, 2, 4, 8, 16}; 32 <= block_words *
- * block_groups <= 256.  Default 4, 0, 128 (1-D, 128 threads).  Results do
- * not depend on the shape (the draws are keyed by site).  It shapes the
- * launches that draw inside the half-sweep: above 102400 thread items, and
- * the sweeps left over after the graph replays below that. */
+ * Philox call serves four rows).  The thread items (4 rows x 1 word) are
+ * numbered along strips of word columns, and each block owns consecutive
+ * items of one strip.  block_words == 0 selects strips of up to 16 words and
+ * block_groups threads per block, in {64, 128, 192, 256}.  Otherwise strips
+ * of up to min(block_words, 16) words, block_words in {16, 32, 64}, and
+ * block_words * block_groups threads, block_groups in {1, 2, 4, 8, 16};
+ * 32 <= block_words * block_groups <= 256.  Default 4, 0, 128 (128 threads).
+ * Results do not depend on the shape (the draws are keyed by site).  It
+ * shapes the launch path's half-sweeps with one lane per item.
+ */
 int ising_set_tiling(ising_lattice *h, int32_t rows_per_thread,
                      int32_t block_words, int32_t block_groups);
 
 /* Lanes per thread item on the launch path: 1, 2, 4 or 8, or 0 (default)
- * for the library's choice by lattice size (4 up to 8192 items, i.e. L up to
- * about 1100; 1 above).  With F lanes, lane q of an item
+ * for the library's choice (1).  With F > 1 lanes, lane q of an item
  * (4 rows x 1 word) draws the fields q, q + F, ... and the lanes merge their
  * accept bits with warp shuffles: F times the threads, each with 1/F of the
- * item's Philox calls.  This fills the GPU for lattices whose one thread
- * per item would leave SMs idle.  It applies to the launches that draw
- * inside the half-sweep (the sweeps left over after the graph replays,
- * whose half-sweeps apply masks drawn ahead).  No counterpart in the paper
+ * item's Philox calls.  No counterpart in the paper
  * (a scheduling choice); results do not depend on it.  Row-packed layout
  * only (EINVAL otherwise; EINVAL for other values). */
 int ising_set_item_lanes(ising_lattice *h, int32_t lanes);
 
 /* Execution path of ising_sweep / ising_sweep_record.  ISING_PATH_LAUNCHES:
- * two kernel launches per sweep, all SMs; up to 102400 thread items (L up
- * to about 4100, either layout) the launches of chunks of up to 32 sweeps are
+ * two kernel launches per sweep, all SMs, each launch's draws running while
+ * the one before finishes; up to 32768 thread items (L up
+ * to about 2350, either layout) the launches of chunks of up to 32 sweeps are
  * captured once into CUDA graphs and replayed (recaptured after
  * ising_set_beta, ising_set_rng, ising_set_tiling, ising_set_item_lanes; a
  * device record index picks the count slots of each replay), because there
- * a half-sweep runs about as long as the host takes to launch it.  These
- * graphs draw the accept masks of up to 8 sweeps at a time on all SMs, into
- * two buffers the library allocates on first use (at most 33.5 MB), and
- * their half-sweeps only apply them.
+ * a half-sweep runs about as long as the host takes to launch it.
  * ISING_PATH_RESIDENT: temporal
  * blocking with the whole lattice on chip -- one block copies both colour
  * arrays into shared memory and runs all requested sweeps there in one

@@ -104,21 +104,10 @@ __device__ __forceinline__ void ci_cl_update(uint64_t* E, const uint64_t* msk, u
     const uint64_t xl = word_ld<false>(oth, o - 1u + par, nw, __LINE__);
     const uint64_t xr = word_ld<false>(oth, o + par, nw, __LINE__);
     const uint64_t p = word_ld<false>(msk, o, nw, __LINE__);
-    // Eq. 3 summed bitwise (as the row-packed kernels do): with x_n = s ^ n
-    // the field's spin bit of x_n is set iff neighbour n is anti-aligned;
-    // a >= 1 is their OR, a >= 2 that two of them are set.  The same
-    // decisions as the carry-free 3-bit field sum of the other interleaved
-    // kernels, in fewer instructions.
-    const uint64_t x1 = s ^ xu, x2 = s ^ xd, x3 = s ^ xl, x4 = s ^ xr;
-    const uint64_t any = x1 | x2 | x3 | x4;
-    const uint64_t ge2 = (x1 & x2) | (x3 & x4) | ((x1 ^ x2) & (x3 ^ x4));
-    const uint64_t accept = ge2 | (any & p) | (~any & (p >> 1));
-    const uint64_t sn = s ^ (accept & kAllFields);
+    const uint64_t sn = ci_flip(s, xu, xd, xl, xr, (uint32_t)p, (uint32_t)(p >> 32));
     word_st(own, o, sn, nw, __LINE__);
     if (RECORD) {
-        const uint64_t pair_other = par ? xl : xr;       // the pair's other word
-        anti += __popcll(sn ^ xu) + __popcll(sn ^ xd) + __popcll(sn ^ xl) + __popcll(sn ^ xr);
-        up += __popcll(sn) + __popcll(pair_other);
+        ci_count(sn, xu, xd, xl, xr, par ? xl : xr, anti, up);    // par ? xl : xr: the pair's other word
     }
 }
 
@@ -359,27 +348,27 @@ ci_cluster_sweeps_kernel(CiClusterArgs a)
     }
 }
 
-// Masks of sweeps j = 0 .. nsweeps-1 after sweep t0, one thread per (sweep,
-// colour, row group q, column pair m) with ci_masks, written as planes:
-// masks[((j * 2 + c) * N + 4 q + e) * L/2 + m], with the bits of a
-// threshold of 2^32 set.
+// Masks of sweeps j = 0 .. nsweeps-1 after sweep t0, one thread per (row group
+// q, column pair m) of a block and one grid layer per (sweep, colour), with
+// ci_masks, written as planes: masks[((j * 2 + c) * N + 4 q + e) * L/2 + m],
+// with the bits of a threshold of 2^32 set.
 template <int ROUNDS>
-__global__ void __launch_bounds__(128)
-ci_cl_mask_draw_kernel(int L, int N, SweepArgs a, uint64_t t0, int nsweeps, uint64_t* __restrict__ masks)
+__global__ void __launch_bounds__(kCiBlockX * kCiBlockY, 8)
+ci_cl_mask_draw_kernel(int L, int N, SweepArgs a, uint64_t t0, uint64_t* __restrict__ masks)
 {
-    const long long Q4 = N / 4, M = L / 2;
-    const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= (long long)nsweeps * 2 * Q4 * M) return;
-    const int m = (int)(k % M);
-    const int q = (int)((k / M) % Q4);
-    const int jc = (int)(k / (M * Q4));                 // sweep * 2 + colour
-    uint64_t packed[4];
-    ci_masks<ROUNDS>(N, q, m, t0 + (uint64_t)(jc >> 1) + 1, jc & 1, a, packed);
-    const uint64_t always = (((uint64_t)a.all1 << 32 | a.all1) & kAllFields) |
-                            ((((uint64_t)a.all0 << 32 | a.all0) & kAllFields) << 1);
+    __shared__ CiRowTable tab;
+    const int x = (int)threadIdx.x % kCiBlockX, y = (int)threadIdx.x / kCiBlockX;
+    const int M = L / 2, m = (int)blockIdx.x * kCiBlockX + x, q = (int)blockIdx.y * kCiBlockY + y;
+    const int jc = (int)blockIdx.z;                     // sweep * 2 + colour
+    const uint64_t t = t0 + (uint64_t)(jc >> 1) + 1;
+    ci_row_keys(tab, N, (int)blockIdx.y * kCiBlockY, t, jc & 1, a);
+    if (m >= M || q >= N / 4) return;
+    ItemMasks acc;
+    ci_masks<ROUNDS>(tab, y, m, t, a, acc);
     uint64_t* plane = masks + (size_t)jc * N * M;
 #pragma unroll
-    for (int e = 0; e < 4; ++e) plane[(size_t)(4 * q + e) * M + m] = packed[e] | always;
+    for (int e = 0; e < 4; ++e)
+        plane[(size_t)(4 * q + e) * M + m] = (uint64_t)acc.m[e][1] << 32 | acc.m[e][0];
 }
 
 // The widest block's columns: c0(b + 1) - c0(b) <= 4 ceil((L / 4) / C).
@@ -500,18 +489,17 @@ cudaError_t ci_cl_mask_draw(int L, const SweepArgs& a, uint64_t t0, int nsweeps,
                             cudaStream_t s)
 {
     const int N = L / 21;
-    const long long threads = (long long)nsweeps * 2 * (N / 4) * (L / 2);
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)((threads + 127) / 128));
-    cfg.blockDim = dim3(128);
+    cfg.gridDim = dim3((L / 2 + kCiBlockX - 1) / kCiBlockX, (N / 4 + kCiBlockY - 1) / kCiBlockY, 2 * nsweeps);
+    cfg.blockDim = dim3(kCiBlockX * kCiBlockY);
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = overlap ? 1 : 0;
-    return a.rounds == 7 ? cudaLaunchKernelEx(&cfg, ci_cl_mask_draw_kernel<7>, L, N, a, t0, nsweeps, masks)
-                         : cudaLaunchKernelEx(&cfg, ci_cl_mask_draw_kernel<10>, L, N, a, t0, nsweeps, masks);
+    return a.rounds == 7 ? cudaLaunchKernelEx(&cfg, ci_cl_mask_draw_kernel<7>, L, N, a, t0, masks)
+                         : cudaLaunchKernelEx(&cfg, ci_cl_mask_draw_kernel<10>, L, N, a, t0, masks);
 }
 
 cudaError_t ci_cluster_sweeps(uint64_t* S, int L, const SweepArgs& a, const ClusterPlan& plan, int nsweeps,

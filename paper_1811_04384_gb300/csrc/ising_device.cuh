@@ -65,16 +65,10 @@ __device__ __forceinline__ void pdl_enter()
     pdl_wait();
 }
 
-// The sweep number of a half-sweep; where the counter is on the device, after
-// the grids that advance it.
-__device__ __forceinline__ uint64_t sweep_number(const SweepArgs& a)
-{
-    if (a.t_base) {
-        pdl_wait();
-        return *a.t_base + a.t_off;
-    }
-    return a.t0 + a.t_off;
-}
+// The sweep number of a half-sweep, read before the wait: the device counter
+// is advanced only by a plain launch at the end of a chunk (or graph), which
+// the half-sweeps of the next chunk start after.
+__device__ __forceinline__ uint64_t sweep_number(const SweepArgs& a) { return (a.t_base ? *a.t_base : a.t0) + a.t_off; }
 
 // ---- Checked build (compiled with -DISING_CHECKED) -------------------------
 // Every lattice-word access of the sweep routines goes through word_ld /
@@ -290,43 +284,50 @@ struct FirstTable {
     }
 };
 
-// Fields k .. 20 of one Philox row group (compile-time k: immediate bit masks).
-template <int k, int ROUNDS, typename First>
-struct FieldLoop {
-    __device__ __forceinline__ static void run(const First& first, const PhiloxRowKey& pk, const PhiloxKeys& rk,
-                                               ItemMasks& acc, uint32_t thr0, uint32_t thr1)
+// The calls of an item's 21 fields, one row group: from the row group's key and
+// the fields' first products.
+template <typename First>
+struct RowCalls {
+    First first;
+    PhiloxRowKey pk;
+    template <int ROUNDS>
+    __device__ __forceinline__ void call(int k, const PhiloxKeys& rk, uint32_t rnd[4]) const
     {
-        uint32_t hi, lo, rnd[4];
+        uint32_t hi, lo;
         first.get(k, hi, lo);
         philox_row_tail<ROUNDS>(pk, rk, hi, lo, rnd);
+    }
+};
+
+// Fields k .. 20 (compile-time k: immediate bit masks); call k gives the draws
+// of field k of four rows.
+template <int k, int ROUNDS, typename Calls>
+struct FieldLoop {
+    __device__ __forceinline__ static void run(const Calls& calls, const PhiloxKeys& rk, ItemMasks& acc,
+                                               uint32_t thr0, uint32_t thr1)
+    {
+        uint32_t rnd[4];
+        calls.template call<ROUNDS>(k, rk, rnd);
         constexpr int half = k <= 10 ? 0 : 1;
         constexpr int B = k <= 10 ? 3 * k : 3 * k - 32;
 #pragma unroll
         for (int e = 0; e < 4; ++e) accept_insert<B>(acc.m[e][half], rnd[e], thr0, thr1);
-        FieldLoop<k + 1, ROUNDS, First>::run(first, pk, rk, acc, thr0, thr1);
+        FieldLoop<k + 1, ROUNDS, Calls>::run(calls, rk, acc, thr0, thr1);
     }
 };
-template <int ROUNDS, typename First>
-struct FieldLoop<kFields, ROUNDS, First> {
-    __device__ __forceinline__ static void run(const First&, const PhiloxRowKey&, const PhiloxKeys&, ItemMasks&,
-                                               uint32_t, uint32_t)
-    {
-    }
+template <int ROUNDS, typename Calls>
+struct FieldLoop<kFields, ROUNDS, Calls> {
+    __device__ __forceinline__ static void run(const Calls&, const PhiloxKeys&, ItemMasks&, uint32_t, uint32_t) {}
 };
 
-// The masks of row group grp at sweep t, colour `colour` (Sec. 2 steps 2-3;
-// one Philox call covers the four rows of one field).
-template <int ROUNDS, typename First>
-__device__ __forceinline__ void draw_item(const First& first, uint32_t grp, uint64_t t, int colour,
-                                          const PhiloxKeys& rk, uint32_t thr0, uint32_t thr1, uint32_t all0w,
-                                          uint32_t all1w, ItemMasks& acc)
+// The masks of the 21 fields of `calls` (Sec. 2 steps 2-3).
+template <int ROUNDS, typename Calls>
+__device__ __forceinline__ void draw_fields(const Calls& calls, const PhiloxKeys& rk, uint32_t thr0, uint32_t thr1,
+                                            uint32_t all0w, uint32_t all1w, ItemMasks& acc)
 {
 #pragma unroll
     for (int e = 0; e < 4; ++e) acc.m[e][0] = acc.m[e][1] = 0;
-    const uint32_t tl = (uint32_t)t;
-    const uint32_t th = ((uint32_t)(t >> 32) << 1) | (uint32_t)colour;
-    const PhiloxRowKey pk = philox_row_key(grp, tl, th, rk);
-    FieldLoop<0, ROUNDS, First>::run(first, pk, rk, acc, thr0, thr1);
+    FieldLoop<0, ROUNDS, Calls>::run(calls, rk, acc, thr0, thr1);
     if (all1w | all0w) {     // a threshold of 2^32 accepts always
         const uint64_t a = ((((uint64_t)all1w << 32 | all1w) & kSpinBits)) |
                            ((((uint64_t)all0w << 32 | all0w) & kSpinBits) << 1);
@@ -336,6 +337,20 @@ __device__ __forceinline__ void draw_item(const First& first, uint32_t grp, uint
             acc.m[e][1] |= (uint32_t)(a >> 32);
         }
     }
+}
+
+// The high counter word of colour c at sweep t.
+__device__ __forceinline__ uint32_t counter_high(uint64_t t, int c) { return ((uint32_t)(t >> 32) << 1) | (uint32_t)c; }
+
+// The masks of row group grp at sweep t, colour `colour` (one Philox call
+// covers the four rows of one field).
+template <int ROUNDS, typename First>
+__device__ __forceinline__ void draw_item(const First& first, uint32_t grp, uint64_t t, int colour,
+                                          const PhiloxKeys& rk, uint32_t thr0, uint32_t thr1, uint32_t all0w,
+                                          uint32_t all1w, ItemMasks& acc)
+{
+    const RowCalls<First> calls = {first, philox_row_key(grp, (uint32_t)t, counter_high(t, colour), rk)};
+    draw_fields<ROUNDS>(calls, rk, thr0, thr1, all0w, all1w, acc);
 }
 
 // Update (and/or record) rows 4 grp .. 4 grp + 3 (those below L) of word

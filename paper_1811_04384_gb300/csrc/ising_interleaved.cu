@@ -66,45 +66,31 @@ __global__ void ci_unpack_kernel(const uint64_t* __restrict__ S, int L, int N, i
         s[(size_t)(I + k * N) * L + J] = ((word >> (3 * k)) & 1ull) ? (int8_t)1 : (int8_t)-1;
 }
 
-// The masks of ci_half_sweep_kernel for the sweeps j = 0 .. nsweeps-1 after
-// sweep (t_base ? *t_base : 0) + t0, drawn ahead on all SMs: one thread per
-// (j, colour, q, m), masks[(((j * 2 + colour) * N/4 + q) * L/2 + m) * 4 + e]
-// = packed masks of word row 4q + e.
-template <int ROUNDS>
-__global__ void __launch_bounds__(128)
-ci_mask_draw_kernel(int L, int N, SweepArgs a, const uint64_t* t_base, uint64_t t0, int nsweeps,
-                    uint64_t* __restrict__ masks)
-{
-    const long long Q = N / 4, M = L / 2;
-    const long long total = (long long)nsweeps * 2 * Q * M;
-    const uint64_t tb = (t_base ? *t_base : 0) + t0 + 1;
-    for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < total;
-         k += (long long)gridDim.x * blockDim.x) {
-        const int m = (int)(k % M);
-        const int q = (int)((k / M) % Q);
-        const int colour = (int)((k / (M * Q)) & 1);
-        const int j = (int)(k / (2 * M * Q));
-        uint64_t packed[4];
-        ci_masks<ROUNDS>(N, q, m, tb + (uint64_t)j, colour, a, packed);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) masks[(size_t)k * 4 + e] = packed[e];
-    }
-}
-
 // One half-sweep of colour C.  Thread (m, q) owns word rows 4q .. 4q+3 and the
 // column pair 2m, 2m+1; in each row it updates the colour-C word
-// J_e = 2m + ((I_e + C) & 1).  Its accept masks come from ci_masks, or with
-// PRE from `masks` (this sweep and colour's block of ci_mask_draw_kernel).
-// RECORD (colour 1) also counts the anti-aligned bonds of the four colour-1
-// words and the up spins of all eight words of the block.
-template <int C, bool UPDATE, bool RECORD, int ROUNDS, bool PRE = false>
-__global__ void __launch_bounds__(128)
-ci_half_sweep_kernel(uint64_t* __restrict__ S, int L, int N, SweepArgs a, const uint64_t* __restrict__ masks)
+// J_e = 2m + ((I_e + C) & 1), with the masks of ci_masks.  The draws need
+// launch operands only and run before the wait for the previous half-sweep
+// (see half_sweep_kernel).  RECORD (colour 1) also counts the anti-aligned
+// bonds of the four colour-1 words and the up spins of all eight words of
+// the block.
+template <int C, bool UPDATE, bool RECORD, int ROUNDS>
+__global__ void __launch_bounds__(kCiBlockX * kCiBlockY, 6)
+ci_half_sweep_kernel(uint64_t* S, int L, int N, SweepArgs a)
 {
-    const int m = blockIdx.x * blockDim.x + threadIdx.x;
-    const int q = blockIdx.y * blockDim.y + threadIdx.y;
+    __shared__ CiRowTable tab;
+    pdl_launch();
+    const int x = (int)threadIdx.x % kCiBlockX, y = (int)threadIdx.x / kCiBlockX;
+    const int m = (int)blockIdx.x * kCiBlockX + x, q = (int)blockIdx.y * kCiBlockY + y;
+    const bool valid = m < L / 2 && q < N / 4;
     uint32_t anti = 0, up = 0;
-    if (m < L / 2 && q < N / 4) {
+    ItemMasks acc;
+    if (UPDATE) {
+        const uint64_t t = sweep_number(a);
+        ci_row_keys(tab, N, (int)blockIdx.y * kCiBlockY, t, C, a);
+        if (valid) ci_masks<ROUNDS>(tab, y, m, t, a, acc);
+    }
+    pdl_wait();
+    if (valid) {
         const uint64_t n = (uint64_t)N * L;
         uint64_t s[4], xl[4], xr[4], xu[4], xd[4], other[4];
         int J[4];
@@ -116,50 +102,22 @@ ci_half_sweep_kernel(uint64_t* __restrict__ S, int L, int N, SweepArgs a, const 
             const int Jr = J[e] == L - 1 ? 0 : J[e] + 1;
             const uint64_t row = (uint64_t)I * L;
             s[e] = word_ld<false>(S, row + J[e], n, __LINE__);
-            xl[e] = word_ld<true>(S, row + Jl, n, __LINE__);
-            xr[e] = word_ld<true>(S, row + Jr, n, __LINE__);
+            xl[e] = word_ld<false>(S, row + Jl, n, __LINE__);
+            xr[e] = word_ld<false>(S, row + Jr, n, __LINE__);
             other[e] = (J[e] & 1) ? xl[e] : xr[e];    // the other word of the column pair
-            xu[e] = I == 0 ? rotate_up(word_ld<true>(S, (uint64_t)(N - 1) * L + J[e], n, __LINE__))
-                           : word_ld<true>(S, (uint64_t)(I - 1) * L + J[e], n, __LINE__);
-            xd[e] = I == N - 1 ? rotate_down(word_ld<true>(S, (uint64_t)J[e], n, __LINE__))
-                               : word_ld<true>(S, (uint64_t)(I + 1) * L + J[e], n, __LINE__);
+            xu[e] = I == 0 ? rotate_up(word_ld<false>(S, (uint64_t)(N - 1) * L + J[e], n, __LINE__))
+                           : word_ld<false>(S, (uint64_t)(I - 1) * L + J[e], n, __LINE__);
+            xd[e] = I == N - 1 ? rotate_down(word_ld<false>(S, (uint64_t)J[e], n, __LINE__))
+                               : word_ld<false>(S, (uint64_t)(I + 1) * L + J[e], n, __LINE__);
         }
-        // c1: r < thr1 at the spin bits; c0 >> 1 of the same word: r < thr0 there
-        // (its other bits fall on no spin bit and are masked below)
-        uint64_t c0[4] = {0, 0, 0, 0}, c1[4] = {0, 0, 0, 0};
-        if (UPDATE) {
-            uint64_t packed[4];
-            if (PRE) {
-#pragma unroll
-                for (int e = 0; e < 4; ++e) packed[e] = __ldg(masks + ((size_t)q * (L / 2) + m) * 4 + e);
-            } else {
-                ci_masks<ROUNDS>(N, q, m, sweep_number(a), C, a, packed);
-            }
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                c1[e] = packed[e];
-                c0[e] = packed[e] >> 1;
-            }
-        }
-        const uint64_t all0 = ((uint64_t)a.all0 << 32 | a.all0) & kAllFields;
-        const uint64_t all1 = ((uint64_t)a.all1 << 32 | a.all1) & kAllFields;
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-            const int I = 4 * q + e;
             uint64_t sn = s[e];
             if (UPDATE) {
-                // Eq. 3: each XOR field is 0/1, so the 3-bit sums hold a = 0..4 without carries
-                const uint64_t A = (s[e] ^ xu[e]) + (s[e] ^ xd[e]) + (s[e] ^ xl[e]) + (s[e] ^ xr[e]);
-                const uint64_t ge2 = ((A >> 1) | (A >> 2)) & kAllFields;           // a >= 2: dE <= 0
-                const uint64_t any = (A | (A >> 1) | (A >> 2)) & kAllFields;       // a >= 1
-                const uint64_t accept = ge2 | (any & (c1[e] | all1)) | (~any & (c0[e] | all0));
-                sn = s[e] ^ (accept & kAllFields);
-                word_st(S, (uint64_t)I * L + J[e], sn, n, __LINE__);
+                sn = ci_flip(s[e], xu[e], xd[e], xl[e], xr[e], acc.m[e][0], acc.m[e][1]);
+                word_st(S, (uint64_t)(4 * q + e) * L + J[e], sn, n, __LINE__);
             }
-            if (RECORD) {
-                anti += __popcll(sn ^ xu[e]) + __popcll(sn ^ xd[e]) + __popcll(sn ^ xl[e]) + __popcll(sn ^ xr[e]);
-                up += __popcll(sn) + __popcll(other[e]);
-            }
+            if (RECORD) ci_count(sn, xu[e], xd[e], xl[e], xr[e], other[e], anti, up);
         }
     }
     if (RECORD) {
@@ -221,7 +179,8 @@ __device__ __forceinline__ void rw_draw(const SweepArgs& a, uint32_t step, uint3
     }
     I = __umulhi(w[0], (uint32_t)N);
     jr = __umulhi(w[1], (uint32_t)h);
-    uint64_t m = 0;
+    uint64_t m = (((uint64_t)a.all1 << 32 | a.all1) & kAllFields) |
+                 ((((uint64_t)a.all0 << 32 | a.all0) & kAllFields) << 1);
 #pragma unroll
     for (int k = 0; k < 21; ++k)
         m |= (uint64_t)(w[2 + k] < a.thr1) << (3 * k) | (uint64_t)(w[2 + k] < a.thr0) << (3 * k + 1);
@@ -277,8 +236,6 @@ ci_rw_phase_kernel(uint64_t* S, int L, int N, int NC, int phase, SweepArgs a, co
     const uint32_t tl = (uint32_t)t;
     const uint32_t x3 = 0x80000000u | ((uint32_t)(t >> 32) << 1) | (uint32_t)phase;
     const ulonglong2* my_draws = PRE ? draws + (size_t)q * U : nullptr;   // this phase's block of draws
-    const uint64_t all1 = ((uint64_t)a.all1 << 32 | a.all1) & kAllFields;
-    const uint64_t all0 = ((uint64_t)a.all0 << 32 | a.all0) & kAllFields;
     constexpr uint32_t B = kRwBuckets - 1;
     const int hw = h + 2;                                // window row: the column before, h, the column after
     const uint64_t n_lat = (uint64_t)N * L, n_win = (uint64_t)N * hw;
@@ -387,14 +344,8 @@ ci_rw_phase_kernel(uint64_t* S, int L, int N, int NC, int phase, SweepArgs a, co
                 didx = row + J;
                 dn = n_lat;
             }
-            // Eq. 3: the 3-bit field sums hold a = 0..4 without carries
-            const uint64_t A = (s ^ xu) + (s ^ xd) + (s ^ xl) + (s ^ xr);
-            const uint64_t ge2 = ((A >> 1) | (A >> 2)) & kAllFields;
-            const uint64_t any = (A | (A >> 1) | (A >> 2)) & kAllFields;
             const uint64_t m = sl_mask[buf][tid];
-            const uint64_t c1 = (m & kAllFields) | all1, c0 = ((m >> 1) & kAllFields) | all0;
-            const uint64_t accept = ge2 | (any & c1) | (~any & c0);
-            word_st(dst, didx, s ^ (accept & kAllFields), dn, __LINE__);
+            word_st(dst, didx, ci_flip(s, xu, xd, xl, xr, (uint32_t)m, (uint32_t)(m >> 32)), dn, __LINE__);
         }
         __syncthreads();
         // the updates that did not run keep their order at the front
@@ -426,55 +377,6 @@ ci_rw_phase_kernel(uint64_t* S, int L, int N, int NC, int phase, SweepArgs a, co
                     n_lat, __LINE__);
         }
     }
-}
-
-// The apply-only half-sweep of the graph replays with one word per thread:
-// thread k updates the colour-C word of word row I = k / (L / 2) in column
-// pair m = k % (L / 2) with its masks from ci_mask_draw_kernel (`masks`: this
-// sweep and colour's block, entry (q * L/2 + m) * 4 + e for I = 4q + e).  The
-// spin logic is ci_half_sweep_kernel's; four times its threads, each with a
-// quarter of the work, so a short half-sweep is not bound by the latency of
-// a few threads' chains.  RECORD counts the colour-1 word's anti-aligned
-// bonds and the up spins of both words of the column pair.
-template <int C, bool RECORD>
-__global__ void __launch_bounds__(128)
-ci_half_sweep_apply_kernel(uint64_t* __restrict__ S, int L, int N, SweepArgs a, const uint64_t* __restrict__ masks)
-{
-    pdl_enter();
-    const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
-    const uint32_t half = (uint32_t)L / 2;
-    uint32_t anti = 0, up = 0;
-    if (k < (uint32_t)N * half) {
-        const uint64_t n = (uint64_t)N * L;
-        const int I = (int)(k / half), m = (int)(k - (uint32_t)I * half);
-        const int J = 2 * m + ((I + C) & 1);
-        const int Jl = J == 0 ? L - 1 : J - 1;
-        const int Jr = J == L - 1 ? 0 : J + 1;
-        const uint64_t row = (uint64_t)I * L;
-        const uint64_t s = word_ld<false>(S, row + J, n, __LINE__);
-        const uint64_t xl = word_ld<true>(S, row + Jl, n, __LINE__);
-        const uint64_t xr = word_ld<true>(S, row + Jr, n, __LINE__);
-        const uint64_t xu = I == 0 ? rotate_up(word_ld<true>(S, (uint64_t)(N - 1) * L + J, n, __LINE__))
-                                   : word_ld<true>(S, (uint64_t)(I - 1) * L + J, n, __LINE__);
-        const uint64_t xd = I == N - 1 ? rotate_down(word_ld<true>(S, (uint64_t)J, n, __LINE__))
-                                       : word_ld<true>(S, (uint64_t)(I + 1) * L + J, n, __LINE__);
-        const uint64_t packed = __ldg(masks + ((size_t)(I >> 2) * half + m) * 4 + (I & 3));
-        const uint64_t all0 = ((uint64_t)a.all0 << 32 | a.all0) & kAllFields;
-        const uint64_t all1 = ((uint64_t)a.all1 << 32 | a.all1) & kAllFields;
-        // Eq. 3: each XOR field is 0/1, so the 3-bit sums hold a = 0..4 without carries
-        const uint64_t A = (s ^ xu) + (s ^ xd) + (s ^ xl) + (s ^ xr);
-        const uint64_t ge2 = ((A >> 1) | (A >> 2)) & kAllFields;
-        const uint64_t any = (A | (A >> 1) | (A >> 2)) & kAllFields;
-        const uint64_t accept = ge2 | (any & (packed | all1)) | (~any & ((packed >> 1) | all0));
-        const uint64_t sn = s ^ (accept & kAllFields);
-        word_st(S, row + J, sn, n, __LINE__);
-        if (RECORD) {
-            const uint64_t other = (J & 1) ? xl : xr;    // the other word of the column pair
-            anti += __popcll(sn ^ xu) + __popcll(sn ^ xd) + __popcll(sn ^ xl) + __popcll(sn ^ xr);
-            up += __popcll(sn) + __popcll(other);
-        }
-    }
-    if (RECORD) block_add_counts(record_counts(a) + 2 * (blockIdx.x % kCountSlots), anti, up);
 }
 
 }  // namespace
@@ -559,59 +461,23 @@ cudaError_t ci_unpack(const uint64_t* S, int L, int8_t* spins, cudaStream_t s)
 }
 
 template <int ROUNDS>
-static void ci_launch_r(dim3 grid, dim3 block, int colour, bool update, bool record, uint64_t* S, int L, int N,
-                        const SweepArgs& a, cudaStream_t s)
+static void ci_launch_r(dim3 grid, int colour, bool update, bool record, uint64_t* S, int L, int N,
+                        const SweepArgs& a, bool in_graphs, cudaStream_t s)
 {
-    if (colour == 0) {
-        if (record) ci_half_sweep_kernel<0, true, true, ROUNDS><<<grid, block, 0, s>>>(S, L, N, a, nullptr);
-        else ci_half_sweep_kernel<0, true, false, ROUNDS><<<grid, block, 0, s>>>(S, L, N, a, nullptr);
-    } else if (!update) {
-        ci_half_sweep_kernel<1, false, true, 10><<<grid, block, 0, s>>>(S, L, N, a, nullptr);
-    } else {
-        if (record) ci_half_sweep_kernel<1, true, true, ROUNDS><<<grid, block, 0, s>>>(S, L, N, a, nullptr);
-        else ci_half_sweep_kernel<1, true, false, ROUNDS><<<grid, block, 0, s>>>(S, L, N, a, nullptr);
-    }
+    const dim3 block(kCiBlockX * kCiBlockY);
+    if (!update) ci_half_sweep_kernel<1, false, true, 10><<<grid, block, 0, s>>>(S, L, N, a);
+    else if (colour == 0) launch_pdl_opt(in_graphs, ci_half_sweep_kernel<0, true, false, ROUNDS>, grid, block, s, S, L, N, a);
+    else if (record) launch_pdl_opt(in_graphs, ci_half_sweep_kernel<1, true, true, ROUNDS>, grid, block, s, S, L, N, a);
+    else launch_pdl_opt(in_graphs, ci_half_sweep_kernel<1, true, false, ROUNDS>, grid, block, s, S, L, N, a);
 }
 
 cudaError_t ci_half_sweep(int colour, bool update, bool record, uint64_t* S, int L, const SweepArgs& a,
-                          cudaStream_t s)
+                          bool in_graphs, cudaStream_t s)
 {
     const int N = L / 21;
-    dim3 block(32, 4);
-    dim3 grid((L / 2 + 31) / 32, (N / 4 + 3) / 4);
-    if (a.rounds == 7) ci_launch_r<7>(grid, block, colour, update, record, S, L, N, a, s);
-    else ci_launch_r<10>(grid, block, colour, update, record, S, L, N, a, s);
-    return cudaGetLastError();
-}
-
-size_t ci_mask_bytes_per_sweep(int L) { return (size_t)8 * (L / 21) * L; }
-
-cudaError_t ci_mask_draw(int L, const SweepArgs& a, const uint64_t* t_base, uint64_t t0, int nsweeps,
-                         uint64_t* masks, int blocks_per_sm, cudaStream_t s)
-{
-    const int N = L / 21;
-    const long long threads = (long long)nsweeps * 2 * (N / 4) * (L / 2);
-    unsigned blocks = (unsigned)((threads + 127) / 128);
-    if (blocks_per_sm > 0) blocks = std::min(blocks, (unsigned)(device_sm_count() * blocks_per_sm));
-    if (a.rounds == 7) ci_mask_draw_kernel<7><<<blocks, 128, 0, s>>>(L, N, a, t_base, t0, nsweeps, masks);
-    else ci_mask_draw_kernel<10><<<blocks, 128, 0, s>>>(L, N, a, t_base, t0, nsweeps, masks);
-    return cudaGetLastError();
-}
-
-cudaError_t ci_half_sweep_pre(int colour, bool record, uint64_t* S, int L, const SweepArgs& a,
-                              const uint64_t* sweep_masks, cudaStream_t s)
-{
-    const int N = L / 21;
-    const uint64_t* m = sweep_masks + (size_t)colour * (N / 4) * (L / 2) * 4;
-    const unsigned threads = (unsigned)N * (unsigned)(L / 2);
-    const dim3 grid((threads + 127) / 128), block(128);
-    // programmatic dependent launch inside the graphs as for the row-packed
-    // apply half-sweeps: up to 8192 and from 80000 thread items
-    const int items = (N / 4) * (L / 2);
-    const bool in_graphs = items <= 8192 || items >= 80000;
-    if (colour == 0) launch_pdl_opt(in_graphs, ci_half_sweep_apply_kernel<0, false>, grid, block, s, S, L, N, a, m);
-    else if (record) launch_pdl_opt(in_graphs, ci_half_sweep_apply_kernel<1, true>, grid, block, s, S, L, N, a, m);
-    else launch_pdl_opt(in_graphs, ci_half_sweep_apply_kernel<1, false>, grid, block, s, S, L, N, a, m);
+    const dim3 grid((L / 2 + kCiBlockX - 1) / kCiBlockX, (N / 4 + kCiBlockY - 1) / kCiBlockY);
+    if (a.rounds == 7) ci_launch_r<7>(grid, colour, update, record, S, L, N, a, in_graphs, s);
+    else ci_launch_r<10>(grid, colour, update, record, S, L, N, a, in_graphs, s);
     return cudaGetLastError();
 }
 

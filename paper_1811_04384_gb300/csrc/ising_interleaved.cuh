@@ -22,26 +22,74 @@ __device__ __forceinline__ uint64_t rotate_down(uint64_t s)  // field k <- field
     return ((s >> 3) | (s << 60)) & kAllFields;
 }
 
-// Accept masks of the words of thread (m, q) of ci_half_sweep_kernel for
-// sweep t, colour C: Philox call k (counter (q + kN/4, m, t, C)) gives the
-// draws of field k of the four words.  packed[e] holds r < thr1 of field k
-// at bit 3k and r < thr0 at bit 3k + 1.
-template <int ROUNDS>
-__device__ __forceinline__ void ci_masks(int N, int q, int m, uint64_t t, int C, const SweepArgs& a,
-                                         uint64_t packed[4])
+// Accept masks of the words of column pair m in word rows 4q .. 4q + 3, colour
+// C, at sweep t: Philox call k (counter (q + kN/4, m, t, C)) gives the draws
+// of field k of the four words, in ItemMasks' form.  Along the 21 calls the
+// column stays and the row group changes, so the first product (column and
+// sweep) is the thread's own, once, and what depends on the row group alone
+// is shared by all columns of a block (ci_row_keys): 15 products per call, as
+// in the row-packed layout, where each call's own row key made them 19.
+constexpr int kCiBlockX = 32, kCiBlockY = 4;      // column pairs x word row groups of a block of 128
+using CiRowTable = uint4[kCiBlockY * kFields];
+
+// All threads of a block of kCiBlockX x kCiBlockY (1-D thread index): the row
+// keys of row groups q0 .. q0 + kCiBlockY - 1.
+__device__ __forceinline__ void ci_row_keys(uint4* tab, int N, int q0, uint64_t t, int C, const SweepArgs& a)
 {
-    const uint32_t tl = (uint32_t)t;
-    const uint32_t th = ((uint32_t)(t >> 32) << 1) | (uint32_t)C;
-#pragma unroll
-    for (int e = 0; e < 4; ++e) packed[e] = 0;
-    for (int k = 0; k < 21; ++k) {
-        const PhiloxRowKey pk = philox_row_key((uint32_t)(q + k * (N / 4)), tl, th, a.rk);
-        uint32_t r[4];
-        philox_row<ROUNDS>(pk, a.rk, (uint32_t)m, r);
-#pragma unroll
-        for (int e = 0; e < 4; ++e)
-            packed[e] |= (uint64_t)(r[e] < a.thr1) << (3 * k) | (uint64_t)(r[e] < a.thr0) << (3 * k + 1);
+    static_assert(kCiBlockX * kCiBlockY >= kCiBlockY * kFields, "one entry per thread");
+    const int e = (int)threadIdx.x;
+    if (e < kCiBlockY * kFields) {
+        const int y = e / kFields, k = e - y * kFields;
+        const PhiloxRowKey pk =
+            philox_row_key((uint32_t)(q0 + y + k * (N / 4)), (uint32_t)t, counter_high(t, C), a.rk);
+        tab[e] = make_uint4(pk.y3k, pk.z1k, pk.hiC, pk.v3);
     }
+    __syncthreads();
+}
+
+struct CiCalls {
+    const uint4* keys;        // the thread's row group in the table
+    uint32_t hi, lo;          // the column's first product
+    template <int ROUNDS>
+    __device__ __forceinline__ void call(int k, const PhiloxKeys& rk, uint32_t rnd[4]) const
+    {
+        const uint4 e = keys[k];
+        const PhiloxRowKey pk = {0, e.x, e.y, e.z, e.w};
+        philox_row_tail<ROUNDS>(pk, rk, hi, lo, rnd);
+    }
+};
+
+// `tab` from ci_row_keys for the thread's t and C; y the row group in it.
+template <int ROUNDS>
+__device__ __forceinline__ void ci_masks(const uint4* tab, int y, int m, uint64_t t, const SweepArgs& a,
+                                         ItemMasks& acc)
+{
+    CiCalls calls;
+    calls.keys = tab + y * kFields;
+    mul_hilo(kPhiloxM0, philox_first_key((uint32_t)t, a.rk) ^ (uint32_t)m, calls.hi, calls.lo);
+    draw_fields<ROUNDS>(calls, a.rk, a.thr0, a.thr1, a.all0, a.all1, acc);
+}
+
+// The update of one word (flip_half on both halves): s, its four neighbours
+// and the masks (lo, hi) of the word.
+__device__ __forceinline__ uint64_t ci_flip(uint64_t s, uint64_t xu, uint64_t xd, uint64_t xl, uint64_t xr,
+                                            uint32_t mlo, uint32_t mhi)
+{
+    const uint32_t lo = flip_half((uint32_t)s, (uint32_t)xu, (uint32_t)xd, (uint32_t)xl, (uint32_t)xr, mlo,
+                                  __funnelshift_r(mlo, mhi, 1), (uint32_t)kAllFields);
+    const uint32_t hi = flip_half((uint32_t)(s >> 32), (uint32_t)(xu >> 32), (uint32_t)(xd >> 32),
+                                  (uint32_t)(xl >> 32), (uint32_t)(xr >> 32), mhi, mhi >> 1,
+                                  (uint32_t)(kAllFields >> 32));
+    return (uint64_t)hi << 32 | lo;
+}
+
+// Anti-aligned bonds of the updated word and the up spins of it and `other`.
+__device__ __forceinline__ void ci_count(uint64_t s, uint64_t xu, uint64_t xd, uint64_t xl, uint64_t xr,
+                                         uint64_t other, uint32_t& anti, uint32_t& up)
+{
+    // three fields of one spin bit each fit one field
+    anti += __popcll((s ^ xu) | (s ^ xd) << 1 | (s ^ xl) << 2) + __popcll(s ^ xr);
+    up += __popcll(s | other << 1);
 }
 
 }  // namespace

@@ -15,19 +15,9 @@ cudaError_t ci_init_hot(uint64_t* S, int L, uint64_t seed, cudaStream_t s);
 cudaError_t ci_init_cold(uint64_t* S, int L, int up, cudaStream_t s);
 cudaError_t ci_pack(uint64_t* S, int L, const int8_t* spins, cudaStream_t s);
 cudaError_t ci_unpack(const uint64_t* S, int L, int8_t* spins, cudaStream_t s);
+// colour 0 does not record; in_graphs as for launch_half_sweep (ising_internal.h).
 cudaError_t ci_half_sweep(int colour, bool update, bool record, uint64_t* S, int L, const SweepArgs& a,
-                          cudaStream_t s);
-// Masks drawn ahead: ci_mask_draw fills `masks` with the accept masks of the
-// nsweeps sweeps after sweep (t_base ? *t_base : 0) + t0 (both colours,
-// ci_mask_bytes_per_sweep(L) bytes per sweep), with at most blocks_per_sm
-// 128-thread blocks per SM (0: one thread per unit); ci_half_sweep_pre
-// applies the block of one sweep (`sweep_masks`) to colour `colour`.
-size_t ci_mask_bytes_per_sweep(int L);
-cudaError_t ci_mask_draw(int L, const SweepArgs& a, const uint64_t* t_base, uint64_t t0, int nsweeps,
-                         uint64_t* masks, int blocks_per_sm, cudaStream_t s);
-cudaError_t ci_half_sweep_pre(int colour, bool record, uint64_t* S, int L, const SweepArgs& a,
-                              const uint64_t* sweep_masks, cudaStream_t s);
-
+                          bool in_graphs, cudaStream_t s);
 // The paper's random-word chain (Sec. 4-5, Appendix A): iteration
 // *a.t_base + a.t_off, phase 0 (the left floor(NC/2) columns of each of the
 // nstrips strips of NC = L / nstrips columns) then phase 1 (the rest), one

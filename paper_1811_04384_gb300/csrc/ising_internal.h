@@ -55,9 +55,8 @@ cudaError_t allow_resident_smem(int bytes);
 cudaError_t launch_resident(uint64_t* w0, uint64_t* w1, const Geom& g, const SweepArgs& a, uint64_t t0, int n,
                             int every, long long* rec, size_t bytes, cudaStream_t s);
 // The on-chip path with masks drawn beforehand: draw the masks of the nsweeps
-// sweeps after sweep (t_base ? *t_base : 0) + t0 (nsweeps * items * 4
-// entries), then run sweeps s_base+1 ..
-// s_base+n of a run reading them (at most kPremaskedMaxItems items, one or
+// sweeps after sweep t0 (nsweeps * items * 4 entries), then run sweeps
+// s_base+1 .. s_base+n of a run reading them (at most kPremaskedMaxItems items, one or
 // two rows per thread of one block; `bytes` = both colour arrays, and
 // allow_resident_smem(bytes) leaves room for 1024 record counters).
 constexpr int kPremaskedMaxItems = 512;
@@ -67,16 +66,8 @@ inline int premasked_rows_per_thread(int items) { return items <= 256 ? 1 : 2; }
 // 32 / 64 / 100 against 0.57 / 0.44 / 0.45 / 0.87 with one, but 0.99
 // against 0.92 at L = 128 (128 items, 32 warps).
 inline int premasked_threads_per_row(int items) { return items <= 100 ? 2 : 1; }
-// blocks_per_sm > 0: at most that many 128-thread blocks per SM, each
-// looping over its share (0: one thread per sweep and item).
-cudaError_t launch_mask_draw(const Geom& g, const SweepArgs& a, const uint64_t* t_base, uint64_t t0, int nsweeps,
-                             ulonglong2* masks, int blocks_per_sm, cudaStream_t s);
-// SMs of the current device (1 if the query fails).
-int device_sm_count();
-// One half-sweep that applies masks drawn by launch_mask_draw (`masks`: the
-// entries of its sweep), one thread per row.
-cudaError_t launch_half_sweep_apply(int colour, bool record, uint64_t* own, const uint64_t* other, const Geom& g,
-                                    const SweepArgs& a, const ulonglong2* masks, cudaStream_t s);
+cudaError_t launch_mask_draw(const Geom& g, const SweepArgs& a, uint64_t t0, int nsweeps, ulonglong2* masks,
+                             cudaStream_t s);
 cudaError_t launch_resident_premasked(uint64_t* w0, uint64_t* w1, const Geom& g, const SweepArgs& a, int s_base,
                                       int n, int every, const ulonglong2* masks, long long* rec, size_t bytes,
                                       cudaStream_t s);
@@ -126,14 +117,12 @@ cudaError_t launch_cluster_sweeps(uint64_t* w0, uint64_t* w1, const Geom& g, con
                                   const ClusterPlan& plan, int nsweeps, const uint64_t* masks, int64_t s0,
                                   int64_t every, const ClusterExchange& x, cudaStream_t s);
 
-// Launch `kernel` with programmatic stream serialization (the kernel calls
-// pdl_enter before its first read): the next launch's setup overlaps the end
-// of the previous one.  On a stream that is being captured into a graph the
-// launch is a plain one unless in_graphs: measured on GB300, programmatic
-// edges made replayed graphs of the fused half-sweeps slower (L = 2016: 531
-// -> 298 spin-updates/ns), while plain stream launches gained (L = 16384:
-// +2.7%, L = 4096: +19%); the apply-only half-sweeps choose by size (see
-// launch_half_sweep_apply).  Errors are left for cudaGetLastError.
+// Launch `kernel` with programmatic stream serialization (every thread of the
+// kernel calls pdl_wait before it reads what an earlier launch writes): the
+// launch's draws overlap the end of the one before.  On a stream that is
+// being captured the launch is a plain one unless in_graphs: a graph captured
+// by the caller keeps full edges; the library's own graphs use programmatic
+// ones.  Errors are left for cudaGetLastError.
 template <typename... Params, typename... Args>
 inline void launch_pdl_opt(bool in_graphs, void (*kernel)(Params...), dim3 grid, dim3 block, cudaStream_t s,
                            Args... args)
@@ -173,10 +162,10 @@ Strips make_strips(const Geom& g, int most);
 // block, else strips of at most bw words and bw * bgrp threads.
 cudaError_t launch_half_sweep(int bw, int bgrp, int colour, bool update, bool record,
                               uint64_t* own, const uint64_t* other, const Geom& g, const SweepArgs& a,
-                              cudaStream_t s);
+                              bool in_graphs, cudaStream_t s);
 
 // A half-sweep that updates, with F = 2, 4 or 8 lanes per thread item.
 cudaError_t launch_half_sweep_lanes(int F, int colour, bool record, uint64_t* own, const uint64_t* other,
-                                    const Geom& g, const SweepArgs& a, cudaStream_t s);
+                                    const Geom& g, const SweepArgs& a, bool in_graphs, cudaStream_t s);
 
 }  // namespace ising

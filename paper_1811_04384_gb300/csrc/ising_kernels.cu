@@ -209,31 +209,26 @@ resident_sweeps_kernel(uint64_t* __restrict__ w0, uint64_t* __restrict__ w1, Geo
 }
 
 // Accept masks of the sweeps j = 0 .. nsweeps-1 that follow sweep t0 (sweep
-// t0 + j + 1), one thread per (j, item), drawn by item_masks_thread: masks[(j * items + item) * 4 + e] = (colour-0, colour-1 packed masks)
-// of row e of the item (item_masks_thread).  The draws depend on the site,
-// sweep and colour only, so a whole run's masks can be drawn at once by every
-// SM before the spins are updated.  t_base (device memory, or null) is added
-// to t0: a graph that is replayed draws for the sweeps after the device sweep
-// counter.
+// t0 + j + 1), one thread per (j, item): masks[(j * items + item) * 4 + e] =
+// (colour-0, colour-1 packed masks) of row e of the item (item_masks_thread).
+// The draws depend on the site, sweep and colour only, so a whole run's masks
+// can be drawn at once by every SM before the spins are updated.
 template <int ROUNDS>
 __global__ void __launch_bounds__(128)
-mask_draw_kernel(Geom g, SweepArgs a, const uint64_t* t_base, uint64_t t0, int nsweeps, ulonglong2* __restrict__ masks)
+mask_draw_kernel(Geom g, SweepArgs a, uint64_t t0, int nsweeps, ulonglong2* __restrict__ masks)
 {
     const int items = ((g.L + 3) / 4) * g.W;
-    const long long total = (long long)nsweeps * items;
-    const uint64_t tb = (t_base ? *t_base : 0) + t0 + 1;
-    for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < total;
-         k += (long long)gridDim.x * blockDim.x) {
-        const int j = (int)(k / items);
-        const int item = (int)(k - (long long)j * items);
-        uint64_t p0[4], p1[4];
-        const uint64_t t = tb + (uint64_t)j;
-        item_masks_thread<ROUNDS>(g, item, t, 0, a, p0);
-        item_masks_thread<ROUNDS>(g, item, t, 1, a, p1);
-        ulonglong2* out = masks + (size_t)k * 4;
+    const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= (long long)nsweeps * items) return;
+    const int j = (int)(k / items);
+    const int item = (int)(k - (long long)j * items);
+    uint64_t p0[4], p1[4];
+    const uint64_t t = t0 + 1 + (uint64_t)j;
+    item_masks_thread<ROUNDS>(g, item, t, 0, a, p0);
+    item_masks_thread<ROUNDS>(g, item, t, 1, a, p1);
+    ulonglong2* out = masks + (size_t)k * 4;
 #pragma unroll
-        for (int e = 0; e < 4; ++e) out[e] = make_ulonglong2(p0[e], p1[e]);
-    }
+    for (int e = 0; e < 4; ++e) out[e] = make_ulonglong2(p0[e], p1[e]);
 }
 
 // The on-chip path with the masks drawn beforehand (mask_draw_kernel): one
@@ -356,57 +351,6 @@ resident_premasked_kernel(uint64_t* __restrict__ w0, uint64_t* __restrict__ w1, 
     }
 }
 
-// One half-sweep of colour C over all SMs with the masks drawn beforehand
-// (mask_draw_kernel): thread k updates row k & 3 of item k >> 2 with the
-// packed masks masks[k] (.x colour 0, .y colour 1), so a launch is short:
-// no Philox work, one row of spin logic per thread.  Same results as
-// half_sweep_kernel.
-template <int C, bool RECORD>
-__global__ void __launch_bounds__(128)
-half_sweep_apply_kernel(uint64_t* __restrict__ own, const uint64_t* __restrict__ other, Geom g, SweepArgs a,
-                        const ulonglong2* __restrict__ masks)
-{
-    pdl_enter();
-    const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
-    const int items = ((g.L + 3) / 4) * g.W;
-    const int item = (int)(k >> 2), e = (int)(k & 3);
-    const int grp = item / g.W;
-    const int w = item - grp * g.W;
-    const int i = grp * 4 + e;
-    uint32_t anti = 0, up = 0;
-    if (item < items && i < g.L) {
-        const uint64_t live = live_mask(g, w);
-        const uint64_t all0 = ((uint64_t)a.all0 << 32 | a.all0) & live;
-        const uint64_t all1 = ((uint64_t)a.all1 << 32 | a.all1) & live;
-        const uint64_t p = C == 0 ? __ldg(&masks[k].x) : __ldg(&masks[k].y);
-        row_apply<C, RECORD>(own, other, g, i, w, live, p, p >> 1, all0, all1, anti, up);
-    }
-    if (RECORD) block_add_counts(record_counts(a) + 2 * (blockIdx.x % kCountSlots), anti, up);
-}
-
-cudaError_t launch_half_sweep_apply(int colour, bool record, uint64_t* own, const uint64_t* other, const Geom& g,
-                                    const SweepArgs& a, const ulonglong2* masks, cudaStream_t s)
-{
-    const uint32_t threads = (uint32_t)(((g.L + 3) / 4) * g.W) * 4;
-    const dim3 block(128), grid((threads + 127) / 128);
-    // Programmatic dependent launch also inside the captured graphs, where the
-    // fused half-sweeps use plain launches: measured on GB300 against plain
-    // launches in the same graphs (sweeps without records, spin-updates/ns),
-    // L = 300 / 512 / 700 / 1008: 35 / 97 / 171 / 314 against 31 / 87 / 156 /
-    // 294, and L = 4096: 1006 against 963, but L = 1500 / 2016 / 2600: 499 /
-    // 651 / 782 against 508 / 681 / 816 (L = 3000: equal).  So it is on up to
-    // 8192 items and from 80000 items.
-    const int items = ((g.L + 3) / 4) * g.W;
-    const bool in_graphs = items <= 8192 || items >= 80000;
-    if (colour == 0)
-        launch_pdl_opt(in_graphs, half_sweep_apply_kernel<0, false>, grid, block, s, own, other, g, a, masks);
-    else if (record)
-        launch_pdl_opt(in_graphs, half_sweep_apply_kernel<1, true>, grid, block, s, own, other, g, a, masks);
-    else
-        launch_pdl_opt(in_graphs, half_sweep_apply_kernel<1, false>, grid, block, s, own, other, g, a, masks);
-    return cudaGetLastError();
-}
-
 // One half-sweep of colour C over all SMs with F lanes per thread item
 // (item_masks, item_apply): for lattices whose one
 // thread per item would leave SMs idle and each thread with a long chain of
@@ -431,27 +375,27 @@ half_sweep_lanes_kernel(uint64_t* __restrict__ own, const uint64_t* __restrict__
 
 template <int F, int ROUNDS>
 static void launch_lanes_r(int colour, bool record, uint64_t* own, const uint64_t* other, const Geom& g,
-                           const SweepArgs& a, cudaStream_t s)
+                           const SweepArgs& a, bool in_graphs, cudaStream_t s)
 {
     const uint32_t threads = (uint32_t)(((g.L + 3) / 4) * g.W) * F;
     const dim3 block(128), grid((threads + 127) / 128);
-    if (colour == 0) launch_pdl(half_sweep_lanes_kernel<0, false, F, ROUNDS>, grid, block, s, own, other, g, a);
-    else if (record) launch_pdl(half_sweep_lanes_kernel<1, true, F, ROUNDS>, grid, block, s, own, other, g, a);
-    else launch_pdl(half_sweep_lanes_kernel<1, false, F, ROUNDS>, grid, block, s, own, other, g, a);
+    if (colour == 0) launch_pdl_opt(in_graphs, half_sweep_lanes_kernel<0, false, F, ROUNDS>, grid, block, s, own, other, g, a);
+    else if (record) launch_pdl_opt(in_graphs, half_sweep_lanes_kernel<1, true, F, ROUNDS>, grid, block, s, own, other, g, a);
+    else launch_pdl_opt(in_graphs, half_sweep_lanes_kernel<1, false, F, ROUNDS>, grid, block, s, own, other, g, a);
 }
 
 // A half-sweep that updates, with F = 2, 4 or 8 lanes per item.
 cudaError_t launch_half_sweep_lanes(int F, int colour, bool record, uint64_t* own, const uint64_t* other,
-                                    const Geom& g, const SweepArgs& a, cudaStream_t s)
+                                    const Geom& g, const SweepArgs& a, bool in_graphs, cudaStream_t s)
 {
     const bool r7 = a.rounds == 7;
     switch (F) {
-    case 2: r7 ? launch_lanes_r<2, 7>(colour, record, own, other, g, a, s)
-               : launch_lanes_r<2, 10>(colour, record, own, other, g, a, s); break;
-    case 4: r7 ? launch_lanes_r<4, 7>(colour, record, own, other, g, a, s)
-               : launch_lanes_r<4, 10>(colour, record, own, other, g, a, s); break;
-    default: r7 ? launch_lanes_r<8, 7>(colour, record, own, other, g, a, s)
-                : launch_lanes_r<8, 10>(colour, record, own, other, g, a, s); break;
+    case 2: r7 ? launch_lanes_r<2, 7>(colour, record, own, other, g, a, in_graphs, s)
+               : launch_lanes_r<2, 10>(colour, record, own, other, g, a, in_graphs, s); break;
+    case 4: r7 ? launch_lanes_r<4, 7>(colour, record, own, other, g, a, in_graphs, s)
+               : launch_lanes_r<4, 10>(colour, record, own, other, g, a, in_graphs, s); break;
+    default: r7 ? launch_lanes_r<8, 7>(colour, record, own, other, g, a, in_graphs, s)
+                : launch_lanes_r<8, 10>(colour, record, own, other, g, a, in_graphs, s); break;
     }
     return cudaGetLastError();
 }
@@ -572,16 +516,16 @@ Strips make_strips(const Geom& g, int most)
 template <int ROUNDS>
 static void launch_half_sweep_r(dim3 grid, dim3 block, int colour, bool update, bool record, uint64_t* own,
                                 const uint64_t* other, const Geom& g, const Strips& st, const SweepArgs& a,
-                                cudaStream_t s)
+                                bool in_graphs, cudaStream_t s)
 {
     if (colour == 0) {
-        if (record) launch_pdl(half_sweep_kernel<0, true, true, ROUNDS>, grid, block, s, own, other, g, st, a);
-        else launch_pdl(half_sweep_kernel<0, true, false, ROUNDS>, grid, block, s, own, other, g, st, a);
+        if (record) launch_pdl_opt(in_graphs, half_sweep_kernel<0, true, true, ROUNDS>, grid, block, s, own, other, g, st, a);
+        else launch_pdl_opt(in_graphs, half_sweep_kernel<0, true, false, ROUNDS>, grid, block, s, own, other, g, st, a);
     } else if (!update) {
         half_sweep_kernel<1, false, true, 10><<<grid, block, 0, s>>>(own, other, g, st, a);
     } else {
-        if (record) launch_pdl(half_sweep_kernel<1, true, true, ROUNDS>, grid, block, s, own, other, g, st, a);
-        else launch_pdl(half_sweep_kernel<1, true, false, ROUNDS>, grid, block, s, own, other, g, st, a);
+        if (record) launch_pdl_opt(in_graphs, half_sweep_kernel<1, true, true, ROUNDS>, grid, block, s, own, other, g, st, a);
+        else launch_pdl_opt(in_graphs, half_sweep_kernel<1, true, false, ROUNDS>, grid, block, s, own, other, g, st, a);
     }
 }
 
@@ -589,14 +533,14 @@ static void launch_half_sweep_r(dim3 grid, dim3 block, int colour, bool update, 
 // strips of up to bw words, bw * bgrp threads.
 cudaError_t launch_half_sweep(int bw, int bgrp, int colour, bool update, bool record,
                               uint64_t* own, const uint64_t* other, const Geom& g, const SweepArgs& a,
-                              cudaStream_t s)
+                              bool in_graphs, cudaStream_t s)
 {
     const Strips st = make_strips(g, bw == 0 ? kStripWords : bw);
     const uint32_t threads = (uint32_t)(bw == 0 ? bgrp : bw * bgrp);
     const uint32_t items = (uint32_t)((g.L + 3) / 4) * st.width;
     dim3 block(threads), grid((items + threads - 1) / threads, st.n);
-    if (a.rounds == 7) launch_half_sweep_r<7>(grid, block, colour, update, record, own, other, g, st, a, s);
-    else launch_half_sweep_r<10>(grid, block, colour, update, record, own, other, g, st, a, s);
+    if (a.rounds == 7) launch_half_sweep_r<7>(grid, block, colour, update, record, own, other, g, st, a, in_graphs, s);
+    else launch_half_sweep_r<10>(grid, block, colour, update, record, own, other, g, st, a, in_graphs, s);
     return cudaGetLastError();
 }
 
@@ -661,29 +605,13 @@ cudaError_t launch_resident(uint64_t* w0, uint64_t* w1, const Geom& g, const Swe
     return cudaGetLastError();
 }
 
-int device_sm_count()
-{
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) !=
-                                                  cudaSuccess || sms < 1) {
-        cudaGetLastError();
-        return 1;
-    }
-    return sms;
-}
-
-// Masks of the nsweeps sweeps following sweep (t_base ? *t_base : 0) + t0
-// into `masks` (nsweeps * items * 4 entries), with at most
-// blocks_per_sm * (the device's SMs) blocks of 128 threads (0: one thread
-// per sweep and item).
-cudaError_t launch_mask_draw(const Geom& g, const SweepArgs& a, const uint64_t* t_base, uint64_t t0, int nsweeps,
-                             ulonglong2* masks, int blocks_per_sm, cudaStream_t s)
+cudaError_t launch_mask_draw(const Geom& g, const SweepArgs& a, uint64_t t0, int nsweeps, ulonglong2* masks,
+                             cudaStream_t s)
 {
     const long long threads = (long long)nsweeps * (((g.L + 3) / 4) * g.W);
-    unsigned blocks = (unsigned)((threads + 127) / 128);
-    if (blocks_per_sm > 0) blocks = std::min(blocks, (unsigned)(device_sm_count() * blocks_per_sm));
-    if (a.rounds == 7) mask_draw_kernel<7><<<blocks, 128, 0, s>>>(g, a, t_base, t0, nsweeps, masks);
-    else mask_draw_kernel<10><<<blocks, 128, 0, s>>>(g, a, t_base, t0, nsweeps, masks);
+    const unsigned blocks = (unsigned)((threads + 127) / 128);
+    if (a.rounds == 7) mask_draw_kernel<7><<<blocks, 128, 0, s>>>(g, a, t0, nsweeps, masks);
+    else mask_draw_kernel<10><<<blocks, 128, 0, s>>>(g, a, t0, nsweeps, masks);
     return cudaGetLastError();
 }
 

@@ -75,9 +75,6 @@ struct ising_lattice {
     bool resident_attr = false;                  // dynamic shared memory attribute set
     ulonglong2* masks = nullptr;                 // lazily allocated: pre-drawn masks of the on-chip path
     size_t mask_bytes = 0;
-    ulonglong2* graph_masks = nullptr;           // two buffers of draw_sweeps() sweeps' masks, drawn inside the graphs
-    cudaStream_t draw_stream = nullptr;          // the graphs' mask draws are captured here, beside the half-sweeps
-    cudaEvent_t fork_ev = nullptr, draw_ev[64] = {}, apply_ev[64] = {};   // kMaxPieces each
     int clusters = 0;                            // clusters of the cluster path's launches (0: automatic)
     uint64_t* xbuf = nullptr;                    // rows between clusters (lazily, several clusters only)
     size_t xbuf_bytes = 0;
@@ -139,7 +136,6 @@ static void free_handle(ising_lattice* h)
     if (h->staging) cudaFree(h->staging);
     if (h->staging2) cudaFree(h->staging2);
     if (h->masks) cudaFree(h->masks);
-    if (h->graph_masks) cudaFree(h->graph_masks);
     if (h->xbuf) cudaFree(h->xbuf);
     if (h->xflag) cudaFree(h->xflag);
     if (h->host_xerr) cudaFreeHost(h->host_xerr);
@@ -151,10 +147,6 @@ static void free_handle(ising_lattice* h)
     if (h->graph_plain) cudaGraphExecDestroy(h->graph_plain);
     if (h->graph_rec) cudaGraphExecDestroy(h->graph_rec);
     if (h->capture_stream) cudaStreamDestroy(h->capture_stream);
-    if (h->draw_stream) cudaStreamDestroy(h->draw_stream);
-    if (h->fork_ev) cudaEventDestroy(h->fork_ev);
-    for (cudaEvent_t ev : h->draw_ev) if (ev) cudaEventDestroy(ev);
-    for (cudaEvent_t ev : h->apply_ev) if (ev) cudaEventDestroy(ev);
     if (h->owns_mem && h->base) cudaFree(h->base);
     if (h->host_counts) cudaFreeHost(h->host_counts);
     delete h;
@@ -297,90 +289,49 @@ static SweepArgs base_args(const ising_lattice* h)
     return a;
 }
 
-// Lanes per thread item on the launch path: the handle's choice, else 4 up
-// to 8192 items (L <= about 1100) and 1 above.  Measured on GB300 (sweeps
-// without records, spin-updates/ns, F = 1 / 2 / 4 / 8 lanes): L = 512:
-// 21 / 27 / 32 / 32; L = 1024: 85 / 102 / 128 / 128; L = 2048: 340 / 340 /
-// 340 / 256; L = 4096: 815 / 680 / 584 / 454.  Below L = 2048 each launch is
-// short and the lanes shorten it further; above, one thread per item fills
-// the GPU and the merge is pure overhead.
-static int item_lanes(const ising_lattice* h)
-{
-    if (h->item_lanes > 0) return h->item_lanes;
-    const int items = ((h->g.L + 3) / 4) * h->g.W;
-    return items <= 8192 ? 4 : 1;
-}
+// Lanes per thread item on the launch path: the handle's choice, else 1.
+// With the draws running while the half-sweep before finishes, splitting an
+// item's draws no longer shortens a launch: measured on GB300 (graph replays,
+// sweeps without records, spin-updates/ns, 1 / 4 lanes) L = 300: 39 / 35;
+// L = 512: 100 / 96; L = 1008: 369 / 324; L = 2016: 1,164 / 751.
+static int item_lanes(const ising_lattice* h) { return h->item_lanes > 0 ? h->item_lanes : 1; }
 
-// One half-sweep of the handle's lattice in its layout.
-static cudaError_t launch_hs_on(const ising_lattice* h, cudaStream_t st, int colour, bool update, bool record,
-                                const SweepArgs& a)
+// One half-sweep of the handle's lattice in its layout on stream `st`
+// (`captured`: into one of the library's own graphs).
+static cudaError_t launch_hs(const ising_lattice* h, cudaStream_t st, bool captured, int colour, bool update,
+                             bool record, const SweepArgs& a)
 {
     if (h->layout == ISING_LAYOUT_COLUMN_INTERLEAVED)
-        return ci_half_sweep(colour, update, record, h->words[0], h->g.L, a, st);
+        return ci_half_sweep(colour, update, record, h->words[0], h->g.L, a, captured, st);
     const int F = item_lanes(h);
     if (update && F > 1)
-        return launch_half_sweep_lanes(F, colour, record, h->words[colour], h->words[1 - colour], h->g, a, st);
+        return launch_half_sweep_lanes(F, colour, record, h->words[colour], h->words[1 - colour], h->g, a, captured,
+                                       st);
     return launch_half_sweep(h->bw, h->bg, colour, update, record, h->words[colour], h->words[1 - colour], h->g, a,
-                             st);
-}
-
-static cudaError_t launch_hs(const ising_lattice* h, int colour, bool update, bool record, const SweepArgs& a)
-{
-    return launch_hs_on(h, h->stream, colour, update, record, a);
+                             captured, st);
 }
 
 // ---- Graph replay of sweep chunks (launch path, small and mid-size lattices)
-// Up to about L = 4100 (102400 thread items) the launch path runs chunks of
-// sweeps as captured CUDA graphs: graph_plain holds kGraphSweeps sweeps, and
-// graph_rec holds max(1, kGraphSweeps / every) record intervals of `every`
-// sweeps, each recording into count slots offset by the device record index
-// (advanced by the graph itself, so one graph serves every record of a
-// chunk).  A graph draws the accept masks of draw_sweeps(h) sweeps at a time
-// on all SMs (mask_draw_kernel, or ci_mask_draw in the column-interleaved
-// layout, from the device sweep counter), and its half-sweeps only apply
-// them (half_sweep_apply_kernel, ci_half_sweep_pre): at these sizes one
-// thread per item leaves SMs idle while each runs its 21 Philox calls in a
-// row, and a half-sweep runs about as long as the host takes to launch it.
-// The draws run on a second branch of the graph, one piece ahead, into two
-// alternating buffers: piece k + 1 is drawn while piece k is applied, and a
-// piece is drawn into a buffer only after the half-sweeps of the piece before
-// have read it.  The kernels' launch operands (thresholds, Philox rounds,
-// launch shape) are baked into the graphs, so every call that changes them
-// drops the graphs.  Measured on GB300, sweeps without records,
-// spin-updates/ns, graphs against plain launches: L = 2600: 814 / 406;
-// L = 3000: 889 / 575; L = 3500: 951 / 729; L = 4096: 996 / 966; but
-// L = 4300: 1010 / 1082, where one thread per item fills the GPU.
+// Up to about L = 2350 (32768 thread items) a half-sweep runs about as long as
+// the host takes to launch it, so the launch path runs chunks of sweeps as
+// captured CUDA graphs: graph_plain holds kGraphSweeps sweeps, and graph_rec
+// holds max(1, kGraphSweeps / every) record intervals of `every` sweeps, each
+// recording into count slots offset by the device record index (advanced by
+// the graph itself, so one graph serves every record of a chunk).  The
+// half-sweeps are those of the plain launches, with the device sweep counter
+// and with programmatic edges: one's draws run while the one before finishes.
+// The kernels' launch operands (thresholds, Philox rounds, launch shape) are
+// baked into the graphs, so every call that changes them drops the graphs.
+// Measured on GB300, sweeps without records, spin-updates/ns, these graphs /
+// plain launches / graphs that drew the masks of up to 8 sweeps on a second
+// branch and applied them in half-sweeps of their own: L = 300: 39 / - / 35;
+// L = 700: 182 / 141 / 170; L = 1008: 382 / 285 / 313; L = 1500: 694 / 604 /
+// 539; L = 2016: 1,164 / 960 / 737; L = 3000: 1,381 / 1,340 / 942; L = 4000:
+// 1,451 / 1,425 / 931; column-interleaved L = 1008: 323 / - / 305; L = 2016:
+// 999 / - / 576; L = 3024: - / 1,380 / 669.
 constexpr int kGraphSweeps = 32;
 constexpr int kGraphMaxEvery = 64;
-constexpr int kGraphMaxItems = 102400;
-constexpr int kMaxDrawSweeps = 8;
-constexpr size_t kGraphMaskBytes = 32u << 20;    // both buffers
-constexpr int kMaxPieces = kGraphMaxEvery;       // a graph holds at most kGraphMaxEvery sweeps
-
-// Sweeps per drawn piece: 8, fewer where two buffers of 8 would pass 32 MB
-// (64 B per item and sweep).
-static int draw_sweeps(const ising_lattice* h)
-{
-    const size_t items = (size_t)((h->g.L + 3) / 4) * h->g.W;
-    return (int)std::max<size_t>(1, std::min<size_t>(kMaxDrawSweeps, kGraphMaskBytes / (2 * 64 * items)));
-}
-
-// Blocks per SM of a graph's mask draws (0: one thread per unit): a capped
-// grid whose blocks loop over the piece leaves room on every SM for the
-// half-sweeps of the piece before, which run beside it on the other branch.
-// Measured on GB300 (sweeps without records, spin-updates/ns, one thread per
-// unit / 2 / 3 blocks per SM), row-packed: L = 1500: 508 / 539 / 532;
-// L = 2016: 680 / 744 / 703; L = 3000: 887 / 941 / 915; L = 4096: 1006 / 923
-// / 1035.  Column-interleaved: L = 1008: 305 / 283 / 291; L = 1512: 388 /
-// 445 / 427; L = 2016: 511 / 575 / 552; L = 3024: 611 / 669 / 645;
-// L = 4032: 683 / 295 / 360 (its half-sweeps use programmatic launches in the
-// graphs from 80,000 items).
-static int draw_blocks_per_sm(const ising_lattice* h)
-{
-    const int items = ((h->g.L + 3) / 4) * h->g.W;      // both layouts: the same thread count
-    if (h->layout == ISING_LAYOUT_COLUMN_INTERLEAVED) return items >= 10000 && items < 80000 ? 2 : 0;
-    return items < 80000 ? 2 : 3;
-}
+constexpr int kGraphMaxItems = 32768;
 
 static bool use_graphs(const ising_lattice* h)
 {
@@ -406,75 +357,23 @@ static int capture_sweeps(ising_lattice* h, int n, int every, cudaGraphExec_t* o
     cudaError_t e = cudaSuccess;
     if (!h->capture_stream) e = cudaStreamCreateWithFlags(&h->capture_stream, cudaStreamNonBlocking);
     if (e != cudaSuccess) { h->capture_stream = nullptr; return cuda_fail(e, "capture stream"); }
-    const bool ci = h->layout == ISING_LAYOUT_COLUMN_INTERLEAVED;
-    const size_t sweep_bytes = ci ? ci_mask_bytes_per_sweep(h->g.L)
-                                  : (size_t)(((h->g.L + 3) / 4) * h->g.W) * 4 * sizeof(ulonglong2);
-    const int D = draw_sweeps(h);
-    if (!h->graph_masks) {
-        e = cudaMalloc(&h->graph_masks, 2 * D * sweep_bytes);
-        if (e != cudaSuccess) { h->graph_masks = nullptr; cuda_fail(e, "cudaMalloc graph masks"); return ISING_ENOMEM; }
-    }
-    if (!h->draw_stream) e = cudaStreamCreateWithFlags(&h->draw_stream, cudaStreamNonBlocking);
-    if (e != cudaSuccess) { h->draw_stream = nullptr; return cuda_fail(e, "draw stream"); }
-    if (!h->fork_ev) e = cudaEventCreateWithFlags(&h->fork_ev, cudaEventDisableTiming);
-    for (int k = 0; k < kMaxPieces && e == cudaSuccess; ++k) {
-        if (!h->draw_ev[k]) e = cudaEventCreateWithFlags(&h->draw_ev[k], cudaEventDisableTiming);
-        if (e == cudaSuccess && !h->apply_ev[k]) e = cudaEventCreateWithFlags(&h->apply_ev[k], cudaEventDisableTiming);
-    }
-    if (e != cudaSuccess) return cuda_fail(e, "graph events");
     SweepArgs a = base_args(h);
     cudaStream_t A = h->capture_stream;
     cudaGraph_t graph = nullptr;
     e = cudaStreamBeginCapture(A, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return cuda_fail(e, "cudaStreamBeginCapture");
     cudaError_t le = cudaSuccess;
-    char* const buffers = reinterpret_cast<char*>(h->graph_masks);
-    // one half-sweep of sweep s from its masks m (this sweep's block in a mask buffer)
-    auto half = [&](int colour, bool rec, const char* m) {
-        if (ci) return ci_half_sweep_pre(colour, rec, h->words[0], h->g.L, a, reinterpret_cast<const uint64_t*>(m), A);
-        return launch_half_sweep_apply(colour, rec, h->words[colour], h->words[1 - colour], h->g, a,
-                                       reinterpret_cast<const ulonglong2*>(m), A);
-    };
-    // the half-sweeps of sweep s (relative to the device counter)
-    auto sweep = [&](int s, const char* m) {
+    for (int s = 1; s <= n && le == cudaSuccess; ++s) {
         a.t_off = (uint32_t)s;
         a.counts = nullptr;
         a.rec_base = nullptr;
-        cudaError_t r = half(0, false, m);
+        le = launch_hs(h, A, true, 0, true, false, a);
         const bool rec = every > 0 && s % every == 0;
         if (rec) {
             a.counts = h->counts + (size_t)(s / every - 1) * kCountSlots * 2;
             a.rec_base = rec_index(h);
         }
-        if (r == cudaSuccess) r = half(1, rec, m);
-        return r;
-    };
-    cudaStream_t B = h->draw_stream;
-    const int np = (n + D - 1) / D;      // <= kMaxPieces
-    auto draw = [&](int k) {       // piece k: sweeps k D + 1 .. into buffer k & 1
-        const int first = k * D;
-        const int count = std::min(D, n - first);
-        char* buf = buffers + (size_t)(k & 1) * D * sweep_bytes;
-        cudaError_t r = ci ? ci_mask_draw(h->g.L, a, h->t_dev, (uint64_t)first, count,
-                                          reinterpret_cast<uint64_t*>(buf), draw_blocks_per_sm(h), B)
-                           : launch_mask_draw(h->g, a, h->t_dev, (uint64_t)first, count,
-                                              reinterpret_cast<ulonglong2*>(buf), draw_blocks_per_sm(h), B);
-        if (r == cudaSuccess) r = cudaEventRecord(h->draw_ev[k], B);
-        return r;
-    };
-    le = cudaEventRecord(h->fork_ev, A);
-    if (le == cudaSuccess) le = cudaStreamWaitEvent(B, h->fork_ev, 0);
-    if (le == cudaSuccess) le = draw(0);
-    for (int k = 0; k < np && le == cudaSuccess; ++k) {
-        if (k + 1 < np) {
-            if (k >= 1) le = cudaStreamWaitEvent(B, h->apply_ev[k - 1], 0);    // buffer (k + 1) & 1 is read
-            if (le == cudaSuccess) le = draw(k + 1);
-        }
-        if (le == cudaSuccess) le = cudaStreamWaitEvent(A, h->draw_ev[k], 0);
-        const char* buf = buffers + (size_t)(k & 1) * D * sweep_bytes;
-        for (int s = k * D + 1; s <= std::min(n, (k + 1) * D) && le == cudaSuccess; ++s)
-            le = sweep(s, buf + (size_t)(s - 1 - k * D) * sweep_bytes);
-        if (le == cudaSuccess) le = cudaEventRecord(h->apply_ev[k], A);
+        if (le == cudaSuccess) le = launch_hs(h, A, true, 1, true, rec, a);
     }
     if (le == cudaSuccess) {
         le = launch_advance_graph(h->t_dev, (uint64_t)n, rec_index(h), every > 0 ? (uint32_t)(n / every) : 0u, A);
@@ -526,11 +425,11 @@ static int run_sweeps(ising_lattice* h, int64_t n, RecOf rec_of)
     }
     for (int64_t s = 1; s <= n; ++s) {
         a.t_off = (uint32_t)s;
-        cudaError_t e = launch_hs(h, 0, true, false, a);
+        cudaError_t e = launch_hs(h, h->stream, false, 0, true, false, a);
         if (e != cudaSuccess) return cuda_fail(e, "half_sweep colour 0");
         const int rec = rec_of(s);
         a.counts = rec >= 0 ? h->counts + (size_t)rec * kCountSlots * 2 : nullptr;
-        e = launch_hs(h, 1, true, rec >= 0, a);
+        e = launch_hs(h, h->stream, false, 1, true, rec >= 0, a);
         if (e != cudaSuccess) return cuda_fail(e, "half_sweep colour 1");
     }
     if (n > 0) {
@@ -621,7 +520,7 @@ static int run_resident(ising_lattice* h, int n, int every)
         }
         for (int done = 0; done < n;) {
             const int part = std::min(n - done, max_sweeps);
-            cudaError_t e = launch_mask_draw(g, a, nullptr, h->t + (uint64_t)done, part, h->masks, 0, h->stream);
+            cudaError_t e = launch_mask_draw(g, a, h->t + (uint64_t)done, part, h->masks, h->stream);
             if (e != cudaSuccess) return cuda_fail(e, "mask_draw_kernel");
             e = launch_resident_premasked(h->words[0], h->words[1], g, a, done, part, every, h->masks, rec,
                                           resident_bytes(g), h->stream);
@@ -956,7 +855,7 @@ static int run_random_words(ising_lattice* h, int64_t n, RecOf rec_of)
         const int rec = rec_of(it);
         if (rec >= 0) {
             a.counts = h->counts + (size_t)rec * kCountSlots * 2;
-            cudaError_t e = ci_half_sweep(1, false, true, h->words[0], h->g.L, a, h->stream);
+            cudaError_t e = ci_half_sweep(1, false, true, h->words[0], h->g.L, a, false, h->stream);
             if (e != cudaSuccess) return cuda_fail(e, "measure");
         }
     }
@@ -1110,7 +1009,7 @@ static int measure(ising_lattice* h, int64_t* E, int64_t* M)
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync counts");
     SweepArgs a = base_args(h);
     a.counts = h->counts;
-    e = launch_hs(h, 1, false, true, a);
+    e = launch_hs(h, h->stream, false, 1, false, true, a);
     if (e != cudaSuccess) return cuda_fail(e, "measure");
     e = cudaMemcpyAsync(h->host_counts, h->counts, bytes, cudaMemcpyDeviceToHost, h->stream);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpyAsync counts");

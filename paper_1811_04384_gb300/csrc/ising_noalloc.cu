@@ -103,11 +103,11 @@ extern "C" int ising_sweep_record_noalloc(uint64_t* dev_words0, uint64_t* dev_wo
     for (int64_t step = 1; step <= n; ++step) {
         a.t_off = (uint32_t)step;
         a.counts = nullptr;
-        e = ising::launch_half_sweep(32, 4, 0, true, false, dev_words0, dev_words1, g, a, s);
+        e = ising::launch_half_sweep(32, 4, 0, true, false, dev_words0, dev_words1, g, a, false, s);
         if (e != cudaSuccess) return ising::cuda_fail(e, "half_sweep colour 0");
         const bool rec = (step % every) == 0;
         if (rec) a.counts = scratch + (size_t)(step / every - 1) * kSlots * 2;
-        e = ising::launch_half_sweep(32, 4, 1, true, rec, dev_words1, dev_words0, g, a, s);
+        e = ising::launch_half_sweep(32, 4, 1, true, rec, dev_words1, dev_words0, g, a, false, s);
         if (e != cudaSuccess) return ising::cuda_fail(e, "half_sweep colour 1");
     }
     if (nrec > 0) {

@@ -53,3 +53,25 @@ def test_strips_batch(ising, threads):
         np.testing.assert_array_equal(E[r], Eo)
         np.testing.assert_array_equal(M[r], Mo)
         np.testing.assert_array_equal(spins[r], s)
+
+
+# word row groups N / 4 = 1, 4, 5 in blocks of 4; column pairs 42, 168, 210 in blocks of 32
+@pytest.mark.parametrize("L", [84, 336, 420])
+@pytest.mark.parametrize("rng,rounds", [(0, 10), (1, 7)])
+@pytest.mark.parametrize("path", [1, 3])
+def test_interleaved_row_keys(ising, L, rng, rounds, path):
+    seed = 0xabcdef0000000011 + L
+    with ising.Lattice(L, seed, layout=ising.ISING_LAYOUT_COLUMN_INTERLEAVED) as lat:
+        lat.set_path(path)
+        lat.set_rng(rng)
+        lat.init_hot()
+        lat.set_beta(0.43)
+        E, M = lat.sweep_record(5, 2)           # launches (no whole graph) or the cluster path
+        E2, M2 = lat.sweep_record(34, 17)       # a replayed graph of the launch path
+        spins = lat.get_spins()
+    s = oracle.init_hot(L, seed)
+    Eo, Mo = oracle.run(s, seed, 0.43, 0, 5, 2, rounds=rounds)
+    Eo2, Mo2 = oracle.run(s, seed, 0.43, 5, 34, 17, rounds=rounds)
+    np.testing.assert_array_equal(np.concatenate([E, E2]), np.concatenate([Eo, Eo2]))
+    np.testing.assert_array_equal(np.concatenate([M, M2]), np.concatenate([Mo, Mo2]))
+    np.testing.assert_array_equal(spins, s)
