@@ -69,9 +69,10 @@ def test_interleaved_row_keys(ising, L, rng, rounds, path):
         E, M = lat.sweep_record(5, 2)           # launches (no whole graph) or the cluster path
         E2, M2 = lat.sweep_record(34, 17)       # a replayed graph of the launch path
         spins = lat.get_spins()
-    s = oracle.init_hot(L, seed)
-    Eo, Mo = oracle.run(s, seed, 0.43, 0, 5, 2, rounds=rounds)
-    Eo2, Mo2 = oracle.run(s, seed, 0.43, 5, 34, 17, rounds=rounds)
+    with oracle.sweep_rounds(rounds):
+        s = oracle.init_hot(L, seed)
+        Eo, Mo = oracle.run(s, seed, 0.43, 0, 5, 2)
+        Eo2, Mo2 = oracle.run(s, seed, 0.43, 5, 34, 17)
     np.testing.assert_array_equal(np.concatenate([E, E2]), np.concatenate([Eo, Eo2]))
     np.testing.assert_array_equal(np.concatenate([M, M2]), np.concatenate([Mo, Mo2]))
     np.testing.assert_array_equal(spins, s)
