@@ -36,7 +36,7 @@ struct BatchTile {
 template <typename Tiles>
 inline void add_tiles(Tiles& tiles, int rep, const Geom& g, int threads)
 {
-    const Strips st = make_strips(g, kStripWords);
+    const Strips st = make_strips(g.W, kStripWords);
     const uint32_t groups = (uint32_t)((g.L + 3) / 4);
     for (uint32_t k = 0; k < st.n; ++k) {
         const bool last = k == st.n - 1;
@@ -79,7 +79,7 @@ batch_half_sweep_kernel(const BatchReplica* __restrict__ reps, const BatchTile* 
     const PhiloxKeys rk = R->rk;
     uint32_t anti = 0, up = 0;
     ItemMasks acc;
-    first_products(tab, w0, width, tile.magic, philox_first_key((uint32_t)t, rk));
+    first_products<kFields, kStripWords>(tab, w0, width, tile.magic, philox_first_key((uint32_t)t, rk));
     if (valid) {
         const FirstTable first = {tab + x};
         if (ROUNDS == 7 || (ROUNDS == 0 && R->rounds == 7))

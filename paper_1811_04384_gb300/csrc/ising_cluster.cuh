@@ -1,6 +1,5 @@
-// Helpers of the cluster kernels (ising_cluster.cu, ising_ci_cluster.cu):
-// asynchronous 16-byte copies into shared memory, with a range-checked form
-// for the checked build, and the flags of the exchanges between clusters.
+// Helpers of the cluster kernel (ising_cluster.cu): the flags of the exchanges
+// between clusters and the agreement on the write-back.
 #pragma once
 #include <cstdint>
 
@@ -8,39 +7,6 @@
 
 namespace ising {
 namespace {
-
-// 16 bytes global -> shared (a 32-bit shared-window address), asynchronously,
-// through L2.
-__device__ __forceinline__ void cl_copy16(uint32_t smem_dst, const void* gmem_src)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_dst), "l"(gmem_src) : "memory");
-}
-
-// cl_copy16 to shared address `dst` from `src`.  In a checked build the
-// copy is skipped and recorded (see word_ld) unless both words of the pair
-// lie in the `dst_words` words from shared address `dst_base` and in the
-// `src_words` words from `src_base`.
-__device__ __forceinline__ void cl_copy_pair(uint32_t dst, uint32_t dst_base, uint64_t dst_words, const uint64_t* src,
-                                             const uint64_t* src_base, uint64_t src_words, uint32_t line)
-{
-#ifdef ISING_CHECKED
-    if (!check_index((uint64_t)(dst - dst_base) / 8 + 1, dst_words, line) ||
-        !check_index((uint64_t)(src - src_base) + 1, src_words, line))
-        return;
-#else
-    (void)dst_base;
-    (void)dst_words;
-    (void)src_base;
-    (void)src_words;
-    (void)line;
-#endif
-    cl_copy16(dst, src);
-}
-
-__device__ __forceinline__ void cl_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-
-template <int N>
-__device__ __forceinline__ void cl_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
 __device__ __forceinline__ int wrap_index(int i, int L) { return i < 0 ? i + L : (i >= L ? i - L : i); }
 
@@ -95,10 +61,6 @@ __device__ __forceinline__ unsigned int cl_load_acquire(const unsigned int* p)
 // proposer ran, so all were resident together.  Normally each block finds
 // the count complete at once, and nobody waits.  On "go" block 0 zeroes the
 // other set for the next piece (the launch before, which used it, has ended).
-// The kernels with more than one word per thread call them through the
-// non-inlined forms below: inlined, they cost the 80-register form a spill
-// in its loop (3% at L = 2016 on GB300); the one-word form runs faster with
-// them inlined (3% at L = 1008).
 constexpr unsigned int kClCheckInNs = 100000000u;   // 0.1 s (on the low 32 bits of the global timer)
 constexpr unsigned int kClNoPiece = 0xffffffffu;
 
@@ -149,16 +111,6 @@ __device__ __forceinline__ bool cl_decide(unsigned int* gate, unsigned int block
         }
     }
     return __syncthreads_or(go) != 0;
-}
-
-__device__ __noinline__ bool cl_count_in_call(unsigned int* gate, unsigned int piece)
-{
-    return cl_count_in(gate, piece);
-}
-
-__device__ __noinline__ bool cl_decide_call(unsigned int* gate, unsigned int blocks, unsigned int piece)
-{
-    return cl_decide(gate, blocks, piece);
 }
 
 // Waits until *f >= want; gives up after kClWaitNs of the GPU's global

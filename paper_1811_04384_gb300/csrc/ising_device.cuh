@@ -228,6 +228,19 @@ __device__ __forceinline__ uint32_t flip_half(uint32_t s, uint32_t u, uint32_t d
     return s ^ lop3<(kLutA | kLutB) & kLutC>(e, m, live);
 }
 
+// flip_half where p and q are zero off the live bits and h1 alone of the
+// neighbours can be set there: A, B and D are zero there, so nothing flips.
+__device__ __forceinline__ uint32_t flip_all(uint32_t s, uint32_t u, uint32_t d, uint32_t h0, uint32_t h1, uint32_t p,
+                                             uint32_t q)
+{
+    constexpr int kOr = (kLutA ^ kLutB) | (kLutA ^ kLutC), kAnd = (kLutA ^ kLutB) & (kLutA ^ kLutC);
+    const uint32_t A = lop3<kOr>(s, u, d), B = lop3<kAnd>(s, u, d);
+    const uint32_t C = lop3<kOr>(s, h0, h1), D = lop3<kAnd>(s, h0, h1);
+    const uint32_t e = lop3<(kLutA | kLutB | kLutC)>(B, D, q);
+    const uint32_t m = lop3<(kLutA & kLutB) | (kLutA & kLutC) | (kLutB & kLutC)>(A, C, p);
+    return lop3<(kLutA ^ (kLutB | kLutC))>(s, e, m);
+}
+
 // Anti-aligned bonds of the updated half word s with its four neighbours, and
 // its up spins plus those of h0, added to anti / up.  Two spin-bit words share
 // one population count (x + 2 y: the fields are three bits wide).
@@ -256,12 +269,17 @@ struct ItemMasks {
 // an add there; as an XOR they stayed on the ALU, 1,243 against 1,394
 // spin-updates/ns at L = 16384).
 template <int B>
-__device__ __forceinline__ void accept_insert(uint32_t& acc, uint32_t r, uint32_t thr0, uint32_t thr1)
+__device__ __forceinline__ void accept_bit(uint32_t& acc, uint32_t r, uint32_t thr)
 {
     asm("{\n\t.reg .pred p;\n\tsetp.lt.u32 p, %1, %2;\n\t@p or.b32 %0, %0, %3;\n\t}"
-        : "+r"(acc) : "r"(r), "r"(thr1), "n"(1u << B));
-    asm("{\n\t.reg .pred p;\n\tsetp.lt.u32 p, %1, %2;\n\t@p or.b32 %0, %0, %3;\n\t}"
-        : "+r"(acc) : "r"(r), "r"(thr0), "n"(2u << B));
+        : "+r"(acc) : "r"(r), "r"(thr), "n"(1u << B));
+}
+
+template <int B>
+__device__ __forceinline__ void accept_insert(uint32_t& acc, uint32_t r, uint32_t thr0, uint32_t thr1)
+{
+    accept_bit<B>(acc, r, thr1);
+    accept_bit<B + 1>(acc, r, thr0);
 }
 
 // The first Philox products of an item's fields: computed (m = m0 + k), or
@@ -457,20 +475,21 @@ struct Strips {
 
 __device__ __forceinline__ uint32_t strip_group(uint32_t q, uint32_t magic) { return magic ? __umulhi(q, magic) : q; }
 
-// All threads of the block: the first products of fields 0 .. 20 of words
-// w0 .. w0 + width - 1 at a sweep (key: philox_first_key), field k of word w0
-// + x in tab[k * kStripWords + x].  The threads fill whole columns of a field
-// at a time (blockDim / width fields per pass).
+// All threads of the block: the first products of fields 0 .. FIELDS - 1 of
+// words w0 .. w0 + width - 1 at a sweep (key: philox_first_key), field k of
+// word w0 + x in tab[k * STRIDE + x].  The threads fill whole columns of a
+// field at a time (blockDim / width fields per pass).
+template <int FIELDS, int STRIDE>
 __device__ __forceinline__ void first_products(uint2* tab, uint32_t w0, uint32_t width, uint32_t magic, uint32_t key)
 {
     const uint32_t k0 = strip_group(threadIdx.x, magic), x = threadIdx.x - k0 * width;
     const uint32_t step = strip_group(blockDim.x, magic);      // >= 2: blocks have at least 32 threads
-    uint32_t m = (w0 + x) * (uint32_t)kFields + k0;
+    uint32_t m = (w0 + x) * (uint32_t)FIELDS + k0;
     if (k0 < step)
-        for (uint32_t k = k0; k < (uint32_t)kFields; k += step, m += step) {
+        for (uint32_t k = k0; k < (uint32_t)FIELDS; k += step, m += step) {
             uint32_t hi, lo;
             mul_hilo(kPhiloxM0, key ^ m, hi, lo);
-            tab[k * kStripWords + x] = make_uint2(hi, lo);
+            tab[k * STRIDE + x] = make_uint2(hi, lo);
         }
     __syncthreads();
 }
@@ -702,7 +721,7 @@ half_sweep_kernel(uint64_t* own, const uint64_t* other, Geom g, Strips st, Sweep
     ItemMasks acc;
     if (UPDATE) {
         const uint64_t t = sweep_number(a);
-        first_products(tab, w0, width, magic, philox_first_key((uint32_t)t, a.rk));
+        first_products<kFields, kStripWords>(tab, w0, width, magic, philox_first_key((uint32_t)t, a.rk));
         if (valid) {
             const FirstTable first = {tab + x};
             draw_item<ROUNDS>(first, grp, t, C, a.rk, a.thr0, a.thr1, a.all0, a.all1, acc);

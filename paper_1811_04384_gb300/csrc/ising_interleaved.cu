@@ -17,6 +17,7 @@
 
 #include "ising_interleaved.h"
 #include "ising_interleaved.cuh"
+#include "ising_dense.cuh"
 #include "ising_internal.h"
 
 namespace ising {
@@ -123,6 +124,69 @@ ci_half_sweep_kernel(uint64_t* S, int L, int N, SweepArgs a)
     if (RECORD) {
         const int slot = (blockIdx.x + gridDim.x * blockIdx.y) % kCountSlots;
         block_add_counts(record_counts(a) + 2 * slot, anti, up);
+    }
+}
+
+// The lattice to the dense form (ising_dense.cuh), and back.  One warp per
+// word row I and 64 columns: lane l holds the words of columns 64 w + 2 l and
+// + 1, whose sites in row i = I + kN are bit l of dense word w of colours i & 1
+// and 1 - (i & 1); a ballot per field gathers them.  Both read and write each
+// word once, coalesced on the word side.
+constexpr int kCiDenseWarps = 4;
+
+__global__ void __launch_bounds__(32 * kCiDenseWarps)
+ci_to_dense_kernel(const uint64_t* __restrict__ S, int L, int N, DenseGeom d, uint32_t* __restrict__ dense)
+{
+    const int w = blockIdx.x * kCiDenseWarps + (int)threadIdx.x / 32, I = blockIdx.y, lane = threadIdx.x & 31;
+    if (w >= d.W) return;                             // uniform over the warp
+    const int J = 64 * w + 2 * lane;
+    const uint64_t n = (uint64_t)N * L, nd = 2 * (uint64_t)L * d.P;
+    uint64_t x = 0, y = 0;
+    if (J < L) {
+        x = word_ld<false>(S, (uint64_t)I * L + J, n, __LINE__);
+        y = word_ld<false>(S, (uint64_t)I * L + J + 1, n, __LINE__);
+    }
+    uint32_t ex = 0, ey = 0;
+    for (int k = 0; k < kFields; ++k) {
+        const uint32_t bx = __ballot_sync(0xffffffffu, (x >> (3 * k)) & 1ull);
+        const uint32_t by = __ballot_sync(0xffffffffu, (y >> (3 * k)) & 1ull);
+        if (lane == k) {
+            ex = bx;
+            ey = by;
+        }
+    }
+    if (lane < kFields) {
+        const int i = I + lane * N, c = i & 1;        // column 2m has colour i & 1
+        half_st(dense, ((uint64_t)c * L + i) * d.P + w, ex, nd, __LINE__);
+        half_st(dense, ((uint64_t)(1 - c) * L + i) * d.P + w, ey, nd, __LINE__);
+        if (w == d.W - 1 && d.P > d.W) {              // the pad word
+            half_st(dense, ((uint64_t)c * L + i) * d.P + w + 1, 0u, nd, __LINE__);
+            half_st(dense, ((uint64_t)(1 - c) * L + i) * d.P + w + 1, 0u, nd, __LINE__);
+        }
+    }
+}
+
+__global__ void __launch_bounds__(32 * kCiDenseWarps)
+ci_from_dense_kernel(uint64_t* __restrict__ S, int L, int N, DenseGeom d, const uint32_t* __restrict__ dense)
+{
+    const int w = blockIdx.x * kCiDenseWarps + (int)threadIdx.x / 32, I = blockIdx.y, lane = threadIdx.x & 31;
+    if (w >= d.W) return;
+    const uint64_t n = (uint64_t)N * L, nd = 2 * (uint64_t)L * d.P;
+    uint32_t ex = 0, ey = 0;
+    if (lane < kFields) {
+        const int i = I + lane * N, c = i & 1;
+        ex = half_ld(dense, ((uint64_t)c * L + i) * d.P + w, nd, __LINE__);
+        ey = half_ld(dense, ((uint64_t)(1 - c) * L + i) * d.P + w, nd, __LINE__);
+    }
+    uint64_t x = 0, y = 0;
+    for (int k = 0; k < kFields; ++k) {
+        x |= (uint64_t)((__shfl_sync(0xffffffffu, ex, k) >> lane) & 1u) << (3 * k);
+        y |= (uint64_t)((__shfl_sync(0xffffffffu, ey, k) >> lane) & 1u) << (3 * k);
+    }
+    const int J = 64 * w + 2 * lane;
+    if (J < L) {
+        word_st(S, (uint64_t)I * L + J, x, n, __LINE__);
+        word_st(S, (uint64_t)I * L + J + 1, y, n, __LINE__);
     }
 }
 
@@ -439,6 +503,22 @@ cudaError_t ci_init_cold(uint64_t* S, int L, int up, cudaStream_t s)
 {
     const size_t n = (size_t)(L / 21) * L;
     ci_fill_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(S, n, up ? kAllFields : 0ull);
+    return cudaGetLastError();
+}
+
+cudaError_t ci_to_dense(const uint64_t* S, int L, uint32_t* dense, cudaStream_t s)
+{
+    const DenseGeom d = dense_geom(L);
+    const dim3 grid((d.W + kCiDenseWarps - 1) / kCiDenseWarps, L / 21);
+    ci_to_dense_kernel<<<grid, 32 * kCiDenseWarps, 0, s>>>(S, L, L / 21, d, dense);
+    return cudaGetLastError();
+}
+
+cudaError_t ci_from_dense(uint64_t* S, int L, const uint32_t* dense, cudaStream_t s)
+{
+    const DenseGeom d = dense_geom(L);
+    const dim3 grid((d.W + kCiDenseWarps - 1) / kCiDenseWarps, L / 21);
+    ci_from_dense_kernel<<<grid, 32 * kCiDenseWarps, 0, s>>>(S, L, L / 21, d, dense);
     return cudaGetLastError();
 }
 

@@ -72,26 +72,29 @@ cudaError_t launch_resident_premasked(uint64_t* w0, uint64_t* w1, const Geom& g,
                                       int n, int every, const ulonglong2* masks, long long* rec, size_t bytes,
                                       cudaStream_t s);
 
-// The cluster path (ising_cluster.cu): one thread-block cluster whose blocks
-// keep the lattice in their shared memory over many sweeps.  cluster_plan
-// picks the launch for side L (false if there is none); launch_cl_mask_draw
-// draws the masks of nsweeps sweeps after sweep (t_base ? *t_base : 0) + t0
-// (cl_mask_bytes_per_sweep bytes each); with `overlap` it is launched with
-// programmatic stream serialization, so that it runs beside the cluster
+// The cluster path (ising_cluster.cu): thread-block clusters whose blocks
+// keep the lattice in their shared memory, one bit per spin, over many
+// sweeps.  A mask buffer has room for kClMaskPad half-sweeps past its last (the
+// launch copies masks that far ahead).  cluster_plan picks the launch for side L of a layout (false if
+// there is none); launch_cl_mask_draw draws the masks of nsweeps sweeps after
+// sweep t0 (cl_mask_bytes_per_sweep bytes each); with `overlap` it is launched
+// with programmatic stream serialization, so that it runs beside the cluster
 // launch before it in the stream (which must not read `masks`).
 // launch_cluster_sweeps runs sweeps s0 + 1 .. s0 + nsweeps of a call from
 // them, recording after every `every`-th (0: none) into count slot
-// s / every - 1 past a.counts.
+// s / every - 1 past a.counts; the lattice is w0, w1 (packed words), or the
+// dense array `dense` (cl_dense_bytes bytes: [colour][row][word], pitch and
+// words of dense_geom) where it is not null.
 struct ClusterPlan {
     int blocks;     // cluster size
     int k;          // half-sweeps per phase = halo rows
-    int q;          // mask slabs in shared memory
-    int ns;         // window words per thread: 1 .. 4
+    int v;          // dense words per unit: 1 or 2
+    int ns;         // units per thread: 1 or 2
     int threads;    // threads per block
     int clusters;   // clusters of a launch (1: the halos never leave the cluster)
 };
 // The rows crossing between the clusters of a launch (clusters > 1): `buf`
-// holds cl_exchange_words(g, plan) words, `flags` 2 per cluster (zero when
+// holds cl_exchange_words(L, plan) words, `flags` 2 per cluster (zero when
 // allocated, then only ever raised), `seq` the flag base of the launch (the
 // caller adds cl_exchange_seqs(plan, nsweeps) after each launch), `err` a
 // word set to 1 when a wait gave up, `wait_add` 0 (a test sets it to a value
@@ -106,14 +109,16 @@ struct ClusterExchange {
     unsigned int piece;            // the launch's piece of the call
     unsigned int absent;           // blocks counted on beyond the launch's (a test hook: 1 gives up)
 };
-bool cluster_plan(const Geom& g, int clusters, ClusterPlan* plan);
+constexpr int kClMaskPad = 8;
+bool cluster_plan(int L, bool interleaved, int clusters, ClusterPlan* plan);
 int cluster_max_active();   // clusters of one launch that can be resident at once (0: none)
-size_t cl_exchange_words(const Geom& g, const ClusterPlan& plan);
+size_t cl_exchange_words(int L, const ClusterPlan& plan);
 unsigned long long cl_exchange_seqs(const ClusterPlan& plan, int nsweeps);
-size_t cl_mask_bytes_per_sweep(const Geom& g);
-cudaError_t launch_cl_mask_draw(const Geom& g, const SweepArgs& a, const uint64_t* t_base, uint64_t t0, int nsweeps,
-                                uint64_t* masks, bool overlap, cudaStream_t s);
-cudaError_t launch_cluster_sweeps(uint64_t* w0, uint64_t* w1, const Geom& g, const SweepArgs& a,
+size_t cl_mask_bytes_per_sweep(int L);
+size_t cl_dense_bytes(int L);
+cudaError_t launch_cl_mask_draw(int L, const SweepArgs& a, uint64_t t0, int nsweeps, uint64_t* masks, bool overlap,
+                                cudaStream_t s);
+cudaError_t launch_cluster_sweeps(uint64_t* w0, uint64_t* w1, uint32_t* dense, const Geom& g, const SweepArgs& a,
                                   const ClusterPlan& plan, int nsweeps, const uint64_t* masks, int64_t s0,
                                   int64_t every, const ClusterExchange& x, cudaStream_t s);
 
@@ -154,8 +159,8 @@ inline void launch_pdl(void (*kernel)(Params...), dim3 grid, dim3 block, cudaStr
 // Geometry checks shared by the entry points.
 bool valid_side(int32_t L);
 
-// Strips of at most `most` (and kStripWords) words for geometry g.
-Strips make_strips(const Geom& g, int most);
+// Strips of at most `most` (<= 16) words for rows of `words` words.
+Strips make_strips(int words, int most);
 
 // One half-sweep of one lattice (update and/or record), or the measurement
 // pass (update = false, record = true, colour 1); bw = 0: bgrp threads a

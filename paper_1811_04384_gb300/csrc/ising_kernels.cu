@@ -498,14 +498,13 @@ SweepArgs make_sweep_args(uint64_t seed, const uint64_t thr[2], const uint64_t* 
     return a;
 }
 
-Strips make_strips(const Geom& g, int most)
+Strips make_strips(int words, int most)
 {
-    most = std::min(most, kStripWords);
     Strips st;
-    st.n = (uint32_t)((g.W + most - 1) / most);
-    st.width = ((uint32_t)g.W + st.n - 1) / st.n;               // strips of about equal width
-    st.n = ((uint32_t)g.W + st.width - 1) / st.width;
-    st.last = (uint32_t)g.W - (st.n - 1) * st.width;
+    st.n = (uint32_t)((words + most - 1) / most);
+    st.width = ((uint32_t)words + st.n - 1) / st.n;               // strips of about equal width
+    st.n = ((uint32_t)words + st.width - 1) / st.width;
+    st.last = (uint32_t)words - (st.n - 1) * st.width;
     // q < 2^18 and width <= 16, so hi32(q * ceil(2^32 / width)) = q / width
     auto magic = [](uint32_t w) { return w == 1 ? 0u : (uint32_t)(((1ull << 32) + w - 1) / w); };
     st.magic = magic(st.width);
@@ -535,7 +534,7 @@ cudaError_t launch_half_sweep(int bw, int bgrp, int colour, bool update, bool re
                               uint64_t* own, const uint64_t* other, const Geom& g, const SweepArgs& a,
                               bool in_graphs, cudaStream_t s)
 {
-    const Strips st = make_strips(g, bw == 0 ? kStripWords : bw);
+    const Strips st = make_strips(g.W, bw == 0 ? kStripWords : std::min(bw, kStripWords));
     const uint32_t threads = (uint32_t)(bw == 0 ? bgrp : bw * bgrp);
     const uint32_t items = (uint32_t)((g.L + 3) / 4) * st.width;
     dim3 block(threads), grid((items + threads - 1) / threads, st.n);

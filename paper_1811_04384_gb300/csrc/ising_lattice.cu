@@ -76,6 +76,7 @@ struct ising_lattice {
     ulonglong2* masks = nullptr;                 // lazily allocated: pre-drawn masks of the on-chip path
     size_t mask_bytes = 0;
     int clusters = 0;                            // clusters of the cluster path's launches (0: automatic)
+    uint32_t* dense = nullptr;                   // column-interleaved layout on the cluster path: its dense rows (lazily)
     uint64_t* xbuf = nullptr;                    // rows between clusters (lazily, several clusters only)
     size_t xbuf_bytes = 0;
     unsigned long long* xflag = nullptr;         // kXWords: their flags, the error word and the agreement words
@@ -136,6 +137,7 @@ static void free_handle(ising_lattice* h)
     if (h->staging) cudaFree(h->staging);
     if (h->staging2) cudaFree(h->staging2);
     if (h->masks) cudaFree(h->masks);
+    if (h->dense) cudaFree(h->dense);
     if (h->xbuf) cudaFree(h->xbuf);
     if (h->xflag) cudaFree(h->xflag);
     if (h->host_xerr) cudaFreeHost(h->host_xerr);
@@ -483,7 +485,7 @@ static bool use_resident(const ising_lattice* h)
     if (items <= kResidentAutoMaxItems) return true;
     if (items > kPremaskedMaxItems) return false;
     ClusterPlan cp;
-    return !cluster_plan(h->g, 1, &cp);
+    return !cluster_plan(h->g.L, false, 1, &cp);
 }
 
 // Pre-drawn masks of the on-chip path: 64 B per item and sweep, drawn for
@@ -541,26 +543,22 @@ static int run_resident(ising_lattice* h, int n, int every)
 // ---- Cluster path (mid-size lattices)
 // Above the on-chip range and up to kClusterMaxL, thread-block clusters keep
 // the lattice in their blocks' shared memory over a whole piece of sweeps
-// (cluster_sweeps_kernel): one cluster, or several (auto_clusters) whose
-// boundary blocks pass their halo rows through a small global buffer.  The
-// masks of each piece are drawn on all SMs into one of two buffers: the draw
-// of piece j + 1 follows the cluster launch of piece j in the stream with
-// programmatic stream serialization, so it runs on the SMs the clusters leave
-// free while piece j is applied, and writes the buffer piece j - 1 read
-// (complete before piece j started).  Replayed graphs of short half-sweeps
-// stay for the launch path (ISING_PATH_LAUNCHES) and, above kClusterMaxL,
-// the fused half-sweeps.  With one cluster (before several), sweeps without
-// records, spin-updates/ns, cluster against graphs: L = 296: 138 / 34;
-// L = 512: 255 / 96; L = 1008: 472 / 313; L = 1150: 499 / 362; but L = 1200:
-// 297 / 368, where the window needs 4 words per thread, which spill
-// registers.  Two 16 MB mask buffers (43-sweep pieces at L = 1008) gave 444
-// there: each launch loads and writes back the lattice and refills the mask
-// ring.  In the column-interleaved layout (one cluster): L = 1008: 373 /
-// 304; L = 1092: 403 / 338; several clusters below (ci_auto_clusters).
+// (cluster_sweeps_kernel), one bit per spin: one cluster, or several
+// (auto_clusters) whose boundary blocks pass their halo rows through a small
+// global buffer.  The masks of each piece are drawn on all SMs into one of two
+// buffers: the draw of piece j + 1 follows the cluster launch of piece j in the
+// stream with programmatic stream serialization, so it runs on the SMs the
+// clusters leave free while piece j is applied, and writes the buffer piece
+// j - 1 read (complete before piece j started).  A call runs as about
+// kClusterPieces pieces, because the first draw and the last apply overlap
+// nothing (us per call for 1 / 4 / 6 / 10 pieces, k = 12: L = 1008 x 500 sweeps
+// 640 / 596 / 589 / 613; L = 1500 x 400 on two clusters 863 / 768 / 749 / 765; L =
+// 296 x 1000: 565 / 563 / 566 / 579).  A column-interleaved lattice is converted
+// to dense rows and back around the call.
 constexpr int kClusterMaxL = 3000;
 constexpr int kCiClusterMaxL = 2604;               // the column-interleaved layout (L % 84 == 0)
 constexpr size_t kClusterMaskBytes = 256u << 20;   // both buffers
-constexpr int kClusterMaxPiece = 256;
+constexpr int kClusterMaxPiece = 256, kClusterMinPiece = 32, kClusterPieces = 4;
 // The words between clusters (xflag, u64 each): 2 flags for each of at most
 // 16 boundaries, the error word of the waits (u32), the agreement words
 // (cl_decide: two sets of {count, verdict} and the first piece given up,
@@ -571,35 +569,15 @@ constexpr int kXWords = kXGate + 3;
 constexpr int kXStatusWords = kXWords - kXErr;
 
 // Clusters of a launch on the automatic path for side L (0: not the cluster
-// path).  Measured on GB300, sweeps without records, spin-updates/ns by
-// clusters 1 .. 7 (graph replays): L = 296: 124 / 86 / 73 / 55 / 29 / 28 / 27
-// (34); L = 700: 302 / 352 / 383 / 381 / 347 / 300 / 300 (173); L = 1008:
-// 439 / 506 / 552 / 667 / 638 / 626 / 598 (311); L = 1300: 240 / 651 / 717 /
-// 739 / 767 / 773 / 723 (399); L = 1500: 409 / 771 / 922 / 904 / 943 / 904 /
-// 880 (539); L = 2016: - / 657 / 993 / 1009 / 982 / 946 / 918 (742);
-// L = 3000: four clusters 980 (939); L = 4096: seven 954 against the fused
-// launches' 1031.  More clusters leave fewer SMs for the mask draws.
-static int auto_clusters(int L)
+// path).  Measured on GB300, a record every 10 sweeps, us per call by clusters
+// 1 / 2 / 3 / 4: L = 700 (1000 sweeps): 872 / 1,125 / 1,088 / 1,101; L = 1008 (500):
+// 570 / 661 / 643 / 671; L = 1300 (500): 883 / 804 / 830 / 850; L = 1500 (400): 814 /
+// 768 / 767 / 795; L = 1700 (400): - / 991 / 951 / 955; L = 2016 (300): - / 955 / 946 /
+// 939; L = 2600 (200): - / - / 1,043 / 1,028; L = 3000: four only.
+static int auto_clusters(int L, bool interleaved)
 {
-    constexpr struct { int max_L, clusters; } kRule[] = {
-        {558, 1}, {898, 3}, {1098, 4}, {1448, 6}, {1698, 5}, {kClusterMaxL, 4}};
-    for (const auto& r : kRule)
-        if (L <= r.max_L) return r.clusters;
-    return 0;
-}
-
-// The same for the column-interleaved layout, whose per-word draws cost more
-// (19 Philox products per call against 16), so the draws on the SMs the
-// clusters leave free bound it sooner.  Measured on GB300, sweeps without
-// records, spin-updates/ns by clusters 1 .. 7 (graph replays): L = 1008:
-// 378 / 397 / 427 / 466 / 441 / 449 / 444 (305); L = 1512: 354 / 567 / 589 /
-// 583 / 578 / 583 / 563 (444); L = 2016: - / 548 / 538 / 651 / 629 / 611 /
-// 598 (574); L = 2520: three to seven 613 / 600 / 655 / 648 / 595 (633);
-// L = 3024: four to seven 620 / 623 / 598 / 588 (666).
-static int ci_auto_clusters(int L)
-{
-    constexpr struct { int max_L, clusters; } kRule[] = {
-        {840, 1}, {1092, 4}, {1764, 3}, {2184, 4}, {kCiClusterMaxL, 5}};
+    constexpr struct { int max_L, clusters; } kRule[] = {{1150, 1}, {1600, 2}, {2400, 3}, {kClusterMaxL, 4}};
+    if (interleaved && L > kCiClusterMaxL) return 0;
     for (const auto& r : kRule)
         if (L <= r.max_L) return r.clusters;
     return 0;
@@ -607,13 +585,12 @@ static int ci_auto_clusters(int L)
 
 static bool plan_cluster_g(const ising_lattice* h, int clusters, ClusterPlan* plan)
 {
-    return h->layout == ISING_LAYOUT_COLUMN_INTERLEAVED ? ci_cluster_plan(h->g.L, clusters, plan)
-                                                        : cluster_plan(h->g, clusters, plan);
+    return cluster_plan(h->g.L, h->layout == ISING_LAYOUT_COLUMN_INTERLEAVED, clusters, plan);
 }
 
 static int auto_clusters_of(const ising_lattice* h)
 {
-    return h->layout == ISING_LAYOUT_COLUMN_INTERLEAVED ? ci_auto_clusters(h->g.L) : auto_clusters(h->g.L);
+    return auto_clusters(h->g.L, h->layout == ISING_LAYOUT_COLUMN_INTERLEAVED);
 }
 
 // The cluster-path launch for h: the clusters set by ising_set_clusters, else
@@ -646,10 +623,11 @@ static int run_cluster(ising_lattice* h, int64_t n, int64_t every, unsigned long
 {
     const Geom& g = h->g;
     const bool ci = h->layout == ISING_LAYOUT_COLUMN_INTERLEAVED;
-    const size_t per_sweep = ci ? ci_cl_mask_bytes_per_sweep(g.L) : cl_mask_bytes_per_sweep(g);
-    const int max_piece =
-        (int)std::max<size_t>(1, std::min<size_t>(kClusterMaxPiece, kClusterMaskBytes / (2 * per_sweep)));
-    const size_t buf = (size_t)std::min<int64_t>(n, max_piece) * per_sweep;
+    const size_t per_sweep = cl_mask_bytes_per_sweep(g.L);
+    const int64_t wanted = std::max<int64_t>(kClusterMinPiece, (n + kClusterPieces - 1) / kClusterPieces);
+    const int max_piece = (int)std::max<size_t>(
+        1, std::min<size_t>((size_t)std::min<int64_t>(wanted, kClusterMaxPiece), kClusterMaskBytes / (2 * per_sweep)));
+    const size_t buf = (size_t)std::min<int64_t>(n, max_piece) * per_sweep + kClMaskPad * per_sweep / 2;
     if (h->mask_bytes < 2 * buf) {
         if (h->masks) cudaFree(h->masks);
         h->masks = nullptr;
@@ -667,9 +645,16 @@ static int run_cluster(ising_lattice* h, int64_t n, int64_t every, unsigned long
     const int64_t np = (n + max_piece - 1) / max_piece;
     auto draw = [&](int64_t j, bool overlap) {
         const uint64_t t0 = h->t + (uint64_t)(j * max_piece);
-        return ci ? ci_cl_mask_draw(g.L, a, t0, part_of(j), masks[j & 1], overlap, h->stream)
-                  : launch_cl_mask_draw(g, a, nullptr, t0, part_of(j), masks[j & 1], overlap, h->stream);
+        return launch_cl_mask_draw(g.L, a, t0, part_of(j), masks[j & 1], overlap, h->stream);
     };
+    // the column-interleaved layout's words become dense rows for the call
+    if (ci && np > 0) {
+        cudaError_t e = cudaSuccess;
+        if (!h->dense) e = cudaMalloc(&h->dense, cl_dense_bytes(g.L));
+        if (e != cudaSuccess) { h->dense = nullptr; cuda_fail(e, "cudaMalloc dense rows"); return ISING_ENOMEM; }
+        e = ci_to_dense(h->words[0], g.L, h->dense, h->stream);
+        if (e != cudaSuccess) return cuda_fail(e, "ci_to_dense");
+    }
     if (np > 0) {
         cudaError_t e = draw(0, false);
         if (e != cudaSuccess) return cuda_fail(e, "cluster mask draw");
@@ -677,7 +662,7 @@ static int run_cluster(ising_lattice* h, int64_t n, int64_t every, unsigned long
     ClusterExchange x = {nullptr, nullptr, 0, nullptr, 0, nullptr, 0, 0};
     const uint64_t t_start = h->t;
     if (plan.clusters > 1) {
-        const size_t xb = (ci ? ci_cl_exchange_words(g.L, plan) : cl_exchange_words(g, plan)) * sizeof(uint64_t);
+        const size_t xb = cl_exchange_words(g.L, plan) * sizeof(uint64_t);
         cudaError_t e = cudaSuccess;
         if (h->xbuf_bytes < xb) {
             if (h->xbuf) cudaFree(h->xbuf);
@@ -712,10 +697,8 @@ static int run_cluster(ising_lattice* h, int64_t n, int64_t every, unsigned long
         }
         if (plan.clusters > 1 && h->absent_after >= 0 && h->absent_after-- == 0)
             x.absent = 1;                            // one block more than the launch has: it gives up
-        cudaError_t e = ci ? ci_cluster_sweeps(h->words[0], g.L, a, plan, part_of(j), masks[j & 1], done, every, x,
-                                               h->stream)
-                           : launch_cluster_sweeps(h->words[0], h->words[1], g, a, plan, part_of(j), masks[j & 1],
-                                                   done, every, x, h->stream);
+        cudaError_t e = launch_cluster_sweeps(h->words[0], h->words[1], ci ? h->dense : nullptr, g, a, plan,
+                                              part_of(j), masks[j & 1], done, every, x, h->stream);
         if (e != cudaSuccess) return cuda_fail(e, "cluster sweeps kernel");
         if (plan.clusters > 1) {
             x.seq += cl_exchange_seqs(plan, part_of(j));
@@ -725,6 +708,10 @@ static int run_cluster(ising_lattice* h, int64_t n, int64_t every, unsigned long
             e = draw(j + 1, true);
             if (e != cudaSuccess) return cuda_fail(e, "cluster mask draw");
         }
+    }
+    if (ci && np > 0) {
+        cudaError_t e = ci_from_dense(h->words[0], g.L, h->dense, h->stream);
+        if (e != cudaSuccess) return cuda_fail(e, "ci_from_dense");
     }
     if (n > 0) {
         cudaError_t e = launch_advance_sweep(h->t_dev, (uint64_t)n, h->stream);
