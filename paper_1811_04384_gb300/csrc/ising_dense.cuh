@@ -127,6 +127,7 @@ __global__ void __launch_bounds__(128, 8)
 dense_mask_draw_kernel(DenseGeom d, Strips st, SweepArgs a, uint64_t t0, uint64_t* __restrict__ masks)
 {
     __shared__ uint2 tab[32 * kDenseStripWords];
+    pdl_launch();      // a launch that applies these masks may start and load its lattice
     const uint32_t w0 = blockIdx.y * st.width;
     const bool last = blockIdx.y == st.n - 1u;
     const uint32_t width = last ? st.last : st.width, magic = last ? st.magic_last : st.magic;

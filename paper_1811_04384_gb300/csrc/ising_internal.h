@@ -61,11 +61,6 @@ cudaError_t launch_resident(uint64_t* w0, uint64_t* w1, const Geom& g, const Swe
 // allow_resident_smem(bytes) leaves room for 1024 record counters).
 constexpr int kPremaskedMaxItems = 512;
 inline int premasked_rows_per_thread(int items) { return items <= 256 ? 1 : 2; }
-// Two threads per row (one per 32-bit half of its word) up to 100 items: on
-// GB300, 1000 recorded sweeps took 0.36 / 0.35 / 0.41 / 0.78 ms at L = 16 /
-// 32 / 64 / 100 against 0.57 / 0.44 / 0.45 / 0.87 with one, but 0.99
-// against 0.92 at L = 128 (128 items, 32 warps).
-inline int premasked_threads_per_row(int items) { return items <= 100 ? 2 : 1; }
 cudaError_t launch_mask_draw(const Geom& g, const SweepArgs& a, uint64_t t0, int nsweeps, ulonglong2* masks,
                              cudaStream_t s);
 cudaError_t launch_resident_premasked(uint64_t* w0, uint64_t* w1, const Geom& g, const SweepArgs& a, int s_base,
@@ -121,6 +116,15 @@ cudaError_t launch_cl_mask_draw(int L, const SweepArgs& a, uint64_t t0, int nswe
 cudaError_t launch_cluster_sweeps(uint64_t* w0, uint64_t* w1, uint32_t* dense, const Geom& g, const SweepArgs& a,
                                   const ClusterPlan& plan, int nsweeps, const uint64_t* masks, int64_t s0,
                                   int64_t every, const ClusterExchange& x, cudaStream_t s);
+
+// The on-chip path up to side kWarpMaxL (ising_warp.cu): sweeps s_base + 1 ..
+// s_base + n of a run in one warp's registers, with masks from
+// launch_cl_mask_draw (launched just before; their buffer has kClMaskPad
+// half-sweeps to spare), (E, M) records into rec (device or pinned host
+// memory), then *t_dev = t_end.
+constexpr int kWarpMaxL = 128;
+cudaError_t launch_warp_sweeps(uint64_t* w0, uint64_t* w1, const Geom& g, const uint64_t* masks, int s_base, int n,
+                               int every, long long* rec, uint64_t* t_dev, uint64_t t_end, cudaStream_t s);
 
 // Launch `kernel` with programmatic stream serialization (every thread of the
 // kernel calls pdl_wait before it reads what an earlier launch writes): the

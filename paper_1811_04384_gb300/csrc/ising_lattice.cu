@@ -492,34 +492,61 @@ static bool use_resident(const ising_lattice* h)
 // at most this many bytes of sweeps at a time.
 constexpr size_t kMaskBufMax = 16u << 20;
 
-// n sweeps with the lattice resident in shared memory, E/M records (if any)
-// written as (E, M) pairs into the count buffer.  Up to kPremaskedMaxItems
-// items the accept masks are drawn first by all SMs (mask_draw_kernel), in
-// pieces of at most kMaskBufMax bytes, and the on-chip kernel only applies
-// them; larger lattices draw inside the on-chip kernel.
-static int run_resident(ising_lattice* h, int n, int every)
+// The mask buffer of the on-chip paths, at least `need` bytes.
+static int ensure_masks(ising_lattice* h, size_t need)
+{
+    if (h->mask_bytes >= need) return ISING_OK;
+    if (h->masks) cudaFree(h->masks);
+    h->masks = nullptr;
+    h->mask_bytes = 0;
+    cudaError_t e = cudaMalloc(&h->masks, need);
+    if (e != cudaSuccess) { h->masks = nullptr; cuda_fail(e, "cudaMalloc masks"); return ISING_ENOMEM; }
+    h->mask_bytes = need;
+    return ISING_OK;
+}
+
+// n sweeps on chip, E/M records (if any) as (E, M) pairs: up to kWarpMaxL in
+// one warp's registers (warp_sweeps_kernel), whose records go straight to the
+// pinned host buffer (*direct = true; they are there once the stream is
+// synchronised); larger lattices in shared memory, records in the count
+// buffer.  The accept masks are drawn first by all SMs, in pieces of at most
+// kMaskBufMax bytes, and the on-chip kernel only applies them; above
+// kPremaskedMaxItems items the on-chip kernel draws them itself.
+static int run_resident(ising_lattice* h, int n, int every, bool* direct)
 {
     const Geom& g = h->g;
+    const SweepArgs a = base_args(h);
+    *direct = g.L <= kWarpMaxL;
+    if (*direct) {
+        const size_t per_sweep = cl_mask_bytes_per_sweep(g.L), pad = kClMaskPad * per_sweep / 2;
+        const int max_sweeps = (int)std::min<size_t>(kMaskBufMax / per_sweep, 65535);      // grid layers of a draw
+        int rc = ensure_masks(h, (size_t)std::min(n, max_sweeps) * per_sweep + pad);
+        if (rc != ISING_OK) return rc;
+        uint64_t* masks = reinterpret_cast<uint64_t*>(h->masks);
+        for (int done = 0; done < n;) {
+            const int part = std::min(n - done, max_sweeps);
+            cudaError_t e = launch_cl_mask_draw(g.L, a, h->t, part, masks, false, h->stream);
+            if (e != cudaSuccess) return cuda_fail(e, "dense_mask_draw_kernel");
+            h->t += (uint64_t)part;
+            e = launch_warp_sweeps(h->words[0], h->words[1], g, masks, done, part, every,
+                                   reinterpret_cast<long long*>(h->host_counts), h->t_dev, h->t, h->stream);
+            if (e != cudaSuccess) return cuda_fail(e, "warp_sweeps_kernel");
+            done += part;
+        }
+        return ISING_OK;
+    }
     if (!h->resident_attr) {
         cudaError_t e = allow_resident_smem((int)kResidentMaxBytes);
         if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute");
         h->resident_attr = true;
     }
-    const SweepArgs a = base_args(h);
     long long* rec = reinterpret_cast<long long*>(h->counts);
     const int items = ((g.L + 3) / 4) * g.W;
     if (items <= kPremaskedMaxItems) {
         const size_t per_sweep = (size_t)items * 4 * sizeof(ulonglong2);
         const int max_sweeps = (int)std::max<size_t>(1, kMaskBufMax / per_sweep);
-        const size_t need = (size_t)std::min(n, max_sweeps) * per_sweep;
-        if (h->mask_bytes < need) {
-            if (h->masks) cudaFree(h->masks);
-            h->masks = nullptr;
-            h->mask_bytes = 0;
-            cudaError_t e = cudaMalloc(&h->masks, need);
-            if (e != cudaSuccess) { h->masks = nullptr; cuda_fail(e, "cudaMalloc masks"); return ISING_ENOMEM; }
-            h->mask_bytes = need;
-        }
+        int rc = ensure_masks(h, (size_t)std::min(n, max_sweeps) * per_sweep);
+        if (rc != ISING_OK) return rc;
         for (int done = 0; done < n;) {
             const int part = std::min(n - done, max_sweeps);
             cudaError_t e = launch_mask_draw(g, a, h->t + (uint64_t)done, part, h->masks, h->stream);
@@ -628,14 +655,8 @@ static int run_cluster(ising_lattice* h, int64_t n, int64_t every, unsigned long
     const int max_piece = (int)std::max<size_t>(
         1, std::min<size_t>((size_t)std::min<int64_t>(wanted, kClusterMaxPiece), kClusterMaskBytes / (2 * per_sweep)));
     const size_t buf = (size_t)std::min<int64_t>(n, max_piece) * per_sweep + kClMaskPad * per_sweep / 2;
-    if (h->mask_bytes < 2 * buf) {
-        if (h->masks) cudaFree(h->masks);
-        h->masks = nullptr;
-        h->mask_bytes = 0;
-        cudaError_t e = cudaMalloc(&h->masks, 2 * buf);
-        if (e != cudaSuccess) { h->masks = nullptr; cuda_fail(e, "cudaMalloc masks"); return ISING_ENOMEM; }
-        h->mask_bytes = 2 * buf;
-    }
+    int rc = ensure_masks(h, 2 * buf);
+    if (rc != ISING_OK) return rc;
     SweepArgs a = base_args(h);
     a.counts = counts;
     uint64_t* masks[2] = {reinterpret_cast<uint64_t*>(h->masks),
@@ -738,7 +759,7 @@ static int run_cluster(ising_lattice* h, int64_t n, int64_t every, unsigned long
             // same results); the automatic path keeps to one cluster from now on.
             const int64_t done = (int64_t)gave_up * max_piece;
             h->multi_gave_up = true;
-            int rc = reset_t(h, t_start + (uint64_t)done);
+            rc = reset_t(h, t_start + (uint64_t)done);
             if (rc != ISING_OK) return rc;
             const int64_t rec_base = (int64_t)(counts - h->counts) / (2 * kCountSlots);
             if (every > 0 && n / every > done / every) {
@@ -886,7 +907,8 @@ extern "C" int ising_sweep(ising_lattice* h, int64_t n)
     if (use_resident(h)) {
         while (n > 0) {
             const int c = (int)std::min<int64_t>(n, 1 << 30);
-            int rc = run_resident(h, c, 0x7fffffff);
+            bool direct;
+            int rc = run_resident(h, c, 0x7fffffff, &direct);
             if (rc != ISING_OK) return rc;
             n -= c;
         }
@@ -938,10 +960,13 @@ extern "C" int ising_sweep_record(ising_lattice* h, int64_t n, int64_t every, in
         while (done_rec < nrec) {
             // at most 2^30 sweeps a launch
             const int64_t chunk = std::min<int64_t>({nrec - done_rec, (int64_t)kRecordsPerChunk, (1 << 30) / every});
-            int rc = run_resident(h, (int)(chunk * every), (int)every);
+            bool direct;
+            int rc = run_resident(h, (int)(chunk * every), (int)every, &direct);
             if (rc != ISING_OK) return rc;
             const size_t bytes = (size_t)chunk * 2 * sizeof(long long);
-            cudaError_t e = cudaMemcpyAsync(h->host_counts, h->counts, bytes, cudaMemcpyDeviceToHost, h->stream);
+            cudaError_t e = cudaSuccess;
+            if (!direct)
+                e = cudaMemcpyAsync(h->host_counts, h->counts, bytes, cudaMemcpyDeviceToHost, h->stream);
             if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
             if (e != cudaSuccess) return cuda_fail(e, "resident records");
             const long long* rec = reinterpret_cast<const long long*>(h->host_counts);
