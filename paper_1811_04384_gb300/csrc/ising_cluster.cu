@@ -610,8 +610,9 @@ cudaError_t launch_cl_mask_draw(int L, const SweepArgs& a, uint64_t t0, int nswe
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = overlap ? 1 : 0;
-    return a.rounds == 7 ? cudaLaunchKernelEx(&cfg, dense_mask_draw_kernel<7>, d, st, a, t0, masks)
-                         : cudaLaunchKernelEx(&cfg, dense_mask_draw_kernel<10>, d, st, a, t0, masks);
+    const DenseOut to = {4u * (uint32_t)d.P, (uint32_t)d.P, (uint32_t)L * (uint32_t)d.P};
+    return a.rounds == 7 ? cudaLaunchKernelEx(&cfg, dense_mask_draw_kernel<7, 1>, d, st, a, t0, to, masks)
+                         : cudaLaunchKernelEx(&cfg, dense_mask_draw_kernel<10, 1>, d, st, a, t0, to, masks);
 }
 
 cudaError_t launch_cluster_sweeps(uint64_t* w0, uint64_t* w1, uint32_t* dense, const Geom& g, const SweepArgs& a,

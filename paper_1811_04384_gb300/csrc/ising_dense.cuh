@@ -81,27 +81,23 @@ __device__ __forceinline__ uint64_t packed_from_dense(uint32_t d0, uint32_t d1, 
     return spread_fields(__funnelshift_r(d0, d1, (kFields * w) & 31));
 }
 
-// Draws of fields 0 .. 31 of a dense word for the four rows of a row group.
-template <int k, int ROUNDS, typename Calls>
+// Draws of fields k .. N - 1 of the FirstTable column for the four rows of a
+// row group, into bits k .. N - 1.
+template <int k, int N, int ROUNDS, typename Calls>
 struct DenseLoop {
     __device__ __forceinline__ static void run(const Calls& calls, const PhiloxKeys& rk, uint32_t (&m1)[4],
                                                uint32_t (&m0)[4], uint32_t thr0, uint32_t thr1)
     {
-        uint32_t rnd[4];
-        calls.template call<ROUNDS>(k, rk, rnd);
+        if constexpr (k < N) {
+            uint32_t rnd[4];
+            calls.template call<ROUNDS>(k, rk, rnd);
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            accept_bit<k>(m1[e], rnd[e], thr1);
-            accept_bit<k>(m0[e], rnd[e], thr0);
+            for (int e = 0; e < 4; ++e) {
+                accept_bit<k>(m1[e], rnd[e], thr1);
+                accept_bit<k>(m0[e], rnd[e], thr0);
+            }
+            DenseLoop<k + 1, N, ROUNDS, Calls>::run(calls, rk, m1, m0, thr0, thr1);
         }
-        DenseLoop<k + 1, ROUNDS, Calls>::run(calls, rk, m1, m0, thr0, thr1);
-    }
-};
-template <int ROUNDS, typename Calls>
-struct DenseLoop<32, ROUNDS, Calls> {
-    __device__ __forceinline__ static void run(const Calls&, const PhiloxKeys&, uint32_t (&)[4], uint32_t (&)[4],
-                                               uint32_t, uint32_t)
-    {
     }
 };
 
@@ -117,39 +113,65 @@ struct DenseFirst {
     }
 };
 
-// The accept masks of sweeps t0 + 1 .. (one per grid layer z), both colours:
-// masks[((z * 2 + c) * L + i) * P + w] = r < thr1 in the low half, r < thr0 in
-// the high half, 0 on dead bits and pad words, set where the threshold is
-// 2^32.  A block owns consecutive items (row group, word) of one strip, as in
-// half_sweep_kernel; its table of first products serves both colours.
-template <int ROUNDS>
+// Where the masks of row 4 grp + e, word w of a half-sweep go, in words:
+// masks[half * plane + grp * group + e * row + w].
+struct DenseOut {
+    uint32_t group, row, plane;
+};
+
+// The accept masks of sweeps t0 + 1 .., half-sweep by half-sweep (half =
+// 2 sweep + colour), one 64-bit word per dense word: r < thr1 in the low half,
+// r < thr0 in the high half, 0 on dead bits and pad words, set where the
+// threshold is 2^32.  A block owns consecutive items (row group, word) of one
+// strip, as in half_sweep_kernel.
+// SPLIT = 1: a grid layer per sweep, a thread draws a whole word for both
+// colours from one table of first products.  SPLIT = 4, for lattices of at most
+// 64 items, where that would leave one half-empty warp per block with a chain
+// of 64 draws: a layer per half-sweep, and a thread draws a quarter of a word
+// (a byte of each mask).  The draws of 10 sweeps of L = 64 are a chain of 8
+// calls then instead of 64.
+template <int ROUNDS, int SPLIT>
 __global__ void __launch_bounds__(128, 8)
-dense_mask_draw_kernel(DenseGeom d, Strips st, SweepArgs a, uint64_t t0, uint64_t* __restrict__ masks)
+dense_mask_draw_kernel(DenseGeom d, Strips st, SweepArgs a, uint64_t t0, DenseOut to, uint64_t* __restrict__ masks)
 {
+    constexpr int N = 32 / SPLIT;
     __shared__ uint2 tab[32 * kDenseStripWords];
     pdl_launch();      // a launch that applies these masks may start and load its lattice
     const uint32_t w0 = blockIdx.y * st.width;
     const bool last = blockIdx.y == st.n - 1u;
     const uint32_t width = last ? st.last : st.width, magic = last ? st.magic_last : st.magic;
-    const uint64_t t = t0 + blockIdx.z + 1;
+    const uint32_t sweep = SPLIT == 1 ? blockIdx.z : blockIdx.z >> 1;
+    const uint64_t t = t0 + sweep + 1;
     first_products<32, kDenseStripWords>(tab, w0, width, magic, philox_first_key((uint32_t)t, a.rk));
-    const uint32_t q = blockIdx.x * blockDim.x + threadIdx.x;
+    const uint32_t thread = blockIdx.x * blockDim.x + threadIdx.x, q = thread / SPLIT, part = thread % SPLIT;
     const uint32_t grp = strip_group(q, magic), x = q - grp * width;
     const int w = (int)(w0 + x);
     if (grp * 4u >= (uint32_t)d.L) return;
-    const uint32_t live = dense_live(d, w);
-    uint64_t* out = masks + ((size_t)blockIdx.z * 2 * d.L + grp * 4u) * d.P + w;
+    const uint32_t live = dense_live(d, w) >> (N * part);
+    const int c0 = SPLIT == 1 ? 0 : blockIdx.z & 1;
+    uint64_t* out = masks + (size_t)(2 * sweep + c0) * to.plane + grp * to.group + w;
 #pragma unroll 1
-    for (int c = 0; c < 2; ++c, out += (size_t)d.L * d.P) {
+    for (int c = c0; c < (SPLIT == 1 ? 2 : c0 + 1); ++c, out += to.plane) {
         uint32_t m1[4] = {0, 0, 0, 0}, m0[4] = {0, 0, 0, 0};
         if (live) {
-            const RowCalls<DenseFirst> calls = {{tab + x}, philox_row_key(grp, (uint32_t)t, counter_high(t, c), a.rk)};
-            DenseLoop<0, ROUNDS, RowCalls<DenseFirst>>::run(calls, a.rk, m1, m0, a.thr0, a.thr1);
+            const RowCalls<DenseFirst> calls = {{tab + x + N * kDenseStripWords * part},
+                                                philox_row_key(grp, (uint32_t)t, counter_high(t, c), a.rk)};
+            DenseLoop<0, N, ROUNDS, RowCalls<DenseFirst>>::run(calls, a.rk, m1, m0, a.thr0, a.thr1);
         }
 #pragma unroll
-        for (int e = 0; e < 4; ++e)
-            if (grp * 4u + e < (uint32_t)d.L)
-                out[(size_t)e * d.P] = (uint64_t)((m0[e] | a.all0) & live) << 32 | ((m1[e] | a.all1) & live);
+        for (int e = 0; e < 4; ++e) {
+            if (grp * 4u + e >= (uint32_t)d.L) continue;
+            m1[e] = (m1[e] | a.all1) & live;
+            m0[e] = (m0[e] | a.all0) & live;
+            if constexpr (SPLIT == 1) {
+                out[(size_t)e * to.row] = (uint64_t)m0[e] << 32 | m1[e];
+            } else {
+                static_assert(N == 8, "a part is a byte");
+                uint8_t* byte = reinterpret_cast<uint8_t*>(out + (size_t)e * to.row) + part;
+                byte[0] = (uint8_t)m1[e];
+                byte[4] = (uint8_t)m0[e];
+            }
+        }
     }
 }
 

@@ -118,11 +118,13 @@ cudaError_t launch_cluster_sweeps(uint64_t* w0, uint64_t* w1, uint32_t* dense, c
                                   int64_t every, const ClusterExchange& x, cudaStream_t s);
 
 // The on-chip path up to side kWarpMaxL (ising_warp.cu): sweeps s_base + 1 ..
-// s_base + n of a run in one warp's registers, with masks from
-// launch_cl_mask_draw (launched just before; their buffer has kClMaskPad
-// half-sweeps to spare), (E, M) records into rec (device or pinned host
-// memory), then *t_dev = t_end.
+// s_base + n of a run in one warp's registers, with the masks that
+// launch_warp_mask_draw (just before; at most 32767 sweeps) left in `masks`,
+// (E, M) records into rec (device or pinned host memory), then *t_dev = t_end.
 constexpr int kWarpMaxL = 128;
+size_t warp_mask_bytes_per_sweep(int L);
+cudaError_t launch_warp_mask_draw(int L, const SweepArgs& a, uint64_t t0, int nsweeps, uint64_t* masks,
+                                  cudaStream_t s);
 cudaError_t launch_warp_sweeps(uint64_t* w0, uint64_t* w1, const Geom& g, const uint64_t* masks, int s_base, int n,
                                int every, long long* rec, uint64_t* t_dev, uint64_t t_end, cudaStream_t s);
 

@@ -518,14 +518,14 @@ static int run_resident(ising_lattice* h, int n, int every, bool* direct)
     const SweepArgs a = base_args(h);
     *direct = g.L <= kWarpMaxL;
     if (*direct) {
-        const size_t per_sweep = cl_mask_bytes_per_sweep(g.L), pad = kClMaskPad * per_sweep / 2;
-        const int max_sweeps = (int)std::min<size_t>(kMaskBufMax / per_sweep, 65535);      // grid layers of a draw
-        int rc = ensure_masks(h, (size_t)std::min(n, max_sweeps) * per_sweep + pad);
+        const size_t per_sweep = warp_mask_bytes_per_sweep(g.L);
+        const int max_sweeps = (int)std::min<size_t>(kMaskBufMax / per_sweep, 32767);      // grid layers of a draw
+        int rc = ensure_masks(h, (size_t)std::min(n, max_sweeps) * per_sweep);
         if (rc != ISING_OK) return rc;
         uint64_t* masks = reinterpret_cast<uint64_t*>(h->masks);
         for (int done = 0; done < n;) {
             const int part = std::min(n - done, max_sweeps);
-            cudaError_t e = launch_cl_mask_draw(g.L, a, h->t, part, masks, false, h->stream);
+            cudaError_t e = launch_warp_mask_draw(g.L, a, h->t, part, masks, h->stream);
             if (e != cudaSuccess) return cuda_fail(e, "dense_mask_draw_kernel");
             h->t += (uint64_t)part;
             e = launch_warp_sweeps(h->words[0], h->words[1], g, masks, done, part, every,

@@ -10,6 +10,8 @@
 // sites and no barrier.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "ising_dense.cuh"
 #include "ising_device.cuh"
 #include "ising_internal.h"
@@ -17,8 +19,17 @@
 namespace ising {
 namespace {
 
-constexpr int kWarpDepth = 8;       // half-sweeps a row's masks are copied ahead
-static_assert(kClMaskPad >= kWarpDepth, "the copies run that far past the last half-sweep");
+// Warp 0 sweeps, warp 4 leaves that scheduler to it, warp 5 copies masks, the
+// others count records.
+constexpr int kWarpThreads = 256, kIdle = 4, kCopier = 5, kCounters = kWarpThreads / 32 - 3;
+
+// Word rows without a pad: one word, or two.
+DenseGeom warp_geom(int L)
+{
+    DenseGeom d = dense_geom(L);
+    d.P = d.W;
+    return d;
+}
 
 // Lane l holds rows RPL l .. RPL l + RPL - 1 (RPL even, so a row's parity is
 // its register's) of W dense words of both colours; lanes past the last row
@@ -44,20 +55,34 @@ struct WarpLattice {
         }
     }
 
-    // One half-sweep of colour C with masks m[row][word] = (r < thr1, r < thr0).
-    // RECORD: the anti-aligned bonds of the updated rows and the up spins of
-    // both colours (live bits only), below nrows of the lane's rows.
-    template <int C, bool RECORD>
-    __device__ __forceinline__ void half_sweep(const uint32_t (&m)[RPL][2 * W], int nrows, const uint32_t (&live)[W],
-                                               uint32_t& anti, uint32_t& up)
+    // Row neighbours of colour C's rows in the other colour: the lanes' edge
+    // rows, and row r's inside the lane.
+    template <int C>
+    __device__ __forceinline__ void edges(uint32_t (&above)[W], uint32_t (&below)[W]) const
     {
-        uint32_t above[W], below[W];
 #pragma unroll
         for (int w = 0; w < W; ++w) {
             const uint32_t bottom = TWO && tail ? x[1 - C][1][w] : x[1 - C][RPL - 1][w];
             above[w] = __shfl_sync(0xffffffffu, bottom, prev);
             below[w] = __shfl_sync(0xffffffffu, x[1 - C][0][w], next);
         }
+    }
+
+    template <int C>
+    __device__ __forceinline__ void vertical(int r, int w, const uint32_t (&above)[W], const uint32_t (&below)[W],
+                                             uint32_t& u, uint32_t& d) const
+    {
+        u = r == 0 ? above[w] : x[1 - C][r > 0 ? r - 1 : 0][w];
+        d = r == RPL - 1 ? below[w] : x[1 - C][r < RPL - 1 ? r + 1 : r][w];
+        if (TWO && r == 1) d = tail ? below[w] : d;
+    }
+
+    // One half-sweep of colour C with masks m[row][word] = (r < thr1, r < thr0).
+    template <int C>
+    __device__ __forceinline__ void half_sweep(const uint32_t (&m)[RPL][2 * W])
+    {
+        uint32_t above[W], below[W];
+        edges<C>(above, below);
 #pragma unroll
         for (int r = 0; r < RPL; ++r) {
             uint32_t h1[W];
@@ -65,76 +90,143 @@ struct WarpLattice {
             else side<false>(x[1 - C][r], h1);
 #pragma unroll
             for (int w = 0; w < W; ++w) {
-                const uint32_t u = r == 0 ? above[w] : x[1 - C][r > 0 ? r - 1 : 0][w];
-                uint32_t d = r == RPL - 1 ? below[w] : x[1 - C][r < RPL - 1 ? r + 1 : r][w];
-                if (TWO && r == 1) d = tail ? below[w] : d;
-                const uint32_t h0 = x[1 - C][r][w];
-                const uint32_t s = flip_all(x[C][r][w], u, d, h0, h1[w], m[r][2 * w], m[r][2 * w + 1]);
-                x[C][r][w] = s;
-                if (RECORD && r < nrows) {
-                    anti += __popc(s ^ u) + __popc(s ^ d) + __popc(s ^ h0) + __popc((s ^ h1[w]) & live[w]);
-                    up += __popc(s) + __popc(h0);
-                }
+                uint32_t u, d;
+                vertical<C>(r, w, above, below, u, d);
+                x[C][r][w] = flip_all(x[C][r][w], u, d, x[1 - C][r][w], h1[w], m[r][2 * w], m[r][2 * w + 1]);
             }
         }
+    }
+
+    // The anti-aligned bonds of colour 1's rows and the up spins of both
+    // colours (live bits only) of a lane with rows.  Bits are added by
+    // three-input adders (sum, carry) and counted as ones, twos and fours: a
+    // population count takes four times the issue slots of a logic operation.
+    __device__ __forceinline__ void count(const uint32_t (&live)[W], uint32_t& anti, uint32_t& up) const
+    {
+        constexpr int kSum = kLutA ^ kLutB ^ kLutC, kCarry = (kLutA & kLutB) | (kLutA & kLutC) | (kLutB & kLutC);
+        uint32_t above[W], below[W], ones = 0, twos = 0, fours = 0, up1 = 0, up2 = 0;
+        edges<1>(above, below);
+#pragma unroll
+        for (int r = 0; r < RPL; ++r) {
+            uint32_t h1[W];
+            if ((r & 1) == 1) side<true>(x[0][r], h1);
+            else side<false>(x[0][r], h1);
+            if (TWO && r >= 2 && tail) continue;
+#pragma unroll
+            for (int w = 0; w < W; ++w) {
+                uint32_t u, d;
+                vertical<1>(r, w, above, below, u, d);
+                const uint32_t s = x[1][r][w], h0 = x[0][r][w];
+                const uint32_t a = s ^ u, b = s ^ d, c = s ^ h0, e = (s ^ h1[w]) & live[w];
+                const uint32_t t1 = lop3<kCarry>(ones, a, b), o = lop3<kSum>(ones, a, b), t2 = lop3<kCarry>(o, c, e);
+                ones = lop3<kSum>(o, c, e);
+                fours += __popc(lop3<kCarry>(twos, t1, t2));
+                twos = lop3<kSum>(twos, t1, t2);
+                up2 += __popc(lop3<kCarry>(up1, s, h0));
+                up1 = lop3<kSum>(up1, s, h0);
+            }
+        }
+        anti = __popc(ones) + 2 * __popc(twos) + 4 * fours;
+        up = __popc(up1) + 2 * up2;
     }
 };
 
 // Sweeps s_base + 1 .. s_base + n of a run with the masks of
-// dense_mask_draw_kernel (P = 2: 16 bytes a row), a record after each of the
-// run's sweeps s with s % every == 0 at records[2 (s / every - 1)] as (E, M);
-// then *t_dev = t_end.  Launched programmatically behind the mask draw, which
-// no kernel overlaps, so the lattice is there before the wait.
-template <int W, int RPL, bool TWO>
-__global__ void __launch_bounds__(32)
+// dense_mask_draw_kernel in the warp_mask_layout form: `rows` of 16 bytes per
+// lane, 2 C of them a sweep.  Warp 0 sweeps; warp kCopier copies the masks
+// into a ring of STAGES stages of K sweeps, and the other warps (on the other
+// schedulers) count the records, (E, M) of the run's sweeps s with s % every == 0 to
+// records[2 (s / every - 1)], from the states that warp 0 leaves in shared
+// memory.  One barrier per stage.  At the end *t_dev = t_end.  Launched
+// programmatically behind the mask draw, which no kernel overlaps, so the
+// lattice is there before the wait.
+template <int W, int RPL, bool TWO, int K, int STAGES>
+__global__ void __launch_bounds__(kWarpThreads)
 warp_sweeps_kernel(uint64_t* __restrict__ w0, uint64_t* __restrict__ w1, Geom g, DenseGeom d,
-                   const uint64_t* __restrict__ masks, int s_base, int n, int every, long long* records,
+                   const uint4* __restrict__ masks, int s_base, int n, int every, long long* records,
                    uint64_t* t_dev, uint64_t t_end)
 {
-    __shared__ __align__(16) uint4 ring[kWarpDepth][RPL][32];
-    const int lane = threadIdx.x, last = (g.L + RPL - 1) / RPL - 1;
-    WarpLattice<W, RPL, TWO> lat;
-    lat.prev = lane == 0 ? last : lane - 1;
-    lat.next = lane == last ? 0 : lane + 1;
-    lat.tail = TWO && lane == last;
-    lat.lsh = (uint32_t)(d.lb - 1);
-    lat.mul = 1u << (d.lb - 1);
-    const int nrows = lane > last ? 0 : min(RPL, g.L - RPL * lane);
+    constexpr int C = W == 1 ? 1 : RPL;          // 16-byte mask chunks of a lane per half-sweep; also of a state
+    static_assert(RPL * W == 2 * C, "a chunk holds the masks of two words");
+    __shared__ uint4 ring[STAGES][2 * K * C][32];
+    __shared__ uint4 state[2][K][C][32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, last = (g.L + RPL - 1) / RPL - 1;
+    const int prev = lane == 0 ? last : lane - 1, next = lane == last ? 0 : lane + 1;
+    const int stages = (n + K - 1) / K;
     uint32_t live[W];
 #pragma unroll
     for (int w = 0; w < W; ++w) live[w] = dense_live(d, w);
-    // masks: the lane's rows (row 0's for rows it does not have, never used)
-    const uint64_t plane = (uint64_t)g.L * d.P, mask_words = (2 * (uint64_t)n + kClMaskPad) * plane;
-    const uint32_t ring_sh = (uint32_t)__cvta_generic_to_shared(&ring[0][0][lane]);
-    constexpr uint32_t kRow = 32 * sizeof(uint4), kSlab = RPL * kRow;
-    const uint64_t* src[RPL];
-#pragma unroll
-    for (int r = 0; r < RPL; ++r) src[r] = masks + (r < nrows ? (uint64_t)(RPL * lane + r) * d.P : 0);
-    auto copy = [&](int slab) {
-#pragma unroll
-        for (int r = 0; r < RPL; ++r) {
+    WarpLattice<W, RPL, TWO> lat;
+    lat.prev = prev;
+    lat.next = next;
+    lat.tail = TWO && lane == last;
+    lat.lsh = (uint32_t)(d.lb - 1);
+    lat.mul = 1u << (d.lb - 1);
+    if (warp != 0) {
+        const long long N = (long long)g.L * g.L;
+        auto copy = [&](int stage) {
+            if (stage < stages && lane <= last) {
+                const int slot = stage % STAGES, rows = 2 * C * min(K, n - stage * K);
+                const uint64_t nl = last + 1u, base = (uint64_t)stage * (2 * K * C) * nl + lane;
+                for (int r = 0; r < rows; ++r) {
 #ifdef ISING_CHECKED
-            if (check_index((uint64_t)(src[r] - masks) + 1, mask_words, __LINE__))
+                    if (!check_index(base + r * nl, (uint64_t)n * (2 * C) * nl, __LINE__)) continue;
 #endif
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(ring_sh + (uint32_t)slab * kSlab + r * kRow),
-                         "l"(src[r]) : "memory");
-            src[r] += plane;
-        }
-        asm volatile("cp.async.commit_group;" ::: "memory");
-    };
-    auto take = [&](int slab, uint32_t (&m)[RPL][2 * W]) {
-        asm volatile("cp.async.wait_group %0;" ::"n"(kWarpDepth - 1) : "memory");
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;"
+                                 ::"r"((uint32_t)__cvta_generic_to_shared(&ring[slot][r][lane])),
+                                   "l"(masks + base + r * nl) : "memory");
+                }
+            }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        };
+        // counter h takes every kCounters-th record of the run: the next one is
+        // after sweep `due` of this launch
+        const int h = warp < kIdle ? warp - 1 : warp - 3;
+        const long long r0 = s_base / every + h;
+        long long due = (r0 + 1) * every - s_base;
+        long long* rec = records + 2 * r0;
+        auto count = [&](int stage) {
+            for (; due <= min((stage + 1) * K, n); due += (long long)kCounters * every, rec += 2 * kCounters) {
+                const int q = (int)due - 1 - stage * K;
 #pragma unroll
-        for (int r = 0; r < RPL; ++r) {
-            const uint32_t at = ring_sh + (uint32_t)slab * kSlab + r * kRow;
-            if constexpr (W == 1)
-                asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(m[r][0]), "=r"(m[r][1]) : "r"(at));
-            else
-                asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
-                             : "=r"(m[r][0]), "=r"(m[r][1]), "=r"(m[r][2]), "=r"(m[r][3]) : "r"(at));
+                for (int c = 0; c < C; ++c) {
+                    const uint4 v = state[stage & 1][q][c][lane];
+                    if constexpr (W == 1) {
+                        lat.x[0][0][0] = v.x; lat.x[0][1][0] = v.y; lat.x[1][0][0] = v.z; lat.x[1][1][0] = v.w;
+                    } else {
+                        lat.x[0][c][0] = v.x; lat.x[0][c][W - 1] = v.y; lat.x[1][c][0] = v.z; lat.x[1][c][W - 1] = v.w;
+                    }
+                }
+                uint32_t anti, up;
+                lat.count(live, anti, up);
+                // both sums in one reduction: anti <= 2 L^2 <= 2^15 and up <= 2^14
+                const uint32_t sum = __reduce_add_sync(0xffffffffu, lane <= last ? anti | up << 16 : 0u);
+                if (lane == 0) {
+                    rec[0] = 2 * (long long)(sum & 0xffffu) - 2 * N;
+                    rec[1] = 2 * (long long)(sum >> 16) - N;
+                }
+            }
+        };
+        pdl_wait();                                 // the masks are drawn
+        if (warp == kCopier) {
+            for (int k = 0; k < STAGES - 1; ++k) copy(k);
+            asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 2) : "memory");
         }
-    };
-    (void)mask_words;
+        __syncthreads();
+        for (int k = 0; k < stages; ++k) {
+            if (warp == kCopier) {
+                copy(k + STAGES - 1);
+                asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 2) : "memory");
+            } else if (warp != kIdle && k > 0) {
+                count(k - 1);
+            }
+            __syncthreads();
+        }
+        if (warp != kCopier && warp != kIdle) count(stages - 1);
+        return;
+    }
+
+    const int nrows = lane > last ? 0 : min(RPL, g.L - RPL * lane);
 #pragma unroll
     for (int c = 0; c < 2; ++c)
 #pragma unroll
@@ -143,39 +235,44 @@ warp_sweeps_kernel(uint64_t* __restrict__ w0, uint64_t* __restrict__ w1, Geom g,
             for (int w = 0; w < W; ++w)
                 lat.x[c][r][w] =
                     r < nrows ? dense_from_packed(c ? w1 : w0, (uint64_t)(RPL * lane + r) * g.P, g, w) : 0u;
-    pdl_wait();                                     // the masks are drawn
+    pdl_wait();
+    __syncthreads();
+    int slot = 0;
+    for (int k = 0; k < stages; ++k) {
+        const int cnt = min(K, n - k * K);
+        uint32_t m[2][RPL][2 * W];
+        auto take = [&](int h) {
 #pragma unroll
-    for (int h = 0; h < kWarpDepth; ++h) copy(h);
-    const long long N = (long long)g.L * g.L;
-    int next_rec = every - s_base % every;          // the next recorded sweep of this launch
-    long long* rec = records + 2 * (s_base / every);
-    for (int s0 = 0; s0 < n; s0 += kWarpDepth / 2) {
-#pragma unroll
-        for (int q = 0; q < kWarpDepth / 2; ++q) {
-            const int s = s0 + q + 1;
-            if (s > n) break;
-            uint32_t m[RPL][2 * W], anti = 0, up = 0;
-            take(2 * q, m);
-            lat.template half_sweep<0, false>(m, nrows, live, anti, up);
-            copy(2 * q);
-            take(2 * q + 1, m);
-            if (s == next_rec) {
-                lat.template half_sweep<1, true>(m, nrows, live, anti, up);
-                // both sums in one reduction: anti <= 2 L^2 <= 2^15 and up <= 2^14
-                const uint32_t sum = __reduce_add_sync(0xffffffffu, anti | up << 16);
-                if (lane == 0) {
-                    rec[0] = 2 * (long long)(sum & 0xffffu) - 2 * N;
-                    rec[1] = 2 * (long long)(sum >> 16) - N;
+            for (int c = 0; c < C; ++c) {
+                const uint4 v = ring[slot][h * C + c][lane];
+                uint32_t(&to)[RPL][2 * W] = m[h & 1];
+                if constexpr (W == 1) {
+                    to[0][0] = v.x; to[0][1] = v.y; to[1][0] = v.z; to[1][1] = v.w;
+                } else {
+                    to[c][0] = v.x; to[c][1] = v.y; to[c][2 * W - 2] = v.z; to[c][2 * W - 1] = v.w;
                 }
-                rec += 2;
-                next_rec = every <= n - s ? s + every : n + 1;
-            } else {
-                lat.template half_sweep<1, false>(m, nrows, live, anti, up);
             }
-            copy(2 * q + 1);
+        };
+        take(0);
+#pragma unroll
+        for (int q = 0; q < K; ++q) {
+            if (q >= cnt) break;
+            take(2 * q + 1);
+            lat.template half_sweep<0>(m[0]);
+            if (q + 1 < K) take(2 * q + 2);
+            lat.template half_sweep<1>(m[1]);
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                if constexpr (W == 1)
+                    state[k & 1][q][c][lane] = make_uint4(lat.x[0][0][0], lat.x[0][1][0], lat.x[1][0][0], lat.x[1][1][0]);
+                else
+                    state[k & 1][q][c][lane] =
+                        make_uint4(lat.x[0][c][0], lat.x[0][c][W - 1], lat.x[1][c][0], lat.x[1][c][W - 1]);
+            }
         }
+        slot = slot + 1 == STAGES ? 0 : slot + 1;
+        __syncthreads();
     }
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
 #pragma unroll
     for (int c = 0; c < 2; ++c)
 #pragma unroll
@@ -196,19 +293,42 @@ warp_sweeps_kernel(uint64_t* __restrict__ w0, uint64_t* __restrict__ w1, Geom g,
 
 }  // namespace
 
+size_t warp_mask_bytes_per_sweep(int L)
+{
+    const DenseGeom d = warp_geom(L);
+    return 2 * (size_t)((L + 3) / 4 * 4) * d.P * sizeof(uint64_t);
+}
+
+cudaError_t launch_warp_mask_draw(int L, const SweepArgs& a, uint64_t t0, int nsweeps, uint64_t* masks,
+                                  cudaStream_t s)
+{
+    const DenseGeom d = warp_geom(L);
+    const Strips st = make_strips(d.P, kDenseStripWords);
+    const uint32_t G = (uint32_t)(L + 3) / 4, threads = 4 * G * d.P;
+    const uint32_t block = std::min((threads + 31) / 32 * 32, 128u);
+    const DenseOut out = d.W == 1 ? DenseOut{4, 1, (uint32_t)L} : DenseOut{2, 2 * G, 8 * G};
+    const dim3 grid((threads + block - 1) / block, 1, 2 * nsweeps);
+    if (a.rounds == 7)
+        dense_mask_draw_kernel<7, 4><<<grid, block, 0, s>>>(d, st, a, t0, out, masks);
+    else
+        dense_mask_draw_kernel<10, 4><<<grid, block, 0, s>>>(d, st, a, t0, out, masks);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_warp_sweeps(uint64_t* w0, uint64_t* w1, const Geom& g, const uint64_t* masks, int s_base, int n,
                                int every, long long* rec, uint64_t* t_dev, uint64_t t_end, cudaStream_t s)
 {
-    const DenseGeom d = dense_geom(g.L);
-    const dim3 one(1), block(32);
+    const DenseGeom d = warp_geom(g.L);
+    const dim3 one(1), block(kWarpThreads);
+    const uint4* m = reinterpret_cast<const uint4*>(masks);
     if (d.W == 1)
-        launch_pdl(warp_sweeps_kernel<1, 2, false>, one, block, s, w0, w1, g, d, masks, s_base, n, every, rec, t_dev,
+        launch_pdl(warp_sweeps_kernel<1, 2, false, 8, 3>, one, block, s, w0, w1, g, d, m, s_base, n, every, rec, t_dev,
                    t_end);
     else if (g.L % 4 == 0)
-        launch_pdl(warp_sweeps_kernel<2, 4, false>, one, block, s, w0, w1, g, d, masks, s_base, n, every, rec, t_dev,
-                   t_end);
+        launch_pdl(warp_sweeps_kernel<2, 4, false, 2, 5>, one, block, s, w0, w1, g, d, m, s_base, n, every, rec,
+                   t_dev, t_end);
     else
-        launch_pdl(warp_sweeps_kernel<2, 4, true>, one, block, s, w0, w1, g, d, masks, s_base, n, every, rec, t_dev,
+        launch_pdl(warp_sweeps_kernel<2, 4, true, 2, 5>, one, block, s, w0, w1, g, d, m, s_base, n, every, rec, t_dev,
                    t_end);
     return cudaGetLastError();
 }
