@@ -58,7 +58,6 @@ namespace ising {
 namespace {
 
 constexpr int kClThreads = 1024;           // most threads of a block
-constexpr size_t kClSmemMax = 220 * 1024;   // dynamic shared memory of a block
 // Most half-sweeps per phase.  A phase's exchange costs about 0.85 us, its halo
 // rows are extra work: measured on GB300 (us of 1000 sweeps, record every 10, k
 // = 8 / 12 / 18 / 24) L = 296: 610 / 565 / 544 / 543; L = 512: 713 / 688 / 652 /
@@ -493,6 +492,10 @@ int g_max_active = 0;
 
 int probe_max_cluster()
 {
+    if (!band_setup()) {
+        cudaGetLastError();
+        return 0;
+    }
     for (ClusterKernel kern : kClusterKernels) {
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
             cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClSmemMax) !=
@@ -564,6 +567,7 @@ bool cluster_plan(int L, bool interleaved, int clusters, ClusterPlan* plan)
     if (c == 0 || clusters < 1 || clusters > g_max_active) return false;
     const int nb = clusters * c, fewest = L / nb;         // blocks of the launch
     if (!cluster_side(L, nb, interleaved)) return false;
+    if (clusters == 1 && band_plan(L, c, plan)) return true;
     const DenseGeom d = dense_geom(L);
     for (int kk = std::min(d.W > kClWideWords ? kClHaloWide : kClHalo, fewest) & ~1; kk >= 2; kk -= 2) {
         const long long rows = (L + nb - 1) / nb + 2 * kk - 2;

@@ -81,6 +81,27 @@ __device__ __forceinline__ uint64_t packed_from_dense(uint32_t d0, uint32_t d1, 
     return spread_fields(__funnelshift_r(d0, d1, (kFields * w) & 31));
 }
 
+// Anti-aligned bonds (four per updated word) and up spins (the word's and its
+// same-column neighbour's) of dense words.  Bits are added by three-input adders
+// (sum, carry) and counted as ones, twos and fours: a population count takes
+// four times the issue slots of a logic operation.
+struct DenseCount {
+    uint32_t ones = 0, twos = 0, fours = 0, up1 = 0, up2 = 0;
+    __device__ __forceinline__ void add(uint32_t s, uint32_t u, uint32_t d, uint32_t h0, uint32_t h1, uint32_t live)
+    {
+        constexpr int kSum = kLutA ^ kLutB ^ kLutC, kCarry = (kLutA & kLutB) | (kLutA & kLutC) | (kLutB & kLutC);
+        const uint32_t a = s ^ u, b = s ^ d, c = s ^ h0, e = (s ^ h1) & live;
+        const uint32_t t1 = lop3<kCarry>(ones, a, b), o = lop3<kSum>(ones, a, b), t2 = lop3<kCarry>(o, c, e);
+        ones = lop3<kSum>(o, c, e);
+        fours += __popc(lop3<kCarry>(twos, t1, t2));
+        twos = lop3<kSum>(twos, t1, t2);
+        up2 += __popc(lop3<kCarry>(up1, s, h0));
+        up1 = lop3<kSum>(up1, s, h0);
+    }
+    __device__ __forceinline__ uint32_t anti() const { return __popc(ones) + 2 * __popc(twos) + 4 * fours; }
+    __device__ __forceinline__ uint32_t up() const { return __popc(up1) + 2 * up2; }
+};
+
 // Draws of fields k .. N - 1 of the FirstTable column for the four rows of a
 // row group, into bits k .. N - 1.
 template <int k, int N, int ROUNDS, typename Calls>

@@ -83,7 +83,7 @@ cudaError_t launch_resident_premasked(uint64_t* w0, uint64_t* w1, const Geom& g,
 struct ClusterPlan {
     int blocks;     // cluster size
     int k;          // half-sweeps per phase = halo rows
-    int v;          // dense words per unit: 1 or 2
+    int v;          // dense words per unit: 1 or 2; 0: band_sweeps_kernel
     int ns;         // units per thread: 1 or 2
     int threads;    // threads per block
     int clusters;   // clusters of a launch (1: the halos never leave the cluster)
@@ -116,6 +116,15 @@ cudaError_t launch_cl_mask_draw(int L, const SweepArgs& a, uint64_t t0, int nswe
 cudaError_t launch_cluster_sweeps(uint64_t* w0, uint64_t* w1, uint32_t* dense, const Geom& g, const SweepArgs& a,
                                   const ClusterPlan& plan, int nsweeps, const uint64_t* masks, int64_t s0,
                                   int64_t every, const ClusterExchange& x, cudaStream_t s);
+
+// The form of the path for one cluster and short rows (ising_band.cu).
+constexpr size_t kClSmemMax = 220 * 1024;   // most dynamic shared memory of a block of the path
+bool band_setup();
+bool band_plan(int L, int blocks, ClusterPlan* plan);
+cudaError_t launch_band_sweeps(uint64_t* w0, uint64_t* w1, uint32_t* dense, const Geom& g,
+                               unsigned long long* counts, const ClusterPlan& plan, int nsweeps,
+                               const uint64_t* masks, int64_t s0, int64_t every, uint64_t* t_dev, uint64_t t_end,
+                               unsigned int* err, cudaStream_t s);
 
 // The on-chip path up to side kWarpMaxL (ising_warp.cu): sweeps s_base + 1 ..
 // s_base + n of a run in one warp's registers, with the masks that

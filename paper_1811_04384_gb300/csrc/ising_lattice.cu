@@ -22,6 +22,7 @@ using namespace ising;
 namespace {
 
 constexpr int kRecordsPerChunk = 1024;           // count slots resident on the device
+constexpr size_t kHostWords = 64;                // words the kernels report to, past the pinned count buffer
 constexpr size_t kCountBytes = (size_t)kRecordsPerChunk * kCountSlots * 2 * sizeof(unsigned long long);
 constexpr size_t kAlign = 256;
 constexpr size_t kResidentMaxBytes = 220 * 1024;   // shared memory for the on-chip path
@@ -59,7 +60,7 @@ struct ising_lattice {
     int8_t* staging2 = nullptr;  // second input buffer of ising_run_states
     cudaStream_t copy_stream = nullptr;          // ising_run_states: host -> device copies
     cudaEvent_t ev_copied[2] = {nullptr, nullptr}, ev_packed[2] = {nullptr, nullptr};
-    unsigned long long* host_counts = nullptr;   // pinned, kCountBytes
+    unsigned long long* host_counts = nullptr;   // pinned, kCountBytes, then the word of gave_up_word
     int bw = 0, bg = 128;                        // half-sweep shape: linear items, 128 threads a block
     int path = ISING_PATH_AUTO;                  // multi-block launches or on-chip resident sweeps
     int rounds = 10;                             // Philox rounds of the sweep draws
@@ -114,6 +115,25 @@ extern "C" size_t ising_bytes_required(int32_t L)
     return 2 * align_up(words_bytes(g), kAlign) + align_up(kCountBytes, kAlign) + kAlign;
 }
 
+// The word a launch sets when one of its waits inside a cluster gave up
+// (band_sweeps_kernel): its sweeps are void, and the next call that waits for
+// results reports it.
+static unsigned int* gave_up_word(ising_lattice* h)
+{
+    return reinterpret_cast<unsigned int*>(reinterpret_cast<char*>(h->host_counts) + kCountBytes);
+}
+
+// Waits for the lattice's stream before results are read.
+static int sync_results(ising_lattice* h)
+{
+    cudaError_t e = cudaStreamSynchronize(h->stream);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize");
+    volatile unsigned int* word = gave_up_word(h);
+    if (*word == 0) return ISING_OK;
+    *word = 0;
+    return ISING_ETIMEOUT;
+}
+
 static int setup_handle(ising_lattice* h, int32_t L, uint64_t seed, char* base)
 {
     h->g = make_geom(L);
@@ -124,8 +144,9 @@ static int setup_handle(ising_lattice* h, int32_t L, uint64_t seed, char* base)
     h->words[1] = reinterpret_cast<uint64_t*>(base + wb);
     h->counts = reinterpret_cast<unsigned long long*>(base + 2 * wb);
     h->t_dev = reinterpret_cast<uint64_t*>(base + 2 * wb + align_up(kCountBytes, kAlign));
-    cudaError_t e = cudaMallocHost(&h->host_counts, kCountBytes);
+    cudaError_t e = cudaMallocHost(&h->host_counts, kCountBytes + kHostWords);
     if (e != cudaSuccess) { h->host_counts = nullptr; return ISING_ENOMEM; }
+    *gave_up_word(h) = 0;
     thresholds_for_beta(0.0, h->thr);
     return ISING_OK;
 }
@@ -194,8 +215,9 @@ extern "C" int ising_create_layout(int32_t L, uint64_t seed, int32_t layout, isi
     h->words[1] = nullptr;
     h->counts = reinterpret_cast<unsigned long long*>(base + sb);
     h->t_dev = reinterpret_cast<uint64_t*>(base + sb + align_up(kCountBytes, kAlign));
-    e = cudaMallocHost(&h->host_counts, kCountBytes);
+    e = cudaMallocHost(&h->host_counts, kCountBytes + kHostWords);
     if (e != cudaSuccess) { h->host_counts = nullptr; free_handle(h); return ISING_ENOMEM; }
+    *gave_up_word(h) = 0;
     thresholds_for_beta(0.0, h->thr);
     int rc = ising_init_cold(h, 1);
     if (rc != ISING_OK) { free_handle(h); return rc; }
@@ -718,8 +740,12 @@ static int run_cluster(ising_lattice* h, int64_t n, int64_t every, unsigned long
         }
         if (plan.clusters > 1 && h->absent_after >= 0 && h->absent_after-- == 0)
             x.absent = 1;                            // one block more than the launch has: it gives up
-        cudaError_t e = launch_cluster_sweeps(h->words[0], h->words[1], ci ? h->dense : nullptr, g, a, plan,
-                                              part_of(j), masks[j & 1], done, every, x, h->stream);
+        cudaError_t e =
+            plan.v == 0 ? launch_band_sweeps(h->words[0], h->words[1], ci ? h->dense : nullptr, g, counts, plan,
+                                             part_of(j), masks[j & 1], done, every, h->t_dev,
+                                             h->t + (uint64_t)(done + part_of(j)), gave_up_word(h), h->stream)
+                        : launch_cluster_sweeps(h->words[0], h->words[1], ci ? h->dense : nullptr, g, a, plan,
+                                                part_of(j), masks[j & 1], done, every, x, h->stream);
         if (e != cudaSuccess) return cuda_fail(e, "cluster sweeps kernel");
         if (plan.clusters > 1) {
             x.seq += cl_exchange_seqs(plan, part_of(j));
@@ -735,7 +761,8 @@ static int run_cluster(ising_lattice* h, int64_t n, int64_t every, unsigned long
         if (e != cudaSuccess) return cuda_fail(e, "ci_from_dense");
     }
     if (n > 0) {
-        cudaError_t e = launch_advance_sweep(h->t_dev, (uint64_t)n, h->stream);
+        // the band kernel sets the counter itself
+        cudaError_t e = plan.v == 0 ? cudaSuccess : launch_advance_sweep(h->t_dev, (uint64_t)n, h->stream);
         if (e != cudaSuccess) return cuda_fail(e, "advance_sweep_kernel");
         h->t += (uint64_t)n;
     }
@@ -1002,8 +1029,8 @@ extern "C" int ising_sweep_record(ising_lattice* h, int64_t n, int64_t every, in
         if (rc != ISING_OK) return rc;
         e = cudaMemcpyAsync(h->host_counts, h->counts, bytes, cudaMemcpyDeviceToHost, h->stream);
         if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpyAsync counts");
-        e = cudaStreamSynchronize(h->stream);
-        if (e != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize");
+        rc = sync_results(h);
+        if (rc != ISING_OK) return rc;
         for (int64_t r = 0; r < chunk; ++r)
             counts_to_EM(h, h->host_counts + (size_t)r * kCountSlots * 2, E ? E + done_rec + r : nullptr,
                          M ? M + done_rec + r : nullptr);
@@ -1025,8 +1052,8 @@ static int measure(ising_lattice* h, int64_t* E, int64_t* M)
     if (e != cudaSuccess) return cuda_fail(e, "measure");
     e = cudaMemcpyAsync(h->host_counts, h->counts, bytes, cudaMemcpyDeviceToHost, h->stream);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpyAsync counts");
-    e = cudaStreamSynchronize(h->stream);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize");
+    const int rc = sync_results(h);
+    if (rc != ISING_OK) return rc;
     counts_to_EM(h, h->host_counts, E, M);
     return ISING_OK;
 }
@@ -1088,9 +1115,7 @@ extern "C" int ising_get_spins(ising_lattice* h, int8_t* out, size_t n)
     if (e != cudaSuccess) return cuda_fail(e, "unpack_kernel");
     e = cudaMemcpyAsync(out, h->staging, n, cudaMemcpyDeviceToHost, h->stream);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpyAsync spins");
-    e = cudaStreamSynchronize(h->stream);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize");
-    return ISING_OK;
+    return sync_results(h);
 }
 
 extern "C" int ising_set_spins(ising_lattice* h, const int8_t* in, size_t n)
@@ -1205,8 +1230,8 @@ extern "C" int ising_run_states(ising_lattice* h, const int8_t* const* states, i
                                 cudaMemcpyDeviceToHost, h->stream);
             if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpyAsync counts");
         }
-        e = cudaStreamSynchronize(h->stream);
-        if (e != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize");
+        rc = sync_results(h);
+        if (rc != ISING_OK) return rc;
         for (int64_t r = 0; r < (k1 - k0) * R; ++r)
             counts_to_EM(h, h->host_counts + (size_t)r * rec_words, E ? E + k0 * R + r : nullptr,
                          M ? M + k0 * R + r : nullptr);
@@ -1225,8 +1250,7 @@ extern "C" int ising_get_words(ising_lattice* h, uint64_t* out, size_t n64)
                                         cudaMemcpyDeviceToHost, h->stream);
         if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpyAsync words");
     }
-    cudaError_t e = cudaStreamSynchronize(h->stream);
-    return e == cudaSuccess ? ISING_OK : cuda_fail(e, "cudaStreamSynchronize");
+    return sync_results(h);
 }
 
 extern "C" int ising_set_words(ising_lattice* h, const uint64_t* in, size_t n64)

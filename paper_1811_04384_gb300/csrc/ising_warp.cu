@@ -98,13 +98,11 @@ struct WarpLattice {
     }
 
     // The anti-aligned bonds of colour 1's rows and the up spins of both
-    // colours (live bits only) of a lane with rows.  Bits are added by
-    // three-input adders (sum, carry) and counted as ones, twos and fours: a
-    // population count takes four times the issue slots of a logic operation.
-    __device__ __forceinline__ void count(const uint32_t (&live)[W], uint32_t& anti, uint32_t& up) const
+    // colours (live bits only) of a lane with rows.
+    __device__ __forceinline__ DenseCount count(const uint32_t (&live)[W]) const
     {
-        constexpr int kSum = kLutA ^ kLutB ^ kLutC, kCarry = (kLutA & kLutB) | (kLutA & kLutC) | (kLutB & kLutC);
-        uint32_t above[W], below[W], ones = 0, twos = 0, fours = 0, up1 = 0, up2 = 0;
+        uint32_t above[W], below[W];
+        DenseCount cnt;
         edges<1>(above, below);
 #pragma unroll
         for (int r = 0; r < RPL; ++r) {
@@ -116,18 +114,10 @@ struct WarpLattice {
             for (int w = 0; w < W; ++w) {
                 uint32_t u, d;
                 vertical<1>(r, w, above, below, u, d);
-                const uint32_t s = x[1][r][w], h0 = x[0][r][w];
-                const uint32_t a = s ^ u, b = s ^ d, c = s ^ h0, e = (s ^ h1[w]) & live[w];
-                const uint32_t t1 = lop3<kCarry>(ones, a, b), o = lop3<kSum>(ones, a, b), t2 = lop3<kCarry>(o, c, e);
-                ones = lop3<kSum>(o, c, e);
-                fours += __popc(lop3<kCarry>(twos, t1, t2));
-                twos = lop3<kSum>(twos, t1, t2);
-                up2 += __popc(lop3<kCarry>(up1, s, h0));
-                up1 = lop3<kSum>(up1, s, h0);
+                cnt.add(x[1][r][w], u, d, x[0][r][w], h1[w], live[w]);
             }
         }
-        anti = __popc(ones) + 2 * __popc(twos) + 4 * fours;
-        up = __popc(up1) + 2 * up2;
+        return cnt;
     }
 };
 
@@ -197,10 +187,9 @@ warp_sweeps_kernel(uint64_t* __restrict__ w0, uint64_t* __restrict__ w1, Geom g,
                         lat.x[0][c][0] = v.x; lat.x[0][c][W - 1] = v.y; lat.x[1][c][0] = v.z; lat.x[1][c][W - 1] = v.w;
                     }
                 }
-                uint32_t anti, up;
-                lat.count(live, anti, up);
-                // both sums in one reduction: anti <= 2 L^2 <= 2^15 and up <= 2^14
-                const uint32_t sum = __reduce_add_sync(0xffffffffu, lane <= last ? anti | up << 16 : 0u);
+                const DenseCount cnt = lat.count(live);
+                // both sums in one reduction: at most 2 L^2 <= 2^15 bonds and 2^14 spins
+                const uint32_t sum = __reduce_add_sync(0xffffffffu, lane <= last ? cnt.anti() | cnt.up() << 16 : 0u);
                 if (lane == 0) {
                     rec[0] = 2 * (long long)(sum & 0xffffu) - 2 * N;
                     rec[1] = 2 * (long long)(sum >> 16) - N;
