@@ -30,7 +30,14 @@ using namespace ising;
 namespace {
 
 constexpr size_t kAlign = 256;
-constexpr int kLanes = 4;   // independent streams an epoch's jobs are split over
+constexpr int kLanes = 4;   // most independent streams an epoch's jobs are split over
+// Sites of all running jobs for each lane of an epoch.  A lane fills the SMs
+// that another's last wave leaves idle, but costs two more launches (4 us of
+// the worker thread) in every sweep, and a lane's half-sweep already starts under
+// the one before it.  Measured on GB300, us of a whole pass with 4 lanes / this
+// rule / 1 lane: 48 jobs of 22e6 sites 7,617 / 5,831 / 6,004; 16 jobs of 8.4e6
+// 6,118 / 2,973 / 2,978; 40 jobs of 1.6e6 6,671 / 2,804 / 2,832.
+constexpr double kLaneSites = 8e6;
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 enum JobState { kQueued = 0, kRunning = 1, kDone = 2, kFailed = 3, kCancelled = 4 };
@@ -225,6 +232,7 @@ int run_epoch(ising_server* s, const std::vector<uint64_t>& run, std::vector<Job
     uint32_t max_n = 0;
     int rounds = 10;                               // 10 if every job uses Philox4x32-10, else per job
     std::vector<double> work(run.size());
+    double sites = 0.0;
     for (size_t a = 0; a < run.size(); ++a) {
         Job& j = *jp[a];
         BatchReplica& R = j.rep;
@@ -238,9 +246,11 @@ int run_epoch(ising_server* s, const std::vector<uint64_t>& run, std::vector<Job
         max_n = std::max(max_n, R.nsweeps);
         if (R.rounds != 10) rounds = 0;
         work[a] = (double)j.g.L * j.g.L * R.nsweeps;
+        sites += (double)j.g.L * j.g.L;
     }
     // lanes: jobs, most work first, to the lane with the least work so far;
     // each lane's tiles are contiguous and it runs on its own stream
+    const int lanes = std::max(1, std::min(kLanes, (int)(sites / kLaneSites)));
     std::vector<size_t> order(run.size());
     for (size_t a = 0; a < order.size(); ++a) order[a] = a;
     std::stable_sort(order.begin(), order.end(), [&](size_t x, size_t y) { return work[x] > work[y]; });
@@ -248,7 +258,7 @@ int run_epoch(ising_server* s, const std::vector<uint64_t>& run, std::vector<Job
     double lane_work[kLanes] = {};
     for (size_t a : order) {
         int best = 0;
-        for (int k = 1; k < kLanes; ++k)
+        for (int k = 1; k < lanes; ++k)
             if (lane_work[k] < lane_work[best]) best = k;
         lane_of[a] = best;
         lane_work[best] += work[a];
