@@ -31,5 +31,16 @@ cudaError_t ci_from_dense(uint64_t* S, int L, const uint32_t* dense, cudaStream_
 bool ci_rw_predraw(int L, int nstrips);
 cudaError_t ci_random_words_iteration(uint64_t* S, int L, int nstrips, const SweepArgs& a, ulonglong2* draws,
                                       cudaStream_t s);
+// The same with the updates planned ahead (ising_words.cu), where a half strip
+// fits (words_planned): words_plan makes the plans of iterations
+// sweep_number(a) .. + iterations - 1 (words_plan_bytes each; at most
+// words_plan_iterations of the n that a call runs), words_run both phases of
+// the plan's iteration `iteration`; *err = 1 when a wait gave up.
+bool words_planned(int L, int nstrips);
+size_t words_plan_bytes(int L, int nstrips);
+int words_plan_iterations(int L, int nstrips, int64_t n);
+cudaError_t words_plan(int L, int nstrips, const SweepArgs& a, int iterations, void* plan, cudaStream_t s);
+cudaError_t words_run(uint64_t* S, int L, int nstrips, const void* plan, int iteration, unsigned int* err,
+                      cudaStream_t s);
 
 }  // namespace ising

@@ -68,7 +68,8 @@ struct ising_lattice {
     int item_lanes = 0;                          // lanes per thread item on the launch path (0: auto)
     int chain = ISING_CHAIN_CHECKERBOARD;        // or the paper's random-word chain (interleaved layout)
     int nstrips = 1;                             // strips of the random-word chain
-    ulonglong2* rw_draws = nullptr;              // random-word chain: the draws of one iteration (lazily)
+    ulonglong2* rw_draws = nullptr;              // random-word chain: the draws of one iteration, or plans (lazily)
+    size_t rw_draws_bytes = 0;
     cudaStream_t capture_stream = nullptr;       // graphs of sweep chunks are captured here
     cudaGraphExec_t graph_plain = nullptr;       // kGraphSweeps sweeps, no record
     cudaGraphExec_t graph_rec = nullptr;         // record intervals of graph_rec_every sweeps, each recorded
@@ -877,16 +878,31 @@ static int run_random_words(ising_lattice* h, int64_t n, RecOf rec_of)
     // the updates' draws are made first on all SMs unless the launch path was
     // chosen or the buffer would be too large; then each block draws its own
     const bool pre = h->path != ISING_PATH_LAUNCHES && ci_rw_predraw(h->g.L, h->nstrips);
-    if (pre && !h->rw_draws) {
-        cudaError_t e = cudaMalloc(&h->rw_draws, ci_rw_draw_bytes(h->g.L, h->nstrips));
+    const bool planned = pre && words_planned(h->g.L, h->nstrips);
+    const int chunk = planned ? words_plan_iterations(h->g.L, h->nstrips, std::max<int64_t>(n, 1)) : 0;
+    const size_t need = planned ? (size_t)chunk * words_plan_bytes(h->g.L, h->nstrips)
+                                : (pre ? ci_rw_draw_bytes(h->g.L, h->nstrips) : 0);
+    if (h->rw_draws_bytes < need) {
+        if (h->rw_draws) cudaFree(h->rw_draws);
+        h->rw_draws_bytes = 0;
+        cudaError_t e = cudaMalloc(&h->rw_draws, need);
         if (e != cudaSuccess) { h->rw_draws = nullptr; cuda_fail(e, "cudaMalloc random-word draws"); return ISING_ENOMEM; }
+        h->rw_draws_bytes = need;
     }
     for (int64_t it = 1; it <= n; ++it) {
         a.t_off = (uint32_t)it;
         a.counts = nullptr;
-        cudaError_t e = ci_random_words_iteration(h->words[0], h->g.L, h->nstrips, a, pre ? h->rw_draws : nullptr,
-                                                  h->stream);
-        if (e != cudaSuccess) return cuda_fail(e, "ci_rw_phase_kernel");
+        cudaError_t e = cudaSuccess;
+        if (planned) {
+            const int k = (int)((it - 1) % chunk);
+            if (k == 0)
+                e = words_plan(h->g.L, h->nstrips, a, (int)std::min<int64_t>(chunk, n - it + 1), h->rw_draws, h->stream);
+            if (e == cudaSuccess)
+                e = words_run(h->words[0], h->g.L, h->nstrips, h->rw_draws, k, gave_up_word(h), h->stream);
+        } else {
+            e = ci_random_words_iteration(h->words[0], h->g.L, h->nstrips, a, pre ? h->rw_draws : nullptr, h->stream);
+        }
+        if (e != cudaSuccess) return cuda_fail(e, "random words");
         const int rec = rec_of(it);
         if (rec >= 0) {
             a.counts = h->counts + (size_t)rec * kCountSlots * 2;

@@ -1,0 +1,356 @@
+// The paper's random-word chain (Sec. 4-5, Appendix A) with its updates planned
+// ahead.  A phase is one sequence of 10 N h word updates per strip, each on the
+// word that its draws choose, and the result must be the sequential chain's,
+// word for word.
+//
+// What bounds it: the longest chain of updates that touch one another (about
+// 120 of the 3,360 of a half strip of 48 x 7 words).  ci_rw_phase_kernel finds
+// the updates that may run in rounds of a window, six block barriers and a
+// table of claims each: 82 us a phase at L = 1008 and 72 strips.  But which
+// updates wait for which depends on the draws alone, not on the spins, so
+// words_plan_kernel works it out beforehand on all SMs, for every phase and
+// iteration of a call at once: each word's updates in sequence order, and with
+// each the number of updates of its four neighbours that come before it.  In
+// words_run_kernel a thread owns a word: it runs its next update as soon as the
+// four neighbours have had exactly that many.  A word's spins (21 bits) and its
+// count of updates share 64 bits of shared memory, so one load gives both and
+// no barrier or fence is needed.  An update that is the oldest of all pending
+// ones never waits, so the phase always ends.  Measured on GB300, 5 iterations
+// of L = 1008 with 72 strips, a record after each: 819 -> @@ us.
+#include <cuda_runtime.h>
+
+#include <algorithm>
+
+#include "ising_device.cuh"
+#include "ising_dense.cuh"
+#include "ising_interleaved.cuh"
+#include "ising_interleaved.h"
+#include "ising_internal.h"
+
+namespace ising {
+namespace {
+
+constexpr int kPlanWarps = 8;
+constexpr size_t kWordsSmemMax = 220 * 1024;
+constexpr int kWordsThreads = 1024;             // most threads of a strip, one or two words each
+constexpr uint32_t kWordsTries = 1u << 24;      // a thread's looks at its neighbours before it gives up
+constexpr size_t kWordsPlanBytes = (size_t)64 << 20;
+constexpr int kWordsPlanIterations = 16;
+constexpr uint32_t kWordBits = (1u << 21) - 1;
+
+// The strips' half strips in a phase.
+struct WordsGeom {
+    int L, N, NC, nstrips;
+    __host__ __device__ int h(int phase) const { return phase == 0 ? NC / 2 : NC - NC / 2; }
+    __host__ __device__ int words(int phase) const { return N * h(phase); }
+    __host__ __device__ uint32_t updates(int phase) const { return 10u * (uint32_t)words(phase); }
+    // plan of an iteration: entries of phase 0's strips, of phase 1's, then the starts
+    __host__ __device__ size_t entry0(int phase, int strip) const
+    {
+        return phase == 0 ? (size_t)strip * updates(0) : (size_t)nstrips * updates(0) + (size_t)strip * updates(1);
+    }
+    __host__ __device__ size_t entries() const { return (size_t)nstrips * (updates(0) + updates(1)); }
+    __host__ __device__ size_t start0(int phase, int strip) const
+    {
+        return phase == 0 ? (size_t)strip * (words(0) + 1)
+                          : (size_t)nstrips * (words(0) + 1) + (size_t)strip * (words(1) + 1);
+    }
+    __host__ __device__ size_t starts() const { return (size_t)nstrips * (words(0) + words(1) + 2); }
+    __host__ __device__ size_t bytes() const { return (entries() * sizeof(uint4) + starts() * 4 + 255) / 256 * 256; }
+};
+
+// An update as its word's thread needs it: x, y the accept masks r < thr1 and
+// r < thr0 of its 21 spins, z the updates of the words above (low half) and
+// below that come before it, w those of the words before and after in the row.
+using Entry = uint4;
+
+__device__ __forceinline__ void words_block(const SweepArgs& a, uint32_t step, uint32_t strip, uint32_t b, uint32_t tl,
+                                            uint32_t x3, uint32_t (&w)[4])
+{
+    w[0] = step;
+    w[1] = strip * 8u + b;
+    w[2] = tl;
+    w[3] = x3;
+#pragma unroll
+    for (int r = 0; r < 10; ++r) philox_round(w[0], w[1], w[2], w[3], a.rk.k0[r], a.rk.k1[r]);
+}
+
+// Accept bits of the draws w[0 .. 3] of spins k0 .. k0 + 3 (those in 0 .. 20).
+template <int K0>
+__device__ __forceinline__ void words_accept(const uint32_t (&w)[4], const SweepArgs& a, uint32_t& m1, uint32_t& m0)
+{
+    if constexpr (K0 >= 0) { accept_bit<(K0 > 0 ? K0 : 0)>(m1, w[0], a.thr1); accept_bit<(K0 > 0 ? K0 : 0)>(m0, w[0], a.thr0); }
+    if constexpr (K0 >= -1) { accept_bit<K0 + 1>(m1, w[1], a.thr1); accept_bit<K0 + 1>(m0, w[1], a.thr0); }
+    accept_bit<K0 + 2>(m1, w[2], a.thr1);
+    accept_bit<K0 + 2>(m0, w[2], a.thr0);
+    if constexpr (K0 + 3 <= 20) { accept_bit<K0 + 3>(m1, w[3], a.thr1); accept_bit<K0 + 3>(m0, w[3], a.thr0); }
+}
+
+// The plan of strip blockIdx.x, phase blockIdx.y, iteration sweep_number(a) +
+// blockIdx.z.  A warp takes a contiguous part of the sequence: first all count
+// their parts' updates of each word, the counts become each part's first update
+// numbers, then each goes through its part 32 updates at a time, with a table of
+// the lanes that update a word.
+__global__ void __launch_bounds__(32 * kPlanWarps)
+words_plan_kernel(WordsGeom g, SweepArgs a, char* __restrict__ plan)
+{
+    extern __shared__ __align__(16) uint32_t plan_smem[];
+    const int phase = blockIdx.y, strip = blockIdx.x, h = g.h(phase), W = g.words(phase);
+    const uint32_t U = g.updates(phase);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    uint32_t* const cnt = plan_smem + (size_t)warp * W;                     // updates of a word before this warp's next
+    uint32_t* const lanes = plan_smem + (size_t)(kPlanWarps + warp) * W;    // this chunk's lanes on a word
+    uint32_t* const start = plan_smem + (size_t)2 * kPlanWarps * W;         // W + 1: first entries of the words
+    uint16_t* const word = reinterpret_cast<uint16_t*>(start + W + 1);      // U: the updates' words
+    plan += (size_t)blockIdx.z * g.bytes();
+    Entry* const entry = reinterpret_cast<Entry*>(plan) + g.entry0(phase, strip);
+    uint32_t* const starts = reinterpret_cast<uint32_t*>(plan + g.entries() * sizeof(Entry)) + g.start0(phase, strip);
+    const uint64_t t = sweep_number(a) + blockIdx.z;
+    const uint32_t x3 = 0x80000000u | ((uint32_t)(t >> 32) << 1) | (uint32_t)phase;
+    const uint32_t part = (U + 32 * kPlanWarps - 1) / (32 * kPlanWarps) * 32;
+    const uint32_t s0 = min(U, (uint32_t)warp * part), s1 = min(U, s0 + part);
+    for (int i = threadIdx.x; i < 2 * kPlanWarps * W; i += blockDim.x) plan_smem[i] = 0;
+    __syncthreads();
+    for (uint32_t s = s0 + lane; s < s1; s += 32) {
+        uint32_t w[4];
+        words_block(a, s, strip, 0, (uint32_t)t, x3, w);
+        const uint32_t x = __umulhi(w[0], (uint32_t)g.N) * (uint32_t)h + __umulhi(w[1], (uint32_t)h);
+        word[s] = (uint16_t)x;
+        atomicAdd(cnt + x, 1u);
+    }
+    __syncthreads();
+    for (int x = threadIdx.x; x < W; x += blockDim.x) {
+        uint32_t run = 0;
+        for (int k = 0; k < kPlanWarps; ++k) {
+            uint32_t* c = plan_smem + (size_t)k * W + x;
+            const uint32_t v = *c;
+            *c = run;
+            run += v;
+        }
+        start[x] = run;
+    }
+    __syncthreads();
+    if (warp == 0) {
+        uint32_t before = 0;
+        for (int x0 = 0; x0 < W; x0 += 32) {
+            const uint32_t v = x0 + lane < W ? start[x0 + lane] : 0u;
+            uint32_t sum = v;
+            for (int d = 1; d < 32; d *= 2) {
+                const uint32_t o = __shfl_up_sync(0xffffffffu, sum, d);
+                if (lane >= d) sum += o;
+            }
+            if (x0 + lane < W) start[x0 + lane] = before + sum - v;
+            before += __shfl_sync(0xffffffffu, sum, 31);
+        }
+        if (lane == 0) start[W] = before;
+    }
+    __syncthreads();
+    for (int x = threadIdx.x; x <= W; x += blockDim.x) starts[x] = start[x];
+    for (uint32_t c0 = s0; c0 < s1; c0 += 32) {
+        const uint32_t s = c0 + lane;
+        const bool live = s < s1;
+        const uint32_t x = live ? word[s] : 0u;
+        if (live) atomicOr(lanes + x, 1u << lane);
+        __syncwarp();
+        Entry e;
+        uint32_t pos = 0, all = 0;
+        if (live) {
+            const uint32_t below = (1u << lane) - 1u, I = x / (uint32_t)h, j = x - I * (uint32_t)h;
+            auto before = [&](uint32_t y) { return cnt[y] + __popc(lanes[y] & below); };
+            const uint32_t up = I == 0 ? x + (uint32_t)(g.N - 1) * h : x - h;
+            const uint32_t dn = I == (uint32_t)g.N - 1 ? j : x + h;
+            e.z = before(up) | before(dn) << 16;
+            e.w = (j > 0 ? before(x - 1) : 0u) | (j + 1 < (uint32_t)h ? before(x + 1) : 0u) << 16;
+            pos = start[x] + before(x);
+            all = lanes[x];
+        }
+        __syncwarp();
+        if (live && lane == __ffs(all) - 1) {
+            cnt[x] += __popc(all);
+            lanes[x] = 0;
+        }
+        __syncwarp();
+        if (!live) continue;
+        uint32_t m1 = 0, m0 = 0, w[4];
+        words_block(a, s, strip, 0, (uint32_t)t, x3, w);
+        words_accept<-2>(w, a, m1, m0);
+        words_block(a, s, strip, 1, (uint32_t)t, x3, w);
+        words_accept<2>(w, a, m1, m0);
+        words_block(a, s, strip, 2, (uint32_t)t, x3, w);
+        words_accept<6>(w, a, m1, m0);
+        words_block(a, s, strip, 3, (uint32_t)t, x3, w);
+        words_accept<10>(w, a, m1, m0);
+        words_block(a, s, strip, 4, (uint32_t)t, x3, w);
+        words_accept<14>(w, a, m1, m0);
+        words_block(a, s, strip, 5, (uint32_t)t, x3, w);
+        words_accept<18>(w, a, m1, m0);
+        e.x = (m1 | a.all1) & kWordBits;
+        e.y = (m0 | a.all0) & kWordBits;
+        entry[pos] = e;
+    }
+}
+
+__device__ __forceinline__ uint64_t word_look(uint32_t addr)
+{
+    uint64_t v;
+    asm volatile("ld.volatile.shared.u64 %0, [%1];" : "=l"(v) : "r"(addr) : "memory");
+    return v;
+}
+
+// A word that a thread owns: its next update and where its neighbours are.
+struct OwnWord {
+    uint32_t at, up, dn;            // shared addresses of the word, of the words above and below
+    uint32_t rot;                   // 1: the word above is in the last row, 2: the word below in the first
+    uint32_t spins, done, count, first;
+    Entry e;
+};
+
+// One phase of one iteration, strip blockIdx.x, from its plan.
+template <int WPT>
+__global__ void __launch_bounds__(kWordsThreads)
+words_run_kernel(uint64_t* S, WordsGeom g, int phase, const char* __restrict__ plan, unsigned int* err)
+{
+    extern __shared__ __align__(16) uint4 run_smem[];
+    const int strip = blockIdx.x, h = g.h(phase), hw = h + 2, W = g.words(phase);
+    const uint32_t U = g.updates(phase);
+    const int col0 = strip * g.NC + (phase == 0 ? 0 : g.NC / 2);
+    const uint64_t n_lat = (uint64_t)g.N * g.L;
+    Entry* const entry = run_smem;                                          // U
+    uint64_t* const win = reinterpret_cast<uint64_t*>(run_smem + U);        // N x (h + 2): spins | updates done << 32
+    const uint64_t n_win = (uint64_t)g.N * hw;
+    uint32_t* const start = reinterpret_cast<uint32_t*>(win + n_win);       // W + 1
+    const Entry* const my_entry = reinterpret_cast<const Entry*>(plan) + g.entry0(phase, strip);
+    const uint32_t* const my_start =
+        reinterpret_cast<const uint32_t*>(plan + g.entries() * sizeof(Entry)) + g.start0(phase, strip);
+    for (uint32_t i = threadIdx.x; i < U; i += blockDim.x)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;"
+                     ::"r"((uint32_t)__cvta_generic_to_shared(entry + i)), "l"(my_entry + i) : "memory");
+    for (int i = threadIdx.x; i <= W; i += blockDim.x) start[i] = __ldg(my_start + i);
+    for (int i = threadIdx.x; i < (int)n_win; i += blockDim.x) {
+        const int I = i / hw;
+        int J = col0 - 1 + i - I * hw;
+        J = J < 0 ? J + g.L : (J >= g.L ? J - g.L : J);
+        word_st(win, (uint64_t)i, pack_fields(word_ld<false>(S, (uint64_t)I * g.L + J, n_lat, __LINE__)), n_win,
+                __LINE__);
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    const uint32_t win_sh = (uint32_t)__cvta_generic_to_shared(win), row = 8u * (uint32_t)hw;
+    OwnWord o[WPT];
+#pragma unroll
+    for (int k = 0; k < WPT; ++k) {
+        const int x = threadIdx.x + k * blockDim.x;
+        o[k].count = o[k].done = 0;
+        if (x >= W) continue;
+        const int I = x / h, j = x - I * h;
+        o[k].at = win_sh + (uint32_t)I * row + 8u * (uint32_t)(j + 1);
+        o[k].up = I == 0 ? o[k].at + (uint32_t)(g.N - 1) * row : o[k].at - row;
+        o[k].dn = I == g.N - 1 ? o[k].at - (uint32_t)(g.N - 1) * row : o[k].at + row;
+        o[k].rot = (I == 0 ? 1u : 0u) | (I == g.N - 1 ? 2u : 0u);
+        o[k].spins = (uint32_t)word_look(o[k].at);
+        o[k].first = start[x];
+        o[k].count = start[x + 1] - o[k].first;
+        if (o[k].count) o[k].e = entry[o[k].first];
+    }
+    // every thread has its own words' spins before any word changes (a word is
+    // written by its own thread only)
+    for (uint32_t tries = 0;; ++tries) {
+        bool pending = false;
+#pragma unroll
+        for (int k = 0; k < WPT; ++k) {
+            OwnWord& w = o[k];
+            if (w.done == w.count) continue;
+            const uint64_t up = word_look(w.up), dn = word_look(w.dn), lf = word_look(w.at - 8), rt = word_look(w.at + 8);
+            // the counts are below 2^16: at most 10 N h <= 2^16 updates
+            const uint32_t z = (uint32_t)(up >> 32) | (uint32_t)(dn >> 32) << 16;
+            const uint32_t v = (uint32_t)(lf >> 32) | (uint32_t)(rt >> 32) << 16;
+            if (z == w.e.z && v == w.e.w) {
+                uint32_t u = (uint32_t)up, d = (uint32_t)dn;
+                if (w.rot & 1) u = (u << 1 | u >> 20) & kWordBits;
+                if (w.rot & 2) d = (d >> 1 | d << 20) & kWordBits;
+                w.spins = flip_all(w.spins, u, d, (uint32_t)lf, (uint32_t)rt, w.e.x, w.e.y);
+                ++w.done;
+                asm volatile("st.volatile.shared.u64 [%0], %1;" ::"r"(w.at), "l"((uint64_t)w.done << 32 | w.spins) : "memory");
+                if (w.done < w.count) w.e = entry[w.first + w.done];
+            }
+            pending = pending || w.done < w.count;
+        }
+        if (!__any_sync(0xffffffffu, pending)) break;
+        if (tries == kWordsTries) {
+            *(volatile unsigned int*)err = 1;
+            break;
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < WPT; ++k) {
+        const int x = threadIdx.x + k * blockDim.x;
+        if (x >= W) continue;
+        const int I = x / h;
+        word_st(S, (uint64_t)I * g.L + col0 + x - I * h, spread_fields(o[k].spins), n_lat, __LINE__);
+    }
+}
+
+WordsGeom words_geom(int L, int nstrips) { return {L, L / 21, L / nstrips, nstrips}; }
+
+size_t plan_smem_bytes(const WordsGeom& g)
+{
+    const size_t W = g.words(1);
+    return (2 * kPlanWarps * W + W + 1) * 4 + ((size_t)g.updates(1) * 2 + 3) / 4 * 4;
+}
+
+size_t run_smem_bytes(const WordsGeom& g, int phase)
+{
+    return g.updates(phase) * sizeof(Entry) + (size_t)g.N * (g.h(phase) + 2) * 8 + ((size_t)g.words(phase) + 1) * 4;
+}
+
+bool words_setup()
+{
+    static const bool ok =      // per process, set once
+        cudaFuncSetAttribute(words_plan_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWordsSmemMax) ==
+            cudaSuccess &&
+        cudaFuncSetAttribute(words_run_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWordsSmemMax) ==
+            cudaSuccess &&
+        cudaFuncSetAttribute(words_run_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWordsSmemMax) ==
+            cudaSuccess;
+    return ok;
+}
+
+}  // namespace
+
+bool words_planned(int L, int nstrips)
+{
+    const WordsGeom g = words_geom(L, nstrips);
+    return g.words(1) <= 2 * kWordsThreads && run_smem_bytes(g, 1) <= kWordsSmemMax &&
+           plan_smem_bytes(g) <= kWordsSmemMax && words_setup();
+}
+
+size_t words_plan_bytes(int L, int nstrips) { return words_geom(L, nstrips).bytes(); }
+
+int words_plan_iterations(int L, int nstrips, int64_t n)
+{
+    const size_t most = std::max<size_t>(1, kWordsPlanBytes / words_plan_bytes(L, nstrips));
+    return (int)std::min<int64_t>(n, std::min<size_t>(most, kWordsPlanIterations));
+}
+
+cudaError_t words_plan(int L, int nstrips, const SweepArgs& a, int iterations, void* plan, cudaStream_t s)
+{
+    const WordsGeom g = words_geom(L, nstrips);
+    words_plan_kernel<<<dim3(nstrips, 2, iterations), 32 * kPlanWarps, plan_smem_bytes(g), s>>>(
+        g, a, static_cast<char*>(plan));
+    return cudaGetLastError();
+}
+
+cudaError_t words_run(uint64_t* S, int L, int nstrips, const void* plan, int iteration, unsigned int* err,
+                      cudaStream_t s)
+{
+    const WordsGeom g = words_geom(L, nstrips);
+    const char* p = static_cast<const char*>(plan) + (size_t)iteration * g.bytes();
+    for (int phase = 0; phase < 2; ++phase) {
+        const int W = g.words(phase), per = W > kWordsThreads ? 2 : 1, threads = ((W + per - 1) / per + 31) / 32 * 32;
+        if (per == 1) words_run_kernel<1><<<nstrips, threads, run_smem_bytes(g, phase), s>>>(S, g, phase, p, err);
+        else words_run_kernel<2><<<nstrips, threads, run_smem_bytes(g, phase), s>>>(S, g, phase, p, err);
+    }
+    return cudaGetLastError();
+}
+
+}  // namespace ising
