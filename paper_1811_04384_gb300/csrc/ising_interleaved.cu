@@ -545,7 +545,7 @@ static void ci_launch_r(dim3 grid, int colour, bool update, bool record, uint64_
                         const SweepArgs& a, bool in_graphs, cudaStream_t s)
 {
     const dim3 block(kCiBlockX * kCiBlockY);
-    if (!update) ci_half_sweep_kernel<1, false, true, 10><<<grid, block, 0, s>>>(S, L, N, a);
+    if (!update) launch_pdl(ci_half_sweep_kernel<1, false, true, 10>, grid, block, s, S, L, N, a);
     else if (colour == 0) launch_pdl_opt(in_graphs, ci_half_sweep_kernel<0, true, false, ROUNDS>, grid, block, s, S, L, N, a);
     else if (record) launch_pdl_opt(in_graphs, ci_half_sweep_kernel<1, true, true, ROUNDS>, grid, block, s, S, L, N, a);
     else launch_pdl_opt(in_graphs, ci_half_sweep_kernel<1, true, false, ROUNDS>, grid, block, s, S, L, N, a);

@@ -35,7 +35,8 @@ cudaError_t ci_random_words_iteration(uint64_t* S, int L, int nstrips, const Swe
 // fits (words_planned): words_plan makes the plans of iterations
 // sweep_number(a) .. + iterations - 1 (words_plan_bytes each; at most
 // words_plan_iterations of the n that a call runs), words_run both phases of
-// the plan's iteration `iteration`; *err = 1 when a wait gave up.
+// the plan's iteration `iteration` (0: right after words_plan, or after the
+// phases before it); *err = 1 when a wait gave up.
 bool words_planned(int L, int nstrips);
 size_t words_plan_bytes(int L, int nstrips);
 int words_plan_iterations(int L, int nstrips, int64_t n);

@@ -144,8 +144,8 @@ cudaError_t launch_warp_sweeps(uint64_t* w0, uint64_t* w1, const Geom& g, const 
 // by the caller keeps full edges; the library's own graphs use programmatic
 // ones.  Errors are left for cudaGetLastError.
 template <typename... Params, typename... Args>
-inline void launch_pdl_opt(bool in_graphs, void (*kernel)(Params...), dim3 grid, dim3 block, cudaStream_t s,
-                           Args... args)
+inline void launch_pdl_with(bool in_graphs, size_t smem, void (*kernel)(Params...), dim3 grid, dim3 block,
+                            cudaStream_t s, Args... args)
 {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     if (!in_graphs && cudaStreamIsCapturing(s, &cs) != cudaSuccess) {
@@ -155,7 +155,7 @@ inline void launch_pdl_opt(bool in_graphs, void (*kernel)(Params...), dim3 grid,
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -163,6 +163,13 @@ inline void launch_pdl_opt(bool in_graphs, void (*kernel)(Params...), dim3 grid,
     cfg.attrs = attr;
     cfg.numAttrs = cs == cudaStreamCaptureStatusNone ? 1 : 0;
     cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+template <typename... Params, typename... Args>
+inline void launch_pdl_opt(bool in_graphs, void (*kernel)(Params...), dim3 grid, dim3 block, cudaStream_t s,
+                           Args... args)
+{
+    launch_pdl_with(in_graphs, 0, kernel, grid, block, s, args...);
 }
 
 template <typename... Params, typename... Args>

@@ -16,7 +16,9 @@
 // count of updates share 64 bits of shared memory, so one load gives both and
 // no barrier or fence is needed.  An update that is the oldest of all pending
 // ones never waits, so the phase always ends.  Measured on GB300, 5 iterations
-// of L = 1008 with 72 strips, a record after each: 819 -> @@ us.
+// of L = 1008 with 72 strips, a record after each: 798 -> 215 us, of which the
+// plans take 54 and a phase 14.  (The plans of later iterations beside the
+// phases, on a second stream: 218.)
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -37,6 +39,8 @@ constexpr uint32_t kWordsTries = 1u << 24;      // a thread's looks at its neigh
 constexpr size_t kWordsPlanBytes = (size_t)64 << 20;
 constexpr int kWordsPlanIterations = 16;
 constexpr uint32_t kWordBits = (1u << 21) - 1;
+constexpr int kWordIndexBits = 12;              // a half strip has at most 2 kWordsThreads words
+static_assert(2 * kWordsThreads <= 1 << kWordIndexBits, "an update's word and four accept bits fit 16 bits");
 
 // The strips' half strips in a phase.
 struct WordsGeom {
@@ -64,26 +68,29 @@ struct WordsGeom {
 // below that come before it, w those of the words before and after in the row.
 using Entry = uint4;
 
-__device__ __forceinline__ void words_block(const SweepArgs& a, uint32_t step, uint32_t strip, uint32_t b, uint32_t tl,
-                                            uint32_t x3, uint32_t (&w)[4])
-{
-    w[0] = step;
-    w[1] = strip * 8u + b;
-    w[2] = tl;
-    w[3] = x3;
-#pragma unroll
-    for (int r = 0; r < 10; ++r) philox_round(w[0], w[1], w[2], w[3], a.rk.k0[r], a.rk.k1[r]);
-}
-
-// Accept bits of the draws w[0 .. 3] of spins k0 .. k0 + 3 (those in 0 .. 20).
-template <int K0>
+// Accept bits of spins K .. of a call's draws w[FROM .. 3] (spins 0 .. 20).
+template <int K, int FROM>
 __device__ __forceinline__ void words_accept(const uint32_t (&w)[4], const SweepArgs& a, uint32_t& m1, uint32_t& m0)
 {
-    if constexpr (K0 >= 0) { accept_bit<(K0 > 0 ? K0 : 0)>(m1, w[0], a.thr1); accept_bit<(K0 > 0 ? K0 : 0)>(m0, w[0], a.thr0); }
-    if constexpr (K0 >= -1) { accept_bit<K0 + 1>(m1, w[1], a.thr1); accept_bit<K0 + 1>(m0, w[1], a.thr0); }
-    accept_bit<K0 + 2>(m1, w[2], a.thr1);
-    accept_bit<K0 + 2>(m0, w[2], a.thr0);
-    if constexpr (K0 + 3 <= 20) { accept_bit<K0 + 3>(m1, w[3], a.thr1); accept_bit<K0 + 3>(m0, w[3], a.thr0); }
+    if constexpr (FROM < 4 && K < 21) {
+        accept_bit<K>(m1, w[FROM], a.thr1);
+        accept_bit<K>(m0, w[FROM], a.thr0);
+        words_accept<K + 1, FROM + 1>(w, a, m1, m0);
+    }
+}
+
+// Calls B .. 5 of an update (the counter of call b is (step, 8 strip + b, t, x3),
+// and draw 4 b + e is the word of spin 4 b + e - 2), with their first products.
+template <int B>
+__device__ __forceinline__ void words_calls(const PhiloxRowKey& row, const uint2 (&first)[6], const SweepArgs& a,
+                                            uint32_t& m1, uint32_t& m0)
+{
+    if constexpr (B < 6) {
+        uint32_t w[4];
+        philox_row_tail<10>(row, a.rk, first[B].x, first[B].y, w);
+        words_accept<4 * B - 2, 0>(w, a, m1, m0);
+        words_calls<B + 1>(row, first, a, m1, m0);
+    }
 }
 
 // The plan of strip blockIdx.x, phase blockIdx.y, iteration sweep_number(a) +
@@ -101,7 +108,7 @@ words_plan_kernel(WordsGeom g, SweepArgs a, char* __restrict__ plan)
     uint32_t* const cnt = plan_smem + (size_t)warp * W;                     // updates of a word before this warp's next
     uint32_t* const lanes = plan_smem + (size_t)(kPlanWarps + warp) * W;    // this chunk's lanes on a word
     uint32_t* const start = plan_smem + (size_t)2 * kPlanWarps * W;         // W + 1: first entries of the words
-    uint16_t* const word = reinterpret_cast<uint16_t*>(start + W + 1);      // U: the updates' words
+    uint16_t* const word = reinterpret_cast<uint16_t*>(start + W + 1);      // U: the updates' words, bits 0 and 1 of both masks
     plan += (size_t)blockIdx.z * g.bytes();
     Entry* const entry = reinterpret_cast<Entry*>(plan) + g.entry0(phase, strip);
     uint32_t* const starts = reinterpret_cast<uint32_t*>(plan + g.entries() * sizeof(Entry)) + g.start0(phase, strip);
@@ -110,12 +117,18 @@ words_plan_kernel(WordsGeom g, SweepArgs a, char* __restrict__ plan)
     const uint32_t part = (U + 32 * kPlanWarps - 1) / (32 * kPlanWarps) * 32;
     const uint32_t s0 = min(U, (uint32_t)warp * part), s1 = min(U, s0 + part);
     for (int i = threadIdx.x; i < 2 * kPlanWarps * W; i += blockDim.x) plan_smem[i] = 0;
+    // the calls' first products, the same for every update of the strip
+    const uint32_t key = philox_first_key((uint32_t)t, a.rk);
+    uint2 first[6];
+#pragma unroll
+    for (int b = 0; b < 6; ++b) mul_hilo(kPhiloxM0, key ^ ((uint32_t)strip * 8u + b), first[b].x, first[b].y);
     __syncthreads();
     for (uint32_t s = s0 + lane; s < s1; s += 32) {
-        uint32_t w[4];
-        words_block(a, s, strip, 0, (uint32_t)t, x3, w);
+        uint32_t w[4], m1 = 0, m0 = 0;
+        philox_row_tail<10>(philox_row_key(s, (uint32_t)t, x3, a.rk), a.rk, first[0].x, first[0].y, w);
         const uint32_t x = __umulhi(w[0], (uint32_t)g.N) * (uint32_t)h + __umulhi(w[1], (uint32_t)h);
-        word[s] = (uint16_t)x;
+        words_accept<0, 2>(w, a, m1, m0);
+        word[s] = (uint16_t)(x | m1 << kWordIndexBits | m0 << (kWordIndexBits + 2));
         atomicAdd(cnt + x, 1u);
     }
     __syncthreads();
@@ -149,7 +162,7 @@ words_plan_kernel(WordsGeom g, SweepArgs a, char* __restrict__ plan)
     for (uint32_t c0 = s0; c0 < s1; c0 += 32) {
         const uint32_t s = c0 + lane;
         const bool live = s < s1;
-        const uint32_t x = live ? word[s] : 0u;
+        const uint32_t kept = live ? word[s] : 0u, x = kept & ((1u << kWordIndexBits) - 1u);
         if (live) atomicOr(lanes + x, 1u << lane);
         __syncwarp();
         Entry e;
@@ -171,19 +184,8 @@ words_plan_kernel(WordsGeom g, SweepArgs a, char* __restrict__ plan)
         }
         __syncwarp();
         if (!live) continue;
-        uint32_t m1 = 0, m0 = 0, w[4];
-        words_block(a, s, strip, 0, (uint32_t)t, x3, w);
-        words_accept<-2>(w, a, m1, m0);
-        words_block(a, s, strip, 1, (uint32_t)t, x3, w);
-        words_accept<2>(w, a, m1, m0);
-        words_block(a, s, strip, 2, (uint32_t)t, x3, w);
-        words_accept<6>(w, a, m1, m0);
-        words_block(a, s, strip, 3, (uint32_t)t, x3, w);
-        words_accept<10>(w, a, m1, m0);
-        words_block(a, s, strip, 4, (uint32_t)t, x3, w);
-        words_accept<14>(w, a, m1, m0);
-        words_block(a, s, strip, 5, (uint32_t)t, x3, w);
-        words_accept<18>(w, a, m1, m0);
+        uint32_t m1 = kept >> kWordIndexBits & 3u, m0 = kept >> (kWordIndexBits + 2);
+        words_calls<1>(philox_row_key(s, (uint32_t)t, x3, a.rk), first, a, m1, m0);
         e.x = (m1 | a.all1) & kWordBits;
         e.y = (m0 | a.all0) & kWordBits;
         entry[pos] = e;
@@ -200,15 +202,23 @@ __device__ __forceinline__ uint64_t word_look(uint32_t addr)
 // A word that a thread owns: its next update and where its neighbours are.
 struct OwnWord {
     uint32_t at, up, dn;            // shared addresses of the word, of the words above and below
-    uint32_t rot;                   // 1: the word above is in the last row, 2: the word below in the first
-    uint32_t spins, done, count, first;
-    Entry e;
+    bool first_row, last_row;
+    uint32_t spins, done, count;
+    uint32_t ahead;                 // shared address of the entry after `next`
+    Entry e, next;                  // its next update and the one after
 };
+
+__device__ __forceinline__ Entry entry_ld(uint32_t addr)
+{
+    Entry e;
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(e.x), "=r"(e.y), "=r"(e.z), "=r"(e.w) : "r"(addr));
+    return e;
+}
 
 // One phase of one iteration, strip blockIdx.x, from its plan.
 template <int WPT>
 __global__ void __launch_bounds__(kWordsThreads)
-words_run_kernel(uint64_t* S, WordsGeom g, int phase, const char* __restrict__ plan, unsigned int* err)
+words_run_kernel(uint64_t* S, WordsGeom g, int phase, bool fresh, const char* __restrict__ plan, unsigned int* err)
 {
     extern __shared__ __align__(16) uint4 run_smem[];
     const int strip = blockIdx.x, h = g.h(phase), hw = h + 2, W = g.words(phase);
@@ -222,10 +232,15 @@ words_run_kernel(uint64_t* S, WordsGeom g, int phase, const char* __restrict__ p
     const Entry* const my_entry = reinterpret_cast<const Entry*>(plan) + g.entry0(phase, strip);
     const uint32_t* const my_start =
         reinterpret_cast<const uint32_t*>(plan + g.entries() * sizeof(Entry)) + g.start0(phase, strip);
+    // the plan is of a launch that this one waits for (fresh), or one that ended
+    // before the launch before passed its wait; the lattice is the launch before's
+    if (fresh) pdl_wait();
     for (uint32_t i = threadIdx.x; i < U; i += blockDim.x)
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;"
                      ::"r"((uint32_t)__cvta_generic_to_shared(entry + i)), "l"(my_entry + i) : "memory");
     for (int i = threadIdx.x; i <= W; i += blockDim.x) start[i] = __ldg(my_start + i);
+    if (!fresh) pdl_wait();
+    pdl_launch();
     for (int i = threadIdx.x; i < (int)n_win; i += blockDim.x) {
         const int I = i / hw;
         int J = col0 - 1 + i - I * hw;
@@ -236,43 +251,55 @@ words_run_kernel(uint64_t* S, WordsGeom g, int phase, const char* __restrict__ p
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
     const uint32_t win_sh = (uint32_t)__cvta_generic_to_shared(win), row = 8u * (uint32_t)hw;
+    const uint32_t entry_sh = (uint32_t)__cvta_generic_to_shared(entry);
     OwnWord o[WPT];
 #pragma unroll
     for (int k = 0; k < WPT; ++k) {
-        const int x = threadIdx.x + k * blockDim.x;
-        o[k].count = o[k].done = 0;
-        if (x >= W) continue;
-        const int I = x / h, j = x - I * h;
+        // a thread without a word looks at word 0's neighbours and never runs
+        const bool has = threadIdx.x + k * blockDim.x < (uint32_t)W;
+        const int x = has ? threadIdx.x + k * blockDim.x : 0, I = x / h, j = x - I * h;
+        o[k].first_row = I == 0;
+        o[k].last_row = I == g.N - 1;
         o[k].at = win_sh + (uint32_t)I * row + 8u * (uint32_t)(j + 1);
-        o[k].up = I == 0 ? o[k].at + (uint32_t)(g.N - 1) * row : o[k].at - row;
-        o[k].dn = I == g.N - 1 ? o[k].at - (uint32_t)(g.N - 1) * row : o[k].at + row;
-        o[k].rot = (I == 0 ? 1u : 0u) | (I == g.N - 1 ? 2u : 0u);
+        o[k].up = o[k].first_row ? o[k].at + (uint32_t)(g.N - 1) * row : o[k].at - row;
+        o[k].dn = o[k].last_row ? o[k].at - (uint32_t)(g.N - 1) * row : o[k].at + row;
         o[k].spins = (uint32_t)word_look(o[k].at);
-        o[k].first = start[x];
-        o[k].count = start[x + 1] - o[k].first;
-        if (o[k].count) o[k].e = entry[o[k].first];
+        o[k].done = 0;
+        o[k].count = has ? start[x + 1] - start[x] : 0u;
+        // two entries past a word's last (never run) are other words', or the window's first bytes
+        o[k].ahead = entry_sh + 16u * (start[x] + 2u);
+        o[k].e = entry_ld(o[k].ahead - 32u);
+        o[k].next = entry_ld(o[k].ahead - 16u);
     }
-    // every thread has its own words' spins before any word changes (a word is
-    // written by its own thread only)
+    // a word changes by its own thread only, so there is no barrier from here on
     for (uint32_t tries = 0;; ++tries) {
         bool pending = false;
 #pragma unroll
         for (int k = 0; k < WPT; ++k) {
             OwnWord& w = o[k];
-            if (w.done == w.count) continue;
             const uint64_t up = word_look(w.up), dn = word_look(w.dn), lf = word_look(w.at - 8), rt = word_look(w.at + 8);
-            // the counts are below 2^16: at most 10 N h <= 2^16 updates
+            // the counts are below 2^16: at most 20,480 updates of a half strip
             const uint32_t z = (uint32_t)(up >> 32) | (uint32_t)(dn >> 32) << 16;
             const uint32_t v = (uint32_t)(lf >> 32) | (uint32_t)(rt >> 32) << 16;
-            if (z == w.e.z && v == w.e.w) {
-                uint32_t u = (uint32_t)up, d = (uint32_t)dn;
-                if (w.rot & 1) u = (u << 1 | u >> 20) & kWordBits;
-                if (w.rot & 2) d = (d >> 1 | d << 20) & kWordBits;
-                w.spins = flip_all(w.spins, u, d, (uint32_t)lf, (uint32_t)rt, w.e.x, w.e.y);
-                ++w.done;
-                asm volatile("st.volatile.shared.u64 [%0], %1;" ::"r"(w.at), "l"((uint64_t)w.done << 32 | w.spins) : "memory");
-                if (w.done < w.count) w.e = entry[w.first + w.done];
-            }
+            const bool ready = w.done < w.count && z == w.e.z && v == w.e.w;
+            // straight-line: the lanes of a warp are seldom ready together
+            uint32_t u = (uint32_t)up, d = (uint32_t)dn;
+            u = w.first_row ? (u << 1 | u >> 20) & kWordBits : u;
+            d = w.last_row ? (d >> 1 | d << 20) & kWordBits : d;
+            const uint32_t spins = flip_all(w.spins, u, d, (uint32_t)lf, (uint32_t)rt, w.e.x, w.e.y);
+            w.spins = ready ? spins : w.spins;
+            w.done += ready;
+            w.ahead += ready ? 16u : 0u;
+            w.e.x = ready ? w.next.x : w.e.x;
+            w.e.y = ready ? w.next.y : w.e.y;
+            w.e.z = ready ? w.next.z : w.e.z;
+            w.e.w = ready ? w.next.w : w.e.w;
+            asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %4, 0;\n\t"
+                         "@p st.volatile.shared.u64 [%5], %6;\n\t"
+                         "@p ld.shared.v4.u32 {%0, %1, %2, %3}, [%7];\n\t}"
+                         : "+r"(w.next.x), "+r"(w.next.y), "+r"(w.next.z), "+r"(w.next.w)
+                         : "r"((uint32_t)ready), "r"(w.at), "l"((uint64_t)w.done << 32 | w.spins), "r"(w.ahead - 16u)
+                         : "memory");
             pending = pending || w.done < w.count;
         }
         if (!__any_sync(0xffffffffu, pending)) break;
@@ -343,12 +370,14 @@ cudaError_t words_plan(int L, int nstrips, const SweepArgs& a, int iterations, v
 cudaError_t words_run(uint64_t* S, int L, int nstrips, const void* plan, int iteration, unsigned int* err,
                       cudaStream_t s)
 {
+    const dim3 grid(nstrips);
     const WordsGeom g = words_geom(L, nstrips);
     const char* p = static_cast<const char*>(plan) + (size_t)iteration * g.bytes();
     for (int phase = 0; phase < 2; ++phase) {
         const int W = g.words(phase), per = W > kWordsThreads ? 2 : 1, threads = ((W + per - 1) / per + 31) / 32 * 32;
-        if (per == 1) words_run_kernel<1><<<nstrips, threads, run_smem_bytes(g, phase), s>>>(S, g, phase, p, err);
-        else words_run_kernel<2><<<nstrips, threads, run_smem_bytes(g, phase), s>>>(S, g, phase, p, err);
+        const bool fresh = iteration == 0 && phase == 0;      // the plan is the launch before
+        launch_pdl_with(false, run_smem_bytes(g, phase), per == 1 ? words_run_kernel<1> : words_run_kernel<2>, grid,
+                        dim3(threads), s, S, g, phase, fresh, p, err);
     }
     return cudaGetLastError();
 }
