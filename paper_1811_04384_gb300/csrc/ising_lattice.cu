@@ -599,16 +599,19 @@ static int run_resident(ising_lattice* h, int n, int every, bool* direct)
 // buffers: the draw of piece j + 1 follows the cluster launch of piece j in the
 // stream with programmatic stream serialization, so it runs on the SMs the
 // clusters leave free while piece j is applied, and writes the buffer piece
-// j - 1 read (complete before piece j started).  A call runs as about
-// kClusterPieces pieces, because the first draw and the last apply overlap
-// nothing (us per call for 1 / 4 / 6 / 10 pieces, k = 12: L = 1008 x 500 sweeps
-// 640 / 596 / 589 / 613; L = 1500 x 400 on two clusters 863 / 768 / 749 / 765; L =
-// 296 x 1000: 565 / 563 / 566 / 579).  A column-interleaved lattice is converted
-// to dense rows and back around the call.
+// j - 1 read (complete before piece j started).  A call runs as up to
+// kClusterPieces equal pieces, because the first draw and the last apply overlap
+// nothing, each of at least kClusterMinPiece or kBandMinPiece sweeps, because a
+// piece's launches cost about 6 us (us per call for 2 / 3 / 4 / 6 / 8 pieces: L = 296,
+// 1000 sweeps 352 / 352 / 357 / 349 / 365, 100 sweeps 66 / 71 / 77 / 81 / 80; L =
+// 1008, 500 sweeps 599 / 567 / 555 / 549 / 546, 100 sweeps 151 / 155 / 167 / - / -; L =
+// 1500, 400 sweeps 828 / 770 / 749 / 741 / 747; L = 2016, 300 sweeps 919 / 948 /
+// 940 / 940 / 932).  A column-interleaved lattice is converted to dense rows and back
+// around the call.
 constexpr int kClusterMaxL = 3000;
 constexpr int kCiClusterMaxL = 2604;               // the column-interleaved layout (L % 84 == 0)
 constexpr size_t kClusterMaskBytes = 256u << 20;   // both buffers
-constexpr int kClusterMaxPiece = 256, kClusterMinPiece = 32, kClusterPieces = 4;
+constexpr int kClusterMaxPiece = 256, kClusterMinPiece = 30, kBandMinPiece = 50, kClusterPieces = 4;
 // The words between clusters (xflag, u64 each): 2 flags for each of at most
 // 16 boundaries, the error word of the waits (u32), the agreement words
 // (cl_decide: two sets of {count, verdict} and the first piece given up,
@@ -674,7 +677,9 @@ static int run_cluster(ising_lattice* h, int64_t n, int64_t every, unsigned long
     const Geom& g = h->g;
     const bool ci = h->layout == ISING_LAYOUT_COLUMN_INTERLEAVED;
     const size_t per_sweep = cl_mask_bytes_per_sweep(g.L);
-    const int64_t wanted = std::max<int64_t>(kClusterMinPiece, (n + kClusterPieces - 1) / kClusterPieces);
+    const int64_t pieces = std::max<int64_t>(
+        1, std::min<int64_t>(kClusterPieces, n / (plan.v == 0 ? kBandMinPiece : kClusterMinPiece)));
+    const int64_t wanted = std::max<int64_t>(1, (n + pieces - 1) / pieces);
     const int max_piece = (int)std::max<size_t>(
         1, std::min<size_t>((size_t)std::min<int64_t>(wanted, kClusterMaxPiece), kClusterMaskBytes / (2 * per_sweep)));
     const size_t buf = (size_t)std::min<int64_t>(n, max_piece) * per_sweep + kClMaskPad * per_sweep / 2;
