@@ -51,6 +51,8 @@ MEASURED_TRAFFIC = {16384: 1.103e8}
 MULWIDE_PER_SITE = 4            # Philox4x32-10 with the counter-independent rounds hoisted:
                                 # 16 multiplies per call, one call per 4 sites (10 per call,
                                 # 2.5 per site, for the opt-in 7-round scheme)
+MULWIDE_SHARED = 3.75           # the half-sweep kernel also shares a call's first product among the
+                                # rows of its block: 15 per call (9 and 2.25 for 7 rounds)
 
 
 def parse():
@@ -493,20 +495,19 @@ def run_plain(args, ising, local):
           "paths": {"resident_on_chip": rate["resident"], "launches": rate["launches"],
                     "graph_captured_batch": rate["graph"]},
           "bit_exact_across_paths": exact,
-          "gpu_launches": 3})      # the timed on-chip call: mask draw, on-chip sweeps, sweep counter
+          "gpu_launches": 2})      # the timed on-chip call: mask draw, on-chip sweeps (which set the counter)
 
 
-# Mid-size lattices, between the on-chip range (L <= 292) and L = 1080:
-# there the automatic path is the cluster path (one thread-block
-# cluster keeps the lattice on chip over pieces of up to 256 sweeps).
+# Mid-size lattices: there the automatic path is the cluster path (one
+# thread-block cluster keeps the lattice on chip over pieces of up to 256 sweeps).
 MIDSIZE_L = [296, 400, 512, 700, 1008]
 
 
 def cluster_launches(L: int, sweeps: int, every: int) -> int:
-    """Kernel launches of ising_sweep_record(sweeps, every) on the cluster
-    path: per chunk of 1024 records, a mask draw and a cluster launch per
-    piece of sweeps (two mask buffers of at most 128 MB, 256 sweeps at most)
-    and one sweep-counter advance."""
+    """Fewest kernel launches of ising_sweep_record(sweeps, every) on the cluster
+    path, with pieces as long as they can be: per chunk of 1024 records, a mask
+    draw and a cluster launch per piece of sweeps (two mask buffers of at most
+    128 MB of packed rows, 256 sweeps at most) and one sweep-counter advance."""
     W = -(-(L // 2) // 21)
     P = W + (W & 1)
     piece = max(1, min(256, (256 << 20) // (2 * 2 * L * P * 8)))
@@ -517,6 +518,24 @@ def cluster_launches(L: int, sweeps: int, every: int) -> int:
         records -= chunk
     if rest > 0:                       # the sweeps after the last record: one ising_sweep
         launches += 2 * -(-rest // piece) + 1
+    return launches
+
+
+def midsize_launches(L: int, sweeps: int, every: int) -> int:
+    """Kernel launches of ising_sweep_record(sweeps, every), sweeps a multiple
+    of every, on one cluster: per chunk of 1024 records, up to four equal pieces
+    of at least 50 sweeps (rows of up to 14 dense words) or 30, 256 at most, each a
+    mask draw and a cluster launch; beyond 14 words a counter advance."""
+    words = -(-(L // 2) // 32)
+    band = words <= 14
+    per_sweep = 2 * L * ((words + 1) // 2 * 2) * 8
+    launches, left = 0, sweeps
+    while left > 0:
+        n = min(left, 1024 * every)
+        pieces = max(1, min(4, n // (50 if band else 30)))
+        piece = min(-(-n // pieces), 256, (256 << 20) // (2 * per_sweep))
+        launches += 2 * -(-n // piece) + (0 if band else 1)
+        left -= n
     return launches
 
 
@@ -558,7 +577,7 @@ def run_midsize(args, ising, local):
                 if name == "cluster":
                     total_updates += L * L * sweeps
                     total_s += dt
-                    launches += cluster_launches(L, sweeps, 10)
+                    launches += midsize_launches(L, sweeps, 10)
             entry["cluster_over_graphs"] = entry["cluster"] / entry["graphs"]
             entry["bit_exact_across_paths"] = bool(np.array_equal(series["cluster"][0], series["graphs"][0]) and
                                                    np.array_equal(series["cluster"][1], series["graphs"][1]))
@@ -665,16 +684,17 @@ def integer_peaks(ising, clocks_summary: dict) -> dict:
     return dict(probe, sm_max_mhz=float(mhz), clock_source=src)
 
 
-def two_pipe_roofline(achieved_sites_per_ns: float, rng: int, peaks: dict) -> dict:
+def two_pipe_roofline(achieved_sites_per_ns: float, rng: int, peaks: dict, mul: float | None = None) -> dict:
     """The two-pipe integer bound, beside the strict multiply-only one: the
     integer work per site over both pipes it can use.  Per site,
-    FMA-heavy only: the Philox multiplies, 2 issue slots each (4 per site;
-    2.5 with 7 rounds); ALU only: the Philox three-input XORs (4.5; 3 with
+    FMA-heavy only: the Philox multiplies, 2 issue slots each (`mul` per
+    site, else 4; 2.5 with 7 rounds); ALU only: the Philox three-input XORs (4.5; 3 with
     7 rounds), the two threshold compares and the word logic (1.1, per
     site of a 21-field word); either pipe: the two accept-bit inserts.  With
     the inserts split to balance, each pipe (64 lanes / clock / SM) carries
     half of the total."""
-    mul = MULWIDE_PER_SITE if rng == 10 else 2.5
+    if mul is None:
+        mul = MULWIDE_PER_SITE if rng == 10 else 2.5
     xors = 4.5 if rng == 10 else 3.0
     # issue slots in units of one 32-bit multiply-add (the FMA-heavy pipe's
     # lane rate); a 32x32->64 product takes mad32 / mulwide of them
@@ -772,7 +792,7 @@ def main():
 
     # roofline of the half-sweep kernel: the 32x32->64 multiplies of Philox4x32-10
     sites_per_launch = L * L // 2
-    mul_per_site = MULWIDE_PER_SITE if args.rng == 10 else 2.5
+    mul_per_site = MULWIDE_SHARED if args.rng == 10 else 2.25
     achieved_mul = sites_per_launch * mul_per_site / half_sweep_s / 1e12
     cs = clocks.summary()
     peaks = integer_peaks(ising, cs)
@@ -849,10 +869,11 @@ def main():
                          "peak_basis": (f"{peaks['sm_count']} SMs x {peaks['mulwide_per_sm_clk']:.1f} "
                                         "mul.wide.u32 per SM per clock (measured, ising_probe_int_pipes) x "
                                         f"{peaks['sm_max_mhz']:.0f} MHz ({peaks['clock_source']}); "
-                                        f"{mul_per_site} per site (16 per Philox4x32-10 call after hoisting, "
-                                        "4 sites per call)"),
+                                        f"{mul_per_site} per site (15 per Philox4x32-10 call after hoisting and "
+                                        "sharing, 4 sites per call)"),
                          "int_pipes": peaks,
-                         "two_pipe": two_pipe_roofline(sites_per_launch / half_sweep_s / 1e9, args.rng, peaks),
+                         "two_pipe": two_pipe_roofline(sites_per_launch / half_sweep_s / 1e9, args.rng, peaks,
+                                                       mul_per_site),
                          "hbm_achieved_gbs": hbm_bytes_per_launch / half_sweep_s / 1e9,
                          "hbm_peak_gbs": hbm_peak,
                          "hbm_frac": hbm_bytes_per_launch / half_sweep_s / 1e9 / hbm_peak},

@@ -129,10 +129,14 @@ int ising_get_thresholds(ising_lattice *h, uint64_t host_thr[2]);
 /* Run n >= 0 full sweeps t+1 .. t+n (t += n).  A sweep is the paper's Monte
  * Carlo iteration (Sec. 2: every spin proposed once), in checkerboard order:
  * all colour-0 sites, then all colour-1 sites.  Asynchronous on the stream
- * (the first call on the on-chip path allocates its mask buffer), except on the cluster path with several clusters, where the
- * call synchronises the stream to read the status of the waits between
- * clusters.  Errors: EINVAL (NULL, n < 0), ENOMEM (that buffer), ETIMEOUT
- * (a wait between clusters gave up; see ising_set_clusters), ECUDA. */
+ * (the first call on the on-chip and cluster paths allocates their buffers),
+ * except on the cluster path with several clusters, where the call
+ * synchronises the stream to read the status of the waits between clusters.
+ * Errors: EINVAL (NULL, n < 0), ENOMEM (a buffer), ETIMEOUT (a wait between
+ * clusters gave up; see ising_set_clusters), ECUDA.  A wait inside a cluster or
+ * of the random-word chain that gives up (none should: both wait for threads
+ * that run at the same time) makes the next call that reads results return
+ * ETIMEOUT. */
 int ising_sweep(ising_lattice *h, int64_t n);
 
 /* Run n sweeps and record E and M after sweeps t+every, t+2*every, ...:
@@ -243,41 +247,33 @@ int ising_set_item_lanes(ising_lattice *h, int32_t lanes);
  * ising_set_beta, ising_set_rng, ising_set_tiling, ising_set_item_lanes; a
  * device record index picks the count slots of each replay), because there
  * a half-sweep runs about as long as the host takes to launch it.
- * ISING_PATH_RESIDENT: temporal
- * blocking with the whole lattice on chip -- one block copies both colour
- * arrays into shared memory and runs all requested sweeps there in one
- * launch (lattices with 2 L pitch 8 bytes <= 220 KB, i.e. L up to about
- * 740; larger -> EINVAL); it removes the per-sweep launch latency that
- * bounds small lattices.  Up to 512 thread items (ceil(L/4) * ceil(L/42),
- * L <= 292) the accept masks of the requested sweeps are first drawn by all
- * SMs into a device buffer the library allocates on first use (up to
- * 16 MB), and the on-chip block only applies them, one or two rows per
- * thread.
+ * ISING_PATH_RESIDENT: temporal blocking with the whole lattice on chip, all
+ * requested sweeps in one launch (lattices with 2 L pitch 8 bytes <= 220 KB,
+ * i.e. L up to about 740; larger -> EINVAL); it removes the per-sweep launch
+ * latency that bounds small lattices.  The accept masks of the requested sweeps
+ * are first drawn by all SMs into a device buffer the library allocates on first
+ * use (up to 16 MB).  Up to L = 128 one warp keeps the lattice in registers; up
+ * to 512 thread items (ceil(L/4) * ceil(L/42), L <= 292) one block keeps it in
+ * shared memory, one or two rows per thread; above, that block also draws.
  * ISING_PATH_CLUSTER: temporal blocking on one thread-block cluster (16
- * blocks where the device runs such a cluster, else 8).  Row-packed
- * lattices with at least two rows per block whose window fits a block's
- * shared memory (L from 32 up to 1600): block b keeps rows b L / C ..
- * (b + 1) L / C - 1 of both colours in shared memory for a piece of up to
- * 256 sweeps.  Column-interleaved lattices (L from 84 up to 1512): block b
- * keeps a band of word columns (multiples of 4) of all N word rows.
- * Otherwise EINVAL, and EINVAL on a device without clusters.  After every
- * k <= 12 half-sweeps each block writes its first and last k own rows (or
- * columns) into its neighbours' shared memory (distributed shared memory)
- * and the blocks pass a cluster barrier; then they run k half-sweeps on
- * their own rows plus halo.  The accept masks of each
- * piece are drawn by the SMs the cluster leaves free, while the piece before
- * is applied, into two device buffers the library allocates on first use (up
- * to 256 MB together; 2 L pitch 8 bytes per sweep).  No spin-waits: only the
- * hardware's block and cluster barriers.
+ * blocks where the device runs such a cluster, else 8): row-packed lattices
+ * with at least two rows per block, L from 32 up to 1600, column-interleaved
+ * ones from 84 up to 1512.  Otherwise EINVAL, and EINVAL on a device without
+ * clusters.  Block b keeps rows b L / C .. (b + 1) L / C - 1 on chip for a piece
+ * of up to 256 sweeps, one bit per spin (a column-interleaved lattice is
+ * converted for the call), and runs k half-sweeps on them and k halo rows on
+ * either side between two exchanges with its neighbours through distributed
+ * shared memory.  The accept masks of each piece are drawn by the SMs the
+ * cluster leaves free, while the piece before is applied, into two device
+ * buffers the library allocates on first use (up to 256 MB together).
  * Both layouts may run several clusters per launch (see
- * ising_set_clusters), which takes the path past the sizes one cluster's
- * shared memory holds.
+ * ising_set_clusters), which takes the path past the sizes of one cluster.
  * ISING_PATH_AUTO (default), row-packed: resident up to 128 thread items
- * (L <= 128), the cluster path above that up to L = 3000 (one cluster up to
- * L = 558, then 3 to 6 by size), the launch path above that (on a device
- * without clusters: resident up to 512 items, L <= 292, then the launch
- * path); column-interleaved: the cluster path up to L = 2604 (one cluster up
- * to L = 840, then 3 to 5), the launch path above.
+ * (L <= 128), the cluster path above that up to L = 3000, the launch path above
+ * that (on a device without clusters: resident up to 512 items, L <= 292, then
+ * the launch path); column-interleaved: the cluster path up to L = 2604, the
+ * launch path above.  Clusters by size: one up to L = 1150, two to 1600, three
+ * to 2400, then four.
  * Results are identical on every path. */
 #define ISING_PATH_AUTO 0
 #define ISING_PATH_LAUNCHES 1
@@ -295,7 +291,7 @@ int ising_get_path(ising_lattice *h, int32_t *path);
  * consecutive row bands.  Inside a cluster the halo rows travel through
  * distributed shared memory; between clusters the two boundary blocks pass
  * them through a small device buffer the library allocates on first use
- * (clusters x 8 k pitch 8 bytes, k <= 12) with release/acquire flags.  A
+ * (8 k rows of one bit per spin per cluster) with release/acquire flags.  A
  * flag wait gives up after one second of the GPU's clock.  A launch with
  * several clusters writes its lattice rows back only if all its blocks were
  * resident together, which all its blocks agree on at their end.  If they
@@ -307,9 +303,8 @@ int ising_get_path(ising_lattice *h, int32_t *path);
  * are void, and the sweep counter has advanced (restore a checkpoint with
  * ising_set_words, or ising_set_spins in the column-interleaved layout, and
  * ising_set_sweep to retry).  A number of clusters the device cannot hold at
- * once, or for which the lattice has no window plan, gives EINVAL.
- * Column-interleaved lattices split their word columns the same way (k halo
- * columns of all word rows between clusters).  Results do not depend on it. */
+ * once, or for which the lattice's side is out of range, gives EINVAL.
+ * Results do not depend on it. */
 int ising_set_clusters(ising_lattice *h, int32_t clusters);
 
 /* Test hook of that wait: the next `launches` cluster-path launches with

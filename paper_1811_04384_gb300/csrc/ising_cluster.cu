@@ -1,5 +1,6 @@
-// Cluster-resident temporal blocking for mid-size lattices (above the
-// one-SM on-chip range, L of about 130 to 3000).
+// Cluster-resident temporal blocking for mid-size lattices (above the on-chip
+// range, L of about 130 to 3000): rows of more than 14 dense words, and several
+// clusters; one cluster on shorter rows is ising_band.cu's.
 //
 // There a half-sweep is short: a launch per half-sweep costs more than its
 // work.  Here one launch of G thread-block clusters (of 16 blocks where the
@@ -34,9 +35,10 @@
 // What bounds it: with 3-bit fields in the window the update itself did (101
 // warp instructions per warp and half-sweep for 32 x 21 sites, on 16 to 96
 // SMs), and more clusters left fewer SMs for the draws.  Dense words take
-// about a tenth of the instructions per site, so from L of about 700 the draws
-// on the other SMs bound the path, and below the latency of a half-sweep
-// (shared-memory round trip and block barrier).
+// about a tenth of the instructions per site, so from L of about 1100 the draws
+// on the other SMs bound the path, and below that the latency of a half-sweep
+// (mask wait, block barrier, shared-memory round trip) does as well: about 1,050 cycles
+// at L = 1008.
 //
 // A wait between clusters that gives up (see cl_wait_flag in
 // ising_cluster.cuh) lets the launch end with void results, and the host

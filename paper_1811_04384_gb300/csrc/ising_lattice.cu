@@ -26,12 +26,10 @@ constexpr size_t kHostWords = 64;                // words the kernels report to,
 constexpr size_t kCountBytes = (size_t)kRecordsPerChunk * kCountSlots * 2 * sizeof(unsigned long long);
 constexpr size_t kAlign = 256;
 constexpr size_t kResidentMaxBytes = 220 * 1024;   // shared memory for the on-chip path
-// auto: on-chip up to 128 thread items (L <= 128), the cluster path above;
-// on a device without thread-block clusters on-chip up to 512 items (L <= 292).
-// Measured on GB300 (sweeps without records / a record after every sweep,
-// spin-updates/ns, on-chip against cluster): L = 100: 16.8 / 12.8 against
-// 16.5 / 9.9; L = 128: 25.8 / 17.7 against 30.6 / 17.2; L = 168: 34.4 / 23.8
-// against 55.8 / 31.0; L = 256: 27.8 / 22.8 against 102 / 59.
+// auto: on-chip up to 128 thread items (L <= 128, one warp), the cluster path
+// above; on a device without thread-block clusters on-chip up to 512 items (L <=
+// 292).  Measured on GB300: a sweep takes 193 ns at L = 128 in one warp, and 260 at
+// L = 130 on a cluster.
 constexpr int kResidentAutoMaxItems = 128;
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
@@ -623,7 +621,7 @@ constexpr int kXStatusWords = kXWords - kXErr;
 
 // Clusters of a launch on the automatic path for side L (0: not the cluster
 // path).  Measured on GB300, a record every 10 sweeps, us per call by clusters
-// 1 / 2 / 3 / 4: L = 700 (1000 sweeps): 872 / 1,125 / 1,088 / 1,101; L = 1008 (500):
+// 1 / 2 / 3 / 4: L = 700 (1000 sweeps): 778 (band_sweeps_kernel) / 1,125 / 1,088 / 1,101; L = 1008 (500):
 // 570 / 661 / 643 / 671; L = 1300 (500): 883 / 804 / 830 / 850; L = 1500 (400): 814 /
 // 768 / 767 / 795; L = 1700 (400): - / 991 / 951 / 955; L = 2016 (300): - / 955 / 946 /
 // 939; L = 2600 (200): - / - / 1,043 / 1,028; L = 3000: four only.

@@ -7,7 +7,12 @@
 // the index arithmetic of a packed word per half-sweep: 0.42 us per recorded
 // sweep at L = 64, 0.92 at L = 128.  In one warp a half-sweep is two shuffles
 // (the rows above and below a lane's own), seven three-input operations per 32
-// sites and no barrier.
+// sites and no barrier.  Measured on GB300: a sweep without a record 69 ns at L
+// = 64 and 193 at L = 128 (there the warp's issue slots bind), 1000 recorded
+// sweeps of L = 64 in 84 us, against 418 in shared memory, 271 with one warp that
+// also copied the masks and counted the records, 159 with three helpers that did
+// both, and 218 ns a sweep at L = 128 with the copying warp on the sweeping warp's
+// scheduler.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -122,8 +127,8 @@ struct WarpLattice {
 };
 
 // Sweeps s_base + 1 .. s_base + n of a run with the masks of
-// dense_mask_draw_kernel in the warp_mask_layout form: `rows` of 16 bytes per
-// lane, 2 C of them a sweep.  Warp 0 sweeps; warp kCopier copies the masks
+// dense_mask_draw_kernel as launch_warp_mask_draw lays them out: rows of 16
+// bytes per lane, 2 C of them a sweep.  Warp 0 sweeps; warp kCopier copies the masks
 // into a ring of STAGES stages of K sweeps, and the other warps (on the other
 // schedulers) count the records, (E, M) of the run's sweeps s with s % every == 0 to
 // records[2 (s / every - 1)], from the states that warp 0 leaves in shared
