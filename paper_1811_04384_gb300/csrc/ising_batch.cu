@@ -23,6 +23,11 @@ namespace {
 
 constexpr size_t kAlign = 256;
 constexpr int kMaxLanes = 8;
+// Sweeps of the short graph that runs what is left of a call after whole
+// chunks.  A chunk's launches past the call's last sweep end at once, but each
+// still takes its 1.2 us or so: 20 sweeps of 64 replicas of L = 32 to 128 took 229
+// us in a chunk of 50 and 190 in two of 10, 256 of L = 32 to 512 614 and 534.
+constexpr int kRestChunk = 10;
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 }  // namespace
@@ -55,12 +60,14 @@ struct ising_batch {
     int8_t* staging = nullptr;
     size_t staging_cap = 0;
     cudaStream_t stream = nullptr;
-    cudaGraphExec_t graph = nullptr;        // captured chunk of sweeps
-    int graph_chunk = 0;
-    int graph_threads = 0;
-    int graph_lanes = 0;
-    int graph_rounds = 0;                   // Philox rounds the graph's kernels are fixed for
-    bool graph_every1 = false;              // colour-1 kernels record every sweep
+    // a captured chunk of sweeps, and what its kernels are fixed for
+    struct Graph {
+        cudaGraphExec_t exec = nullptr;
+        int chunk = 0, threads = 0, lanes = 0;
+        int rounds = 0;                     // Philox rounds
+        bool every1 = false;                // colour-1 kernels record every sweep
+    };
+    Graph graph, rest;                      // of `chunk` sweeps, of kRestChunk
 };
 
 namespace {
@@ -69,7 +76,8 @@ void free_batch(ising_batch* b)
 {
     if (!b) return;
     if (b->stream) cudaStreamSynchronize(b->stream);
-    if (b->graph) cudaGraphExecDestroy(b->graph);
+    for (ising_batch::Graph* g : {&b->graph, &b->rest})
+        if (g->exec) cudaGraphExecDestroy(g->exec);
     cudaFree(b->arena);
     cudaFree(b->d_reps);
     cudaFree(b->d_tiles);
@@ -111,6 +119,10 @@ int build_tiles(ising_batch* b)
             add_tiles(tiles, r, b->geom[r], b->threads);
         }
         b->lane_ntiles[k] = (int)tiles.size() - b->lane_tile0[k];
+    }
+    for (ising_batch::Graph* g : {&b->graph, &b->rest}) {      // they hold the old table's address
+        if (g->exec) cudaGraphExecDestroy(g->exec);
+        g->exec = nullptr;
     }
     if (b->d_tiles) cudaFree(b->d_tiles);
     b->d_tiles = nullptr;
@@ -157,18 +169,16 @@ void launch_batch_pair(int rounds, bool every1, dim3 grid, dim3 block, cudaStrea
     else launch_batch_pair_r<10>(every1, grid, block, st, reps, tiles, chunk_base, s);
 }
 
-// One chunk of sweeps as a graph: lane 0 on the batch's stream, lanes
+// A chunk of sweeps as a graph: lane 0 on the batch's stream, lanes
 // 1.. forked from it and joined back before the chunk counter advances.
 // The kernels are fixed for the batch's Philox rounds and for records every
 // sweep, so the graph is recaptured when either changes.
-int capture_graph(ising_batch* b, int rounds, bool every1)
+int capture_graph(ising_batch* b, ising_batch::Graph& g, int chunk, int rounds, bool every1)
 {
-    if (b->graph && b->graph_chunk == b->chunk && b->graph_threads == b->threads && b->graph_lanes == b->lanes &&
-        b->graph_rounds == rounds && b->graph_every1 == every1)
+    if (g.exec && g.chunk == chunk && g.threads == b->threads && g.lanes == b->lanes && g.rounds == rounds &&
+        g.every1 == every1)
         return ISING_OK;
-    b->graph_rounds = rounds;
-    b->graph_every1 = every1;
-    if (b->graph) { cudaGraphExecDestroy(b->graph); b->graph = nullptr; }
+    if (g.exec) { cudaGraphExecDestroy(g.exec); g.exec = nullptr; }
     int rc = ensure_lane_streams(b);
     if (rc != ISING_OK) return rc;
     cudaStream_t st[kMaxLanes];
@@ -179,12 +189,12 @@ int capture_graph(ising_batch* b, int rounds, bool every1)
     cudaError_t le = cudaEventRecord(b->fork, b->stream);
     for (int k = 1; k < b->lanes && le == cudaSuccess; ++k)
         if (b->lane_ntiles[k] > 0) le = cudaStreamWaitEvent(st[k], b->fork, 0);
-    for (int s = 1; s <= b->chunk && le == cudaSuccess; ++s) {
+    for (int s = 1; s <= chunk && le == cudaSuccess; ++s) {
         for (int k = 0; k < b->lanes && le == cudaSuccess; ++k) {
             const int nt = b->lane_ntiles[k];
             if (nt == 0) continue;
             const BatchTile* tiles = b->d_tiles + b->lane_tile0[k];
-            launch_batch_pair(b->graph_rounds, b->graph_every1, dim3(nt), dim3(b->threads), st[k], b->d_reps, tiles,
+            launch_batch_pair(rounds, every1, dim3(nt), dim3(b->threads), st[k], b->d_reps, tiles,
                               b->d_chunk_base, (uint32_t)s);
             le = cudaGetLastError();
         }
@@ -195,18 +205,20 @@ int capture_graph(ising_batch* b, int rounds, bool every1)
         if (le == cudaSuccess) le = cudaStreamWaitEvent(b->stream, b->join[k], 0);
     }
     if (le == cudaSuccess) {
-        batch_advance_kernel<<<1, 1, 0, b->stream>>>(b->d_chunk_base, (uint32_t)b->chunk);
+        batch_advance_kernel<<<1, 1, 0, b->stream>>>(b->d_chunk_base, (uint32_t)chunk);
         le = cudaGetLastError();
     }
     e = cudaStreamEndCapture(b->stream, &graph);
     if (le != cudaSuccess) { if (graph) cudaGraphDestroy(graph); return cuda_fail(le, "batch capture launch"); }
     if (e != cudaSuccess) return cuda_fail(e, "cudaStreamEndCapture");
-    e = cudaGraphInstantiate(&b->graph, graph, 0);
+    e = cudaGraphInstantiate(&g.exec, graph, 0);
     cudaGraphDestroy(graph);
-    if (e != cudaSuccess) { b->graph = nullptr; return cuda_fail(e, "cudaGraphInstantiate"); }
-    b->graph_chunk = b->chunk;
-    b->graph_threads = b->threads;
-    b->graph_lanes = b->lanes;
+    if (e != cudaSuccess) { g.exec = nullptr; return cuda_fail(e, "cudaGraphInstantiate"); }
+    g.chunk = chunk;
+    g.threads = b->threads;
+    g.lanes = b->lanes;
+    g.rounds = rounds;
+    g.every1 = every1;
     return ISING_OK;
 }
 
@@ -360,11 +372,23 @@ extern "C" int ising_batch_sweep(ising_batch* b, const int64_t* sweeps, int64_t 
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync counts");
     e = cudaMemsetAsync(b->d_chunk_base, 0, sizeof(uint32_t), b->stream);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync chunk");
-    int rc = capture_graph(b, b->h_reps[0].rounds == 7 ? 7 : 10, every == 1);
-    if (rc != ISING_OK) return rc;
-    const int64_t nlaunch = (max_s + b->chunk - 1) / b->chunk;
-    for (int64_t k = 0; k < nlaunch; ++k) {
-        e = cudaGraphLaunch(b->graph, b->stream);
+    // whole chunks, then the rest in short ones unless those would come to a chunk
+    int64_t chunks = max_s / b->chunk, rests = (max_s % b->chunk + kRestChunk - 1) / kRestChunk;
+    if (rests * kRestChunk >= b->chunk) {
+        chunks += 1;
+        rests = 0;
+    }
+    const int rounds = b->h_reps[0].rounds == 7 ? 7 : 10;
+    if (chunks > 0) {
+        int rc = capture_graph(b, b->graph, b->chunk, rounds, every == 1);
+        if (rc != ISING_OK) return rc;
+    }
+    if (rests > 0) {
+        int rc = capture_graph(b, b->rest, kRestChunk, rounds, every == 1);
+        if (rc != ISING_OK) return rc;
+    }
+    for (int64_t k = 0; k < chunks + rests; ++k) {
+        e = cudaGraphLaunch(k < chunks ? b->graph.exec : b->rest.exec, b->stream);
         if (e != cudaSuccess) return cuda_fail(e, "cudaGraphLaunch");
     }
     e = cudaMemcpyAsync(b->h_counts, b->d_counts, need * sizeof(unsigned long long), cudaMemcpyDeviceToHost,
