@@ -66,8 +66,10 @@ constexpr int kClThreads = 1024;           // most threads of a block
 // 641; L = 1008 (500 sweeps): 666 / 640 / 615 / 615; but L = 1700 (400 sweeps, two
 // clusters) 12 / 18: 991 / 1023; L = 2600 (200, four): 1,028 / 1,042.
 constexpr int kClHalo = 18, kClHaloWide = 12, kClWideWords = 21;   // 12 from rows of more than 21 words (L > 1344)
-// Up to this many window words: one word per unit (L = 512: 688 us against 846
-// with two, L = 700, above it: 872 with two against 982).
+// Up to this many window words: one word per unit (one cluster, before short
+// rows had their own form: L = 512 688 us against 846 with two, L = 700, above it:
+// 872 with two against 982).  Since then: small windows of several clusters, and
+// L <= 128 on this path.
 constexpr long long kClOneWord = 512;
 
 struct ClusterArgs {
