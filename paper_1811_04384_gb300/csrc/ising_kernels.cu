@@ -13,6 +13,7 @@
 #include <type_traits>
 
 #include "../../include/ising.h"
+#include "ising_dense.cuh"
 #include "ising_device.cuh"
 #include "ising_internal.h"
 
@@ -77,23 +78,79 @@ __global__ void init_cold_kernel(uint64_t* __restrict__ w0, uint64_t* __restrict
     w1[(size_t)i * g.P + w] = v;
 }
 
-// int8 spins of row blockIdx.x (> 0 is up) -> that row's words of both
-// colours.  The row is first staged in shared memory (16-byte loads when
-// vec16: `in` 16-byte aligned and L % 16 == 0), so the input is read once
-// and coalesced; `in` may be device memory or pinned host memory mapped into
-// the device's address space.  Dynamic shared memory: L bytes.
-__global__ void pack_rows_kernel(uint64_t* __restrict__ w0, uint64_t* __restrict__ w1, Geom g,
-                                 const int8_t* __restrict__ in, int vec16)
+// Four spins (bytes of v, > 0 is up) as four bits.
+__device__ __forceinline__ uint32_t spin_nibble(uint32_t v)
 {
-    extern __shared__ __align__(16) int8_t row_s[];
+    const uint32_t g = ((v & 0x7f7f7f7fu) + 0x7f7f7f7fu) & ~v & 0x80808080u;    // bit 7 of a byte: > 0
+    return (g * 0x00204081u) >> 28;
+}
+
+// Bits 0 and 2 of the bytes of v as eight bits.
+__device__ __forceinline__ uint32_t even_bits(uint32_t v)
+{
+    const uint32_t p = (v & 0x01010101u) | (v >> 1 & 0x02020202u);
+    return (p | p >> 6 | p >> 12 | p >> 18) & 0xffu;
+}
+
+// int8 spins of row blockIdx.x (> 0 is up) -> that row's words of both colours;
+// `in` may be device memory or pinned host memory mapped into the device's
+// address space.  In three steps through shared memory: four spins to a byte
+// of four bits (16 bytes a load when the rows are 16-byte aligned, else 4 with a
+// shift by the row's offset, or single bytes when `in` itself is not 4-byte
+// aligned), those to dense bits of the two colours, and 21 of those to a word.
+// Gathering each word's 21 bytes from a staged row took 14.4 us at L = 4096 and
+// 49 at L = 5000, where the rows were staged byte by byte: 10.6 and 18.5 so.
+// Launches that wait (pdl_wait) may start beside it.
+// Dynamic shared memory: pack_smem(L) bytes.
+constexpr int kPackAlign16 = 2, kPackAlign4 = 1;      // `aligned`: else 0
+__host__ __device__ inline uint32_t pack_nibbles(int L) { return (uint32_t)(L / 4 + 1 + 15) / 16 * 16; }
+__host__ __device__ inline uint32_t pack_dense(int L) { return (uint32_t)(L / 64 + 3); }   // words of a colour
+inline size_t pack_smem(int L) { return pack_nibbles(L) + 8 * (size_t)pack_dense(L); }
+
+__global__ void pack_rows_kernel(uint64_t* __restrict__ w0, uint64_t* __restrict__ w1, Geom g,
+                                 const int8_t* __restrict__ in, int aligned)
+{
+    extern __shared__ __align__(16) uint8_t nibbles[];
+    pdl_launch();
+    const uint32_t nn = pack_nibbles(g.L), nd = pack_dense(g.L);
+    uint32_t* const dense = reinterpret_cast<uint32_t*>(nibbles + nn);      // [parity of j][nd]
     const int i = blockIdx.x;
     const int8_t* src = in + (size_t)i * g.L;
-    if (vec16) {
+    if (aligned == kPackAlign16) {
         const uint4* s4 = reinterpret_cast<const uint4*>(src);
-        uint4* d4 = reinterpret_cast<uint4*>(row_s);
-        for (int k = threadIdx.x; k < g.L / 16; k += blockDim.x) d4[k] = s4[k];
+        uint32_t* n4 = reinterpret_cast<uint32_t*>(nibbles);
+        for (int k = threadIdx.x; k < g.L / 16; k += blockDim.x) {
+            const uint4 v = s4[k];
+            n4[k] = spin_nibble(v.x) | spin_nibble(v.y) << 8 | spin_nibble(v.z) << 16 | spin_nibble(v.w) << 24;
+        }
+    } else if (aligned == kPackAlign4) {
+        // rows begin at offset 0 or 2 of a 4-byte word
+        const uint32_t* s1 = reinterpret_cast<const uint32_t*>(reinterpret_cast<uintptr_t>(src) & ~(uintptr_t)3);
+        const uint32_t* const end = reinterpret_cast<const uint32_t*>(in + (size_t)g.L * g.L);
+        const bool half = (reinterpret_cast<uintptr_t>(src) & 2) != 0;
+        for (int k = threadIdx.x; 4 * k < g.L; k += blockDim.x) {
+            uint32_t v = s1[k];
+            if (half) v = __funnelshift_r(v, s1 + k + 1 < end ? s1[k + 1] : 0u, 16);
+            nibbles[k] = (uint8_t)spin_nibble(v);
+        }
     } else {
-        for (int k = threadIdx.x; k < g.L; k += blockDim.x) row_s[k] = src[k];
+        for (int k = threadIdx.x; 4 * k < g.L; k += blockDim.x) {
+            uint32_t v = 0;
+            for (int e = 0; e < 4 && 4 * k + e < g.L; ++e) v |= (uint32_t)(uint8_t)src[4 * k + e] << (8 * e);
+            nibbles[k] = (uint8_t)spin_nibble(v);
+        }
+    }
+    __syncthreads();
+    // 64 spins to 32 bits of either parity of j; what lies past the row is cut off below
+    for (uint32_t k = threadIdx.x; k < nd; k += blockDim.x) {
+        uint32_t e = 0, o = 0;
+        if (16 * k < nn) {
+            const uint4 v = reinterpret_cast<const uint4*>(nibbles)[k];
+            e = even_bits(v.x) | even_bits(v.y) << 8 | even_bits(v.z) << 16 | even_bits(v.w) << 24;
+            o = even_bits(v.x >> 1) | even_bits(v.y >> 1) << 8 | even_bits(v.z >> 1) << 16 | even_bits(v.w >> 1) << 24;
+        }
+        dense[k] = e;
+        dense[nd + k] = o;
     }
     __syncthreads();
     for (int t = threadIdx.x; t < 2 * g.P; t += blockDim.x) {
@@ -101,10 +158,9 @@ __global__ void pack_rows_kernel(uint64_t* __restrict__ w0, uint64_t* __restrict
         const int w = t - c * g.P;
         uint64_t word = 0;
         if (w < g.W) {
-            const int nf = (w == g.W - 1) ? g.rlast : kFields;
-            const int par = (i + c) & 1;
-            const int8_t* r = row_s + 2 * w * kFields + par;
-            for (int k = 0; k < nf; ++k) word |= (uint64_t)(r[2 * k] > 0) << (3 * k);
+            const uint32_t* d = dense + ((i + c) & 1) * nd + (kFields * w >> 5);
+            const uint32_t bits = __funnelshift_r(d[0], d[1], (kFields * w) & 31);
+            word = spread_fields(w == g.W - 1 ? bits & ((1u << g.rlast) - 1u) : bits);
         }
         (c ? w1 : w0)[(size_t)i * g.P + w] = word;
     }
@@ -539,8 +595,10 @@ namespace ising {
 
 cudaError_t launch_pack_rows(uint64_t* w0, uint64_t* w1, const Geom& g, const int8_t* src, cudaStream_t s)
 {
-    const int vec16 = ((uintptr_t)src % 16 == 0) && (g.L % 16 == 0);
-    pack_rows_kernel<<<g.L, 256, g.L, s>>>(w0, w1, g, src, vec16);
+    const int aligned = (uintptr_t)src % 16 == 0 && g.L % 16 == 0 ? kPackAlign16
+                        : (uintptr_t)src % 4 == 0                 ? kPackAlign4
+                                                                  : 0;
+    pack_rows_kernel<<<g.L, 256, pack_smem(g.L), s>>>(w0, w1, g, src, aligned);
     return cudaGetLastError();
 }
 

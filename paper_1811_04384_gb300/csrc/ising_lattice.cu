@@ -432,9 +432,13 @@ static int replay_plain(ising_lattice* h, int64_t* n)
 // rec_of(s) >= 0.  Then advances the counter by n.  The launches take the
 // sweep counter from the host, so that their draws need no device memory;
 // where the stream is being captured they read the device's, which a replay
-// advances.
-template <typename RecOf>
-static int run_sweeps(ising_lattice* h, int64_t n, RecOf rec_of)
+// advances.  after_first() comes after the first launch.  With `owed` the
+// device counter may stay behind, by the sweeps added to *owed.
+struct NoHook {
+    cudaError_t operator()() const { return cudaSuccess; }
+};
+template <typename RecOf, typename First = NoHook>
+static int run_sweeps(ising_lattice* h, int64_t n, RecOf rec_of, First after_first = First(), int64_t* owed = nullptr)
 {
     SweepArgs a = base_args(h);
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -449,13 +453,17 @@ static int run_sweeps(ising_lattice* h, int64_t n, RecOf rec_of)
     for (int64_t s = 1; s <= n; ++s) {
         a.t_off = (uint32_t)s;
         cudaError_t e = launch_hs(h, h->stream, false, 0, true, false, a);
+        if (e == cudaSuccess && s == 1) e = after_first();
         if (e != cudaSuccess) return cuda_fail(e, "half_sweep colour 0");
         const int rec = rec_of(s);
         a.counts = rec >= 0 ? h->counts + (size_t)rec * kCountSlots * 2 : nullptr;
         e = launch_hs(h, h->stream, false, 1, true, rec >= 0, a);
         if (e != cudaSuccess) return cuda_fail(e, "half_sweep colour 1");
     }
-    if (n > 0) {
+    if (owed && !a.t_base) {
+        *owed += n;
+        h->t += (uint64_t)n;
+    } else if (n > 0) {
         cudaError_t e = launch_advance_sweep(h->t_dev, (uint64_t)n, h->stream);
         if (e != cudaSuccess) return cuda_fail(e, "advance_sweep_kernel");
         h->t += (uint64_t)n;
@@ -1216,11 +1224,12 @@ extern "C" int ising_run_states(ising_lattice* h, const int8_t* const* states, i
     const int64_t group = R > 0 ? std::max<int64_t>(1, kRecordsPerChunk / R) : (int64_t)nstates;
     for (int64_t k0 = 0; k0 < nstates; k0 += group) {
         const int64_t k1 = std::min<int64_t>(nstates, k0 + group);
+        int64_t owed = 0;                                      // sweeps by which the device counter lags
         cudaError_t e = cudaSuccess;
         if (R > 0)
             e = cudaMemsetAsync(h->counts, 0, (size_t)(k1 - k0) * R * rec_words * sizeof(unsigned long long),
                                 h->stream);
-        for (int64_t k = k0; k < k1 && e == cudaSuccess; ++k) {
+        for (int64_t k = k0; k < k1 && e == cudaSuccess && rc == ISING_OK; ++k) {
             const int b = (int)(k & 1);
             // state k -> input buffer b, once the pack that last read buffer b is done;
             // this copy runs while the sweeps of state k - 1 are on the device
@@ -1230,18 +1239,29 @@ extern "C" int ising_run_states(ising_lattice* h, const int8_t* const* states, i
             if (e == cudaSuccess) e = cudaStreamWaitEvent(h->stream, h->ev_copied[b], 0);
             if (e != cudaSuccess) break;
             e = launch_pack_rows(h->words[0], h->words[1], g, stage[b], h->stream);
-            if (e == cudaSuccess) e = cudaEventRecord(h->ev_packed[b], h->stream);
             if (e != cudaSuccess) break;
             const int64_t base = (k - k0) * R;
+            const auto packed = [h, b] { return cudaEventRecord(h->ev_packed[b], h->stream); };
             ClusterPlan cp;
-            if (use_cluster(h, &cp))
+            if (use_cluster(h, &cp)) {
+                e = packed();
+                if (e != cudaSuccess) break;
                 rc = run_cluster(h, sweeps, every, h->counts + (size_t)base * rec_words, cp);
-            else
+            } else if (sweeps == 0) {
+                e = packed();
+            } else {
+                // the event is recorded after the first half-sweep, so that it does not
+                // come between that launch and the pack kernel it starts beside
                 rc = run_sweeps(h, sweeps, [every, base](int64_t s) {
                     return (s % every == 0) ? (int)(base + s / every - 1) : -1;
-                });
-            if (rc != ISING_OK) return rc;
+                }, packed, &owed);
+            }
         }
+        if (owed > 0) {
+            const cudaError_t e1 = launch_advance_sweep(h->t_dev, (uint64_t)owed, h->stream);
+            if (e == cudaSuccess) e = e1;
+        }
+        if (rc != ISING_OK) return rc;
         if (e != cudaSuccess) return cuda_fail(e, "run_states");
         if (R > 0) {
             const size_t nrec = (size_t)(k1 - k0) * R;
