@@ -16,9 +16,11 @@
 // count of updates share 64 bits of shared memory, so one load gives both and
 // no barrier or fence is needed.  An update that is the oldest of all pending
 // ones never waits, so the phase always ends.  Measured on GB300, 5 iterations
-// of L = 1008 with 72 strips, a record after each: 798 -> 215 us, of which the
+// of L = 1008 with 72 strips, a record after each: 798 -> 213 us, of which the
 // plans take 54 and a phase 14.  (The plans of later iterations beside the
-// phases, on a second stream: 218.)
+// phases, on a second stream: 218 against 215.)  A phase is bound by latency: 15%
+// fewer instructions a look (the turns at the top and bottom rows in the warps that
+// have them, four looks to a test for the end) gave 1 to 3%.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -35,7 +37,8 @@ namespace {
 constexpr int kPlanWarps = 8;
 constexpr size_t kWordsSmemMax = 220 * 1024;
 constexpr int kWordsThreads = 1024;             // most threads of a strip, one or two words each
-constexpr uint32_t kWordsTries = 1u << 24;      // a thread's looks at its neighbours before it gives up
+constexpr int kWordsLooks = 4;                  // a thread's looks at its neighbours between two tests for the end
+constexpr uint32_t kWordsTries = 1u << 22;      // such rounds of looks before it gives up
 constexpr size_t kWordsPlanBytes = (size_t)64 << 20;
 constexpr int kWordsPlanIterations = 16;
 constexpr uint32_t kWordBits = (1u << 21) - 1;
@@ -271,37 +274,47 @@ words_run_kernel(uint64_t* S, WordsGeom g, int phase, bool fresh, const char* __
         o[k].e = entry_ld(o[k].ahead - 32u);
         o[k].next = entry_ld(o[k].ahead - 16u);
     }
+    // rows whose neighbours come from across the top or bottom row: few warps have any
+    bool edge = false;
+#pragma unroll
+    for (int k = 0; k < WPT; ++k) edge = edge || o[k].first_row || o[k].last_row;
+    edge = __any_sync(0xffffffffu, edge);
     // a word changes by its own thread only, so there is no barrier from here on
+    auto look = [&](OwnWord& w) {
+        const uint64_t up = word_look(w.up), dn = word_look(w.dn), lf = word_look(w.at - 8), rt = word_look(w.at + 8);
+        // the counts are below 2^16: at most 20,480 updates of a half strip
+        const uint32_t z = (uint32_t)(up >> 32) | (uint32_t)(dn >> 32) << 16;
+        const uint32_t v = (uint32_t)(lf >> 32) | (uint32_t)(rt >> 32) << 16;
+        const bool ready = w.done < w.count && z == w.e.z && v == w.e.w;
+        // straight-line: the lanes of a warp are seldom ready together
+        uint32_t u = (uint32_t)up, d = (uint32_t)dn;
+        if (edge) {
+            u = w.first_row ? (u << 1 | u >> 20) & kWordBits : u;
+            d = w.last_row ? (d >> 1 | d << 20) & kWordBits : d;
+        }
+        const uint32_t spins = flip_all(w.spins, u, d, (uint32_t)lf, (uint32_t)rt, w.e.x, w.e.y);
+        w.spins = ready ? spins : w.spins;
+        w.done += ready;
+        w.ahead += ready ? 16u : 0u;
+        w.e.x = ready ? w.next.x : w.e.x;
+        w.e.y = ready ? w.next.y : w.e.y;
+        w.e.z = ready ? w.next.z : w.e.z;
+        w.e.w = ready ? w.next.w : w.e.w;
+        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %4, 0;\n\t"
+                     "@p st.volatile.shared.u64 [%5], %6;\n\t"
+                     "@p ld.shared.v4.u32 {%0, %1, %2, %3}, [%7];\n\t}"
+                     : "+r"(w.next.x), "+r"(w.next.y), "+r"(w.next.z), "+r"(w.next.w)
+                     : "r"((uint32_t)ready), "r"(w.at), "l"((uint64_t)w.done << 32 | w.spins), "r"(w.ahead - 16u)
+                     : "memory");
+    };
     for (uint32_t tries = 0;; ++tries) {
         bool pending = false;
 #pragma unroll
-        for (int k = 0; k < WPT; ++k) {
-            OwnWord& w = o[k];
-            const uint64_t up = word_look(w.up), dn = word_look(w.dn), lf = word_look(w.at - 8), rt = word_look(w.at + 8);
-            // the counts are below 2^16: at most 20,480 updates of a half strip
-            const uint32_t z = (uint32_t)(up >> 32) | (uint32_t)(dn >> 32) << 16;
-            const uint32_t v = (uint32_t)(lf >> 32) | (uint32_t)(rt >> 32) << 16;
-            const bool ready = w.done < w.count && z == w.e.z && v == w.e.w;
-            // straight-line: the lanes of a warp are seldom ready together
-            uint32_t u = (uint32_t)up, d = (uint32_t)dn;
-            u = w.first_row ? (u << 1 | u >> 20) & kWordBits : u;
-            d = w.last_row ? (d >> 1 | d << 20) & kWordBits : d;
-            const uint32_t spins = flip_all(w.spins, u, d, (uint32_t)lf, (uint32_t)rt, w.e.x, w.e.y);
-            w.spins = ready ? spins : w.spins;
-            w.done += ready;
-            w.ahead += ready ? 16u : 0u;
-            w.e.x = ready ? w.next.x : w.e.x;
-            w.e.y = ready ? w.next.y : w.e.y;
-            w.e.z = ready ? w.next.z : w.e.z;
-            w.e.w = ready ? w.next.w : w.e.w;
-            asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %4, 0;\n\t"
-                         "@p st.volatile.shared.u64 [%5], %6;\n\t"
-                         "@p ld.shared.v4.u32 {%0, %1, %2, %3}, [%7];\n\t}"
-                         : "+r"(w.next.x), "+r"(w.next.y), "+r"(w.next.z), "+r"(w.next.w)
-                         : "r"((uint32_t)ready), "r"(w.at), "l"((uint64_t)w.done << 32 | w.spins), "r"(w.ahead - 16u)
-                         : "memory");
-            pending = pending || w.done < w.count;
-        }
+        for (int n = 0; n < kWordsLooks; ++n)
+#pragma unroll
+            for (int k = 0; k < WPT; ++k) look(o[k]);
+#pragma unroll
+        for (int k = 0; k < WPT; ++k) pending = pending || o[k].done < o[k].count;
         if (!__any_sync(0xffffffffu, pending)) break;
         if (tries == kWordsTries) {
             *(volatile unsigned int*)err = 1;
