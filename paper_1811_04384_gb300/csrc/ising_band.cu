@@ -53,6 +53,7 @@ struct BandArgs {
     const uint64_t* masks;      // masks[(h * L + i) * d.P + w]: half-sweep h of the launch, row i, word w
     int64_t s0, every;          // as ClusterArgs
     unsigned long long* counts;
+    int slots;                  // count slots of a record, a power of two
     uint64_t* t_dev;            // set to t_end at the end
     uint64_t t_end;
     unsigned int* err;          // set to 1 when a wait for rows gives up
@@ -265,7 +266,7 @@ band_sweeps_kernel(BandArgs a)
             const int64_t due = (a.s0 / a.every + 1) * a.every;                 // first recorded sweep of the call > s0
             if (due - a.s0 <= a.nsweeps) {
                 rec_j = (int)(due - a.s0);
-                rec = a.counts + ((size_t)(due / a.every - 1) * kCountSlots + q % kCountSlots) * 2;
+                rec = a.counts + ((size_t)(due / a.every - 1) * a.slots + (q & (a.slots - 1))) * 2;
             }
         }
         const uint32_t to_own = in_block(win_sh, b), to_up = in_block(win_sh, bp), to_dn = in_block(win_sh, bn);
@@ -308,7 +309,7 @@ band_sweeps_kernel(BandArgs a)
                         atomicAdd(rec, (unsigned long long)(sum & 0xffffu));
                         atomicAdd(rec + 1, (unsigned long long)(sum >> 16));
                     }
-                    rec += 2 * kCountSlots;
+                    rec += 2 * a.slots;
                     rec_j = a.every <= a.nsweeps - j ? j + (int)a.every : a.nsweeps + 1;
                 }
             }
@@ -405,7 +406,7 @@ bool band_setup()
 }
 
 cudaError_t launch_band_sweeps(uint64_t* w0, uint64_t* w1, uint32_t* dense, const Geom& g,
-                               unsigned long long* counts, const ClusterPlan& plan, int nsweeps,
+                               unsigned long long* counts, int slots, const ClusterPlan& plan, int nsweeps,
                                const uint64_t* masks, int64_t s0, int64_t every, uint64_t* t_dev, uint64_t t_end,
                                unsigned int* err, cudaStream_t s)
 {
@@ -422,6 +423,7 @@ cudaError_t launch_band_sweeps(uint64_t* w0, uint64_t* w1, uint32_t* dense, cons
     a.s0 = s0;
     a.every = every;
     a.counts = counts;
+    a.slots = slots;
     a.t_dev = t_dev;
     a.t_end = t_end;
     a.err = err;

@@ -83,7 +83,8 @@ struct ClusterArgs {
     const uint64_t* masks;      // masks[(h * L + i) * d.P + w]: half-sweep h = 2 j + c of the launch, row i, word w
     int64_t s0;                 // the launch runs sweeps s0 + 1 .. s0 + nsweeps of the call
     int64_t every;              // record after sweeps s with s % every == 0 (0: none)
-    unsigned long long* counts; // count slots (32 per record); record r of the call -> slot r
+    unsigned long long* counts; // count slots; record r of the call -> slots r `slots` ..
+    int slots;                  // of a record, a power of two
     int G;                      // clusters of the launch: blocks g C .. g C + C - 1 form cluster g
     uint64_t* xbuf;             // G > 1: halo rows between clusters, [boundary][dir][parity][colour], k x d.P / 2 words
     unsigned long long* xflag;  // G > 1: [boundary][dir] sequence flags
@@ -224,7 +225,7 @@ __device__ __forceinline__ void cl_half_sweep(const uint32_t (&m)[NS][2 * V], ui
                 cl_update<V, C, false>(m[j], win0, win_bytes, P4, slot[j], last_lo, live_last, anti, up);
         }
     }
-    if (RECORD) block_add_counts(counts + 2 * (blockIdx.x % kCountSlots), anti, up);
+    if (RECORD) block_add_counts(counts, anti, up);
 }
 
 // V: dense words per unit; NS: units per thread: the block has ceil(units /
@@ -405,7 +406,7 @@ cluster_sweeps_kernel(ClusterArgs a)
         const int64_t first = (a.s0 / a.every + 1) * a.every;          // first recorded sweep of the call > s0
         if (first - a.s0 <= a.nsweeps) {
             rec_j = (int)(first - a.s0);
-            rec_counts = a.counts + (size_t)(first / a.every - 1) * 2 * kCountSlots;
+            rec_counts = a.counts + ((size_t)(first / a.every - 1) * a.slots + (blockIdx.x & (a.slots - 1))) * 2;
         }
     }
     // d: the half-sweep's number in the phase
@@ -421,7 +422,7 @@ cluster_sweeps_kernel(ClusterArgs a)
         __syncthreads();
         if (++j == rec_j) {
             cl_half_sweep<V, 1, true, NS>(m, smem_sh, win_bytes, P4, slot, d + 1, last_lo, live_last, rec_counts);
-            rec_counts += 2 * kCountSlots;
+            rec_counts += 2 * a.slots;
             rec_j = a.every <= a.nsweeps - j ? j + (int)a.every : a.nsweeps + 1;
         } else {
             cl_half_sweep<V, 1, false, NS>(m, smem_sh, win_bytes, P4, slot, d + 1, last_lo, live_last, nullptr);
@@ -624,7 +625,7 @@ cudaError_t launch_cl_mask_draw(int L, const SweepArgs& a, uint64_t t0, int nswe
 }
 
 cudaError_t launch_cluster_sweeps(uint64_t* w0, uint64_t* w1, uint32_t* dense, const Geom& g, const SweepArgs& a,
-                                  const ClusterPlan& plan, int nsweeps, const uint64_t* masks, int64_t s0,
+                                  int slots, const ClusterPlan& plan, int nsweeps, const uint64_t* masks, int64_t s0,
                                   int64_t every, const ClusterExchange& x, cudaStream_t s)
 {
     const int nb = plan.clusters * plan.blocks;
@@ -641,6 +642,7 @@ cudaError_t launch_cluster_sweeps(uint64_t* w0, uint64_t* w1, uint32_t* dense, c
     ca.s0 = s0;
     ca.every = every;
     ca.counts = a.counts;
+    ca.slots = slots;
     ca.G = plan.clusters;
     ca.xbuf = x.buf;
     ca.xflag = x.flags;

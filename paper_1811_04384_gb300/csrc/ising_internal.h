@@ -76,8 +76,8 @@ cudaError_t launch_resident_premasked(uint64_t* w0, uint64_t* w1, const Geom& g,
 // with programmatic stream serialization, so that it runs beside the cluster
 // launch before it in the stream (which must not read `masks`).
 // launch_cluster_sweeps runs sweeps s0 + 1 .. s0 + nsweeps of a call from
-// them, recording after every `every`-th (0: none) into count slot
-// s / every - 1 past a.counts; the lattice is w0, w1 (packed words), or the
+// them, recording after every `every`-th (0: none) into the count slots
+// (`slots` of them) s / every - 1 past a.counts; the lattice is w0, w1 (packed words), or the
 // dense array `dense` (cl_dense_bytes bytes: [colour][row][word], pitch and
 // words of dense_geom) where it is not null.
 struct ClusterPlan {
@@ -114,7 +114,7 @@ size_t cl_dense_bytes(int L);
 cudaError_t launch_cl_mask_draw(int L, const SweepArgs& a, uint64_t t0, int nsweeps, uint64_t* masks, bool overlap,
                                 cudaStream_t s);
 cudaError_t launch_cluster_sweeps(uint64_t* w0, uint64_t* w1, uint32_t* dense, const Geom& g, const SweepArgs& a,
-                                  const ClusterPlan& plan, int nsweeps, const uint64_t* masks, int64_t s0,
+                                  int slots, const ClusterPlan& plan, int nsweeps, const uint64_t* masks, int64_t s0,
                                   int64_t every, const ClusterExchange& x, cudaStream_t s);
 
 // The form of the path for one cluster and short rows (ising_band.cu).
@@ -122,7 +122,7 @@ constexpr size_t kClSmemMax = 220 * 1024;   // most dynamic shared memory of a b
 bool band_setup();
 bool band_plan(int L, int blocks, ClusterPlan* plan);
 cudaError_t launch_band_sweeps(uint64_t* w0, uint64_t* w1, uint32_t* dense, const Geom& g,
-                               unsigned long long* counts, const ClusterPlan& plan, int nsweeps,
+                               unsigned long long* counts, int slots, const ClusterPlan& plan, int nsweeps,
                                const uint64_t* masks, int64_t s0, int64_t every, uint64_t* t_dev, uint64_t t_end,
                                unsigned int* err, cudaStream_t s);
 

@@ -677,8 +677,10 @@ static bool use_cluster(const ising_lattice* h, ClusterPlan* plan)
 }
 
 // n sweeps on the cluster path; every > 0: after every `every`-th sweep s of
-// the n, a record into count slot s / every - 1 past `counts`.
-static int run_cluster(ising_lattice* h, int64_t n, int64_t every, unsigned long long* counts, const ClusterPlan& plan)
+// the n, a record into the count slots s / every - 1 past `counts` (`slots` a record;
+// kCountSlots with several clusters, whose calls may end on the launch path).
+static int run_cluster(ising_lattice* h, int64_t n, int64_t every, unsigned long long* counts, const ClusterPlan& plan,
+                       int slots = kCountSlots)
 {
     const Geom& g = h->g;
     const bool ci = h->layout == ISING_LAYOUT_COLUMN_INTERLEAVED;
@@ -753,10 +755,10 @@ static int run_cluster(ising_lattice* h, int64_t n, int64_t every, unsigned long
         if (plan.clusters > 1 && h->absent_after >= 0 && h->absent_after-- == 0)
             x.absent = 1;                            // one block more than the launch has: it gives up
         cudaError_t e =
-            plan.v == 0 ? launch_band_sweeps(h->words[0], h->words[1], ci ? h->dense : nullptr, g, counts, plan,
+            plan.v == 0 ? launch_band_sweeps(h->words[0], h->words[1], ci ? h->dense : nullptr, g, counts, slots, plan,
                                              part_of(j), masks[j & 1], done, every, h->t_dev,
                                              h->t + (uint64_t)(done + part_of(j)), gave_up_word(h), h->stream)
-                        : launch_cluster_sweeps(h->words[0], h->words[1], ci ? h->dense : nullptr, g, a, plan,
+                        : launch_cluster_sweeps(h->words[0], h->words[1], ci ? h->dense : nullptr, g, a, slots, plan,
                                                 part_of(j), masks[j & 1], done, every, x, h->stream);
         if (e != cudaSuccess) return cuda_fail(e, "cluster sweeps kernel");
         if (plan.clusters > 1) {
@@ -992,10 +994,11 @@ extern "C" int ising_sweep(ising_lattice* h, int64_t n)
     return ISING_OK;
 }
 
-static void counts_to_EM(const ising_lattice* h, const unsigned long long* slots, int64_t* E, int64_t* M)
+static void counts_to_EM(const ising_lattice* h, const unsigned long long* slots, int64_t* E, int64_t* M,
+                         int n = kCountSlots)
 {
     unsigned long long anti = 0, up = 0;
-    for (int k = 0; k < kCountSlots; ++k) {
+    for (int k = 0; k < n; ++k) {
         anti += slots[2 * k];
         up += slots[2 * k + 1];
     }
@@ -1037,7 +1040,12 @@ extern "C" int ising_sweep_record(ising_lattice* h, int64_t n, int64_t every, in
     ClusterPlan cp;
     while (done_rec < nrec) {
         const int64_t chunk = (nrec - done_rec) < kRecordsPerChunk ? (nrec - done_rec) : kRecordsPerChunk;
-        const size_t bytes = (size_t)chunk * kCountSlots * 2 * sizeof(unsigned long long);
+        // one cluster adds few counts to a record (64 warps, or 16 blocks): one slot,
+        // and a 32nd of the clearing, copying and adding up (500 sweeps, all recorded,
+        // of L = 160: 241 -> 219 us; of L = 296: 292 -> 287)
+        const bool cluster = h->chain == ISING_CHAIN_CHECKERBOARD && use_cluster(h, &cp);
+        const int slots = cluster && cp.clusters == 1 ? 1 : kCountSlots;
+        const size_t bytes = (size_t)chunk * slots * 2 * sizeof(unsigned long long);
         cudaError_t e = cudaMemsetAsync(h->counts, 0, bytes, h->stream);
         if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync counts");
         int rc;
@@ -1045,8 +1053,8 @@ extern "C" int ising_sweep_record(ising_lattice* h, int64_t n, int64_t every, in
             rc = run_random_words(h, chunk * every, [every](int64_t s) {
                 return (s % every == 0) ? (int)(s / every - 1) : -1;
             });
-        else if (use_cluster(h, &cp))
-            rc = run_cluster(h, chunk * every, every, h->counts, cp);
+        else if (cluster)
+            rc = run_cluster(h, chunk * every, every, h->counts, cp, slots);
         else if (use_graphs(h) && every <= kGraphMaxEvery)
             rc = replay_records(h, chunk, (int)every);
         else
@@ -1059,8 +1067,8 @@ extern "C" int ising_sweep_record(ising_lattice* h, int64_t n, int64_t every, in
         rc = sync_results(h);
         if (rc != ISING_OK) return rc;
         for (int64_t r = 0; r < chunk; ++r)
-            counts_to_EM(h, h->host_counts + (size_t)r * kCountSlots * 2, E ? E + done_rec + r : nullptr,
-                         M ? M + done_rec + r : nullptr);
+            counts_to_EM(h, h->host_counts + (size_t)r * slots * 2, E ? E + done_rec + r : nullptr,
+                         M ? M + done_rec + r : nullptr, slots);
         done_rec += chunk;
     }
     const int64_t rest = n - nrec * every;
