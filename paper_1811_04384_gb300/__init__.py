@@ -237,7 +237,7 @@ class Lattice:
     def sweep_record(self, n: int, every: int = 1):
         """Run n sweeps; returns int64 arrays E, M recorded every `every` sweeps (ising_sweep_record)."""
         k = n // every
-        slots = max(k, 1)
+        slots = operator.index(max(k, 1))                  # a Python int: 8 slots may pass the type of n
         out = np.zeros(2 * slots, dtype=np.int64)          # E, then M
         first = ctypes.c_int64.from_buffer(out)
         _check(load().ising_sweep_record(self._h, int(n), int(every), ctypes.byref(first),
