@@ -313,6 +313,14 @@ int ising_set_clusters(ising_lattice *h, int32_t clusters);
  * ISING_ETIMEOUT (the GPU keeps running; nothing traps).  0 clears it. */
 int ising_cluster_inject_stall(ising_lattice *h, int32_t launches);
 
+/* Test hook of the waits that ising_sweep reports late: the next `launches`
+ * launches of one cluster on rows of 3 to 14 dense words (L of about 130 to
+ * 896), or phases of the random-word chain on half strips that fit in shared
+ * memory, wait for what never comes.  The wait gives up after a second or so,
+ * the launch ends (one on a cluster leaves the lattice as it was), and the next
+ * call that reads results returns ISING_ETIMEOUT.  0 clears it. */
+int ising_inject_wait_stall(ising_lattice *h, int32_t launches);
+
 /* Test hook of that agreement: the launch with several clusters that comes
  * after `after` (>= 0) more such launches counts on one block more than it
  * has, so its blocks agree after 0.1 s that not all were resident and write

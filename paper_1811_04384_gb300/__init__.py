@@ -210,6 +210,11 @@ class Lattice:
         """Test hook (ising_cluster_inject_stall): the next launches' waits between clusters give up."""
         _check(load().ising_cluster_inject_stall(self._h, int(launches)), "ising_cluster_inject_stall")
 
+    def inject_wait_stall(self, launches: int = 1):
+        """Test hook (ising_inject_wait_stall): the waits inside a cluster, or of
+        the random-word chain, of the next such launches give up."""
+        _check(load().ising_inject_wait_stall(self._h, int(launches)), "ising_inject_wait_stall")
+
     def inject_absent(self, after: int = 0):
         """Test hook (ising_cluster_inject_absent): the launch with several
         clusters after `after` more of them counts on one block more than it

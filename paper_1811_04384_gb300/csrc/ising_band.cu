@@ -57,6 +57,7 @@ struct BandArgs {
     uint64_t* t_dev;            // set to t_end at the end
     uint64_t t_end;
     unsigned int* err;          // set to 1 when a wait for rows gives up
+    int stall;                  // 1: the first wait is for rows that never come (a test hook)
 };
 
 // A lane's row of both colours.  The side neighbour of a site of colour C is at
@@ -142,9 +143,9 @@ __device__ __forceinline__ uint32_t in_block(uint32_t addr, int rank)
 
 // Waits for the completion of the barrier's phase of that parity.  The rows
 // come from blocks of the same cluster, which run at the same time, so they
-// come; all the same the wait gives up after kClWaitNs, sets *err and lets the
-// launch end with void results.
-__device__ __forceinline__ void wait_rows(uint32_t bar, uint32_t parity, unsigned int* err)
+// come; all the same the wait gives up after kClWaitNs, sets *err and returns
+// false.
+__device__ __forceinline__ bool wait_rows(uint32_t bar, uint32_t parity, unsigned int* err)
 {
     unsigned long long t0 = 0;
     for (int tries = 0;; ++tries) {
@@ -152,16 +153,30 @@ __device__ __forceinline__ void wait_rows(uint32_t bar, uint32_t parity, unsigne
         asm volatile("{\n\t.reg .pred p;\n\t"
                      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
                      "selp.u32 %0, 1, 0, p;\n\t}" : "=r"(done) : "r"(bar), "r"(parity) : "memory");
-        if (done) return;
+        if (done) return true;
         if (tries < 1000) continue;
-        if (*(volatile unsigned int*)err != 0) return;
+        if (*(volatile unsigned int*)err != 0) return false;
         const unsigned long long t = cl_globaltimer();
         if (t0 == 0) t0 = t;
         if (t - t0 > kClWaitNs) {
             *(volatile unsigned int*)err = 1;
-            return;
+            return false;
         }
     }
+}
+
+// The end of a launch in which a block gave up, for every thread of every
+// block once none sends any more: rows that are still on their way reach the
+// windows (a millisecond is a thousand times what one takes) before any block
+// leaves.
+__device__ __forceinline__ void drain_rows(cg::cluster_group cluster)
+{
+    constexpr unsigned long long kDrainNs = 1000000;
+    if (threadIdx.x == 0) {
+        const unsigned long long t0 = cl_globaltimer();
+        while (cl_globaltimer() - t0 < kDrainNs) __nanosleep(1000);
+    }
+    cluster.sync();
 }
 
 template <int W>
@@ -198,13 +213,16 @@ band_sweeps_kernel(BandArgs a)
         if (r >= S - k) half_st(win_dn, at(par, c, r - (S - k), w), v, win_words, __LINE__);
     };
     const uint32_t win_sh = (uint32_t)__cvta_generic_to_shared(win);
-    // arrivals of the windows' rows, one barrier per parity
-    __shared__ uint64_t rows_bar[2];
+    // arrivals of the windows' rows, one barrier per parity; one that nothing arrives at
+    __shared__ uint64_t rows_bar[3];
+    __shared__ unsigned int gave_up;         // a block of the cluster gave up
     const uint32_t bar_sh = (uint32_t)__cvta_generic_to_shared(rows_bar);
     const uint32_t window_bytes = (uint32_t)R * 2u * WV * 16u;
     if (threadIdx.x == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar_sh) : "memory");
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar_sh + 8u) : "memory");
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar_sh + 16u) : "memory");
+        gave_up = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     const int half_sweeps = 2 * a.nsweeps, phases = (half_sweeps + k - 1) / k;
@@ -239,10 +257,11 @@ band_sweeps_kernel(BandArgs a)
         }
     if (warp >= kBandWarps) copy(0);
     cluster.sync();
+    bool stopped = false;                    // uniform over the block: one of its waits gave up
     if (warp >= kBandWarps) {
-        for (int p = 0; p < phases; ++p) {
+        for (int p = 0; p < phases && !stopped; ++p) {
             if (p + 1 < phases) copy(p + 1);
-            __syncthreads();
+            stopped = __syncthreads_or(0) != 0;
         }
     } else {
         // lane l: window row first + l; the own rows at lanes k .. k + own - 1
@@ -274,8 +293,9 @@ band_sweeps_kernel(BandArgs a)
         for (int p = 0; p < phases; ++p) {
             const int nh = min(k, half_sweeps - p * k);
             // window p (the first: by the cluster barrier) and the count of the next one's bytes
-            if (p > 0) wait_rows(bar_sh + 8u * (p & 1), (p - 1) >> 1 & 1, a.err);
-            if (threadIdx.x == 0 && p + 1 < phases)
+            const bool come =
+                p == 0 || wait_rows(bar_sh + (a.stall ? 16u : 8u * (p & 1)), (p - 1) >> 1 & 1, a.err);
+            if (threadIdx.x == 0 && come && p + 1 < phases)
                 asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
                              ::"r"(bar_sh + 8u * ((p + 1) & 1)), "r"(window_bytes) : "memory");
 #pragma unroll
@@ -316,8 +336,10 @@ band_sweeps_kernel(BandArgs a)
             // All warps have loaded their rows of window p, so the neighbours may write
             // the window after next (they cannot be there before this block's rows of
             // the next one reach them), the masks of phase p + 1 are in the ring, and
-            // those of phase p are no longer needed.
-            __syncthreads();
+            // those of phase p are no longer needed.  A block that gave up sends
+            // nothing more.
+            stopped = __syncthreads_or(!come) != 0;
+            if (stopped) break;
             if (is_own) {
                 // row `row` of the window; row + Sp of the block's above, row - S of the block's below
                 const int r = row - k, to = (p + 1) & 1;
@@ -337,7 +359,12 @@ band_sweeps_kernel(BandArgs a)
         }
     }
     // the own rows are in the window; no block leaves while another may still use its barriers
+    if (stopped && threadIdx.x < C) *cluster.map_shared_rank(&gave_up, threadIdx.x) = 1;
     cluster.sync();
+    if (gave_up) {                           // nobody writes back: the launch leaves the lattice as it was
+        drain_rows(cluster);
+        return;
+    }
     const int par = phases & 1;
     if (blockIdx.x == 0 && threadIdx.x == 0) *a.t_dev = a.t_end;
     if (a.dense) {
@@ -408,7 +435,7 @@ bool band_setup()
 cudaError_t launch_band_sweeps(uint64_t* w0, uint64_t* w1, uint32_t* dense, const Geom& g,
                                unsigned long long* counts, int slots, const ClusterPlan& plan, int nsweeps,
                                const uint64_t* masks, int64_t s0, int64_t every, uint64_t* t_dev, uint64_t t_end,
-                               unsigned int* err, cudaStream_t s)
+                               unsigned int* err, bool stall, cudaStream_t s)
 {
     BandArgs a;
     a.w[0] = w0;
@@ -427,6 +454,7 @@ cudaError_t launch_band_sweeps(uint64_t* w0, uint64_t* w1, uint32_t* dense, cons
     a.t_dev = t_dev;
     a.t_end = t_end;
     a.err = err;
+    a.stall = stall;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(plan.blocks);
     cfg.blockDim = dim3(kBandThreads);

@@ -36,12 +36,13 @@ cudaError_t ci_random_words_iteration(uint64_t* S, int L, int nstrips, const Swe
 // sweep_number(a) .. + iterations - 1 (words_plan_bytes each; at most
 // words_plan_iterations of the n that a call runs), words_run both phases of
 // the plan's iteration `iteration` (0: right after words_plan, or after the
-// phases before it); *err = 1 when a wait gave up.
+// phases before it); *err = 1 when a wait gave up; the first `stalls` (0 .. 2)
+// phases wait for what never comes (a test hook).
 bool words_planned(int L, int nstrips);
 size_t words_plan_bytes(int L, int nstrips);
 int words_plan_iterations(int L, int nstrips, int64_t n);
 cudaError_t words_plan(int L, int nstrips, const SweepArgs& a, int iterations, void* plan, cudaStream_t s);
 cudaError_t words_run(uint64_t* S, int L, int nstrips, const void* plan, int iteration, unsigned int* err,
-                      cudaStream_t s);
+                      int stalls, cudaStream_t s);
 
 }  // namespace ising

@@ -124,7 +124,7 @@ bool band_plan(int L, int blocks, ClusterPlan* plan);
 cudaError_t launch_band_sweeps(uint64_t* w0, uint64_t* w1, uint32_t* dense, const Geom& g,
                                unsigned long long* counts, int slots, const ClusterPlan& plan, int nsweeps,
                                const uint64_t* masks, int64_t s0, int64_t every, uint64_t* t_dev, uint64_t t_end,
-                               unsigned int* err, cudaStream_t s);
+                               unsigned int* err, bool stall, cudaStream_t s);
 
 // The on-chip path up to side kWarpMaxL (ising_warp.cu): sweeps s_base + 1 ..
 // s_base + n of a run in one warp's registers, with the masks that

@@ -83,6 +83,8 @@ struct ising_lattice {
     unsigned long long xseq = 0;                 // flag base of the next launch
     unsigned int* host_xerr = nullptr;           // pinned copy of the error and agreement words
     int stall_launches = 0;                      // test hook: launches whose waits between clusters give up
+    int wait_stalls = 0;                         // test hook: launches whose waits inside a cluster, or of the
+                                                 // random-word chain, give up
     int absent_after = -1;                       // test hook: the launch after this many more counts on one
                                                  // block more than it has (-1: none)
     bool multi_gave_up = false;                  // a launch's blocks were not all resident: auto keeps to one cluster
@@ -754,10 +756,12 @@ static int run_cluster(ising_lattice* h, int64_t n, int64_t every, unsigned long
         }
         if (plan.clusters > 1 && h->absent_after >= 0 && h->absent_after-- == 0)
             x.absent = 1;                            // one block more than the launch has: it gives up
+        const bool stall = plan.v == 0 && h->wait_stalls > 0;
+        if (stall) --h->wait_stalls;
         cudaError_t e =
             plan.v == 0 ? launch_band_sweeps(h->words[0], h->words[1], ci ? h->dense : nullptr, g, counts, slots, plan,
                                              part_of(j), masks[j & 1], done, every, h->t_dev,
-                                             h->t + (uint64_t)(done + part_of(j)), gave_up_word(h), h->stream)
+                                             h->t + (uint64_t)(done + part_of(j)), gave_up_word(h), stall, h->stream)
                         : launch_cluster_sweeps(h->words[0], h->words[1], ci ? h->dense : nullptr, g, a, slots, plan,
                                                 part_of(j), masks[j & 1], done, every, x, h->stream);
         if (e != cudaSuccess) return cuda_fail(e, "cluster sweeps kernel");
@@ -838,6 +842,13 @@ extern "C" int ising_cluster_inject_stall(ising_lattice* h, int32_t launches)
     return ISING_OK;
 }
 
+extern "C" int ising_inject_wait_stall(ising_lattice* h, int32_t launches)
+{
+    if (!h || launches < 0) return ISING_EINVAL;
+    h->wait_stalls = launches;
+    return ISING_OK;
+}
+
 extern "C" int ising_cluster_inject_absent(ising_lattice* h, int32_t after)
 {
     if (!h || after < -1) return ISING_EINVAL;
@@ -910,8 +921,10 @@ static int run_random_words(ising_lattice* h, int64_t n, RecOf rec_of)
             const int k = (int)((it - 1) % chunk);
             if (k == 0)
                 e = words_plan(h->g.L, h->nstrips, a, (int)std::min<int64_t>(chunk, n - it + 1), h->rw_draws, h->stream);
+            const int stalls = std::min(h->wait_stalls, 2);
+            h->wait_stalls -= stalls;
             if (e == cudaSuccess)
-                e = words_run(h->words[0], h->g.L, h->nstrips, h->rw_draws, k, gave_up_word(h), h->stream);
+                e = words_run(h->words[0], h->g.L, h->nstrips, h->rw_draws, k, gave_up_word(h), stalls, h->stream);
         } else {
             e = ci_random_words_iteration(h->words[0], h->g.L, h->nstrips, a, pre ? h->rw_draws : nullptr, h->stream);
         }

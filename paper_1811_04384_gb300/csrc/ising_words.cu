@@ -221,7 +221,8 @@ __device__ __forceinline__ Entry entry_ld(uint32_t addr)
 // One phase of one iteration, strip blockIdx.x, from its plan.
 template <int WPT>
 __global__ void __launch_bounds__(kWordsThreads)
-words_run_kernel(uint64_t* S, WordsGeom g, int phase, bool fresh, const char* __restrict__ plan, unsigned int* err)
+words_run_kernel(uint64_t* S, WordsGeom g, int phase, bool fresh, const char* __restrict__ plan, unsigned int* err,
+                 uint32_t stall)
 {
     extern __shared__ __align__(16) uint4 run_smem[];
     const int strip = blockIdx.x, h = g.h(phase), hw = h + 2, W = g.words(phase);
@@ -273,6 +274,7 @@ words_run_kernel(uint64_t* S, WordsGeom g, int phase, bool fresh, const char* __
         o[k].ahead = entry_sh + 16u * (start[x] + 2u);
         o[k].e = entry_ld(o[k].ahead - 32u);
         o[k].next = entry_ld(o[k].ahead - 16u);
+        o[k].e.z |= stall;               // a test hook: a count that no word reaches
     }
     // rows whose neighbours come from across the top or bottom row: few warps have any
     bool edge = false;
@@ -381,7 +383,7 @@ cudaError_t words_plan(int L, int nstrips, const SweepArgs& a, int iterations, v
 }
 
 cudaError_t words_run(uint64_t* S, int L, int nstrips, const void* plan, int iteration, unsigned int* err,
-                      cudaStream_t s)
+                      int stalls, cudaStream_t s)
 {
     const dim3 grid(nstrips);
     const WordsGeom g = words_geom(L, nstrips);
@@ -390,7 +392,7 @@ cudaError_t words_run(uint64_t* S, int L, int nstrips, const void* plan, int ite
         const int W = g.words(phase), per = W > kWordsThreads ? 2 : 1, threads = ((W + per - 1) / per + 31) / 32 * 32;
         const bool fresh = iteration == 0 && phase == 0;      // the plan is the launch before
         launch_pdl_with(false, run_smem_bytes(g, phase), per == 1 ? words_run_kernel<1> : words_run_kernel<2>, grid,
-                        dim3(threads), s, S, g, phase, fresh, p, err);
+                        dim3(threads), s, S, g, phase, fresh, p, err, phase < stalls ? 0x8000u : 0u);
     }
     return cudaGetLastError();
 }
