@@ -136,7 +136,8 @@ int ising_get_thresholds(ising_lattice *h, uint64_t host_thr[2]);
  * clusters gave up; see ising_set_clusters), ECUDA.  A wait inside a cluster or
  * of the random-word chain that gives up (none should: both wait for threads
  * that run at the same time) makes the next call that reads results return
- * ETIMEOUT. */
+ * ETIMEOUT, unless new spins are set before it (ising_init_hot, ising_init_cold,
+ * ising_set_spins, ising_set_words, ising_run_states). */
 int ising_sweep(ising_lattice *h, int64_t n);
 
 /* Run n sweeps and record E and M after sweeps t+every, t+2*every, ...:
@@ -144,8 +145,8 @@ int ising_sweep(ising_lattice *h, int64_t n);
  * each; either may be NULL.  n >= 0, 1 <= every <= 2^22.  Synchronises the stream.
  * The counts come from the reduction fused into the colour-1 half-sweep.
  * Errors: EINVAL (NULL, n < 0, every out of range), ENOMEM (the mask
- * buffer of the on-chip path), ETIMEOUT (as for
- * ising_sweep), ECUDA. */
+ * buffer of the on-chip path), ETIMEOUT (as for ising_sweep, and a wait that
+ * gave up since results were last read), ECUDA. */
 int ising_sweep_record(ising_lattice *h, int64_t n, int64_t every,
                        int64_t *host_E, int64_t *host_M);
 

@@ -45,6 +45,7 @@ cudaError_t launch_pack_rows(uint64_t* w0, uint64_t* w1, const Geom& g, const in
 cudaError_t launch_advance_sweep(uint64_t* t_base, uint64_t n, cudaStream_t s);
 cudaError_t launch_advance_graph(uint64_t* t_base, uint64_t n, uint32_t* rec_base, uint32_t inc, cudaStream_t s);
 cudaError_t launch_set_sweep(uint64_t* t_base, uint64_t t, cudaStream_t s);
+cudaError_t launch_clear_word(unsigned int* word, cudaStream_t s);   // *word = 0 (pinned host memory)
 // Philox4x32-10 of n counters (4 words each) under key `seed` (test hook).
 cudaError_t launch_philox_blocks(const uint32_t* ctr, uint32_t* out, int64_t n, uint64_t seed, cudaStream_t s);
 // The on-chip path: allow `bytes` of dynamic shared memory for its kernels

@@ -204,6 +204,8 @@ __global__ void set_sweep_kernel(uint64_t* t_base, uint64_t t)
     if (threadIdx.x == 0 && blockIdx.x == 0) *t_base = t;
 }
 
+__global__ void clear_word_kernel(unsigned int* word) { *word = 0; }
+
 // Temporal blocking with the whole lattice on chip: one block copies both
 // colour arrays into shared memory, runs sweeps t0+1 .. t0+n there (a block
 // barrier between half-sweeps), records E and M after every `every`-th sweep
@@ -617,6 +619,12 @@ cudaError_t launch_advance_graph(uint64_t* t_base, uint64_t n, uint32_t* rec_bas
 cudaError_t launch_set_sweep(uint64_t* t_base, uint64_t t, cudaStream_t s)
 {
     set_sweep_kernel<<<1, 1, 0, s>>>(t_base, t);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_clear_word(unsigned int* word, cudaStream_t s)
+{
+    clear_word_kernel<<<1, 1, 0, s>>>(word);
     return cudaGetLastError();
 }
 

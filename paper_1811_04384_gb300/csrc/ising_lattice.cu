@@ -83,6 +83,7 @@ struct ising_lattice {
     unsigned long long xseq = 0;                 // flag base of the next launch
     unsigned int* host_xerr = nullptr;           // pinned copy of the error and agreement words
     int stall_launches = 0;                      // test hook: launches whose waits between clusters give up
+    bool may_give_up = false;                    // a launch that sets gave_up_word is not yet looked at
     int wait_stalls = 0;                         // test hook: launches whose waits inside a cluster, or of the
                                                  // random-word chain, give up
     int absent_after = -1;                       // test hook: the launch after this many more counts on one
@@ -129,10 +130,22 @@ static int sync_results(ising_lattice* h)
 {
     cudaError_t e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize");
+    h->may_give_up = false;
     volatile unsigned int* word = gave_up_word(h);
     if (*word == 0) return ISING_OK;
     *word = 0;
     return ISING_ETIMEOUT;
+}
+
+// New spins take the place of what a launch that gave up has left: its word is
+// cleared in the stream, after the launches that may yet set it.
+static int forget_gave_up(ising_lattice* h)
+{
+    if (!h->may_give_up) return ISING_OK;
+    cudaError_t e = launch_clear_word(gave_up_word(h), h->stream);
+    if (e != cudaSuccess) return cuda_fail(e, "clear_word_kernel");
+    h->may_give_up = false;
+    return ISING_OK;
 }
 
 static int setup_handle(ising_lattice* h, int32_t L, uint64_t seed, char* base)
@@ -263,6 +276,8 @@ extern "C" int ising_init_hot(ising_lattice* h)
 {
     TraceRange trace("ising_init_hot");
     if (!h) return ISING_EINVAL;
+    const int rc = forget_gave_up(h);
+    if (rc != ISING_OK) return rc;
     if (h->layout == ISING_LAYOUT_COLUMN_INTERLEAVED) {
         cudaError_t e = ci_init_hot(h->words[0], h->g.L, h->seed, h->stream);
         if (e != cudaSuccess) return cuda_fail(e, "ci_init_hot");
@@ -280,6 +295,8 @@ extern "C" int ising_init_hot(ising_lattice* h)
 extern "C" int ising_init_cold(ising_lattice* h, int8_t spin)
 {
     if (!h || (spin != 1 && spin != -1)) return ISING_EINVAL;
+    const int rc = forget_gave_up(h);
+    if (rc != ISING_OK) return rc;
     if (h->layout == ISING_LAYOUT_COLUMN_INTERLEAVED) {
         cudaError_t e = ci_init_cold(h->words[0], h->g.L, spin > 0 ? 1 : 0, h->stream);
         if (e != cudaSuccess) return cuda_fail(e, "ci_init_cold");
@@ -758,6 +775,7 @@ static int run_cluster(ising_lattice* h, int64_t n, int64_t every, unsigned long
             x.absent = 1;                            // one block more than the launch has: it gives up
         const bool stall = plan.v == 0 && h->wait_stalls > 0;
         if (stall) --h->wait_stalls;
+        if (plan.v == 0) h->may_give_up = true;
         cudaError_t e =
             plan.v == 0 ? launch_band_sweeps(h->words[0], h->words[1], ci ? h->dense : nullptr, g, counts, slots, plan,
                                              part_of(j), masks[j & 1], done, every, h->t_dev,
@@ -923,6 +941,7 @@ static int run_random_words(ising_lattice* h, int64_t n, RecOf rec_of)
                 e = words_plan(h->g.L, h->nstrips, a, (int)std::min<int64_t>(chunk, n - it + 1), h->rw_draws, h->stream);
             const int stalls = std::min(h->wait_stalls, 2);
             h->wait_stalls -= stalls;
+            h->may_give_up = true;
             if (e == cudaSuccess)
                 e = words_run(h->words[0], h->g.L, h->nstrips, h->rw_draws, k, gave_up_word(h), stalls, h->stream);
         } else {
@@ -1034,11 +1053,12 @@ extern "C" int ising_sweep_record(ising_lattice* h, int64_t n, int64_t every, in
             int rc = run_resident(h, (int)(chunk * every), (int)every, &direct);
             if (rc != ISING_OK) return rc;
             const size_t bytes = (size_t)chunk * 2 * sizeof(long long);
-            cudaError_t e = cudaSuccess;
-            if (!direct)
-                e = cudaMemcpyAsync(h->host_counts, h->counts, bytes, cudaMemcpyDeviceToHost, h->stream);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-            if (e != cudaSuccess) return cuda_fail(e, "resident records");
+            if (!direct) {
+                cudaError_t e = cudaMemcpyAsync(h->host_counts, h->counts, bytes, cudaMemcpyDeviceToHost, h->stream);
+                if (e != cudaSuccess) return cuda_fail(e, "resident records");
+            }
+            rc = sync_results(h);
+            if (rc != ISING_OK) return rc;
             const long long* rec = reinterpret_cast<const long long*>(h->host_counts);
             for (int64_t r = 0; r < chunk; ++r) {
                 if (E) E[done_rec + r] = rec[2 * r];
@@ -1171,6 +1191,7 @@ extern "C" int ising_set_spins(ising_lattice* h, const int8_t* in, size_t n)
     TraceRange trace("ising_set_spins");
     if (!h || !in || n != (size_t)h->g.L * h->g.L) return ISING_EINVAL;
     int rc = ensure_staging(h);
+    if (rc == ISING_OK) rc = forget_gave_up(h);
     if (rc != ISING_OK) return rc;
     const Geom& g = h->g;
     // Pinned host memory is read by the pack kernel itself (one pass over the
@@ -1238,6 +1259,7 @@ extern "C" int ising_run_states(ising_lattice* h, const int8_t* const* states, i
         return ISING_OK;
     }
     int rc = ensure_pipeline(h);
+    if (rc == ISING_OK) rc = forget_gave_up(h);
     if (rc != ISING_OK) return rc;
     const Geom& g = h->g;
     int8_t* stage[2] = {h->staging, h->staging2};
@@ -1319,6 +1341,8 @@ extern "C" int ising_set_words(ising_lattice* h, const uint64_t* in, size_t n64)
     if (h->layout != ISING_LAYOUT_ROW_PACKED) return ISING_EINVAL;   // row-packed words only
     const size_t per = (size_t)h->g.L * h->g.P;
     if (n64 != 2 * per) return ISING_EINVAL;
+    const int rc = forget_gave_up(h);
+    if (rc != ISING_OK) return rc;
     for (int c = 0; c < 2; ++c) {
         cudaError_t e = cudaMemcpyAsync(h->words[c], in + c * per, per * sizeof(uint64_t),
                                         cudaMemcpyHostToDevice, h->stream);
