@@ -210,7 +210,12 @@ int ising_set_words(ising_lattice *h, const uint64_t *host_in, size_t n64);
 int ising_layout(ising_lattice *h, int32_t *W, int32_t *pitch, int32_t *last_fields);
 
 /* Sweep counter t (checkpoint / resume: with the counter-based draws a run
- * resumed at t is bit-identical to an uninterrupted one). */
+ * resumed at t is bit-identical to an uninterrupted one).  Sweeps of the launch
+ * path that a caller captures into a graph of its own count on the device, once
+ * for every replay, and the launch path's calls after them go on from there.
+ * The host does not see replays: ising_get_sweep counts the captured call once,
+ * and before a call on another path ising_set_sweep has to say where the run
+ * stands. */
 int ising_get_sweep(ising_lattice *h, uint64_t *t);
 int ising_set_sweep(ising_lattice *h, uint64_t t);
 

@@ -54,8 +54,7 @@ struct BandArgs {
     int64_t s0, every;          // as ClusterArgs
     unsigned long long* counts;
     int slots;                  // count slots of a record, a power of two
-    uint64_t* t_dev;            // set to t_end at the end
-    uint64_t t_end;
+    uint64_t* t_dev;            // advanced by nsweeps at the end
     unsigned int* err;          // set to 1 when a wait for rows gives up
     int stall;                  // 1: the first wait is for rows that never come (a test hook)
 };
@@ -361,12 +360,13 @@ band_sweeps_kernel(BandArgs a)
     // the own rows are in the window; no block leaves while another may still use its barriers
     if (stopped && threadIdx.x < C) *cluster.map_shared_rank(&gave_up, threadIdx.x) = 1;
     cluster.sync();
+    if (blockIdx.x == 0 && threadIdx.x == 0)
+        atomicAdd(reinterpret_cast<unsigned long long*>(a.t_dev), (unsigned long long)a.nsweeps);
     if (gave_up) {                           // nobody writes back: the launch leaves the lattice as it was
         drain_rows(cluster);
         return;
     }
     const int par = phases & 1;
-    if (blockIdx.x == 0 && threadIdx.x == 0) *a.t_dev = a.t_end;
     if (a.dense) {
         for (int c = 0; c < 2; ++c)
             for (int e = threadIdx.x; e < S * W; e += kBandThreads) {
@@ -434,7 +434,7 @@ bool band_setup()
 
 cudaError_t launch_band_sweeps(uint64_t* w0, uint64_t* w1, uint32_t* dense, const Geom& g,
                                unsigned long long* counts, int slots, const ClusterPlan& plan, int nsweeps,
-                               const uint64_t* masks, int64_t s0, int64_t every, uint64_t* t_dev, uint64_t t_end,
+                               const uint64_t* masks, int64_t s0, int64_t every, uint64_t* t_dev,
                                unsigned int* err, bool stall, cudaStream_t s)
 {
     BandArgs a;
@@ -452,7 +452,6 @@ cudaError_t launch_band_sweeps(uint64_t* w0, uint64_t* w1, uint32_t* dense, cons
     a.counts = counts;
     a.slots = slots;
     a.t_dev = t_dev;
-    a.t_end = t_end;
     a.err = err;
     a.stall = stall;
     cudaLaunchConfig_t cfg = {};

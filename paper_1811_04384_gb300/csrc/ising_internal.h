@@ -124,19 +124,19 @@ bool band_setup();
 bool band_plan(int L, int blocks, ClusterPlan* plan);
 cudaError_t launch_band_sweeps(uint64_t* w0, uint64_t* w1, uint32_t* dense, const Geom& g,
                                unsigned long long* counts, int slots, const ClusterPlan& plan, int nsweeps,
-                               const uint64_t* masks, int64_t s0, int64_t every, uint64_t* t_dev, uint64_t t_end,
+                               const uint64_t* masks, int64_t s0, int64_t every, uint64_t* t_dev,
                                unsigned int* err, bool stall, cudaStream_t s);
 
 // The on-chip path up to side kWarpMaxL (ising_warp.cu): sweeps s_base + 1 ..
 // s_base + n of a run in one warp's registers, with the masks that
 // launch_warp_mask_draw (just before; at most 32767 sweeps) left in `masks`,
-// (E, M) records into rec (device or pinned host memory), then *t_dev = t_end.
+// (E, M) records into rec (device or pinned host memory), then *t_dev += n.
 constexpr int kWarpMaxL = 128;
 size_t warp_mask_bytes_per_sweep(int L);
 cudaError_t launch_warp_mask_draw(int L, const SweepArgs& a, uint64_t t0, int nsweeps, uint64_t* masks,
                                   cudaStream_t s);
 cudaError_t launch_warp_sweeps(uint64_t* w0, uint64_t* w1, const Geom& g, const uint64_t* masks, int s_base, int n,
-                               int every, long long* rec, uint64_t* t_dev, uint64_t t_end, cudaStream_t s);
+                               int every, long long* rec, uint64_t* t_dev, cudaStream_t s);
 
 // Launch `kernel` with programmatic stream serialization (every thread of the
 // kernel calls pdl_wait before it reads what an earlier launch writes): the

@@ -46,6 +46,7 @@ struct ising_lattice {
     Geom g;
     uint64_t seed = 0;
     uint64_t t = 0;              // host copy of the sweep counter
+    bool t_on_device = false;    // a caller's graph holds sweeps: only the device counter knows how many ran
     double beta = 0.0;
     uint64_t thr[2] = {0, 0};
     cudaStream_t stream = nullptr;
@@ -451,7 +452,8 @@ static int replay_plain(ising_lattice* h, int64_t* n)
 // rec_of(s) >= 0.  Then advances the counter by n.  The launches take the
 // sweep counter from the host, so that their draws need no device memory;
 // where the stream is being captured they read the device's, which a replay
-// advances.  after_first() comes after the first launch.  With `owed` the
+// advances, and from then on all the handle's launches do, as the host does not
+// see the replays.  after_first() comes after the first launch.  With `owed` the
 // device counter may stay behind, by the sweeps added to *owed.
 struct NoHook {
     cudaError_t operator()() const { return cudaSuccess; }
@@ -465,7 +467,8 @@ static int run_sweeps(ising_lattice* h, int64_t n, RecOf rec_of, First after_fir
         cudaGetLastError();
         cs = cudaStreamCaptureStatusActive;
     }
-    if (cs == cudaStreamCaptureStatusNone) {
+    if (cs != cudaStreamCaptureStatusNone) h->t_on_device = true;
+    if (!h->t_on_device) {
         a.t_base = nullptr;
         a.t0 = h->t;
     }
@@ -575,10 +578,10 @@ static int run_resident(ising_lattice* h, int n, int every, bool* direct)
             const int part = std::min(n - done, max_sweeps);
             cudaError_t e = launch_warp_mask_draw(g.L, a, h->t, part, masks, h->stream);
             if (e != cudaSuccess) return cuda_fail(e, "dense_mask_draw_kernel");
-            h->t += (uint64_t)part;
             e = launch_warp_sweeps(h->words[0], h->words[1], g, masks, done, part, every,
-                                   reinterpret_cast<long long*>(h->host_counts), h->t_dev, h->t, h->stream);
+                                   reinterpret_cast<long long*>(h->host_counts), h->t_dev, h->stream);
             if (e != cudaSuccess) return cuda_fail(e, "warp_sweeps_kernel");
+            h->t += (uint64_t)part;
             done += part;
         }
         return ISING_OK;
@@ -778,8 +781,8 @@ static int run_cluster(ising_lattice* h, int64_t n, int64_t every, unsigned long
         if (plan.v == 0) h->may_give_up = true;
         cudaError_t e =
             plan.v == 0 ? launch_band_sweeps(h->words[0], h->words[1], ci ? h->dense : nullptr, g, counts, slots, plan,
-                                             part_of(j), masks[j & 1], done, every, h->t_dev,
-                                             h->t + (uint64_t)(done + part_of(j)), gave_up_word(h), stall, h->stream)
+                                             part_of(j), masks[j & 1], done, every, h->t_dev, gave_up_word(h), stall,
+                                             h->stream)
                         : launch_cluster_sweeps(h->words[0], h->words[1], ci ? h->dense : nullptr, g, a, slots, plan,
                                                 part_of(j), masks[j & 1], done, every, x, h->stream);
         if (e != cudaSuccess) return cuda_fail(e, "cluster sweeps kernel");
@@ -797,7 +800,7 @@ static int run_cluster(ising_lattice* h, int64_t n, int64_t every, unsigned long
         if (e != cudaSuccess) return cuda_fail(e, "ci_from_dense");
     }
     if (n > 0) {
-        // the band kernel sets the counter itself
+        // the band kernel advances the counter itself
         cudaError_t e = plan.v == 0 ? cudaSuccess : launch_advance_sweep(h->t_dev, (uint64_t)n, h->stream);
         if (e != cudaSuccess) return cuda_fail(e, "advance_sweep_kernel");
         h->t += (uint64_t)n;

@@ -132,14 +132,14 @@ struct WarpLattice {
 // into a ring of STAGES stages of K sweeps, and the other warps (on the other
 // schedulers) count the records, (E, M) of the run's sweeps s with s % every == 0 to
 // records[2 (s / every - 1)], from the states that warp 0 leaves in shared
-// memory.  One barrier per stage.  At the end *t_dev = t_end.  Launched
+// memory.  One barrier per stage.  At the end *t_dev += n.  Launched
 // programmatically behind the mask draw, which no kernel overlaps, so the
 // lattice is there before the wait.
 template <int W, int RPL, bool TWO, int K, int STAGES>
 __global__ void __launch_bounds__(kWarpThreads)
 warp_sweeps_kernel(uint64_t* __restrict__ w0, uint64_t* __restrict__ w1, Geom g, DenseGeom d,
                    const uint4* __restrict__ masks, int s_base, int n, int every, long long* records,
-                   uint64_t* t_dev, uint64_t t_end)
+                   uint64_t* t_dev)
 {
     constexpr int C = W == 1 ? 1 : RPL;          // 16-byte mask chunks of a lane per half-sweep; also of a state
     static_assert(RPL * W == 2 * C, "a chunk holds the masks of two words");
@@ -282,7 +282,7 @@ warp_sweeps_kernel(uint64_t* __restrict__ w0, uint64_t* __restrict__ w1, Geom g,
                         lattice_words(g), __LINE__);
             }
         }
-    if (lane == 0) *t_dev = t_end;
+    if (lane == 0) atomicAdd(reinterpret_cast<unsigned long long*>(t_dev), (unsigned long long)n);
 }
 
 }  // namespace
@@ -310,20 +310,19 @@ cudaError_t launch_warp_mask_draw(int L, const SweepArgs& a, uint64_t t0, int ns
 }
 
 cudaError_t launch_warp_sweeps(uint64_t* w0, uint64_t* w1, const Geom& g, const uint64_t* masks, int s_base, int n,
-                               int every, long long* rec, uint64_t* t_dev, uint64_t t_end, cudaStream_t s)
+                               int every, long long* rec, uint64_t* t_dev, cudaStream_t s)
 {
     const DenseGeom d = warp_geom(g.L);
     const dim3 one(1), block(kWarpThreads);
     const uint4* m = reinterpret_cast<const uint4*>(masks);
     if (d.W == 1)
-        launch_pdl(warp_sweeps_kernel<1, 2, false, 8, 3>, one, block, s, w0, w1, g, d, m, s_base, n, every, rec, t_dev,
-                   t_end);
+        launch_pdl(warp_sweeps_kernel<1, 2, false, 8, 3>, one, block, s, w0, w1, g, d, m, s_base, n, every, rec, t_dev);
     else if (g.L % 4 == 0)
         launch_pdl(warp_sweeps_kernel<2, 4, false, 2, 5>, one, block, s, w0, w1, g, d, m, s_base, n, every, rec,
-                   t_dev, t_end);
+                   t_dev);
     else
-        launch_pdl(warp_sweeps_kernel<2, 4, true, 2, 5>, one, block, s, w0, w1, g, d, m, s_base, n, every, rec, t_dev,
-                   t_end);
+        launch_pdl(warp_sweeps_kernel<2, 4, true, 2, 5>, one, block, s, w0, w1, g, d, m, s_base, n, every, rec,
+                   t_dev);
     return cudaGetLastError();
 }
 
