@@ -240,7 +240,9 @@ int ising_set_tiling(ising_lattice *h, int32_t rows_per_thread,
  * for the library's choice (1).  With F > 1 lanes, lane q of an item
  * (4 rows x 1 word) draws the fields q, q + F, ... and the lanes merge their
  * accept bits with warp shuffles: F times the threads, each with 1/F of the
- * item's Philox calls.  No counterpart in the paper
+ * item's Philox calls.  It applies to launches outside the replayed graphs
+ * (the sweeps that fill no whole graph, and sides without graphs); the graphs
+ * use 1.  No counterpart in the paper
  * (a scheduling choice); results do not depend on it.  Row-packed layout
  * only (EINVAL otherwise; EINVAL for other values). */
 int ising_set_item_lanes(ising_lattice *h, int32_t lanes);
@@ -250,9 +252,9 @@ int ising_set_item_lanes(ising_lattice *h, int32_t lanes);
  * the one before finishes; up to 32768 thread items (L up
  * to about 2350, either layout) the launches of chunks of up to 32 sweeps are
  * captured once into CUDA graphs and replayed (recaptured after
- * ising_set_beta, ising_set_rng, ising_set_tiling, ising_set_item_lanes; a
- * device record index picks the count slots of each replay), because there
- * a half-sweep runs about as long as the host takes to launch it.
+ * ising_set_beta, ising_set_rng, ising_set_tiling; a device record index picks
+ * the count slots of each replay), because there a half-sweep runs about as long
+ * as the host takes to launch it.
  * ISING_PATH_RESIDENT: temporal blocking with the whole lattice on chip, all
  * requested sweeps in one launch (lattices with 2 L pitch 8 bytes <= 220 KB,
  * i.e. L up to about 740; larger -> EINVAL); it removes the per-sweep launch

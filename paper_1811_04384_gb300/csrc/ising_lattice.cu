@@ -332,12 +332,18 @@ static SweepArgs base_args(const ising_lattice* h)
     return a;
 }
 
-// Lanes per thread item on the launch path: the handle's choice, else 1.
-// With the draws running while the half-sweep before finishes, splitting an
-// item's draws no longer shortens a launch: measured on GB300 (graph replays,
-// sweeps without records, spin-updates/ns, 1 / 4 lanes) L = 300: 39 / 35;
-// L = 512: 100 / 96; L = 1008: 369 / 324; L = 2016: 1,164 / 751.
-static int item_lanes(const ising_lattice* h) { return h->item_lanes > 0 ? h->item_lanes : 1; }
+// Lanes per thread item on the launch path: the handle's choice, else 1, and 1
+// in the library's graphs.  With the draws running while the half-sweep before
+// finishes, splitting an item's draws no longer shortens a launch: measured on
+// GB300 (graph replays, sweeps without records, spin-updates/ns, 1 / 4 lanes)
+// L = 300: 39 / 35; L = 512: 100 / 96; L = 1008: 369 / 324; L = 2016: 1,164 /
+// 751; 8 lanes took 64 sweeps of L = 1024 from 215 us to 336 and of 2048 from
+// 376 to 660.  A handle's lanes apply where a launch costs the host more than
+// the GPU: the sweeps outside the graphs.
+static int item_lanes(const ising_lattice* h, bool captured)
+{
+    return h->item_lanes > 0 && !captured ? h->item_lanes : 1;
+}
 
 // One half-sweep of the handle's lattice in its layout on stream `st`
 // (`captured`: into one of the library's own graphs).
@@ -346,7 +352,7 @@ static cudaError_t launch_hs(const ising_lattice* h, cudaStream_t st, bool captu
 {
     if (h->layout == ISING_LAYOUT_COLUMN_INTERLEAVED)
         return ci_half_sweep(colour, update, record, h->words[0], h->g.L, a, captured, st);
-    const int F = item_lanes(h);
+    const int F = item_lanes(h, captured);
     if (update && F > 1)
         return launch_half_sweep_lanes(F, colour, record, h->words[colour], h->words[1 - colour], h->g, a, captured,
                                        st);
@@ -1412,7 +1418,6 @@ extern "C" int ising_set_item_lanes(ising_lattice* h, int32_t lanes)
     if (h->layout != ISING_LAYOUT_ROW_PACKED) return ISING_EINVAL;   // row-packed words only
     if (lanes != 0 && lanes != 1 && lanes != 2 && lanes != 4 && lanes != 8) return ISING_EINVAL;
     h->item_lanes = lanes;
-    drop_graphs(h);
     return ISING_OK;
 }
 

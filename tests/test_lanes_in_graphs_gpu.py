@@ -1,0 +1,56 @@
+"""Lanes per item (ising_set_item_lanes) leave the replayed graphs alone: whole
+graphs take the same time whatever the lanes, and sweeps in and outside the
+graphs are the oracle's."""
+import time
+
+import numpy as np
+import pytest
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ising():
+    import paper_1811_04384_gb300 as p
+    p.load()
+    return p
+
+
+@pytest.mark.parametrize("lanes", [2, 4, 8])
+def test_series(ising, lanes):
+    L, seed, n = 258, 5, 71                    # two graphs of 32 and 7 sweeps outside them
+    with ising.Lattice(L, seed) as lat:
+        lat.set_path(ising.ISING_PATH_LAUNCHES)
+        lat.init_hot()
+        lat.set_beta(0.44)
+        lat.sweep(33)
+        lat.set_item_lanes(lanes)              # the graph is there already
+        E, M = lat.sweep_record(n, 1)
+        S = lat.get_spins()
+    s = oracle.init_hot(L, seed)
+    oracle.run(s, seed, 0.44, 0, 33, 33)
+    Eo, Mo = oracle.run(s, seed, 0.44, 33, n, 1)
+    np.testing.assert_array_equal(E, Eo)
+    np.testing.assert_array_equal(M, Mo)
+    np.testing.assert_array_equal(S, s)
+
+
+# 64 sweeps, two whole graphs, took 376 us with 1 lane and 660 with 8 while the lanes applied to them
+def test_time(ising):
+    def best(lanes):
+        with ising.Lattice(2048, 5) as lat:
+            lat.set_path(ising.ISING_PATH_LAUNCHES)
+            lat.set_item_lanes(lanes)
+            lat.init_hot()
+            lat.set_beta(0.44)
+            times = []
+            for _ in range(8):
+                lat.energy()
+                t = time.perf_counter()
+                lat.sweep(64)
+                lat.energy()
+                times.append(time.perf_counter() - t)
+        return min(times)
+    assert best(8) < 1.3 * best(1)
