@@ -43,3 +43,34 @@ def test_counts_that_are_no_integers(monkeypatch, n):
     lat._h = None
     with pytest.raises(TypeError):
         lat.sweep_record(n, 1)
+
+
+@pytest.mark.parametrize("counts", [[], [0], [3], [2, 0, 5], [1] * 32, list(range(33)), [4] * 300])
+def test_arrays_of_a_batch(counts):
+    arrays, addresses = p._records(counts)
+    assert len(arrays) == len(addresses) == len(counts)
+    for k, (a, n) in enumerate(zip(arrays, counts)):
+        assert a.shape == (n,) and a.dtype == np.int64 and a.flags["C_CONTIGUOUS"] and not a.any()
+        if n:
+            assert addresses[k] == a.ctypes.data
+        a[:] = k
+    for k, a in enumerate(arrays):
+        assert (a == k).all()                         # none lies over another
+
+
+@pytest.mark.parametrize("counts,error", [([1, -1], ValueError), ([2.0], TypeError)])
+def test_arrays_of_a_batch_refused(counts, error):
+    with pytest.raises(error):
+        p._records(counts)
+
+
+def test_arrays_of_one_replica_take_microseconds():
+    """Two such calls are in every Batch.sweep (20 us each while they used NumPy
+    throughout, against the 6 us of an array and a ctypes pointer)."""
+    import timeit
+
+    def pointer():
+        a = np.zeros(20, dtype=np.int64)
+        return a, p._ptr_array([a], ctypes.c_int64)
+    pointer_s, records_s = (min(timeit.repeat(f, number=200, repeat=20)) for f in (pointer, lambda: p._records([20])))
+    assert records_s < 2 * pointer_s
