@@ -187,6 +187,15 @@ __device__ __forceinline__ void cl_update(const uint32_t (&m)[2 * V], uint32_t w
     }
 }
 
+// Draws of at most this many threads (one a dense word and sweep), which leave
+// most SMs idle for a chain of 64 calls, go to eight times the threads with a
+// chain of 8 (SPLIT in dense_mask_draw_kernel): us of a call of 5 recorded sweeps,
+// whole / split: L = 64 43 / 36, 512 39 / 34, 1008 (20,160 threads) 53 / 48, 1400
+// (38,500) 68 / 63, 1600 (52,000) 75 / 72; but of 10 of L = 1500 (90,000) 80 / 85.
+// Not beside a launch that applies masks: there the split costs SM time (300 of L =
+// 512 198 / 208).
+constexpr long long kSplitThreads = 50000;
+
 // Asynchronous copy of a unit's masks (V words of (r < thr1, r < thr0)) from p
 // to shared address dst.
 template <int V>
@@ -609,9 +618,10 @@ cudaError_t launch_cl_mask_draw(int L, const SweepArgs& a, uint64_t t0, int nswe
 {
     const DenseGeom d = dense_geom(L);
     const Strips st = make_strips(d.P, kDenseStripWords);
-    const uint32_t items = (uint32_t)((L + 3) / 4) * st.width;
+    const uint32_t groups = (uint32_t)(L + 3) / 4, items = groups * st.width;
+    const bool split = !overlap && (long long)groups * d.P * nsweeps <= kSplitThreads;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((items + 127) / 128, st.n, nsweeps);
+    cfg.gridDim = split ? dim3((4 * items + 127) / 128, st.n, 2 * nsweeps) : dim3((items + 127) / 128, st.n, nsweeps);
     cfg.blockDim = dim3(128);
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
@@ -620,8 +630,9 @@ cudaError_t launch_cl_mask_draw(int L, const SweepArgs& a, uint64_t t0, int nswe
     cfg.attrs = attr;
     cfg.numAttrs = overlap ? 1 : 0;
     const DenseOut to = {4u * (uint32_t)d.P, (uint32_t)d.P, (uint32_t)L * (uint32_t)d.P};
-    return a.rounds == 7 ? cudaLaunchKernelEx(&cfg, dense_mask_draw_kernel<7, 1>, d, st, a, t0, to, masks)
-                         : cudaLaunchKernelEx(&cfg, dense_mask_draw_kernel<10, 1>, d, st, a, t0, to, masks);
+    const auto draw = split ? (a.rounds == 7 ? dense_mask_draw_kernel<7, 4> : dense_mask_draw_kernel<10, 4>)
+                            : (a.rounds == 7 ? dense_mask_draw_kernel<7, 1> : dense_mask_draw_kernel<10, 1>);
+    return cudaLaunchKernelEx(&cfg, draw, d, st, a, t0, to, masks);
 }
 
 cudaError_t launch_cluster_sweeps(uint64_t* w0, uint64_t* w1, uint32_t* dense, const Geom& g, const SweepArgs& a,

@@ -146,12 +146,13 @@ struct DenseOut {
 // threshold is 2^32.  A block owns consecutive items (row group, word) of one
 // strip, as in half_sweep_kernel.
 // SPLIT = 1: a grid layer per sweep, a thread draws a whole word for both
-// colours from one table of first products.  SPLIT = 4, for lattices of at most
-// 64 items, where that would leave one half-empty warp per block with a chain
-// of 64 draws: a layer per half-sweep, and a thread draws a quarter of a word
-// (a byte of each mask).  The draws of 10 sweeps of L = 64 are a chain of 8
-// calls then instead of 64 (a call of 10 sweeps 24.1 -> 20.4 us); 1024 sweeps
-// of L = 64 take 4.1 us.  Without a split: 1,744 sites/ns at L = 2016.
+// colours from one table of first products.  SPLIT = 4, for the on-chip warp's
+// lattices of at most 64 items and the cluster path's short draws
+// (kSplitThreads), where that would leave most SMs without a warp and the others
+// with a chain of 64 draws: a layer per half-sweep, and a thread draws a quarter
+// of a word (a byte of each mask).  The draws of 10 sweeps of L = 64 are a chain
+// of 8 calls then instead of 64 (a call of 10 sweeps on chip 24.1 -> 20.4 us); 1024
+// sweeps of L = 64 take 4.1 us.  Without a split: 1,744 sites/ns at L = 2016.
 template <int ROUNDS, int SPLIT>
 __global__ void __launch_bounds__(128, 8)
 dense_mask_draw_kernel(DenseGeom d, Strips st, SweepArgs a, uint64_t t0, DenseOut to, uint64_t* __restrict__ masks)
