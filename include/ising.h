@@ -281,7 +281,8 @@ int ising_set_item_lanes(ising_lattice *h, int32_t lanes);
  * that (on a device without clusters: resident up to 512 items, L <= 292, then
  * the launch path); column-interleaved: the cluster path up to L = 2604, the
  * launch path above.  Clusters by size: one up to L = 1150, two to 1600, three
- * to 2400, then four.
+ * to 2400, then four; a call of at most 20 sweeps takes one where the lattice
+ * fits it.
  * Results are identical on every path. */
 #define ISING_PATH_AUTO 0
 #define ISING_PATH_LAUNCHES 1

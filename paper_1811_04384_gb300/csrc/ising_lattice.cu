@@ -680,28 +680,40 @@ static int auto_clusters_of(const ising_lattice* h)
     return auto_clusters(h->g.L, h->layout == ISING_LAYOUT_COLUMN_INTERLEAVED);
 }
 
-// The cluster-path launch for h: the clusters set by ising_set_clusters, else
+// A call of at most kShortCall sweeps has nothing to overlap its first draw
+// with, and one cluster saves the exchange's status words, their copy and the
+// wait for it: us of a recorded call of 5 / 10 / 20 / 50 sweeps with one cluster
+// against two, L = 1200: 52 / 64 / 88 / 145 against 63 / 74 / 90 / 151; L = 1600: 63
+// / 79 / 113 / 212 against 73 / 86 / 112 / 201; interleaved L = 1512: 66 / 76 / 105 /
+// 181 against 78 / 84 / 116 / 186.
+constexpr int kShortCall = 20;
+
+// The cluster-path launch of n sweeps for h: the clusters set by
+// ising_set_clusters, else one for a short call if one holds the lattice, else
 // the automatic count, or fewer where the device holds fewer clusters at
 // once; one cluster on the automatic path once a launch found its blocks
 // not all resident together (other work held SMs); `forced`
 // (ISING_PATH_CLUSTER) also takes one cluster at any size it fits.
-static bool plan_cluster(const ising_lattice* h, ClusterPlan* plan, bool forced)
+static bool plan_cluster(const ising_lattice* h, ClusterPlan* plan, bool forced, int64_t n)
 {
     if (h->clusters > 0) return plan_cluster_g(h, h->clusters, plan);
     int G0 = auto_clusters_of(h);
+    if (n <= kShortCall && G0 > 1 && plan_cluster_g(h, 1, plan)) return true;
     if (h->multi_gave_up && h->path == ISING_PATH_AUTO) G0 = std::min(G0, 1);
     for (int G = G0; G >= 1; --G)
         if (plan_cluster_g(h, G, plan)) return true;
     return forced && plan_cluster_g(h, 1, plan);
 }
 
-static bool use_cluster(const ising_lattice* h, ClusterPlan* plan)
+// Whether a call of n sweeps takes the cluster path (which does not depend on
+// n), and its launch.
+static bool use_cluster(const ising_lattice* h, ClusterPlan* plan, int64_t n)
 {
     if (h->chain != ISING_CHAIN_CHECKERBOARD) return false;
-    if (h->path == ISING_PATH_CLUSTER) return plan_cluster(h, plan, true);
+    if (h->path == ISING_PATH_CLUSTER) return plan_cluster(h, plan, true, n);
     if (h->path != ISING_PATH_AUTO || use_resident(h)) return false;
     if (h->clusters == 0 && auto_clusters_of(h) == 0) return false;
-    return plan_cluster(h, plan, false);
+    return plan_cluster(h, plan, false, n);
 }
 
 // n sweeps on the cluster path; every > 0: after every `every`-th sweep s of
@@ -902,7 +914,7 @@ extern "C" int ising_set_path(ising_lattice* h, int32_t path)
     if (path == ISING_PATH_RESIDENT && (h->layout != ISING_LAYOUT_ROW_PACKED || resident_bytes(h->g) > kResidentMaxBytes))
         return ISING_EINVAL;
     ClusterPlan cp;
-    if (path == ISING_PATH_CLUSTER && !plan_cluster(h, &cp, true)) return ISING_EINVAL;
+    if (path == ISING_PATH_CLUSTER && !plan_cluster(h, &cp, true, INT64_MAX)) return ISING_EINVAL;
     h->path = path;
     h->multi_gave_up = false;
     return ISING_OK;
@@ -914,7 +926,7 @@ extern "C" int ising_get_path(ising_lattice* h, int32_t* path)
     ClusterPlan cp;
     if (h->chain == ISING_CHAIN_RANDOM_WORDS) *path = h->path;
     else if (use_resident(h)) *path = ISING_PATH_RESIDENT;
-    else if (use_cluster(h, &cp)) *path = ISING_PATH_CLUSTER;
+    else if (use_cluster(h, &cp, INT64_MAX)) *path = ISING_PATH_CLUSTER;
     else *path = ISING_PATH_LAUNCHES;
     return ISING_OK;
 }
@@ -1012,7 +1024,7 @@ extern "C" int ising_sweep(ising_lattice* h, int64_t n)
         return ISING_OK;
     }
     ClusterPlan cp;
-    if (use_cluster(h, &cp)) {
+    if (use_cluster(h, &cp, n)) {
         while (n > 0) {
             const int64_t c = n > (1 << 30) ? (1 << 30) : n;
             int rc = run_cluster(h, c, 0, h->counts, cp);
@@ -1085,7 +1097,7 @@ extern "C" int ising_sweep_record(ising_lattice* h, int64_t n, int64_t every, in
         // one cluster adds few counts to a record (64 warps, or 16 blocks): one slot,
         // and a 32nd of the clearing, copying and adding up (500 sweeps, all recorded,
         // of L = 160: 241 -> 219 us; of L = 296: 292 -> 287)
-        const bool cluster = h->chain == ISING_CHAIN_CHECKERBOARD && use_cluster(h, &cp);
+        const bool cluster = h->chain == ISING_CHAIN_CHECKERBOARD && use_cluster(h, &cp, chunk * every);
         const int slots = cluster && cp.clusters == 1 ? 1 : kCountSlots;
         const size_t bytes = (size_t)chunk * slots * 2 * sizeof(unsigned long long);
         cudaError_t e = cudaMemsetAsync(h->counts, 0, bytes, h->stream);
@@ -1295,7 +1307,7 @@ extern "C" int ising_run_states(ising_lattice* h, const int8_t* const* states, i
             const int64_t base = (k - k0) * R;
             const auto packed = [h, b] { return cudaEventRecord(h->ev_packed[b], h->stream); };
             ClusterPlan cp;
-            if (use_cluster(h, &cp)) {
+            if (use_cluster(h, &cp, sweeps)) {
                 e = packed();
                 if (e != cudaSuccess) break;
                 rc = run_cluster(h, sweeps, every, h->counts + (size_t)base * rec_words, cp);
