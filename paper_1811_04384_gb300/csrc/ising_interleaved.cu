@@ -131,14 +131,21 @@ ci_half_sweep_kernel(uint64_t* S, int L, int N, SweepArgs a)
 // word row I and 64 columns: lane l holds the words of columns 64 w + 2 l and
 // + 1, whose sites in row i = I + kN are bit l of dense word w of colours i & 1
 // and 1 - (i & 1); a ballot per field gathers them.  Both read and write each
-// word once, coalesced on the word side.
+// word once, coalesced on the word side.  As plain launches around a call they
+// cost a short one 5 us (one sweep of L = 168 27.9 us, 22.8 before there was a
+// dense form).  So the first is launched programmatically behind the draw of the
+// call's first masks, which it shares nothing with: the draw is a plain launch, so
+// the lattice is there, and all that is left is to end after it.
 constexpr int kCiDenseWarps = 4;
 
 __global__ void __launch_bounds__(32 * kCiDenseWarps)
 ci_to_dense_kernel(const uint64_t* __restrict__ S, int L, int N, DenseGeom d, uint32_t* __restrict__ dense)
 {
     const int w = blockIdx.x * kCiDenseWarps + (int)threadIdx.x / 32, I = blockIdx.y, lane = threadIdx.x & 31;
-    if (w >= d.W) return;                             // uniform over the warp
+    if (w >= d.W) {                                   // uniform over the warp
+        pdl_wait();
+        return;
+    }
     const int J = 64 * w + 2 * lane;
     const uint64_t n = (uint64_t)N * L, nd = 2 * (uint64_t)L * d.P;
     uint64_t x = 0, y = 0;
@@ -164,11 +171,16 @@ ci_to_dense_kernel(const uint64_t* __restrict__ S, int L, int N, DenseGeom d, ui
             half_st(dense, ((uint64_t)(1 - c) * L + i) * d.P + w + 1, 0u, nd, __LINE__);
         }
     }
+    pdl_wait();
 }
 
+// Also *t_dev += n, if not null.
 __global__ void __launch_bounds__(32 * kCiDenseWarps)
-ci_from_dense_kernel(uint64_t* __restrict__ S, int L, int N, DenseGeom d, const uint32_t* __restrict__ dense)
+ci_from_dense_kernel(uint64_t* S, int L, int N, DenseGeom d, const uint32_t* dense, unsigned long long* t_dev,
+                     unsigned long long n_sweeps)
 {
+    pdl_wait();
+    if (t_dev && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) atomicAdd(t_dev, n_sweeps);
     const int w = blockIdx.x * kCiDenseWarps + (int)threadIdx.x / 32, I = blockIdx.y, lane = threadIdx.x & 31;
     if (w >= d.W) return;
     const uint64_t n = (uint64_t)N * L, nd = 2 * (uint64_t)L * d.P;
@@ -513,15 +525,19 @@ cudaError_t ci_to_dense(const uint64_t* S, int L, uint32_t* dense, cudaStream_t 
 {
     const DenseGeom d = dense_geom(L);
     const dim3 grid((d.W + kCiDenseWarps - 1) / kCiDenseWarps, L / 21);
-    ci_to_dense_kernel<<<grid, 32 * kCiDenseWarps, 0, s>>>(S, L, L / 21, d, dense);
+    launch_pdl(ci_to_dense_kernel, grid, dim3(32 * kCiDenseWarps), s, S, L, L / 21, d, dense);
     return cudaGetLastError();
 }
 
-cudaError_t ci_from_dense(uint64_t* S, int L, const uint32_t* dense, cudaStream_t s)
+cudaError_t ci_from_dense(uint64_t* S, int L, const uint32_t* dense, uint64_t* t_dev, int64_t n, bool beside,
+                          cudaStream_t s)
 {
     const DenseGeom d = dense_geom(L);
     const dim3 grid((d.W + kCiDenseWarps - 1) / kCiDenseWarps, L / 21);
-    ci_from_dense_kernel<<<grid, 32 * kCiDenseWarps, 0, s>>>(S, L, L / 21, d, dense);
+    const dim3 block(32 * kCiDenseWarps);
+    auto* t = reinterpret_cast<unsigned long long*>(t_dev);
+    if (beside) launch_pdl(ci_from_dense_kernel, grid, block, s, S, L, L / 21, d, dense, t, (unsigned long long)n);
+    else ci_from_dense_kernel<<<grid, block, 0, s>>>(S, L, L / 21, d, dense, t, (unsigned long long)n);
     return cudaGetLastError();
 }
 

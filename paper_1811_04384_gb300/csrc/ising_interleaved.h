@@ -25,9 +25,14 @@ cudaError_t ci_half_sweep(int colour, bool update, bool record, uint64_t* S, int
 bool ci_valid_strips(int32_t L, int32_t nstrips);   // nstrips divides L, L / nstrips >= 2
 size_t ci_rw_draw_bytes(int L, int nstrips);
 // The lattice to and from the dense array of the cluster path (cl_dense_bytes
-// in ising_internal.h): rows of one bit per spin, both colours.
+// in ising_internal.h): rows of one bit per spin, both colours.  ci_to_dense
+// comes directly after a plain launch that triggers its dependents and writes
+// neither array; it runs beside that launch and ends after it.  ci_from_dense
+// also advances *t_dev (if not null) by n, and with `beside` its blocks are placed
+// while the launch before, which triggers its dependents, runs.
 cudaError_t ci_to_dense(const uint64_t* S, int L, uint32_t* dense, cudaStream_t s);
-cudaError_t ci_from_dense(uint64_t* S, int L, const uint32_t* dense, cudaStream_t s);
+cudaError_t ci_from_dense(uint64_t* S, int L, const uint32_t* dense, uint64_t* t_dev, int64_t n, bool beside,
+                          cudaStream_t s);
 bool ci_rw_predraw(int L, int nstrips);
 cudaError_t ci_random_words_iteration(uint64_t* S, int L, int nstrips, const SweepArgs& a, ulonglong2* draws,
                                       cudaStream_t s);

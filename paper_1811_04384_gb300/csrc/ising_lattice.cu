@@ -744,17 +744,16 @@ static int run_cluster(ising_lattice* h, int64_t n, int64_t every, unsigned long
         const uint64_t t0 = h->t + (uint64_t)(j * max_piece);
         return launch_cl_mask_draw(g.L, a, t0, part_of(j), masks[j & 1], overlap, h->stream);
     };
-    // the column-interleaved layout's words become dense rows for the call
-    if (ci && np > 0) {
-        cudaError_t e = cudaSuccess;
-        if (!h->dense) e = cudaMalloc(&h->dense, cl_dense_bytes(g.L));
+    if (ci && np > 0 && !h->dense) {
+        cudaError_t e = cudaMalloc(&h->dense, cl_dense_bytes(g.L));
         if (e != cudaSuccess) { h->dense = nullptr; cuda_fail(e, "cudaMalloc dense rows"); return ISING_ENOMEM; }
-        e = ci_to_dense(h->words[0], g.L, h->dense, h->stream);
-        if (e != cudaSuccess) return cuda_fail(e, "ci_to_dense");
     }
     if (np > 0) {
         cudaError_t e = draw(0, false);
         if (e != cudaSuccess) return cuda_fail(e, "cluster mask draw");
+        // the column-interleaved layout's words become dense rows for the call
+        if (ci) e = ci_to_dense(h->words[0], g.L, h->dense, h->stream);
+        if (e != cudaSuccess) return cuda_fail(e, "ci_to_dense");
     }
     ClusterExchange x = {nullptr, nullptr, 0, nullptr, 0, nullptr, 0, 0};
     const uint64_t t_start = h->t;
@@ -813,14 +812,14 @@ static int run_cluster(ising_lattice* h, int64_t n, int64_t every, unsigned long
             if (e != cudaSuccess) return cuda_fail(e, "cluster mask draw");
         }
     }
-    if (ci && np > 0) {
-        cudaError_t e = ci_from_dense(h->words[0], g.L, h->dense, h->stream);
-        if (e != cudaSuccess) return cuda_fail(e, "ci_from_dense");
-    }
     if (n > 0) {
-        // the band kernel advances the counter itself
-        cudaError_t e = plan.v == 0 ? cudaSuccess : launch_advance_sweep(h->t_dev, (uint64_t)n, h->stream);
-        if (e != cudaSuccess) return cuda_fail(e, "advance_sweep_kernel");
+        // the band kernel advances the counter itself, else the words' launch does or one of its own.  That
+        // launch's blocks wait on their SMs beside a single piece only: longer they would keep others' out
+        uint64_t* const t_dev = plan.v == 0 ? nullptr : h->t_dev;
+        cudaError_t e = cudaSuccess;
+        if (ci) e = ci_from_dense(h->words[0], g.L, h->dense, t_dev, n, np == 1, h->stream);
+        else if (t_dev) e = launch_advance_sweep(t_dev, (uint64_t)n, h->stream);
+        if (e != cudaSuccess) return cuda_fail(e, "end of a cluster call");
         h->t += (uint64_t)n;
     }
     if (plan.clusters > 1) {
