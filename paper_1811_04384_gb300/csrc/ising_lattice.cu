@@ -640,12 +640,15 @@ static int run_resident(ising_lattice* h, int n, int every, bool* direct)
 // 1000 sweeps 352 / 352 / 357 / 349 / 365, 100 sweeps 66 / 71 / 77 / 81 / 80; L =
 // 1008, 500 sweeps 599 / 567 / 555 / 549 / 546, 100 sweeps 151 / 155 / 167 / - / -; L =
 // 1500, 400 sweeps 828 / 770 / 749 / 741 / 747; L = 2016, 300 sweeps 919 / 948 /
-// 940 / 940 / 932).  A column-interleaved lattice is converted to dense rows and back
+// 940 / 940 / 932), and of at least kPieceSites draws, which take 0.6 us: below
+// that there is nothing to overlap (100 sweeps of L = 128 in 2 pieces 77 us, in one
+// 63; of 100 84 and 68).  A column-interleaved lattice is converted to dense rows and back
 // around the call.
 constexpr int kClusterMaxL = 3000;
 constexpr int kCiClusterMaxL = 2604;               // the column-interleaved layout (L % 84 == 0)
 constexpr size_t kClusterMaskBytes = 256u << 20;   // both buffers
 constexpr int kClusterMaxPiece = 256, kClusterMinPiece = 30, kBandMinPiece = 50, kClusterPieces = 4;
+constexpr int64_t kPieceSites = 1000000;
 // The words between clusters (xflag, u64 each): 2 flags for each of at most
 // 16 boundaries, the error word of the waits (u32), the agreement words
 // (cl_decide: two sets of {count, verdict} and the first piece given up,
@@ -726,7 +729,8 @@ static int run_cluster(ising_lattice* h, int64_t n, int64_t every, unsigned long
     const bool ci = h->layout == ISING_LAYOUT_COLUMN_INTERLEAVED;
     const size_t per_sweep = cl_mask_bytes_per_sweep(g.L);
     const int64_t pieces = std::max<int64_t>(
-        1, std::min<int64_t>(kClusterPieces, n / (plan.v == 0 ? kBandMinPiece : kClusterMinPiece)));
+        1, std::min<int64_t>({(int64_t)kClusterPieces, n / (plan.v == 0 ? kBandMinPiece : kClusterMinPiece),
+                              n * g.L * g.L / kPieceSites}));
     const int64_t wanted = std::max<int64_t>(1, (n + pieces - 1) / pieces);
     const int max_piece = (int)std::max<size_t>(
         1, std::min<size_t>((size_t)std::min<int64_t>(wanted, kClusterMaxPiece), kClusterMaskBytes / (2 * per_sweep)));
