@@ -73,31 +73,42 @@ __global__ void ci_unpack_kernel(const uint64_t* __restrict__ S, int L, int N, i
 // launch operands only and run before the wait for the previous half-sweep
 // (see half_sweep_kernel).  RECORD (colour 1) also counts the anti-aligned
 // bonds of the four colour-1 words and the up spins of all eight words of
-// the block.
-template <int C, bool UPDATE, bool RECORD, int ROUNDS>
+// the block.  SPLIT, for sides with few threads (kCiSplitMaxL): the four warps of
+// a block share one row group, and a thread draws a quarter of the fields and
+// updates one row.
+template <int C, bool UPDATE, bool RECORD, int ROUNDS, bool SPLIT>
 __global__ void __launch_bounds__(kCiBlockX * kCiBlockY, 6)
 ci_half_sweep_kernel(uint64_t* S, int L, int N, SweepArgs a)
 {
-    __shared__ CiRowTable tab;
+    constexpr int GROUPS = SPLIT ? 1 : kCiBlockY, ROWS = SPLIT ? 1 : 4;
+    __shared__ uint4 tab[GROUPS * kFields];
+    __shared__ uint2 parts[SPLIT ? 4 : 1][4][kCiBlockX];
     pdl_launch();
     const int x = (int)threadIdx.x % kCiBlockX, y = (int)threadIdx.x / kCiBlockX;
-    const int m = (int)blockIdx.x * kCiBlockX + x, q = (int)blockIdx.y * kCiBlockY + y;
+    const int m = (int)blockIdx.x * kCiBlockX + x, q = (int)blockIdx.y * GROUPS + (SPLIT ? 0 : y);
+    const int e0 = SPLIT ? y : 0;                  // the thread's first row of the group
     const bool valid = m < L / 2 && q < N / 4;
     uint32_t anti = 0, up = 0;
     ItemMasks acc;
     if (UPDATE) {
         const uint64_t t = sweep_number(a);
-        ci_row_keys(tab, N, (int)blockIdx.y * kCiBlockY, t, C, a);
-        if (valid) ci_masks<ROUNDS>(tab, y, m, t, a, acc);
+        ci_row_keys<GROUPS>(tab, N, (int)blockIdx.y * GROUPS, t, C, a);
+        if constexpr (SPLIT) {
+            const uint2 r = ci_masks_split<ROUNDS>(tab, parts, y, x, m, t, a);
+            acc.m[0][0] = r.x;
+            acc.m[0][1] = r.y;
+        } else {
+            if (valid) ci_masks<ROUNDS>(tab, y, m, t, a, acc);
+        }
     }
     pdl_wait();
     if (valid) {
         const uint64_t n = (uint64_t)N * L;
-        uint64_t s[4], xl[4], xr[4], xu[4], xd[4], other[4];
-        int J[4];
+        uint64_t s[ROWS], xl[ROWS], xr[ROWS], xu[ROWS], xd[ROWS], other[ROWS];
+        int J[ROWS];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const int I = 4 * q + e;
+        for (int e = 0; e < ROWS; ++e) {
+            const int I = 4 * q + e0 + e;
             J[e] = 2 * m + ((I + C) & 1);
             const int Jl = J[e] == 0 ? L - 1 : J[e] - 1;
             const int Jr = J[e] == L - 1 ? 0 : J[e] + 1;
@@ -112,11 +123,11 @@ ci_half_sweep_kernel(uint64_t* S, int L, int N, SweepArgs a)
                                : word_ld<false>(S, (uint64_t)(I + 1) * L + J[e], n, __LINE__);
         }
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
+        for (int e = 0; e < ROWS; ++e) {
             uint64_t sn = s[e];
             if (UPDATE) {
                 sn = ci_flip(s[e], xu[e], xd[e], xl[e], xr[e], acc.m[e][0], acc.m[e][1]);
-                word_st(S, (uint64_t)(4 * q + e) * L + J[e], sn, n, __LINE__);
+                word_st(S, (uint64_t)(4 * q + e0 + e) * L + J[e], sn, n, __LINE__);
             }
             if (RECORD) ci_count(sn, xu[e], xd[e], xl[e], xr[e], other[e], anti, up);
         }
@@ -559,24 +570,34 @@ cudaError_t ci_unpack(const uint64_t* S, int L, int8_t* spins, cudaStream_t s)
     return cudaGetLastError();
 }
 
-template <int ROUNDS>
-static void ci_launch_r(dim3 grid, int colour, bool update, bool record, uint64_t* S, int L, int N,
-                        const SweepArgs& a, bool in_graphs, cudaStream_t s)
+// Up to this side a half-sweep is the chain of one thread's 21 calls and four
+// rows, on SMs with few warps.  64 sweeps in graphs, us, with the masks drawn in
+// launches of their own before / whole / split: L = 84 166 / 156 / 123; 252 184 /
+// 192 / 148; 504 190 / 197 / 154; 1008 222 / 208 / 165; 1512 329 / 228 / 195.
+constexpr int kCiSplitMaxL = 1512;
+
+template <int ROUNDS, bool SPLIT>
+static void ci_launch_r(int colour, bool update, bool record, uint64_t* S, int L, const SweepArgs& a, bool in_graphs,
+                        cudaStream_t s)
 {
-    const dim3 block(kCiBlockX * kCiBlockY);
-    if (!update) launch_pdl(ci_half_sweep_kernel<1, false, true, 10>, grid, block, s, S, L, N, a);
-    else if (colour == 0) launch_pdl_opt(in_graphs, ci_half_sweep_kernel<0, true, false, ROUNDS>, grid, block, s, S, L, N, a);
-    else if (record) launch_pdl_opt(in_graphs, ci_half_sweep_kernel<1, true, true, ROUNDS>, grid, block, s, S, L, N, a);
-    else launch_pdl_opt(in_graphs, ci_half_sweep_kernel<1, true, false, ROUNDS>, grid, block, s, S, L, N, a);
+    const int N = L / 21, groups = SPLIT ? 1 : kCiBlockY;
+    const dim3 grid((L / 2 + kCiBlockX - 1) / kCiBlockX, (N / 4 + groups - 1) / groups), block(kCiBlockX * kCiBlockY);
+    if (!update) launch_pdl(ci_half_sweep_kernel<1, false, true, 10, SPLIT>, grid, block, s, S, L, N, a);
+    else if (colour == 0) launch_pdl_opt(in_graphs, ci_half_sweep_kernel<0, true, false, ROUNDS, SPLIT>, grid, block, s, S, L, N, a);
+    else if (record) launch_pdl_opt(in_graphs, ci_half_sweep_kernel<1, true, true, ROUNDS, SPLIT>, grid, block, s, S, L, N, a);
+    else launch_pdl_opt(in_graphs, ci_half_sweep_kernel<1, true, false, ROUNDS, SPLIT>, grid, block, s, S, L, N, a);
 }
 
 cudaError_t ci_half_sweep(int colour, bool update, bool record, uint64_t* S, int L, const SweepArgs& a,
                           bool in_graphs, cudaStream_t s)
 {
-    const int N = L / 21;
-    const dim3 grid((L / 2 + kCiBlockX - 1) / kCiBlockX, (N / 4 + kCiBlockY - 1) / kCiBlockY);
-    if (a.rounds == 7) ci_launch_r<7>(grid, colour, update, record, S, L, N, a, in_graphs, s);
-    else ci_launch_r<10>(grid, colour, update, record, S, L, N, a, in_graphs, s);
+    if (L <= kCiSplitMaxL) {
+        if (a.rounds == 7) ci_launch_r<7, true>(colour, update, record, S, L, a, in_graphs, s);
+        else ci_launch_r<10, true>(colour, update, record, S, L, a, in_graphs, s);
+    } else {
+        if (a.rounds == 7) ci_launch_r<7, false>(colour, update, record, S, L, a, in_graphs, s);
+        else ci_launch_r<10, false>(colour, update, record, S, L, a, in_graphs, s);
+    }
     return cudaGetLastError();
 }
 
