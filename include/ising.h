@@ -558,7 +558,8 @@ int ising_autotune(int32_t L, int32_t sweeps, int32_t *best_block_words, int32_t
 
 /* Batch (arguments as ising_batch_create): threads per tile {64, 128, 256}
  * x graph chunk {10, 50, 200} x lanes {1, 2, 4}, `sweeps` timed sweeps per
- * replica with E/M every `every`-th sweep (1 <= every <= sweeps; the
+ * replica (1..100000, rounded up to a multiple of 200, after 200 that are not
+ * timed) with E/M every `every`-th sweep (1 <= every <= sweeps; the
  * kernels differ for every == 1).  Outputs may be NULL. */
 int ising_batch_autotune(int32_t n, const int32_t *L, const double *beta, const uint64_t *seed,
                          const uint8_t *hot, int64_t sweeps, int64_t every, int32_t *best_threads,

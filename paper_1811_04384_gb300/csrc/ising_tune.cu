@@ -105,9 +105,13 @@ extern "C" int ising_batch_autotune(int32_t n, const int32_t* L, const double* b
     const int threads[3] = {64, 128, 256};
     const int chunks[3] = {10, 50, 200};
     const int lanes[3] = {1, 2, 4};
+    // A call that is no multiple of a candidate's chunk runs the rest in other
+    // graphs than the candidate's, so all run whole chunks of the longest; the
+    // warm-up does too, and has captured what the timed call replays.
+    sweeps = (sweeps + chunks[2] - 1) / chunks[2] * chunks[2];
     double updates = 0.0;
     for (int r = 0; r < n; ++r) updates += (double)L[r] * L[r] * (double)sweeps;
-    std::vector<int64_t> sw(n, sweeps);
+    const std::vector<int64_t> sw(n, sweeps), warm(n, chunks[2]);
     std::vector<std::vector<int8_t>> ref(n), got(n);
     double best = -1.0;
     int bt = 128, bc = 50, bl = 4;
@@ -120,8 +124,7 @@ extern "C" int ising_batch_autotune(int32_t n, const int32_t* L, const double* b
             if (rc != ISING_OK) return rc;
             rc = ising_batch_set_tiling(b, threads[ti], chunks[ci]);
             if (rc == ISING_OK) rc = ising_batch_set_lanes(b, lanes[li]);
-            std::vector<int64_t> one(n, 1);
-            if (rc == ISING_OK) rc = ising_batch_sweep(b, one.data(), every == 1 ? 1 : 2, nullptr, nullptr);   // warm-up
+            if (rc == ISING_OK) rc = ising_batch_sweep(b, warm.data(), every, nullptr, nullptr);
             // ising_batch_sweep synchronises the batch's stream, so the host clock times it
             const auto t0 = std::chrono::steady_clock::now();
             if (rc == ISING_OK) rc = ising_batch_sweep(b, sw.data(), every, nullptr, nullptr);
