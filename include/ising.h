@@ -433,7 +433,10 @@ int ising_batch_get_sweep(ising_batch *b, int32_t r, uint64_t *t);
 int ising_batch_set_rng(ising_batch *b, int32_t scheme);
 
 /* Threads per tile (64, 128 or 256; default 128) and sweeps per captured
- * graph (1 .. 1024; default 50).  Rebuilds the tile table.  Results do not
+ * graph, a chunk (1 .. 1024; default 50).  A call runs whole chunks, then what
+ * is left in graphs of 10 sweeps, or in one more chunk where that leaves fewer
+ * than 10 sweeps of it without work, or at most 4 for each graph of 10.
+ * Rebuilds the tile table.  Results do not
  * depend on either. */
 int ising_batch_set_tiling(ising_batch *b, int32_t threads_per_tile, int32_t graph_chunk);
 

@@ -26,8 +26,14 @@ constexpr int kMaxLanes = 8;
 // Sweeps of the short graph that runs what is left of a call after whole
 // chunks.  A chunk's launches past the call's last sweep end at once, but each
 // still takes its 1.2 us or so: 20 sweeps of 64 replicas of L = 32 to 128 took 229
-// us in a chunk of 50 and 190 in two of 10, 256 of L = 32 to 512 614 and 534.
-constexpr int kRestChunk = 10;
+// us in a chunk of 50 and 190 in two of 10, 256 of L = 32 to 512 614 and 534.  But
+// a graph more costs what kRestEmpty sweeps without work do (us of either with 1
+// and 4 lanes: one replica of L = 64 2.3, 0.5; 63 of L = 32 to 128 4.5 and 8.9, 0.7;
+// 12 of L = 64 to 2048 7.1 and 9.8, 2.2; 256 of L = 32 to 512 7.4 and 10, 2.6), so a
+// whole chunk runs the rest where it has no more of these than that: 1000 sweeps
+// of a replica of L = 64 with chunks of 1024 took 3,371 us in a hundred short
+// graphs.
+constexpr int kRestChunk = 10, kRestEmpty = 4;
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 }  // namespace
@@ -372,9 +378,10 @@ extern "C" int ising_batch_sweep(ising_batch* b, const int64_t* sweeps, int64_t 
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync counts");
     e = cudaMemsetAsync(b->d_chunk_base, 0, sizeof(uint32_t), b->stream);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync chunk");
-    // whole chunks, then the rest in short ones unless those would come to a chunk
-    int64_t chunks = max_s / b->chunk, rests = (max_s % b->chunk + kRestChunk - 1) / kRestChunk;
-    if (rests * kRestChunk >= b->chunk) {
+    // whole chunks, then the rest in short ones unless those would come to a chunk or cost more than one
+    const int64_t rest = max_s % b->chunk;
+    int64_t chunks = max_s / b->chunk, rests = (rest + kRestChunk - 1) / kRestChunk;
+    if (rests > 0 && (rests * kRestChunk >= b->chunk || b->chunk - rest <= kRestEmpty * rests)) {
         chunks += 1;
         rests = 0;
     }
