@@ -357,13 +357,15 @@ int ising_cluster_inject_absent(ising_lattice *h, int32_t after);
  * chain the functions' "sweep" is the paper's iteration (10 update attempts
  * per spin on average, Table 2), and t counts iterations.  The strips of a
  * phase run in parallel, each strip's updates in its own sequence order, so
- * the result equals the sequential chain's.  Execution: the draws of an
- * iteration's updates are made first on all SMs, into a buffer of
- * 160 L^2 / 21 bytes the library allocates on first use (up to 256 MB,
- * L <= about 5900); with ISING_PATH_LAUNCHES, or above that size, each strip
- * draws its own updates.  A strip whose words fit in shared memory (N (h + 2)
- * words <= 160 KB) keeps them there for the phase.  Results are the same on
- * every form.  Errors: EINVAL (bad chain, nstrips not dividing L or
+ * the result equals the sequential chain's.  Execution: the updates of an
+ * iteration are drawn first on all SMs (L up to about 5900; with
+ * ISING_PATH_LAUNCHES, or above that size, each strip draws its own).  A half strip
+ * of up to about 1,280 words (N h) also has its updates planned ahead, each with
+ * what it waits for, for up to 16 iterations at a time.  Both go to one buffer that
+ * the library allocates on first use and keeps: about 165 L^2 / 21 bytes for each
+ * iteration, of which it holds up to 16, as many as 64 MB do (8 at L = 1008, one from
+ * L = 2900 on, 256 MB at most), or fewer where memory is short.  A wider one whose words fit in shared memory (N (h + 2) words <=
+ * 160 KB) keeps them there for the phase.  Results are the same on every form.  Errors: EINVAL (bad chain, nstrips not dividing L or
  * L / nstrips < 2, a row-packed lattice). */
 #define ISING_CHAIN_CHECKERBOARD 0
 #define ISING_CHAIN_RANDOM_WORDS 1

@@ -38,14 +38,16 @@ cudaError_t ci_random_words_iteration(uint64_t* S, int L, int nstrips, const Swe
                                       cudaStream_t s);
 // The same with the updates planned ahead (ising_words.cu), where a half strip
 // fits (words_planned): words_plan makes the plans of iterations
-// sweep_number(a) .. + iterations - 1 (words_plan_bytes each; at most
-// words_plan_iterations of the n that a call runs), words_run both phases of
+// sweep_number(a) .. + iterations - 1 (words_plan_bytes each; a buffer of
+// words_buffer_bytes holds `iterations` of them, or ci_rw_draw_bytes, for any
+// number of strips; words_most_iterations is as many as pay), words_run both phases of
 // the plan's iteration `iteration` (0: right after words_plan, or after the
 // phases before it); *err = 1 when a wait gave up; the first `stalls` (0 .. 2)
 // phases wait for what never comes (a test hook).
 bool words_planned(int L, int nstrips);
 size_t words_plan_bytes(int L, int nstrips);
-int words_plan_iterations(int L, int nstrips, int64_t n);
+size_t words_buffer_bytes(int L, int iterations);
+int words_most_iterations(int L);
 cudaError_t words_plan(int L, int nstrips, const SweepArgs& a, int iterations, void* plan, cudaStream_t s);
 cudaError_t words_run(uint64_t* S, int L, int nstrips, const void* plan, int iteration, unsigned int* err,
                       int stalls, cudaStream_t s);

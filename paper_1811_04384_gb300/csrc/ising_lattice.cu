@@ -68,7 +68,7 @@ struct ising_lattice {
     int chain = ISING_CHAIN_CHECKERBOARD;        // or the paper's random-word chain (interleaved layout)
     int nstrips = 1;                             // strips of the random-word chain
     ulonglong2* rw_draws = nullptr;              // random-word chain: the draws of one iteration, or plans (lazily)
-    size_t rw_draws_bytes = 0;
+    size_t rw_draws_bytes = 0;                   // words_buffer_bytes of as many iterations as there was room for
     cudaStream_t capture_stream = nullptr;       // graphs of sweep chunks are captured here
     cudaGraphExec_t graph_plain = nullptr;       // kGraphSweeps sweeps, no record
     cudaGraphExec_t graph_rec = nullptr;         // record intervals of graph_rec_every sweeps, each recorded
@@ -945,16 +945,22 @@ static int run_random_words(ising_lattice* h, int64_t n, RecOf rec_of)
     // chosen or the buffer would be too large; then each block draws its own
     const bool pre = h->path != ISING_PATH_LAUNCHES && ci_rw_predraw(h->g.L, h->nstrips);
     const bool planned = pre && words_planned(h->g.L, h->nstrips);
-    const int chunk = planned ? words_plan_iterations(h->g.L, h->nstrips, std::max<int64_t>(n, 1)) : 0;
-    const size_t need = planned ? (size_t)chunk * words_plan_bytes(h->g.L, h->nstrips)
-                                : (pre ? ci_rw_draw_bytes(h->g.L, h->nstrips) : 0);
-    if (h->rw_draws_bytes < need) {
-        if (h->rw_draws) cudaFree(h->rw_draws);
-        h->rw_draws_bytes = 0;
-        cudaError_t e = cudaMalloc(&h->rw_draws, need);
-        if (e != cudaSuccess) { h->rw_draws = nullptr; cuda_fail(e, "cudaMalloc random-word draws"); return ISING_ENOMEM; }
-        h->rw_draws_bytes = need;
+    // one buffer for good, whatever the strips and sweeps of the calls: a caller's graph of sweeps holds its
+    // address, and a stream that is being captured cannot wait for another.  Fewer iterations of plans where
+    // memory is short.
+    for (int its = words_most_iterations(h->g.L); pre && !h->rw_draws; its /= 2) {
+        const size_t bytes = words_buffer_bytes(h->g.L, its);
+        cudaError_t e = cudaMalloc(&h->rw_draws, bytes);
+        if (e == cudaSuccess) {
+            h->rw_draws_bytes = bytes;
+            break;
+        }
+        h->rw_draws = nullptr;
+        if (its == 1) { cuda_fail(e, "cudaMalloc random-word draws"); return ISING_ENOMEM; }
+        cudaGetLastError();
     }
+    const int chunk = planned ? (int)std::min<int64_t>(words_most_iterations(h->g.L),
+                                                       h->rw_draws_bytes / words_plan_bytes(h->g.L, h->nstrips)) : 0;
     for (int64_t it = 1; it <= n; ++it) {
         a.t_off = (uint32_t)it;
         a.counts = nullptr;

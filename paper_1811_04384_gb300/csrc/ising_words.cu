@@ -39,7 +39,7 @@ constexpr size_t kWordsSmemMax = 220 * 1024;
 constexpr int kWordsThreads = 1024;             // most threads of a strip, one or two words each
 constexpr int kWordsLooks = 4;                  // a thread's looks at its neighbours between two tests for the end
 constexpr uint32_t kWordsTries = 1u << 22;      // such rounds of looks before it gives up
-constexpr size_t kWordsPlanBytes = (size_t)64 << 20;
+constexpr size_t kWordsPlanBytes = (size_t)64 << 20;      // of a handle's plans (at least one iteration's)
 constexpr int kWordsPlanIterations = 16;
 constexpr uint32_t kWordBits = (1u << 21) - 1;
 constexpr int kWordIndexBits = 12;              // a half strip has at most 2 kWordsThreads words
@@ -368,10 +368,16 @@ bool words_planned(int L, int nstrips)
 
 size_t words_plan_bytes(int L, int nstrips) { return words_geom(L, nstrips).bytes(); }
 
-int words_plan_iterations(int L, int nstrips, int64_t n)
+// The starts of any number of strips come to at most N L + L.
+size_t words_buffer_bytes(int L, int iterations)
 {
-    const size_t most = std::max<size_t>(1, kWordsPlanBytes / words_plan_bytes(L, nstrips));
-    return (int)std::min<int64_t>(n, std::min<size_t>(most, kWordsPlanIterations));
+    const size_t NL = (size_t)(L / 21) * L;
+    return (size_t)iterations * ((10 * NL * sizeof(Entry) + (NL + L) * 4 + 255) / 256 * 256);
+}
+
+int words_most_iterations(int L)
+{
+    return (int)std::max<size_t>(1, std::min<size_t>(kWordsPlanBytes / words_buffer_bytes(L, 1), kWordsPlanIterations));
 }
 
 cudaError_t words_plan(int L, int nstrips, const SweepArgs& a, int iterations, void* plan, cudaStream_t s)
