@@ -53,6 +53,7 @@
 #include "ising_dense.cuh"
 #include "ising_device.cuh"
 #include "ising_internal.h"
+#include "ising_per_device.h"
 
 namespace cg = cooperative_groups;
 
@@ -500,23 +501,19 @@ size_t cl_smem_bytes(const DenseGeom& d, const ClusterPlan& p)
            (size_t)kDepth[form(p)] * kClThreads * p.ns * p.v * sizeof(uint64_t);
 }
 
-// Clusters of the largest size that can be resident at once (set by
-// probe_max_cluster).
-int g_max_active = 0;
+// The blocks of the largest cluster a device runs (0: none), and how many such
+// clusters can be resident at once.
+struct MaxCluster {
+    int size = 0, active = 0;
+};
 
-int probe_max_cluster()
+MaxCluster probe_max_cluster()
 {
-    if (!band_setup()) {
-        cudaGetLastError();
-        return 0;
-    }
+    if (!band_setup()) return {};
     for (ClusterKernel kern : kClusterKernels) {
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
-            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClSmemMax) !=
-                cudaSuccess) {
-            cudaGetLastError();
-            return 0;
-        }
+            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClSmemMax) != cudaSuccess)
+            return {};
     }
     for (int c : {16, 8}) {
         cudaLaunchConfig_t cfg = {};
@@ -537,24 +534,21 @@ int probe_max_cluster()
             ok = ok && cudaOccupancyMaxActiveClusters(&nc, kern, &cfg) == cudaSuccess && nc >= 1;
             active = std::min(active, nc);
         }
-        if (ok) {
-            g_max_active = active;
-            return c;
-        }
+        if (ok) return {c, active};
         cudaGetLastError();
     }
-    return 0;
+    return {};
 }
 
-int max_cluster_size()
+MaxCluster max_cluster()
 {
-    static const int c = probe_max_cluster();   // per process, set once
-    return c;
+    static PerDevice<MaxCluster> m;
+    return m.get(probe_max_cluster);
 }
 
 }  // namespace
 
-int cluster_max_active() { return max_cluster_size() == 0 ? 0 : g_max_active; }
+int cluster_max_active() { return max_cluster().active; }
 
 // The sides a launch of `blocks` blocks takes (the path's range): at least two
 // rows per block (four columns in the column-interleaved layout), and up to
@@ -577,8 +571,9 @@ bool cluster_side(int L, int blocks, bool interleaved)
 // units per thread and fits in shared memory.
 bool cluster_plan(int L, bool interleaved, int clusters, ClusterPlan* plan)
 {
-    const int c = max_cluster_size();
-    if (c == 0 || clusters < 1 || clusters > g_max_active) return false;
+    const MaxCluster most = max_cluster();
+    const int c = most.size;
+    if (c == 0 || clusters < 1 || clusters > most.active) return false;
     const int nb = clusters * c, fewest = L / nb;         // blocks of the launch
     if (!cluster_side(L, nb, interleaved)) return false;
     if (clusters == 1 && band_plan(L, c, plan)) return true;

@@ -19,6 +19,7 @@
 #include "ising_interleaved.cuh"
 #include "ising_dense.cuh"
 #include "ising_internal.h"
+#include "ising_per_device.h"
 
 namespace ising {
 namespace {
@@ -489,15 +490,17 @@ cudaError_t ci_random_words_iteration(uint64_t* S, int L, int nstrips, const Swe
     const int N = L / 21, NC = L / nstrips;
     const size_t win_bytes = (size_t)N * (NC - NC / 2 + 2) * sizeof(uint64_t);
     const bool win = win_bytes <= kRwWinBytesMax;
-    static bool attr_set = false;   // per process; the attribute is per function
-    if (win && !attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(ci_rw_phase_kernel<true, true>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRwWinBytesMax);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(ci_rw_phase_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)kRwWinBytesMax);
+    static PerDevice<cudaError_t> attr;
+    if (win) {
+        const cudaError_t e = attr.get([] {
+            const cudaError_t r = cudaFuncSetAttribute(
+                ci_rw_phase_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRwWinBytesMax);
+            return r != cudaSuccess ? r
+                                    : cudaFuncSetAttribute(ci_rw_phase_kernel<false, true>,
+                                                           cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                           (int)kRwWinBytesMax);
+        });
         if (e != cudaSuccess) return e;
-        attr_set = true;
     }
     const bool pre = draws != nullptr;
     if (pre) {

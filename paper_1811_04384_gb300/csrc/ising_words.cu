@@ -30,6 +30,7 @@
 #include "ising_interleaved.cuh"
 #include "ising_interleaved.h"
 #include "ising_internal.h"
+#include "ising_per_device.h"
 
 namespace ising {
 namespace {
@@ -347,14 +348,13 @@ size_t run_smem_bytes(const WordsGeom& g, int phase)
 
 bool words_setup()
 {
-    static const bool ok =      // per process, set once
-        cudaFuncSetAttribute(words_plan_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWordsSmemMax) ==
-            cudaSuccess &&
-        cudaFuncSetAttribute(words_run_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWordsSmemMax) ==
-            cudaSuccess &&
-        cudaFuncSetAttribute(words_run_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWordsSmemMax) ==
-            cudaSuccess;
-    return ok;
+    static PerDevice<bool> ok;
+    return ok.get([] {
+        constexpr auto kSmem = cudaFuncAttributeMaxDynamicSharedMemorySize;
+        return cudaFuncSetAttribute(words_plan_kernel, kSmem, (int)kWordsSmemMax) == cudaSuccess &&
+               cudaFuncSetAttribute(words_run_kernel<1>, kSmem, (int)kWordsSmemMax) == cudaSuccess &&
+               cudaFuncSetAttribute(words_run_kernel<2>, kSmem, (int)kWordsSmemMax) == cudaSuccess;
+    });
 }
 
 }  // namespace
