@@ -120,11 +120,17 @@ struct BandRow {
     }
 };
 
-// A row to a window of a block of the cluster; its 16 ceil(W / 4) bytes count
-// towards the block's barrier `bar`.
+// A row to a window of a block of the cluster, at byte `off` of its `bytes` at
+// `win`; its 16 ceil(W / 4) bytes count towards the block's barrier `bar`.
 template <int W>
-__device__ __forceinline__ void send(uint32_t to, uint32_t bar, const uint32_t (&x)[W])
+__device__ __forceinline__ void send(uint32_t win, uint32_t off, uint32_t bytes, uint32_t bar, const uint32_t (&x)[W])
 {
+#ifdef ISING_CHECKED
+    if (!check_index((uint64_t)off + (W + 3) / 4 * 16 - 1, bytes, __LINE__)) return;
+#else
+    (void)bytes;
+#endif
+    const uint32_t to = win + off;
 #pragma unroll
     for (int w = 0; w < W; w += 4)
         asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
@@ -239,6 +245,8 @@ band_sweeps_kernel(BandArgs a)
                 for (int h = 0; h < nh; ++h, src += plane, dst += slab * 16u) {
 #ifdef ISING_CHECKED
                     if (!check_index((uint64_t)(src - a.masks) + 1, (uint64_t)half_sweeps * plane, __LINE__)) continue;
+                    if (!check_index((dst - (uint32_t)__cvta_generic_to_shared(ring)) / 16u, 2u * k * slab, __LINE__))
+                        continue;
 #endif
                     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
                 }
@@ -301,7 +309,7 @@ band_sweeps_kernel(BandArgs a)
             for (int c = 0; c < 2; ++c)
 #pragma unroll
                 for (int q = 0; q < WV; ++q) {
-                    const uint4 v = *reinterpret_cast<const uint4*>(win + at(p & 1, c, row, 4 * q));
+                    const uint4 v = vector_ld(win, at(p & 1, c, row, 4 * q), win_words, __LINE__);
                     const uint32_t e[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
                     for (int w = 4 * q; w < min(W, 4 * q + 4); ++w) x.x[c][w] = e[w - 4 * q];
@@ -309,6 +317,9 @@ band_sweeps_kernel(BandArgs a)
             const uint4* m = ring + (p & 1) * k * slab + row * MP;
             uint4 m0[CH];
             auto load = [&](uint4 (&to)[CH], const uint4* from) {
+#ifdef ISING_CHECKED
+                if (!check_index((uint64_t)(from - ring) + CH - 1, 2u * k * slab + win_words / 4u, __LINE__)) from = ring;
+#endif
 #pragma unroll
                 for (int c = 0; c < CH; ++c) to[c] = from[c];
             };
@@ -346,9 +357,9 @@ band_sweeps_kernel(BandArgs a)
                 for (int c = 0; c < 2; ++c) {
                     const uint32_t o = 4u * at(to, c, row, 0), bar = 8u * to;
                     if (p + 1 < phases) {
-                        send(to_own + o, bar_own + bar, x.x[c]);
-                        if (r < k) send(to_up + o + 4u * WP * Sp, bar_up + bar, x.x[c]);
-                        if (r >= S - k) send(to_dn + o - 4u * WP * S, bar_dn + bar, x.x[c]);
+                        send(to_own, o, 4u * win_words, bar_own + bar, x.x[c]);
+                        if (r < k) send(to_up, o + 4u * WP * Sp, 4u * win_words, bar_up + bar, x.x[c]);
+                        if (r >= S - k) send(to_dn, o - 4u * WP * S, 4u * win_words, bar_dn + bar, x.x[c]);
                     } else {
 #pragma unroll
                         for (int w = 0; w < W; ++w) half_st(win, at(to, c, row, w), x.x[c][w], win_words, __LINE__);

@@ -172,7 +172,10 @@ dense_mask_draw_kernel(DenseGeom d, Strips st, SweepArgs a, uint64_t t0, DenseOu
     if (grp * 4u >= (uint32_t)d.L) return;
     const uint32_t live = dense_live(d, w) >> (N * part);
     const int c0 = SPLIT == 1 ? 0 : blockIdx.z & 1;
-    uint64_t* out = masks + (size_t)(2 * sweep + c0) * to.plane + grp * to.group + w;
+    uint64_t out = (uint64_t)(2 * sweep + c0) * to.plane + grp * to.group + w;
+#ifdef ISING_CHECKED
+    const uint64_t n = (uint64_t)gridDim.z * (SPLIT == 1 ? 2 : 1) * to.plane;
+#endif
 #pragma unroll 1
     for (int c = c0; c < (SPLIT == 1 ? 2 : c0 + 1); ++c, out += to.plane) {
         uint32_t m1[4] = {0, 0, 0, 0}, m0[4] = {0, 0, 0, 0};
@@ -186,11 +189,15 @@ dense_mask_draw_kernel(DenseGeom d, Strips st, SweepArgs a, uint64_t t0, DenseOu
             if (grp * 4u + e >= (uint32_t)d.L) continue;
             m1[e] = (m1[e] | a.all1) & live;
             m0[e] = (m0[e] | a.all0) & live;
+            uint64_t* const word = masks + out + (uint64_t)e * to.row;
+#ifdef ISING_CHECKED
+            if (!check_index(out + (uint64_t)e * to.row, n, __LINE__)) continue;
+#endif
             if constexpr (SPLIT == 1) {
-                out[(size_t)e * to.row] = (uint64_t)m0[e] << 32 | m1[e];
+                *word = (uint64_t)m0[e] << 32 | m1[e];
             } else {
                 static_assert(N == 8, "a part is a byte");
-                uint8_t* byte = reinterpret_cast<uint8_t*>(out + (size_t)e * to.row) + part;
+                uint8_t* byte = reinterpret_cast<uint8_t*>(word) + part;
                 byte[0] = (uint8_t)m1[e];
                 byte[4] = (uint8_t)m0[e];
             }

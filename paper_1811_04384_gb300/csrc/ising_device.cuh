@@ -59,11 +59,6 @@ __device__ __forceinline__ unsigned long long* record_counts(const SweepArgs& a)
 // launch operands only) overlaps the end of the previous grid.
 __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_enter()
-{
-    pdl_launch();
-    pdl_wait();
-}
 
 // The sweep number of a half-sweep, read before the wait: the device counter
 // is advanced only by a plain launch at the end of a chunk (or graph), which
@@ -135,6 +130,15 @@ __device__ __forceinline__ void half_st(uint32_t* p, uint64_t idx, uint32_t v, u
     if (!check_index(idx, n, line)) return;
 #endif
     p[idx] = v;
+}
+
+// Four 32-bit words from p[idx] on, idx a multiple of four.
+__device__ __forceinline__ uint4 vector_ld(const uint32_t* p, uint32_t idx, uint64_t n, uint32_t line)
+{
+#ifdef ISING_CHECKED
+    if (!check_index((uint64_t)idx + 3, n, line)) return make_uint4(0, 0, 0, 0);
+#endif
+    return *reinterpret_cast<const uint4*>(p + idx);
 }
 
 // The word, or the 32-bit half of one, at byte offset `o` of an array of n words.

@@ -162,7 +162,7 @@ __global__ void pack_rows_kernel(uint64_t* __restrict__ w0, uint64_t* __restrict
             const uint32_t bits = __funnelshift_r(d[0], d[1], (kFields * w) & 31);
             word = spread_fields(w == g.W - 1 ? bits & ((1u << g.rlast) - 1u) : bits);
         }
-        (c ? w1 : w0)[(size_t)i * g.P + w] = word;
+        word_st(c ? w1 : w0, (uint64_t)i * g.P + w, word, lattice_words(g), __LINE__);
     }
 }
 

@@ -192,13 +192,24 @@ words_plan_kernel(WordsGeom g, SweepArgs a, char* __restrict__ plan)
         words_calls<1>(philox_row_key(s, (uint32_t)t, x3, a.rk), first, a, m1, m0);
         e.x = (m1 | a.all1) & kWordBits;
         e.y = (m0 | a.all0) & kWordBits;
+#ifdef ISING_CHECKED
+        if (!check_index(pos, U, __LINE__)) continue;
+#endif
         entry[pos] = e;
     }
 }
 
-__device__ __forceinline__ uint64_t word_look(uint32_t addr)
+// The word at a shared address, one of the n at `win`.
+__device__ __forceinline__ uint64_t word_look(uint32_t addr, uint32_t win, uint64_t n, uint32_t line)
 {
     uint64_t v;
+#ifdef ISING_CHECKED
+    if (!check_index((addr - win) / 8u, n, line)) return 0;
+#else
+    (void)win;
+    (void)n;
+    (void)line;
+#endif
     asm volatile("ld.volatile.shared.u64 %0, [%1];" : "=l"(v) : "r"(addr) : "memory");
     return v;
 }
@@ -212,9 +223,17 @@ struct OwnWord {
     Entry e, next;                  // its next update and the one after
 };
 
-__device__ __forceinline__ Entry entry_ld(uint32_t addr)
+// The entry at a shared address, one of the n at `first`.
+__device__ __forceinline__ Entry entry_ld(uint32_t addr, uint32_t first, uint32_t n, uint32_t line)
 {
     Entry e;
+#ifdef ISING_CHECKED
+    if (!check_index((addr - first) / 16u, n, line)) return make_uint4(0, 0, 0, 0);
+#else
+    (void)first;
+    (void)n;
+    (void)line;
+#endif
     asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(e.x), "=r"(e.y), "=r"(e.z), "=r"(e.w) : "r"(addr));
     return e;
 }
@@ -268,13 +287,13 @@ words_run_kernel(uint64_t* S, WordsGeom g, int phase, bool fresh, const char* __
         o[k].at = win_sh + (uint32_t)I * row + 8u * (uint32_t)(j + 1);
         o[k].up = o[k].first_row ? o[k].at + (uint32_t)(g.N - 1) * row : o[k].at - row;
         o[k].dn = o[k].last_row ? o[k].at - (uint32_t)(g.N - 1) * row : o[k].at + row;
-        o[k].spins = (uint32_t)word_look(o[k].at);
+        o[k].spins = (uint32_t)word_look(o[k].at, win_sh, n_win, __LINE__);
         o[k].done = 0;
         o[k].count = has ? start[x + 1] - start[x] : 0u;
         // two entries past a word's last (never run) are other words', or the window's first bytes
         o[k].ahead = entry_sh + 16u * (start[x] + 2u);
-        o[k].e = entry_ld(o[k].ahead - 32u);
-        o[k].next = entry_ld(o[k].ahead - 16u);
+        o[k].e = entry_ld(o[k].ahead - 32u, entry_sh, U + 2, __LINE__);
+        o[k].next = entry_ld(o[k].ahead - 16u, entry_sh, U + 2, __LINE__);
         o[k].e.z |= stall;               // a test hook: a count that no word reaches
     }
     // rows whose neighbours come from across the top or bottom row: few warps have any
@@ -284,11 +303,15 @@ words_run_kernel(uint64_t* S, WordsGeom g, int phase, bool fresh, const char* __
     edge = __any_sync(0xffffffffu, edge);
     // a word changes by its own thread only, so there is no barrier from here on
     auto look = [&](OwnWord& w) {
-        const uint64_t up = word_look(w.up), dn = word_look(w.dn), lf = word_look(w.at - 8), rt = word_look(w.at + 8);
+        const uint64_t up = word_look(w.up, win_sh, n_win, __LINE__), dn = word_look(w.dn, win_sh, n_win, __LINE__);
+        const uint64_t lf = word_look(w.at - 8, win_sh, n_win, __LINE__), rt = word_look(w.at + 8, win_sh, n_win, __LINE__);
         // the counts are below 2^16: at most 20,480 updates of a half strip
         const uint32_t z = (uint32_t)(up >> 32) | (uint32_t)(dn >> 32) << 16;
         const uint32_t v = (uint32_t)(lf >> 32) | (uint32_t)(rt >> 32) << 16;
-        const bool ready = w.done < w.count && z == w.e.z && v == w.e.w;
+        bool ready = w.done < w.count && z == w.e.z && v == w.e.w;
+#ifdef ISING_CHECKED
+        ready = ready && check_index((w.ahead - entry_sh) / 16u, U + 2, __LINE__);
+#endif
         // straight-line: the lanes of a warp are seldom ready together
         uint32_t u = (uint32_t)up, d = (uint32_t)dn;
         if (edge) {
