@@ -552,9 +552,9 @@ int ising_server_inject_fault(ising_server *srv, int32_t epochs);
  * ising_batch_set_tiling); the Python binding keeps the choices in a JSON
  * table. */
 
-/* Single lattice of side L: the launch shapes of ising_set_tiling (1-D with
- * 64/128/192/256 threads, eleven 2-D block_words x block_groups) with one
- * thread per item, the 1-D shape with 2, 4 and 8 lanes per item
+/* Single lattice of side L: the launch shapes of ising_set_tiling that differ
+ * (64, 128, 192 and 256 threads a block, and 32 as 16 x 2) with one thread per
+ * item, 128 threads with 2, 4 and 8 lanes per item
  * (ising_set_item_lanes) and, if the lattice fits, the on-chip path;
  * `sweeps` timed sweeps each (1..100000) from a hot start at T = 2.269.
  * best_item_lanes is 0 for the on-chip path.  Outputs may be NULL. */

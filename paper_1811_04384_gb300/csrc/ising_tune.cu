@@ -68,11 +68,11 @@ extern "C" int ising_autotune(int32_t L, int32_t sweeps, int32_t* best_bw, int32
 {
     if (!ising::valid_side(L) || sweeps < 1 || sweeps > 100000) return ISING_EINVAL;
     const int P = ISING_PATH_LAUNCHES;
-    std::vector<Candidate> cands = {{0, 128, P, 1},  {0, 64, P, 1},   {0, 192, P, 1},  {0, 256, P, 1},
-                                    {32, 4, P, 1},   {16, 2, P, 1},   {16, 4, P, 1},   {16, 8, P, 1},
-                                    {16, 16, P, 1},  {32, 1, P, 1},   {32, 2, P, 1},   {32, 8, P, 1},
-                                    {64, 1, P, 1},   {64, 2, P, 1},   {64, 4, P, 1},   {0, 128, P, 2},
-                                    {0, 128, P, 4},  {0, 128, P, 8},  {0, 128, ISING_PATH_RESIDENT, 0}};
+    // strips hold at most 16 words, so shapes of as many threads are one shape: 16 x 2 stands for the
+    // only count that is not among the linear ones
+    std::vector<Candidate> cands = {{0, 128, P, 1}, {0, 64, P, 1},  {0, 192, P, 1},
+                                    {0, 256, P, 1}, {16, 2, P, 1},  {0, 128, P, 2},
+                                    {0, 128, P, 4}, {0, 128, P, 8}, {0, 128, ISING_PATH_RESIDENT, 0}};
     std::vector<uint64_t> ref, words;
     double best = -1.0;
     Candidate pick = cands[0];
