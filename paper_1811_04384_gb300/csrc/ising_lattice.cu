@@ -46,7 +46,9 @@ struct ising_lattice {
     Geom g;
     uint64_t seed = 0;
     uint64_t t = 0;              // host copy of the sweep counter
-    bool t_on_device = false;    // a caller's graph holds sweeps: only the device counter knows how many ran
+    bool captured = false;       // a caller's graph holds sweeps: only the device counter knows how many ran, and
+                                 // it holds the addresses of the masks
+    std::vector<void*> retired;  // buffers that such a graph may hold, kept until the end
     double beta = 0.0;
     uint64_t thr[2] = {0, 0};
     cudaStream_t stream = nullptr;
@@ -173,6 +175,7 @@ static void free_handle(ising_lattice* h)
     if (h->staging) cudaFree(h->staging);
     if (h->staging2) cudaFree(h->staging2);
     if (h->masks) cudaFree(h->masks);
+    for (void* p : h->retired) cudaFree(p);
     if (h->dense) cudaFree(h->dense);
     if (h->xbuf) cudaFree(h->xbuf);
     if (h->xflag) cudaFree(h->xflag);
@@ -468,13 +471,7 @@ template <typename RecOf, typename First = NoHook>
 static int run_sweeps(ising_lattice* h, int64_t n, RecOf rec_of, First after_first = First(), int64_t* owed = nullptr)
 {
     SweepArgs a = base_args(h);
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(h->stream, &cs) != cudaSuccess) {
-        cudaGetLastError();
-        cs = cudaStreamCaptureStatusActive;
-    }
-    if (cs != cudaStreamCaptureStatusNone) h->t_on_device = true;
-    if (!h->t_on_device) {
+    if (!h->captured) {
         a.t_base = nullptr;
         a.t0 = h->t;
     }
@@ -549,11 +546,20 @@ static bool use_resident(const ising_lattice* h)
 // at most this many bytes of sweeps at a time.
 constexpr size_t kMaskBufMax = 16u << 20;
 
-// The mask buffer of the on-chip paths, at least `need` bytes.
+// The mask buffer of the on-chip paths, at least `need` bytes.  One that a
+// caller's graph may hold outlives the larger one that takes its place.
 static int ensure_masks(ising_lattice* h, size_t need)
 {
     if (h->mask_bytes >= need) return ISING_OK;
-    if (h->masks) cudaFree(h->masks);
+    if (h->masks && h->captured) {
+        try {
+            h->retired.push_back(h->masks);
+        } catch (const std::bad_alloc&) {
+            return ISING_ENOMEM;
+        }
+    } else if (h->masks) {
+        cudaFree(h->masks);
+    }
     h->masks = nullptr;
     h->mask_bytes = 0;
     cudaError_t e = cudaMalloc(&h->masks, need);
@@ -1013,6 +1019,13 @@ extern "C" int ising_sweep(ising_lattice* h, int64_t n)
 {
     TraceRange trace("ising_sweep");
     if (!h || n < 0) return ISING_EINVAL;
+    // the one call that sweeps without waiting for the stream, so the one that can be captured
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(h->stream, &cs) != cudaSuccess) {
+        cudaGetLastError();
+        cs = cudaStreamCaptureStatusActive;
+    }
+    if (cs != cudaStreamCaptureStatusNone) h->captured = true;
     if (h->chain == ISING_CHAIN_RANDOM_WORDS) {
         while (n > 0) {
             const int64_t c = n > (1 << 30) ? (1 << 30) : n;
