@@ -96,8 +96,8 @@ __device__ __forceinline__ uint32_t even_bits(uint32_t v)
 // `in` may be device memory or pinned host memory mapped into the device's
 // address space.  In three steps through shared memory: four spins to a byte
 // of four bits (16 bytes a load when the rows are 16-byte aligned, else 4 with a
-// shift by the row's offset, or single bytes when `in` itself is not 4-byte
-// aligned), those to dense bits of the two colours, and 21 of those to a word.
+// shift by the row's offset, or a byte per lane and a ballot when `in` itself is
+// not 4-byte aligned: four bytes a thread took 0.5 us more), those to dense bits of the two colours, and 21 of those to a word.
 // Gathering each word's 21 bytes from a staged row took 14.4 us at L = 4096 and
 // 49 at L = 5000, where the rows were staged byte by byte: 10.6 and 18.5 so.
 // Launches that wait (pdl_wait) may start beside it.
@@ -134,10 +134,12 @@ __global__ void pack_rows_kernel(uint64_t* __restrict__ w0, uint64_t* __restrict
             nibbles[k] = (uint8_t)spin_nibble(v);
         }
     } else {
-        for (int k = threadIdx.x; 4 * k < g.L; k += blockDim.x) {
-            uint32_t v = 0;
-            for (int e = 0; e < 4 && 4 * k + e < g.L; ++e) v |= (uint32_t)(uint8_t)src[4 * k + e] << (8 * e);
-            nibbles[k] = (uint8_t)spin_nibble(v);
+        // a byte per lane, 32 bits at a time
+        const int lane = threadIdx.x & 31;
+        for (int j0 = (int)threadIdx.x - lane; j0 < g.L; j0 += blockDim.x) {
+            const uint32_t up = __ballot_sync(0xffffffffu, j0 + lane < g.L && src[j0 + lane] > 0);
+            const uint32_t k = (uint32_t)j0 / 4 + lane;
+            if (lane < 8 && k < nn) nibbles[k] = (uint8_t)(up >> (4 * lane) & 15u);
         }
     }
     __syncthreads();
