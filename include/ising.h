@@ -237,7 +237,8 @@ int ising_set_tiling(ising_lattice *h, int32_t rows_per_thread,
                      int32_t block_words, int32_t block_groups);
 
 /* Lanes per thread item on the launch path: 1, 2, 4 or 8, or 0 (default)
- * for the library's choice (1).  With F > 1 lanes, lane q of an item
+ * for the library's choice (4 up to 8192 items, i.e. L up to 1168; 1
+ * above).  With F > 1 lanes, lane q of an item
  * (4 rows x 1 word) draws the fields q, q + F, ... and the lanes merge their
  * accept bits with warp shuffles: F times the threads, each with 1/F of the
  * item's Philox calls.  It applies to launches outside the replayed graphs

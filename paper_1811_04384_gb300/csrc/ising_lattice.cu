@@ -335,17 +335,22 @@ static SweepArgs base_args(const ising_lattice* h)
     return a;
 }
 
-// Lanes per thread item on the launch path: the handle's choice, else 1, and 1
-// in the library's graphs.  With the draws running while the half-sweep before
-// finishes, splitting an item's draws no longer shortens a launch: measured on
-// GB300 (graph replays, sweeps without records, spin-updates/ns, 1 / 4 lanes)
-// L = 300: 39 / 35; L = 512: 100 / 96; L = 1008: 369 / 324; L = 2016: 1,164 /
-// 751; 8 lanes took 64 sweeps of L = 1024 from 215 us to 336 and of 2048 from
-// 376 to 660.  A handle's lanes apply where a launch costs the host more than
-// the GPU: the sweeps outside the graphs.
+// Lanes per thread item on the launch path.  In the library's graphs 1: with the
+// draws running while the half-sweep before finishes, splitting an item's draws
+// no longer shortens a launch: measured on GB300 (graph replays, sweeps without
+// records, spin-updates/ns, 1 / 4 lanes) L = 300: 39 / 35; L = 512: 100 / 96;
+// L = 1008: 369 / 324; L = 2016: 1,164 / 751; 8 lanes took 64 sweeps of L = 1024
+// from 215 us to 336 and of 2048 from 376 to 660.  Outside them, where a call is
+// few launches that the host makes, the handle's choice, else 4 up to 8192 items (L
+// up to 1168) and 1 above: us of a call of 1 / 5 recorded sweeps, 1 against
+// 4 lanes, L = 64: 24.4 / 43.2 against 22.4 / 36.6; L = 512: 30.6 / 45.1 against 23.4
+// / 37.7; L = 1008: 30.7 / 45.2 against 24.4 / 43.9; L = 1500: 30.7 / 45.0 against
+// 30.5 / 45.1; L = 2016: 30.6 / 45.3 against 30.6 / 48.0.
 static int item_lanes(const ising_lattice* h, bool captured)
 {
-    return h->item_lanes > 0 && !captured ? h->item_lanes : 1;
+    if (captured) return 1;
+    if (h->item_lanes > 0) return h->item_lanes;
+    return ((h->g.L + 3) / 4) * h->g.W <= 8192 ? 4 : 1;
 }
 
 // One half-sweep of the handle's lattice in its layout on stream `st`

@@ -54,3 +54,33 @@ def test_time(ising):
                 times.append(time.perf_counter() - t)
         return min(times)
     assert best(8) < 1.3 * best(1)
+
+
+# the library's choice of lanes outside the graphs: one sweep of L = 512 took 27.5 us with four, and 30.6 while it was one
+def test_short_calls_choose_lanes(ising):
+    def best(lanes):
+        with ising.Lattice(512, 5) as lat:
+            lat.set_path(ising.ISING_PATH_LAUNCHES)
+            lat.set_item_lanes(lanes)
+            lat.init_hot()
+            lat.set_beta(0.44)
+            times = []
+            for _ in range(300):
+                t = time.perf_counter()
+                lat.sweep_record(5, 5)
+                times.append(time.perf_counter() - t)
+        return sorted(times)[60]
+    assert best(0) < 0.95 * best(1)
+
+
+@pytest.mark.parametrize("L", [4, 46, 1168, 1170])      # the smallest, and 8176 and 8204 items
+def test_choice_series(ising, L):
+    def series(lanes):
+        with ising.Lattice(L, 6) as lat:
+            lat.set_path(ising.ISING_PATH_LAUNCHES)
+            lat.set_item_lanes(lanes)
+            lat.init_hot()
+            lat.set_beta(0.44)
+            return [*lat.sweep_record(7, 1), lat.get_spins()]
+    for a, b in zip(series(0), series(1)):
+        np.testing.assert_array_equal(a, b)
