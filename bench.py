@@ -524,15 +524,16 @@ def cluster_launches(L: int, sweeps: int, every: int) -> int:
 def midsize_launches(L: int, sweeps: int, every: int) -> int:
     """Kernel launches of ising_sweep_record(sweeps, every), sweeps a multiple
     of every, on one cluster: per chunk of 1024 records, up to four equal pieces
-    of at least 50 sweeps (rows of up to 14 dense words) or 30, 256 at most, each a
-    mask draw and a cluster launch; beyond 14 words a counter advance."""
+    of at least 50 sweeps (rows of up to 14 dense words) or 30 and 10^6 draws, 256
+    sweeps at most, each a mask draw and a cluster launch; beyond 14 words a counter
+    advance."""
     words = -(-(L // 2) // 32)
     band = words <= 14
     per_sweep = 2 * L * ((words + 1) // 2 * 2) * 8
     launches, left = 0, sweeps
     while left > 0:
         n = min(left, 1024 * every)
-        pieces = max(1, min(4, n // (50 if band else 30)))
+        pieces = max(1, min(4, n // (50 if band else 30), n * L * L // 10**6))
         piece = min(-(-n // pieces), 256, (256 << 20) // (2 * per_sweep))
         launches += 2 * -(-n // piece) + (0 if band else 1)
         left -= n

@@ -443,7 +443,7 @@ int ising_batch_set_rng(ising_batch *b, int32_t scheme);
  * depend on either. */
 int ising_batch_set_tiling(ising_batch *b, int32_t threads_per_tile, int32_t graph_chunk);
 
-/* Lanes (1 .. 8; default 2): the replicas are split, largest first, into
+/* Lanes (1 .. 8; default 4): the replicas are split, largest first, into
  * `lanes` groups of about equal work (sum of L^2), and each group is an
  * independent branch of the captured graph, so the blocks of one lane can
  * fill SMs that another lane's last wave of blocks leaves idle.  No
@@ -586,8 +586,9 @@ int ising_probe_int_pipes(double *mulwide_per_sm_clk, double *mad32_per_sm_clk, 
 /* Memory-safety check of the checked build (no counterpart in the paper).  A
  * library built with -DISING_CHECKED (paper_1811_04384_gb300.build.build(
  * checked=True), libising_checked.so) range-checks every lattice-word index of
- * the sweep, apply, batch, on-chip, column-interleaved and random-word
- * kernels against the array it indexes; an index out of range is not
+ * the sweep, apply, batch, on-chip, cluster, column-interleaved and random-word
+ * kernels, and those of the masks, plans and rows that they pass on, against
+ * the array it indexes; an index out of range is not
  * accessed (loads give 0, stores are dropped, nothing traps) and the first
  * one is recorded on the device.  *checked = 1 for that build, 0 for the
  * normal one (whose kernels check nothing).  *first_violation = 0 if no index
@@ -617,9 +618,9 @@ int ising_check_status(int32_t *checked, uint64_t *first_violation);
  * cudaStream_t `stream` (NULL = legacy default stream); the call
  * synchronises it before returning.
  *
- * Scratch: the count slots, per-record results and sweep counter live in one
- * fixed file-scope device array of about 528 KB, which every GPU that loads
- * the library holds until the process exits.  It holds at most
+ * Scratch: the count slots and per-record results live in one fixed file-scope
+ * device array of about 528 KB, which every GPU that loads the library holds
+ * until the process exits.  It holds at most
  * ISING_NOALLOC_MAX_RECORDS records per call; n / every above that returns
  * ISING_EINVAL before any device work.  The first call on each device looks
  * up the array's device address (cudaGetSymbolAddress) with that device
@@ -631,8 +632,8 @@ int ising_check_status(int32_t *checked, uint64_t *first_violation);
  * (each call clears the slots it uses first): calls that overlap on the GPU,
  * on any streams, race and give wrong results.
  *
- * Execution: two plain half-sweep launches per sweep with a fixed 2-D shape
- * (32 words x 4 row groups per block), no CUDA graphs and no on-chip path,
+ * Execution: two half-sweep launches per sweep with a fixed shape (strips of
+ * up to 16 words, 128 threads a block), no CUDA graphs and no on-chip path,
  * so small lattices run at the plain-launch rate, far below
  * ising_sweep_record's; results are identical (the draws are keyed by site).
  * Errors: EINVAL (NULL words, bad L, n < 0, every < 1, beta < 0 or NaN, too

@@ -510,7 +510,7 @@ __device__ __forceinline__ void sweep_item(uint64_t* own, const uint64_t* other,
     apply_item<C, true, RECORD>(own, other, g, grp, w, acc, anti, up);
 }
 
-// ---- Split forms of sweep_rows -------------------------------------------
+// ---- Split forms of an item's step ---------------------------------------
 // The work of an item in two parts: its accept masks (the Philox draws
 // against the thresholds; they depend on the site, sweep and colour only,
 // never on the spins) and their application to the item's rows.  So the
@@ -518,7 +518,8 @@ __device__ __forceinline__ void sweep_item(uint64_t* own, const uint64_t* other,
 // before the spins they apply to exist: F lanes per item on the launch path
 // for lattices too small to fill the GPU with one thread per item, and all
 // masks of a run drawn beforehand for the on-chip path.  The draws and the
-// accept rule are those of sweep_rows, so the results are bit-identical.  All
+// accept rule are those of draw_item and apply_item, so the results are
+// bit-identical.  All
 // lanes of a warp must call the lane forms (shuffles); an item past the end
 // (`valid` = false) is drawn as item 0 and never applied.
 
@@ -569,7 +570,7 @@ __device__ __forceinline__ void item_masks_lanes(const Geom& g, int item, int q,
 }
 
 // Apply the masks m1 (r < thr1) and m0 (r < thr0) of row i, word w of colour
-// C: the spin logic of sweep_rows for one row.  all0 / all1 are the "always"
+// C: the spin logic of apply_item for one row.  all0 / all1 are the "always"
 // masks (thresholds of 2^32) and live the row's live spin bits.  RECORD adds
 // the row's anti-aligned bonds and up spins to anti / up (colour 1).
 template <int C, bool RECORD>
@@ -584,7 +585,7 @@ __device__ __forceinline__ void row_apply(uint64_t* __restrict__ own, const uint
     const uint64_t u = word_ld<false>(other, (uint32_t)wrap_row(i - 1, g.L) * P + (uint32_t)w, n, __LINE__);
     const uint64_t d = word_ld<false>(other, (uint32_t)wrap_row(i + 1, g.L) * P + (uint32_t)w, n, __LINE__);
     const uint64_t h0 = word_ld<false>(other, o + (uint32_t)w, n, __LINE__);
-    // horizontal neighbour at m - 1 ((i + C) even) or m + 1 (odd), as in sweep_rows
+    // horizontal neighbour at m - 1 ((i + C) even) or m + 1 (odd), as in apply_item
     const bool left = ((i + C) & 1) == 0;
     const int ws = left ? ((w > 0) ? w - 1 : g.W - 1) : ((w < g.W - 1) ? w + 1 : 0);
     const int sh = (left ? (w > 0) : (w < g.W - 1)) ? 60 : 3 * (g.rlast - 1);
