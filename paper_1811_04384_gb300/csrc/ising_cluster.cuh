@@ -50,9 +50,10 @@ __device__ __forceinline__ unsigned int cl_load_acquire(const unsigned int* p)
 // are stale.  So a launch writes its lattice rows back only if all its blocks
 // were resident together, and all its blocks agree on that:
 //   gate[0..3]  two sets of {blocks counted in, verdict}, used by alternate
-//               pieces of a call (both zeroed before the call's first launch);
+//               pieces (numbered on through the calls; both are zero before the first);
 //   gate[4]     the first piece of the call whose launch gave up (kClNoPiece
-//               before it; the launches after it in the call do nothing).
+//               before it; the launches after it in the call do nothing, and the
+//               next call begins anew).
 // Every block counts in as it starts (cl_count_in, no wait) and decides at
 // its end, before the write-back (cl_decide): it proposes "go" (1) if it sees
 // all blocks counted in, else, after kClCheckInNs, "give up" (2).  The first

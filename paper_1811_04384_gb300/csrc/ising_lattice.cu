@@ -84,6 +84,7 @@ struct ising_lattice {
     size_t xbuf_bytes = 0;
     unsigned long long* xflag = nullptr;         // kXWords: their flags, the error word and the agreement words
     unsigned long long xseq = 0;                 // flag base of the next launch
+    unsigned int xpiece = 0;                     // number of the next launch among those that agree (0: words not set up)
     unsigned int* host_xerr = nullptr;           // pinned copy of the error and agreement words
     int stall_launches = 0;                      // test hook: launches whose waits between clusters give up
     bool may_give_up = false;                    // a launch that sets gave_up_word is not yet looked at
@@ -772,6 +773,7 @@ static int run_cluster(ising_lattice* h, int64_t n, int64_t every, unsigned long
     }
     ClusterExchange x = {nullptr, nullptr, 0, nullptr, 0, nullptr, 0, 0};
     const uint64_t t_start = h->t;
+    unsigned int piece0 = 0;                         // number of the call's first piece
     if (plan.clusters > 1) {
         const size_t xb = cl_exchange_words(g.L, plan) * sizeof(uint64_t);
         cudaError_t e = cudaSuccess;
@@ -791,16 +793,22 @@ static int run_cluster(ising_lattice* h, int64_t n, int64_t every, unsigned long
             h->xseq = 0;
         }
         unsigned int* gate = reinterpret_cast<unsigned int*>(h->xflag + kXGate);
-        // both agreement sets undecided, no piece given up
-        e = cudaMemsetAsync(gate, 0, 4 * sizeof(unsigned int), h->stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(gate + 4, 0xff, sizeof(unsigned int), h->stream);
-        if (e != cudaSuccess) return cuda_fail(e, "cluster agreement words");
+        // both agreement sets undecided, no piece given up: so does a call leave them whose launches all went
+        // on, and the next one numbers its pieces from there (two memsets were 2 us of a call)
+        if (h->xpiece == 0 || h->xpiece > 1u << 31) {
+            e = cudaMemsetAsync(gate, 0, 4 * sizeof(unsigned int), h->stream);
+            if (e == cudaSuccess) e = cudaMemsetAsync(gate + 4, 0xff, sizeof(unsigned int), h->stream);
+            if (e != cudaSuccess) return cuda_fail(e, "cluster agreement words");
+            h->xpiece = 1;
+        }
+        piece0 = h->xpiece;
+        h->xpiece = 0;                               // until the call has gone through
         x = {h->xbuf, h->xflag, h->xseq, reinterpret_cast<unsigned int*>(h->xflag + kXErr), 0, gate, 0, 0};
     }
     for (int64_t j = 0; j < np; ++j) {
         const int64_t done = j * max_piece;
         x.wait_add = 0;
-        x.piece = (unsigned int)j;
+        x.piece = piece0 + (unsigned int)j;
         x.absent = 0;
         if (plan.clusters > 1 && h->stall_launches > 0) {
             --h->stall_launches;
@@ -855,7 +863,7 @@ static int run_cluster(ising_lattice* h, int64_t n, int64_t every, unsigned long
             // it.  The pieces before it stand; its records are cleared and the
             // rest of the call runs on the launch path (the same draws, so the
             // same results); the automatic path keeps to one cluster from now on.
-            const int64_t done = (int64_t)gave_up * max_piece;
+            const int64_t done = (int64_t)(gave_up - piece0) * max_piece;
             h->multi_gave_up = true;
             rc = reset_t(h, t_start + (uint64_t)done);
             if (rc != ISING_OK) return rc;
@@ -870,6 +878,7 @@ static int run_cluster(ising_lattice* h, int64_t n, int64_t every, unsigned long
                 return (every > 0 && (done + s) % every == 0) ? (int)(rec_base + (done + s) / every - 1) : -1;
             });
         }
+        h->xpiece = piece0 + (unsigned int)np;
         // a wait between clusters that gave up while all were resident voids
         // the sweeps (the counter has advanced; the caller restores a
         // checkpoint to retry)

@@ -16,7 +16,7 @@
 // count of updates share 64 bits of shared memory, so one load gives both and
 // no barrier or fence is needed.  An update that is the oldest of all pending
 // ones never waits, so the phase always ends.  Measured on GB300, 5 iterations
-// of L = 1008 with 72 strips, a record after each: 798 -> 213 us, of which the
+// of L = 1008 with 72 strips, a record after each: 798 -> 202 us, of which the
 // plans take 54 and a phase 14.  (The plans of later iterations beside the
 // phases, on a second stream: 218 against 215.)  A phase is bound by latency: 15%
 // fewer instructions a look (the turns at the top and bottom rows in the warps that
