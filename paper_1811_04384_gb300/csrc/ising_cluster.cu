@@ -94,7 +94,7 @@ struct ClusterArgs {
     unsigned int* xerr;         // set to 1 when a wait for a flag gives up
     unsigned int* gate;         // G > 1: the words the blocks agree through (cl_count_in, cl_decide)
     unsigned int gate_blocks;   // blocks that must have counted in (the launch's; one more in a test)
-    unsigned int piece;         // the launch's piece of the call
+    unsigned int piece;         // the launch's number among those that agree
 };
 
 // Shared memory by 32-bit address: a half-sweep is short, and with generic

@@ -102,7 +102,7 @@ struct ClusterExchange {
     unsigned int* err;
     unsigned long long wait_add;   // added to the flag values a launch waits for (a test hook: nonzero stalls it)
     unsigned int* gate;            // the launch's agreement words (cl_count_in, cl_decide)
-    unsigned int piece;            // the launch's piece of the call
+    unsigned int piece;            // the launch's number among those that agree
     unsigned int absent;           // blocks counted on beyond the launch's (a test hook: 1 gives up)
 };
 constexpr int kClMaskPad = 8;
