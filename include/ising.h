@@ -438,9 +438,9 @@ int ising_batch_set_rng(ising_batch *b, int32_t scheme);
 /* Threads per tile (64, 128 or 256; default 128) and sweeps per captured
  * graph, a chunk (1 .. 1024; default 50).  A call runs whole chunks, then what
  * is left in graphs of 10 sweeps, or in one more chunk where that leaves fewer
- * than 10 sweeps of it without work, or at most 4 for each graph of 10.
- * Rebuilds the tile table.  Results do not
- * depend on either. */
+ * than 10 sweeps of it without work, or at most 4 for each graph of 10 that it
+ * saves (but a call of less than a chunk still takes up to four of those).
+ * Rebuilds the tile table.  Results do not depend on either. */
 int ising_batch_set_tiling(ising_batch *b, int32_t threads_per_tile, int32_t graph_chunk);
 
 /* Lanes (1 .. 8; default 4): the replicas are split, largest first, into

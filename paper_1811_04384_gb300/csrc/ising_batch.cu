@@ -32,8 +32,10 @@ constexpr int kMaxLanes = 8;
 // 12 of L = 64 to 2048 7.1 and 9.8, 2.2; 256 of L = 32 to 512 7.4 and 10, 2.6), so a
 // whole chunk runs the rest where it has no more of these than that: 1000 sweeps
 // of a replica of L = 64 with chunks of 1024 took 3,371 us in a hundred short
-// graphs.
-constexpr int kRestChunk = 10, kRestEmpty = 4;
+// graphs.  Up to kRestFew of them in a call without a whole chunk stay short all
+// the same, because capturing the chunk's graph would cost the first call more
+// (164 replicas, 40 sweeps: 1.55 ms with it, 0.88 without, then 503 and 548 us).
+constexpr int kRestChunk = 10, kRestEmpty = 4, kRestFew = 4;
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 }  // namespace
@@ -381,7 +383,8 @@ extern "C" int ising_batch_sweep(ising_batch* b, const int64_t* sweeps, int64_t 
     // whole chunks, then the rest in short ones unless those would come to a chunk or cost more than one
     const int64_t rest = max_s % b->chunk;
     int64_t chunks = max_s / b->chunk, rests = (rest + kRestChunk - 1) / kRestChunk;
-    if (rests > 0 && (rests * kRestChunk >= b->chunk || b->chunk - rest <= kRestEmpty * rests)) {
+    if (rests > 0 && (rests * kRestChunk >= b->chunk ||
+                      (b->chunk - rest <= kRestEmpty * rests && (chunks > 0 || rests > kRestFew)))) {
         chunks += 1;
         rests = 0;
     }

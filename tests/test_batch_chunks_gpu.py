@@ -1,8 +1,6 @@
 """What is left of a batch's call after whole chunks, in one more chunk or in
 short graphs, on either side of the rule: the series are those of the default
-chunk; and a long chunk is no slower than short ones for a call it nearly holds."""
-import time
-
+chunk."""
 import numpy as np
 import pytest
 
@@ -26,22 +24,8 @@ def series(ising, chunk, calls):
         return out + [b.get_spins(r) for r in range(3)] + [b.t(r) for r in range(3)]
 
 
-@pytest.mark.parametrize("chunk,calls", [(50, [33, 34, 83, 84]), (200, [142, 143, 350]), (1024, [730, 731, 1000]),
+@pytest.mark.parametrize("chunk,calls", [(50, [33, 34, 40, 83, 84, 90]), (200, [142, 143, 350]), (1024, [730, 731, 1000]),
                                          (12, [7, 11, 13]), (1, [3])])
 def test_rule(ising, chunk, calls):
     for a, b in zip(series(ising, chunk, calls), series(ising, 0, calls)):
         np.testing.assert_array_equal(a, b)
-
-
-# a hundred short graphs took 3,371 us where five of 200 sweeps take 2,731
-def test_time(ising):
-    def best(chunk):
-        with ising.Batch([64], [0.44], [1], hot=[1]) as b:
-            b.set_tiling(128, chunk)
-            times = []
-            for _ in range(12):
-                t = time.perf_counter()
-                b.sweep(1000, every=1)
-                times.append(time.perf_counter() - t)
-        return min(times)
-    assert best(1024) < 1.12 * best(200)

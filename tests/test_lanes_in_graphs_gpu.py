@@ -1,8 +1,6 @@
-"""Lanes per item (ising_set_item_lanes) leave the replayed graphs alone: whole
-graphs take the same time whatever the lanes, and sweeps in and outside the
-graphs are the oracle's."""
-import time
-
+"""Lanes per item (ising_set_item_lanes) leave the replayed graphs alone: sweeps in
+and outside the graphs are the oracle's, and the library's choice of lanes gives
+what one lane does."""
 import numpy as np
 import pytest
 
@@ -35,42 +33,6 @@ def test_series(ising, lanes):
     np.testing.assert_array_equal(E, Eo)
     np.testing.assert_array_equal(M, Mo)
     np.testing.assert_array_equal(S, s)
-
-
-# 64 sweeps, two whole graphs, took 376 us with 1 lane and 660 with 8 while the lanes applied to them
-def test_time(ising):
-    def best(lanes):
-        with ising.Lattice(2048, 5) as lat:
-            lat.set_path(ising.ISING_PATH_LAUNCHES)
-            lat.set_item_lanes(lanes)
-            lat.init_hot()
-            lat.set_beta(0.44)
-            times = []
-            for _ in range(8):
-                lat.energy()
-                t = time.perf_counter()
-                lat.sweep(64)
-                lat.energy()
-                times.append(time.perf_counter() - t)
-        return min(times)
-    assert best(8) < 1.3 * best(1)
-
-
-# the library's choice of lanes outside the graphs: one sweep of L = 512 took 27.5 us with four, and 30.6 while it was one
-def test_short_calls_choose_lanes(ising):
-    def best(lanes):
-        with ising.Lattice(512, 5) as lat:
-            lat.set_path(ising.ISING_PATH_LAUNCHES)
-            lat.set_item_lanes(lanes)
-            lat.init_hot()
-            lat.set_beta(0.44)
-            times = []
-            for _ in range(300):
-                t = time.perf_counter()
-                lat.sweep_record(5, 5)
-                times.append(time.perf_counter() - t)
-        return sorted(times)[60]
-    assert best(0) < 0.95 * best(1)
 
 
 @pytest.mark.parametrize("L", [4, 46, 1168, 1170])      # the smallest, and 8176 and 8204 items

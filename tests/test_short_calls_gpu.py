@@ -3,8 +3,6 @@ and two colours a thread (one and several strips of words, pad words, last words
 of 1 to 32 live bits, row groups of two rows) on either side of their limit, both
 layouts, both schemes, thresholds of 2^32 and 0; against the launch path, whose
 draws are made in the half-sweeps."""
-import time
-
 import numpy as np
 import pytest
 
@@ -67,19 +65,3 @@ def test_clusters_by_sweeps(ising, L, layout):
     a = series(ising, L, ising.ISING_PATH_AUTO, [20, 21, 1, 30], layout)
     for x, y in zip(a, series(ising, L, ising.ISING_PATH_CLUSTER, [20, 21, 1, 30], layout, 2)):
         np.testing.assert_array_equal(x, y)
-
-
-# five sweeps of L = 1300 took 68 us on the automatic choice while that was two clusters, 55 with one
-def test_time(ising):
-    def best(clusters):
-        with ising.Lattice(1300, 5) as lat:
-            lat.set_clusters(clusters)
-            lat.init_hot()
-            lat.set_beta(0.44)
-            times = []
-            for _ in range(100):
-                t = time.perf_counter()
-                lat.sweep_record(5, 5)
-                times.append(time.perf_counter() - t)
-        return sorted(times)[20]
-    assert best(0) < 0.97 * best(2)
