@@ -1033,9 +1033,10 @@ extern "C" int ising_sweep(ising_lattice* h, int64_t n)
 {
     TraceRange trace("ising_sweep");
     if (!h || n < 0) return ISING_EINVAL;
-    // the one call that sweeps without waiting for the stream, so the one that can be captured
+    // the one call that sweeps without waiting for the stream, so the one that can be captured (on any stream but
+    // the legacy one)
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(h->stream, &cs) != cudaSuccess) {
+    if (h->stream && cudaStreamIsCapturing(h->stream, &cs) != cudaSuccess) {
         cudaGetLastError();
         cs = cudaStreamCaptureStatusActive;
     }
